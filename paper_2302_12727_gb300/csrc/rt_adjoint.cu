@@ -14,61 +14,274 @@
 // The fix-up E <- max(E, 0) is treated as inactive.
 //
 // The forward pass keeps the state every ckpt_every steps; the reverse pass recomputes each
-// segment with the forward kernels (bitwise the same states) and walks it backwards.  Pair
-// terms are evaluated by both particles in the pair's canonical orientation (k < l), each
-// keeping its own side, so the reductions are per particle, fixed-order and atomic-free.
+// segment with the forward kernels (bitwise the same states) and walks it backwards.  Each
+// pair's terms are evaluated once, in its canonical orientation (k < l), into slots that its
+// two particles then sum, so the reductions are per particle, fixed-order and atomic-free.
 #include "rt_pair.cuh"
 
 namespace rt {
 
 static inline unsigned nblk_(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
-// J(u)^T pb for the M1 flux contracted with A (m1_dot_): u = (E, F), pb = dL/d(flux).
-// Derivatives of (F.A, c^2 E [a(u) A + b(u) u/|F|^2 (F.A) F]) with u = min(|F|^2/(cE)^2, 1),
-// a = (1 - chi)/2, b = (3 chi - 1)/(2u), both functions of s = sqrt(4 - 3u).
+// J(U)^T pb for the M1 flux contracted with A (m1_terms): U = (E, F), pb = dL/d(flux).  With
+// e = cE, f = F/e, u = f.f, s = sqrt(4 - 3u) and g = 3/(2 + s) the flux rows are
+// Pi = c e (a A + g (f.A) f), a = (s - 1)/3, and a' = -1/(2s), g' = g^2/(2s), so
+//   d(p.Pi)/de = c [(a + u/s) p.A - (g + u g^2/s) (f.A)(p.f)]
+//   d(p.Pi)/dF = c [(g^2 (f.A)(p.f) - p.A)/s f + g ((p.f) A + (f.A) p)];
+// where |f| > 1 is clipped, Pi = c e (f.A) f / u.  f keeps every term scale-free.
 template <class T>
 __device__ __forceinline__ void m1_vjp(const T u4[4], T Ax, T Ay, T Az, T c, const T pb[4], T ub[4]) {
-    const T E = u4[0], Fx = u4[1], Fy = u4[2], Fz = u4[3];
     ub[0] = T(0);
     ub[1] = pb[0] * Ax;
     ub[2] = pb[0] * Ay;
     ub[3] = pb[0] * Az;
-    if (!(E > T(0))) return;
-    const T FA = Fx * Ax + Fy * Ay + Fz * Az;
-    const T phA = pb[1] * Ax + pb[2] * Ay + pb[3] * Az;
-    const T phF = pb[1] * Fx + pb[2] * Fy + pb[3] * Fz;
-    const T F2 = Fx * Fx + Fy * Fy + Fz * Fz;
-    const T c2 = c * c;
-    const T u = F2 / (c2 * E * E);
+    const T e = c * u4[0];
+    if (!(e > tiny_<T>())) return;
+    const T ie = rcp_fast(e);
+    const T fx = u4[1] * ie, fy = u4[2] * ie, fz = u4[3] * ie;
+    const T fA = fx * Ax + fy * Ay + fz * Az;
+    const T pA = pb[1] * Ax + pb[2] * Ay + pb[3] * Az;
+    const T pf = pb[1] * fx + pb[2] * fy + pb[3] * fz;
+    const T u = fx * fx + fy * fy + fz * fz;
+    T ce, cf, cg;   // d/de, and the coefficients of f and of (p.f) A + (f.A) p
     if (u > T(1)) {
-        // clamped: flux = c^2 E (F.A) F / |F|^2
-        const T iF2 = T(1) / F2;
-        ub[0] += c2 * FA * phF * iF2;
-        const T k1 = c2 * E * iF2;
-        const T k2 = T(2) * c2 * E * FA * phF * iF2 * iF2;
-        ub[1] += k1 * (phF * Ax + FA * pb[1]) - k2 * Fx;
-        ub[2] += k1 * (phF * Ay + FA * pb[2]) - k2 * Fy;
-        ub[3] += k1 * (phF * Az + FA * pb[3]) - k2 * Fz;
-        return;
+        cg = rcp_fast(u);
+        ce = cg * fA * pf;
+        cf = T(-2) * cg * ce;
+    } else {
+        T is;
+        const T s = sqrt_fast(fma_rn(T(-3), u, T(4)), is);
+        cg = T(3) * rcp_fast(T(2) + s);
+        const T h = cg * fA * pf;             // g (f.A)(p.f)
+        const T k = cg * h - pA;
+        ce = (s - T(1)) * T(1.0 / 3.0) * pA - h - u * is * k;
+        cf = is * k;
     }
-    const T s = sqrt(T(4) - T(3) * u);
-    const T sp = T(-1.5) / s;                      // ds/du
-    const T q5 = T(5) + T(2) * s, q4 = T(4) + T(2) * s;
-    const T a = (T(1) + s - T(2) * u) / q5;
-    const T ap = ((sp - T(2)) * q5 - (T(1) + s - T(2) * u) * T(2) * sp) / (q5 * q5);
-    const T b = T(6) * (T(1) + T(1) / q4) / q5;
-    const T bp = T(6) * ((T(-2) * sp / (q4 * q4)) * q5 - (T(1) + T(1) / q4) * T(2) * sp) / (q5 * q5);
-    const T iE = T(1) / E;
-    ub[0] += c2 * (a - T(2) * u * ap) * phA - (T(2) * u * bp + b) * FA * phF * iE * iE;
-    const T cf = T(2) * ap * iE * phA + T(2) * bp * FA * phF * iE * iE * iE / c2;
-    const T bE = b * iE;
-    ub[1] += cf * Fx + bE * (phF * Ax + FA * pb[1]);
-    ub[2] += cf * Fy + bE * (phF * Ay + FA * pb[2]);
-    ub[3] += cf * Fz + bE * (phF * Az + FA * pb[3]);
+    cg *= c;
+    cf *= c;
+    ub[0] = c * (c * ce);
+    ub[1] += cf * fx + cg * (pf * Ax + fA * pb[1]);
+    ub[2] += cf * fy + cg * (pf * Ay + fA * pb[2]);
+    ub[3] += cf * fz + cg * (pf * Az + fA * pb[3]);
 }
 
-// adjoint of the flux stage for group g0 + g of a group chunk of GC: one thread per (particle i,
-// group), over i's whole row; the pair geometry is recomputed by each group's thread
+// which particle's slope the limiter chose: 1 for k, 2 for l, 0 for none (opposite signs or a
+// zero slope); equal slopes count as l's, as in minmod_
+template <class T>
+__device__ __forceinline__ int slope_of(T dqk, T dql, T s) {
+    return s == T(0) ? 0 : (fabs(dqk) < fabs(dql) ? 1 : 2);
+}
+
+// sink factor of particle p over one step
+template <class T>
+__device__ __forceinline__ T grey_sink(const FluxExtra<T>& x, int64_t p, T dt) {
+    return x.alpha ? fmax_(T(1) - x.c * x.alpha[p] * dt, T(0)) : T(1);
+}
+
+// mu_i = -dt omega_i sink_i lambda_i for every component: the derivative of the loss with
+// respect to the flux sum of particle i
+template <class T>
+__global__ void __launch_bounds__(256) k_adj_mu(PairArgs<T> a, FluxExtra<T> x, const T* __restrict__ lam,
+                                                T* __restrict__ mu) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = t / a.G;
+    if (i >= a.n) return;
+    const T dt = (T)(*x.dt_dev);
+    const T f = -dt * a.omega[i], sk = grey_sink(x, i, dt);
+    T l[4];
+    vload<4>(lam + 4 * t, l);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) l[q] = f * (l[q] * sk);
+    vstore<4>(mu + 4 * t, l);
+}
+
+// Adjoint of the flux of each unordered pair, once, by one thread, for the groups [g0, g0 + GC):
+// the slot gets dL/dQ_k through the left state, dL/dQ_l through the right state and dL/ds of
+// the slope (12 values a group), sel the particle whose slope each component took (2 bits
+// each).  Evaluating the pair for each of its particles, as a kernel over rows does, costs
+// twice the double instructions that bound it: 4.26 ms a step in double on 32,768 particles and
+// two groups, against 0.53 ms for this pass and its gather.
+template <class T, int GC>
+__global__ void __launch_bounds__(128) k_adj_pair(PairArgs<T> a, T c, const T* __restrict__ mu,
+                                                  const T* __restrict__ W, T* __restrict__ slots,
+                                                  uint8_t* __restrict__ sel, int g0) {
+    const int64_t slot = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (slot >= a.n_pairs) return;
+    const int G = a.G, RS = 4 * G;
+    const int2 kl = a.ends[slot];
+    const int64_t i = kl.x, j = kl.y;
+    PairGeo<T> p;
+    T sk, sl;
+    load_pair_geo(a, slot, i, j, c, p, sk, sl);
+    const T wl = T(1) - p.wk;
+#pragma unroll
+    for (int g = 0; g < GC; ++g) {
+        const int gg = g0 + g;
+        T uk[4], ul[4], gk[12], gl[12], mk[4], ml[4], L[4], R[4];
+        vload<4>(W + i * RS + 4 * gg, uk);
+        vload<4>(W + j * RS + 4 * gg, ul);
+        vload<12>(a.grad + i * 12 * G + 12 * gg, gk);
+        vload<12>(a.grad + j * 12 * G + 12 * gg, gl);
+        vload<4>(mu + i * RS + 4 * gg, mk);
+        vload<4>(mu + j * RS + 4 * gg, ml);
+        unsigned code = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const T dqk = gk[3 * q] * p.dx + gk[3 * q + 1] * p.dy + gk[3 * q + 2] * p.dz;
+            const T dql = gl[3 * q] * p.dx + gl[3 * q + 1] * p.dy + gl[3 * q + 2] * p.dz;
+            const T s = minmod_(dqk, dql);
+            code |= (unsigned)slope_of(dqk, dql, s) << (2 * q);
+            L[q] = fma_rn(p.wk, s, uk[q]);
+            R[q] = fma_rn(-wl, s, ul[q]);
+            mk[q] -= ml[q];
+        }
+        // half the surface: the central flux is the mean of the two states' fluxes
+        T jL[4], jR[4], sb[4];
+        m1_vjp(L, p.hx, p.hy, p.hz, c, mk, jL);
+        m1_vjp(R, p.hx, p.hy, p.hz, c, mk, jR);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            jL[q] += p.diss * mk[q];
+            jR[q] -= p.diss * mk[q];
+            sb[q] = p.wk * jL[q] - wl * jR[q];
+        }
+        T* o = slots + (slot * GC + g) * 12;
+        vstore<4>(o, jL);
+        vstore<4>(o + 4, jR);
+        vstore<4>(o + 8, sb);
+        sel[slot * GC + g] = (uint8_t)code;
+    }
+}
+
+// d = x_l - x_k of a slot: kept, or from the two positions
+template <class T>
+__device__ __forceinline__ void pair_sep(const PairArgs<T>& a, int64_t slot, int64_t k, int64_t l, T& dx, T& dy, T& dz) {
+    if constexpr (std::is_same<T, double>::value) {
+        if (a.pg) {
+            const double* p = reinterpret_cast<const double*>(a.pg + slot);
+            const double2 v = *reinterpret_cast<const double2*>(p);
+            dx = v.x;
+            dy = v.y;
+            dz = p[2];
+            return;
+        }
+    }
+    const T* tag = nullptr;
+    sep(a.sp, load_pos(tag, a.pos, k), load_pos(tag, a.pos, l), dx, dy, dz);
+}
+
+// Particle i's share of its slots, one thread per (particle, group): Ubar through its own
+// states, gbar = sum of dL/ds d over the slots whose slope it gave, gamma = omega Bp gbar
+template <class T, int GC>
+__global__ void __launch_bounds__(128) k_adj_gather(PairArgs<T> a, FluxExtra<T> x, const T* __restrict__ lam,
+                                                    const T* __restrict__ slots, const uint8_t* __restrict__ sel,
+                                                    T* __restrict__ ubar, T* __restrict__ gam, int g0) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = t / GC;
+    if (i >= a.n) return;
+    const int g = (int)(t - i * GC), gg = g0 + g;
+    const int G = a.G, RS = 4 * G;
+    T ub[4], gb[4][3];
+    vload<4>(lam + i * RS + 4 * gg, ub);
+    const T sk = grey_sink(x, i, (T)(*x.dt_dev));
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        ub[q] *= sk;
+        gb[q][0] = gb[q][1] = gb[q][2] = T(0);
+    }
+    auto add = [&](int64_t slot, int64_t k, int64_t l, int side) {
+        T v[4], sb[4], dx, dy, dz;
+        const T* o = slots + (slot * GC + g) * 12;
+        vload<4>(o + 4 * (side - 1), v);
+        vload<4>(o + 8, sb);
+        const unsigned code = sel[slot * GC + g];
+        pair_sep(a, slot, k, l, dx, dy, dz);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            ub[q] += v[q];
+            const T b = ((code >> (2 * q)) & 3u) == (unsigned)side ? sb[q] : T(0);
+            gb[q][0] += b * dx;
+            gb[q][1] += b * dy;
+            gb[q][2] += b * dz;
+        }
+    };
+    const int64_t r0 = a.row_off[i], s0 = a.up_off[i], s1 = a.up_off[i + 1];
+    const int nl = a.n_low[i];
+    const int32_t* ls = a.low_slot + (r0 - s0);
+#pragma unroll 2
+    for (int e = 0; e < nl; ++e) add(ls[e], a.cols[r0 + e], i, 2);
+#pragma unroll 2
+    for (int64_t s = s0; s < s1; ++s) add(s, i, a.cols[r0 + nl + (s - s0)], 1);
+    vstore<4>(ubar + i * RS + 4 * gg, ub);
+    // gamma_i = omega_i Bp_i gbar_i (the gradient is omega_i Bp_i sum_j (Q_j - Q_i) w d, Bp symmetric)
+    T Mi[6], out[12];
+    const T om = a.omega[i];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) Mi[k] = om * a.geo[8 * i + 2 + k];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sym_mv(Mi, gb[q][0], gb[q][1], gb[q][2], out[3 * q], out[3 * q + 1], out[3 * q + 2]);
+    vstore<12>(gam + i * 12 * G + 12 * gg, out);
+}
+
+// Transpose of the gradient operator by pairs: v = d . (gamma_k w(r/H_k) + gamma_l w(r/H_l)) is
+// what lambda_k loses and lambda_l gains; the gather below sums the slots in row order
+template <class T, int GC>
+__global__ void __launch_bounds__(128) k_adj_grad_pair(PairArgs<T> a, T c, const T* __restrict__ gam,
+                                                       T* __restrict__ pairbuf, int g0) {
+    const int64_t slot = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (slot >= a.n_pairs) return;
+    const int G = a.G;
+    const int2 kl = a.ends[slot];
+    PairGeo<T> p;
+    T sk, sl;
+    load_pair_geo(a, slot, kl.x, kl.y, c, p, sk, sl);
+    const T kx = sk * p.dx, ky = sk * p.dy, kz = sk * p.dz, lx = sl * p.dx, ly = sl * p.dy, lz = sl * p.dz;
+#pragma unroll
+    for (int g = 0; g < GC; ++g) {
+        T gk[12], gl[12], v[4];
+        vload<12>(gam + (int64_t)kl.x * 12 * G + 12 * (g0 + g), gk);
+        vload<12>(gam + (int64_t)kl.y * 12 * G + 12 * (g0 + g), gl);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            v[q] = gk[3 * q] * kx + gk[3 * q + 1] * ky + gk[3 * q + 2] * kz + gl[3 * q] * lx + gl[3 * q + 1] * ly +
+                   gl[3 * q + 2] * lz;
+        vstore<4>(pairbuf + (slot * GC + g) * 4, v);
+    }
+}
+
+template <class T, int GC>
+__global__ void __launch_bounds__(128) k_adj_grad_gather(PairArgs<T> a, const T* __restrict__ ubar,
+                                                         const T* __restrict__ pairbuf, T* __restrict__ lam_out,
+                                                         int g0) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = t / GC;
+    if (i >= a.n) return;
+    const int g = (int)(t - i * GC);
+    const int64_t o = i * 4 * a.G + 4 * (g0 + g);
+    T acc[4], v[4];
+    vload<4>(ubar + o, acc);
+    const T* pb = pairbuf + 4 * g;
+    const int64_t s0 = a.up_off[i], s1 = a.up_off[i + 1];
+    const int nl = a.n_low[i];
+    const int32_t* ls = a.low_slot + (a.row_off[i] - s0);
+#pragma unroll 4
+    for (int e = 0; e < nl; ++e) {
+        vload<4>(pb + (int64_t)ls[e] * 4 * GC, v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] += v[q];
+    }
+#pragma unroll 4
+    for (int64_t s = s0; s < s1; ++s) {
+        vload<4>(pb + s * 4 * GC, v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] -= v[q];
+    }
+    vstore<4>(lam_out + o, acc);
+}
+
+// The same two stages without per-pair slots, for sets whose slots device memory does not hold
+// (run_adjoint): one thread per (particle i, group) over i's whole row, every pair evaluated by
+// both of its particles.
 template <class T, int GC>
 __global__ void __launch_bounds__(128) k_adj_flux(PairArgs<T> a, FluxExtra<T> x, const T* __restrict__ lam,
                                                   const T* __restrict__ W, T* __restrict__ ubar, T* __restrict__ gam,
@@ -80,12 +293,7 @@ __global__ void __launch_bounds__(128) k_adj_flux(PairArgs<T> a, FluxExtra<T> x,
     const T* tag = nullptr;
     const int G = a.G, RS = 4 * G;
     const T dt = (T)(*x.dt_dev);
-    auto sink_of = [&](int64_t p) {
-        T sk = T(1);
-        if (x.alpha) sk = fmax_(T(1) - x.c * x.alpha[p] * dt, T(0));
-        return sk;
-    };
-    const T sink_i = sink_of(i), om_i = a.omega[i];
+    const T sink_i = grey_sink(x, i, dt), om_i = a.omega[i];
     T li[4], mui[4], ub[4], gb[4][3];
     vload<4>(lam + i * RS + 4 * gg, li);
 #pragma unroll
@@ -111,18 +319,12 @@ __global__ void __launch_bounds__(128) k_adj_flux(PairArgs<T> a, FluxExtra<T> x,
         T dx, dy, dz;
         if (ik) sep(a.sp, pi, pj, dx, dy, dz);
         else sep(a.sp, pj, pi, dx, dy, dz);       // d = x_l - x_k
-        T r = sqrt_(dx * dx + dy * dy + dz * dz);
-        T sk = spline_w_(r * gk8[0]), sl = spline_w_(r * gl8[0]);
-        T M[6];
-#pragma unroll
-        for (int q = 0; q < 6; ++q) M[q] = gk8[2 + q] * sk + gl8[2 + q] * sl;
-        T Ax, Ay, Az;
-        sym_mv(M, dx, dy, dz, Ax, Ay, Az);
-        const T diss = T(0.5) * x.c * sqrt_(Ax * Ax + Ay * Ay + Az * Az);
-        const T ih = rcp_(gk8[1] + gl8[1]);
-        const T wk = gk8[1] * ih, wl = gl8[1] * ih;
+        PairGeo<T> p;
+        T sk, sl;
+        pair_geo(dx, dy, dz, gk8, gl8, x.c, p, sk, sl);
+        const T wk = p.wk, wl = T(1) - p.wk;
         // mu of the other particle
-        const T sink_j = sink_of(j), om_j = a.omega[j];
+        const T sink_j = grey_sink(x, j, dt), om_j = a.omega[j];
         T lj[4], uj[4], grj[12];
         vload<4>(lam + j * RS + 4 * gg, lj);
         vload<4>(W + j * RS + 4 * gg, uj);
@@ -138,8 +340,7 @@ __global__ void __launch_bounds__(128) k_adj_flux(PairArgs<T> a, FluxExtra<T> x,
             T dqk = gk[3 * q] * dx + gk[3 * q + 1] * dy + gk[3 * q + 2] * dz;
             T dql = gl[3 * q] * dx + gl[3 * q + 1] * dy + gl[3 * q + 2] * dz;
             s[q] = minmod_(dqk, dql);
-            bool pos = dqk > T(0) && dql > T(0), neg = dqk < T(0) && dql < T(0);
-            sel[q] = (pos || neg) ? (((pos && dqk < dql) || (neg && dqk > dql)) ? 1 : 2) : 0;
+            sel[q] = slope_of(dqk, dql, s[q]);
             L[q] = fma_rn(wk, s[q], uk[q]);
             R[q] = fma_rn(-wl, s[q], ul[q]);
         }
@@ -152,12 +353,12 @@ __global__ void __launch_bounds__(128) k_adj_flux(PairArgs<T> a, FluxExtra<T> x,
             pb[q] = muk - mul;
         }
         T jL[4], jR[4];
-        m1_vjp(L, Ax, Ay, Az, x.c, pb, jL);
-        m1_vjp(R, Ax, Ay, Az, x.c, pb, jR);
+        m1_vjp(L, p.hx, p.hy, p.hz, x.c, pb, jL);   // half the surface: the mean of the fluxes
+        m1_vjp(R, p.hx, p.hy, p.hz, x.c, pb, jR);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const T Lb = T(0.5) * jL[q] + diss * pb[q];
-            const T Rb = T(0.5) * jR[q] - diss * pb[q];
+            const T Lb = jL[q] + p.diss * pb[q];
+            const T Rb = jR[q] - p.diss * pb[q];
             const T sb = wk * Lb - wl * Rb;
             ub[q] += ik ? Lb : Rb;
             const bool mine = ik ? (sel[q] == 1) : (sel[q] == 2);
@@ -260,6 +461,33 @@ static void launch_adj_step(rt_ctx* c, cudaStream_t s, const T* lamN, const T* W
     x.clamp = 0;
     x.clamp_count = nullptr;
     const int G = c->cfg.n_groups;
+    if (c->adj_slots.p) {
+        T* mu = c->adj_x.as<T>();      // free between the forward steps
+        T* slots = c->adj_slots.as<T>();
+        uint8_t* sel = c->adj_sel.as<uint8_t>();
+        T* pb = c->pairbuf.as<T>();
+        const unsigned nbp = nblk_(std::max<int64_t>(a.n_pairs, 1), 128);
+        k_adj_mu<T><<<nblk_(c->n * G, 256), 256, 0, s>>>(a, x, lamN, mu);
+        ++c->launches;
+        for (int g0 = 0; g0 < G; g0 += kMaxGC) {
+            const int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+            const unsigned nbg = nblk_(c->n * gc, 128);
+#define RT_ADJ_PAIRS(GC_)                                                                      \
+    k_adj_pair<T, GC_><<<nbp, 128, 0, s>>>(a, x.c, mu, W, slots, sel, g0);                      \
+    k_adj_gather<T, GC_><<<nbg, 128, 0, s>>>(a, x, lamN, slots, sel, ub, gam, g0);             \
+    k_adj_grad_pair<T, GC_><<<nbp, 128, 0, s>>>(a, x.c, gam, pb, g0);                           \
+    k_adj_grad_gather<T, GC_><<<nbg, 128, 0, s>>>(a, ub, pb, lamO, g0);
+            switch (gc) {
+                case 1: RT_ADJ_PAIRS(1) break;
+                case 2: RT_ADJ_PAIRS(2) break;
+                case 3: RT_ADJ_PAIRS(3) break;
+                default: RT_ADJ_PAIRS(4) break;
+            }
+#undef RT_ADJ_PAIRS
+            c->launches += 4;
+        }
+        return;
+    }
     for (int g0 = 0; g0 < G; g0 += kMaxGC) {
         int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
         const unsigned nbg = nblk_(c->n * gc, 128);
@@ -299,15 +527,31 @@ rt_status run_adjoint(rt_ctx* c, int n_sub, int k, bool has_src, bool has_alpha,
     RT_TRY(ensure(c, c->adj_ub, S, "adjoint"));
     RT_TRY(ensure(c, c->adj_gam, 3 * S, "adjoint"));
     RT_TRY(ensure(c, c->adj_lam, S, "adjoint"));
+    // slots of 12 values and a code byte per pair and group of a chunk, where they take no more
+    // than half of the memory that is free
+    const size_t pg = (size_t)std::max<int64_t>(c->n_directed / 2, 1) * (G < kMaxGC ? G : kMaxGC);
+    if (c->adj_slots.bytes < pg * 12 * ts || c->adj_sel.bytes < pg) {
+        size_t free_b = 0, total_b = 0;
+        free_buf(c->adj_slots);
+        free_buf(c->adj_sel);
+        RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+        if (pg * (12 * ts + 1) <= free_b / 2) {
+            RT_TRY(ensure(c, c->adj_slots, pg * 12 * ts, "adjoint slots"));
+            RT_TRY(ensure(c, c->adj_sel, pg, "adjoint slots"));
+        }
+    }
     char* ck = c->ck.as<char>();
     char* seg = c->seg.as<char>();
     void* X = c->adj_x.p;
     void* W = c->adj_w.p;
 
     // forward pass with a checkpoint every k steps
+    const int n_last = (nck - 1) * k;
     RT_CUDA(c, cudaMemcpyAsync(X, U0s, S, cudaMemcpyDeviceToDevice, st));
     for (int t = 0; t < n_sub; ++t) {
         if (t % k == 0) RT_CUDA(c, cudaMemcpyAsync(ck + (size_t)(t / k) * S, X, S, cudaMemcpyDeviceToDevice, st));
+        // the last segment, the first to be walked back, is kept whole as it passes
+        if (t > n_last) RT_CUDA(c, cudaMemcpyAsync(seg + (size_t)(t - n_last) * S, X, S, cudaMemcpyDeviceToDevice, st));
         if (t == n_sub - 1) break;      // the final state is not needed
         RT_TRY(launch_step(c, st, X, W, has_src, has_alpha));
         std::swap(X, W);
@@ -320,7 +564,7 @@ rt_status run_adjoint(rt_ctx* c, int n_sub, int k, bool has_src, bool has_alpha,
         const int n0 = m * k;
         const int len = (n_sub - n0) < k ? (n_sub - n0) : k;
         RT_CUDA(c, cudaMemcpyAsync(seg, ck + (size_t)m * S, S, cudaMemcpyDeviceToDevice, st));
-        for (int t = 0; t + 1 < len; ++t) {
+        for (int t = 0; t + 1 < len && m < nck - 1; ++t) {
             RT_CUDA(c, cudaMemcpyAsync(c->adj_x.p, seg + (size_t)t * S, S, cudaMemcpyDeviceToDevice, st));
             RT_TRY(launch_step(c, st, c->adj_x.p, seg + (size_t)(t + 1) * S, has_src, has_alpha));
         }

@@ -40,7 +40,7 @@ rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what) {
     return RT_OK;
 }
 
-static void free_buf(DevBuf& b) {
+void free_buf(DevBuf& b) {
     if (b.p) cudaFree(b.p);
     b.p = nullptr;
     b.bytes = 0;
@@ -120,6 +120,26 @@ static rt_status ensure_state(rt_ctx* c) {
     // per-pair flux slots of one group chunk (at most 4 groups)
     const int gc = G < kMaxGC ? G : kMaxGC;
     RT_TRY(ensure(c, c->pairbuf, (size_t)std::max<int64_t>(c->n_directed / 2, 1) * 4 * gc * tsize(c), "pair fluxes"));
+    // double path: the kept pair geometry (80 bytes a pair and 24 an entry), where it takes no
+    // more than a quarter of the memory that is free; without it the kernels compute it
+    if (c->fp64) {
+        c->pair_geo_ready = false;
+        const size_t P = (size_t)std::max<int64_t>(c->n_directed / 2, 1);
+        const size_t need = P * (64 + 16 + 48), have = c->pair_geo.bytes + c->pair_w.bytes + c->row_wd.bytes;
+        size_t free_b = 0, total_b = 0;
+        const bool fits = P * 64 <= c->pair_geo.bytes && P * 16 <= c->pair_w.bytes && P * 48 <= c->row_wd.bytes;
+        if (!fits) RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
+        if (fits || need <= (free_b + have) / 4) {
+            RT_TRY(ensure(c, c->pair_geo, P * 64, "pair geometry"));
+            RT_TRY(ensure(c, c->pair_w, P * 16, "pair geometry"));
+            RT_TRY(ensure(c, c->row_wd, P * 48, "pair geometry"));
+        } else {
+            free_buf(c->pair_geo);
+            free_buf(c->pair_w);
+            free_buf(c->row_wd);
+            ++g_generation;
+        }
+    }
     if (!c->fp64 && G <= kMaxGC)
         RT_TRY(ensure(c, c->frec, (size_t)(12 + 16 * G + kRowRot) * n * 4, "packed flux rows"));
     return RT_OK;
@@ -283,6 +303,7 @@ rt_status rt_gradients(rt_ctx* c, const void* U, void* gradU) {
     RT_TRY(check_ready(c));
     if (!U || !gradU) return fail(c, RT_ERR_INVALID, "NULL array");
     const int G = c->cfg.n_groups;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(launch_gradient(c, c->stream, c->U_a.p));
     RT_TRY(state_out(c, c->grad_t.p, gradU, 12 * G, 12 * G, 0));
@@ -295,6 +316,7 @@ rt_status rt_step_bins(rt_ctx* c, void* U, const double* Lsrc, const double* alp
     if (!c->has_bins) return fail(c, RT_ERR_STATE, "rt_set_time_bins has not been called since rt_neighbours");
     const int G = c->cfg.n_groups;
     const bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(set_step_inputs(c, c->dt_min, Lsrc, alpha));
     RT_CUDA(c, cudaMemsetAsync(c->acc_t.p, 0, (size_t)32 * G * c->n, c->stream));   // 32 B per (particle, group)
@@ -309,6 +331,7 @@ rt_status rt_drift(rt_ctx* c, void* U, const double* v, double dt_drift) {
     if (!U || !v) return fail(c, RT_ERR_INVALID, "NULL array");
     if (!std::isfinite(dt_drift)) return fail(c, RT_ERR_INVALID, "dt_drift must be finite");
     const int G = c->cfg.n_groups;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(launch_gradient(c, c->stream, c->U_a.p));
     RT_TRY(launch_drift(c, c->stream, c->U_a.p, v, dt_drift));
@@ -322,6 +345,7 @@ rt_status rt_transport_step(rt_ctx* c, double dt, void* U, const double* Lsrc, c
     if (!std::isfinite(dt) || dt < 0) return fail(c, RT_ERR_INVALID, "dt must be finite and >= 0");
     const int G = c->cfg.n_groups;
     bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     if (c->profiling) {
@@ -342,6 +366,7 @@ rt_status rt_transport_step_given_gradients(rt_ctx* c, double dt, void* U, const
     if (!U || !gradU) return fail(c, RT_ERR_INVALID, "U_dev or gradU_dev is NULL");
     if (!std::isfinite(dt) || dt < 0) return fail(c, RT_ERR_INVALID, "dt must be finite and >= 0");
     const int G = c->cfg.n_groups;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(state_in(c, gradU, c->grad_t.p, 12 * G, 12 * G, 0));
     RT_TRY(set_step_inputs(c, dt, nullptr, alpha));
@@ -380,6 +405,7 @@ rt_status rt_subcycle(rt_ctx* c, int32_t n_sub, double dt, void* U, const double
     const int G = c->cfg.n_groups;
     bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
     bool has_alpha = alpha != nullptr;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     // sub-cycles after the first take their injection from the previous gather
@@ -439,6 +465,7 @@ rt_status rt_adjoint(rt_ctx* c, int32_t n_sub, double dt, int32_t ckpt_every, co
     if (!std::isfinite(dt) || dt < 0) return fail(c, RT_ERR_INVALID, "dt must be finite and >= 0");
     const int G = c->cfg.n_groups;
     bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     RT_TRY(ensure(c, c->lam_a, (size_t)4 * G * c->n * tsize(c), "adjoint"));
     RT_TRY(ensure(c, c->lam_b, (size_t)4 * G * c->n * tsize(c), "adjoint"));
@@ -638,6 +665,7 @@ rt_status rt_autotune(rt_ctx* c, const void* U, double dt, int32_t n_sub, const 
     const int G = c->cfg.n_groups;
     const bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
     const bool has_alpha = alpha != nullptr;
+    RT_TRY(prepare_pair_geometry(c));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     const rt_tuning saved = c->tune;
     int best_k = -1;
@@ -725,7 +753,8 @@ void rt_destroy(rt_ctx* c) {
                       &c->sigma_d, &c->bins_s, &c->bins_tmp, &c->acc_t, &c->bins_nmin, &c->order_b, &c->order_m,
                       &c->order_q, &c->bin_keys, &c->bin_keys2, &c->bin_vals, &c->bin_cub, &c->bin_hist, &c->alpha_s,
                       &c->L_dev, &c->dt_dev, &c->energy_part, &c->ck, &c->seg, &c->lam_a, &c->lam_b, &c->adj_w,
-                      &c->adj_x, &c->adj_ub, &c->adj_gam, &c->adj_lam};
+                      &c->adj_x, &c->adj_ub, &c->adj_gam, &c->adj_lam, &c->pair_geo, &c->pair_w, &c->row_wd, &c->adj_slots,
+                      &c->adj_sel};
     for (DevBuf* b : bufs) free_buf(*b);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
     delete c;

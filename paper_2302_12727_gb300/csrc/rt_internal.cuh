@@ -94,6 +94,11 @@ struct rt_ctx {
     rt::DevBuf pkeys, pkeys_alt;                        // (row, col) keys of the sort-based build
     rt::DevBuf n_low, n_up, up_off, low_slot, pair_ends; // lower / upper split, pair slots
     rt::DevBuf pairbuf;                                 // per-pair fluxes of one group chunk
+    // double path: geometry of every pair and weights of every row entry, kept from the first
+    // transport call after a build (empty when device memory is short)
+    rt::DevBuf pair_geo, pair_w, row_wd;
+    bool pair_geo_ready = false;
+    rt::DevBuf adj_slots, adj_sel;                      // adjoint: per-pair values of one group chunk
     // sizes that captured graphs bake in besides buffer addresses (pair count, injection
     // targets and entries): a rebuild that changes them drops the graphs
     std::vector<int64_t> graph_shape;
@@ -158,6 +163,7 @@ namespace rt {
 rt_status fail(rt_ctx* c, rt_status s, const std::string& msg);
 rt_status cuda_fail(rt_ctx* c, cudaError_t e, const char* what);
 rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what);
+void free_buf(DevBuf& b);
 // HLL wave speeds over (f, theta), [RT_WAVE_NF][RT_WAVE_NTH] each (rt_hll.cu)
 void build_wave_table(double* lmax, double* lmin);
 // record a start event before a profiled launch (returns the index, or -1 when off)
@@ -192,6 +198,8 @@ rt_status field_out(rt_ctx* c, const double* src_sorted, double* dst_user, int c
 rt_status set_step_inputs(rt_ctx* c, double dt, const double* Lsrc, const double* alpha);
 // fills inj_dense from the inputs of set_step_inputs (when on and there are targets)
 rt_status set_dense_injection(rt_ctx* c, bool on);
+// double path: computes the kept pair geometry if the buffers are there and it is not valid
+rt_status prepare_pair_geometry(rt_ctx* c);
 // rt_wait_selftest's kernel: *ran_out = the bounded wait on a never-completed barrier ran out
 rt_status wait_selftest(rt_ctx* c, unsigned long long budget, bool* ran_out);
 // one sub-cycle: injection (if inject_first), gradients, pair fluxes, update and sink; with

@@ -3,6 +3,8 @@
 // branch-free form, position / geometry / state record access, and the pair flux.
 #pragma once
 
+#include <type_traits>
+
 #include "rt_internal.cuh"
 
 namespace rt {
@@ -40,9 +42,14 @@ __device__ __forceinline__ T spline_w_(T q) {
 
 // minmod of Eq. rt-minmod (both positive -> min, both negative -> max, else 0) as the median
 // of a, b and 0: max(min(a, b), min(max(a, b), 0)), four min/max and no compare or select
-template <class T>
-__device__ __forceinline__ T minmod_(T a, T b) {
-    return fmax_(fmin_(a, b), fmin_(fmax_(a, b), T(0)));
+__device__ __forceinline__ float minmod_(float a, float b) {
+    return fmax_(fmin_(a, b), fmin_(fmax_(a, b), 0.f));
+}
+// the same in double with one instruction of the double pipe (a compare; the signs are
+// compared as integers) instead of four min/max of a compare each
+__device__ __forceinline__ double minmod_(double a, double b) {
+    const double m = fabs(a) < fabs(b) ? a : b;
+    return (__double2hiint(a) ^ __double2hiint(b)) < 0 ? 0.0 : m;
 }
 
 // smallest normal number: a product or reciprocal below it is flushed by the approximate
@@ -60,33 +67,78 @@ __device__ __forceinline__ float rsqrt_(float x) {
     return y;
 }
 
-// M1 flux of one group contracted with A, in branch-free form (Eq. eddington-group):
-// (F . A, c^2 E [(1 - chi)/2 A + (3 chi - 1)/2 (n . A) n]), n = F/|F|, f = |F|/(cE) clipped
-// to 1.  The factors are bounded for every state: (1 - chi)/2 = (1 + s - 2u)/(5 + 2s) and
-// (3 chi - 1)/2 = 3u/(2 + s) with u = f^2, s = sqrt(4 - 3u), and the direction enters as
-// F/|F|, so no (cE)^-2 can overflow.  cE not a normal number (E <= 0 included) gives zero
-// pressure; F not normal gives the isotropic closure.
+// ------------------------------------------------------------------------------------
+// 1/x and sqrt(x) in double for normal x whose result is normal: the hardware's
+// approximations refined by one third-order step of the error e = 1 - x y (Householder's
+// iteration; the series of 1/(1 - e) and of (1 - e)^(-1/2) cut after e^2), three and five
+// instructions of the double pipe instead of the eight to twenty of the IEEE routines.  The
+// double path's time is that pipe's, which runs at 1/64 of the float rate.
+__device__ __forceinline__ double rcp_fast(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+// sqrt(x), and its reciprocal in `inv`
+__device__ __forceinline__ double sqrt_fast(double x, double& inv) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double t = x * y;
+    const double e = fma(-t, y, 1.0);
+    const double p = e * fma(e, 0.375, 0.5);
+    inv = fma(y, p, y);
+    return fma(t, p, t);
+}
+__device__ __forceinline__ double sqrt_fast(double x) {
+    double inv;
+    return sqrt_fast(x, inv);
+}
+__device__ __forceinline__ float rcp_fast(float x) { return rcp_(x); }
+__device__ __forceinline__ float sqrt_fast(float x) { return sqrt_(x); }
+__device__ __forceinline__ float sqrt_fast(float x, float& inv) {
+    inv = rsqrt_(x);
+    return x * inv;
+}
+
+// max(E, 0) and u = F2 / max(F2, cE^2), iq = 1 / max(F2, cE^2); both zero when that maximum
+// is not a normal number (|F| and cE below the square root of the smallest one: isotropic)
+__device__ __forceinline__ float pos_part(float v) { return fmaxf(v, 0.f); }
+__device__ __forceinline__ double pos_part(double v) { return __double2hiint(v) < 0 ? 0.0 : v; }
+__device__ __forceinline__ void m1_ratio(float F2, float cE, float& u, float& iq) {
+    iq = rcp_(fmaxf(fmaxf(F2, cE * cE), tiny_<float>()));
+    u = fminf(F2 * iq, 1.f);
+}
+__device__ __forceinline__ void m1_ratio(double F2, double cE, double& u, double& iq) {
+    // non-negative doubles compare like integers: no instruction of the double pipe
+    const double c2 = cE * cE;
+    const double q = __double_as_longlong(F2) > __double_as_longlong(c2) ? F2 : c2;
+    const bool ok = (unsigned)__double2hiint(q) - 0x00100000u < 0x7fd00000u - 0x00100000u;
+    const double r = rcp_fast(q);
+    iq = ok ? r : 0.0;
+    u = ok ? F2 * r : 0.0;
+}
+
+// M1 flux of one group contracted with A (Eq. eddington-group): F . A for the energy and
+// P A + t F for the flux, with
+//   P = c^2 E (1 - chi)/2,  t = c^2 E (3 chi - 1)/2 (F . A)/|F|^2.
+// With f = |F|/(cE) clipped to 1, u = f^2 and s = sqrt(4 - 3u), the printed
+// chi = (3 + 4u)/(5 + 2s) is (5 - 2s)/3, because (5 + 2s)(5 - 2s) = 3 (3 + 4u); hence
+// (3 chi - 1)/2 = 2 - s = 3u/(2 + s) and (1 - chi)/2 = (1 - 3u/(2 + s))/3.  The clip is the
+// maximum in q = max(|F|^2, (cE)^2), u = |F|^2/q, and (3 chi - 1)/2 / |F|^2 = 3/((2 + s) q):
+// the direction F/|F| needs no root of its own, and three special functions a state remain
+// of five.  E <= 0 gives zero pressure.
 template <class T>
-__device__ __forceinline__ void m1_dot_(T E, T Fx, T Fy, T Fz, T Ax, T Ay, T Az, T c, T& oE, T& oFx, T& oFy,
-                                        T& oFz) {
-    const T FA = Fx * Ax + Fy * Ay + Fz * Az;
-    oE = FA;
-    const T cE1 = c * E;
-    const bool pos = cE1 > tiny_<T>();
+__device__ __forceinline__ void m1_terms(T E, T Fx, T Fy, T Fz, T Ax, T Ay, T Az, T c, T& FA, T& P, T& t) {
+    FA = Fx * Ax + Fy * Ay + Fz * Az;
+    const T cE = pos_part(c * E);
     const T F2 = Fx * Fx + Fy * Fy + Fz * Fz;
-    const bool dir = F2 > tiny_<T>();
-    const T iFn = rsqrt_(dir ? F2 : T(1));
-    const T icE = rcp_(pos ? cE1 : T(1));
-    const T f = dir ? fmin_(F2 * iFn * icE, T(1)) : T(0);
-    const T u = f * f;
-    const T s = sqrt_(T(4) - T(3) * u);
-    const T a_iso = (T(1) + s - T(2) * u) * rcp_(T(5) + T(2) * s);
-    const T a_dir = T(3) * u * rcp_(T(2) + s);
-    const T cE = pos ? c * cE1 : T(0);
-    const T t = ((a_dir * FA) * iFn) * iFn;
-    oFx = cE * (a_iso * Ax + t * Fx);
-    oFy = cE * (a_iso * Ay + t * Fy);
-    oFz = cE * (a_iso * Az + t * Fz);
+    T u, iq;
+    m1_ratio(F2, cE, u, iq);
+    const T s = sqrt_fast(fma_rn(T(-3), u, T(4)));
+    const T r = T(3) * rcp_fast(T(2) + s);
+    const T cc = c * cE;
+    P = cc * fma_rn(-u * r, T(1.0 / 3.0), T(1.0 / 3.0));
+    t = (cc * (iq * r)) * FA;
 }
 
 // ------------------------------------------------------------------------------------
@@ -215,6 +267,13 @@ __device__ __forceinline__ void vstore(double* p, const double* o) {
     for (int k = 0; k < K; k += 2) *reinterpret_cast<double2*>(p + k) = make_double2(o[k], o[k + 1]);
 }
 
+// Geometry of pair (k, l) as the flux needs it: d = x_l - x_k, half the surface A/2 with
+// A = A_kl (Eq. HopkinsAij), diss = c |A| / 2, wk = h_k / (h_k + h_l)
+template <class T>
+struct PairGeo {
+    T dx, dy, dz, hx, hy, hz, diss, wk;
+};
+
 template <class T>
 struct PairArgs {
     const void* pos;          // uint4[N] or double[4N]
@@ -229,6 +288,10 @@ struct PairArgs {
     const int64_t* up_off;    // first pair slot of each row
     const int32_t* low_slot;  // slot of each lower entry's pair
     const int2* ends;         // (k, l) of each pair slot
+    // double path: the pairs' geometry, computed once per build (prepare_pair_geometry), or null
+    const PairGeo<T>* pg;     // [P]
+    const T* wd;              // [2P][3] per row entry: w(r_ij / H_i) d_ij
+    const T* wkl;             // [P][2] w(r / H_k), w(r / H_l)
     int64_t n_pairs;
     int G;
     // packed flux-input rows [N][kRowRot + RW], RW = 12 + 16G logical words {pos (4), geo
@@ -318,27 +381,80 @@ __device__ __forceinline__ void wave_speeds_(const T* __restrict__ tab, T E, T F
     lmin = c * (w00 * a.y + w10 * b.y + w01 * d.y + w11 * e.y);
 }
 
-// Flux of pair (k, l) for one group, k = this particle as the left state: face states
-// (Eq. rt-riemann-problem with s = minmod(grad Q_k . d, grad Q_l . d)), M1 fluxes
-// (Eq. eddington-group), GLF (Eq. riemann-GLF).  The face states use explicit fma so that
-// the evaluation by l (with -d and the roles swapped) gives exactly -phi.
+// from d and the two particles' geometry records {1/H, h, Bp xx yy zz xy xz yz}:
+// A_kl = (Bp_k w_k + Bp_l w_l) d; also the two spline weights
+template <class T>
+__device__ __forceinline__ void pair_geo(T dx, T dy, T dz, const T gk[8], const T gl[8], T c, PairGeo<T>& p, T& sk,
+                                         T& sl) {
+    const T r = sqrt_(dx * dx + dy * dy + dz * dz);
+    sk = spline_w_(r * gk[0]);
+    sl = spline_w_(r * gl[0]);
+    const T hk = T(0.5) * sk, hl = T(0.5) * sl;
+    T M[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) M[q] = gk[2 + q] * hk + gl[2 + q] * hl;
+    p.dx = dx;
+    p.dy = dy;
+    p.dz = dz;
+    sym_mv(M, dx, dy, dz, p.hx, p.hy, p.hz);
+    p.diss = c * sqrt_(p.hx * p.hx + p.hy * p.hy + p.hz * p.hz);
+    p.wk = gk[1] * rcp_(gk[1] + gl[1]);
+}
+
+// the geometry of slot's pair (i, j): read where it is kept, else computed; sk, sl are the
+// spline weights where the caller uses them
+template <class T>
+__device__ __forceinline__ void load_pair_geo(const PairArgs<T>& a, int64_t slot, int64_t i, int64_t j, T c,
+                                              PairGeo<T>& p, T& sk, T& sl) {
+    if constexpr (std::is_same<T, double>::value) {
+        if (a.pg) {
+            vload<8>(reinterpret_cast<const T*>(a.pg + slot), reinterpret_cast<T*>(&p));
+            sk = a.wkl[2 * slot];
+            sl = a.wkl[2 * slot + 1];
+            return;
+        }
+    }
+    const T* tag = nullptr;
+    const Pos<T> pi = load_pos(tag, a.pos, i), pj = load_pos(tag, a.pos, j);
+    T gi8[8], gj8[8], dx, dy, dz;
+    vload<8>(a.geo + 8 * i, gi8);
+    vload<8>(a.geo + 8 * j, gj8);
+    sep(a.sp, pi, pj, dx, dy, dz);              // d = x_l - x_k
+    pair_geo(dx, dy, dz, gi8, gj8, c, p, sk, sl);
+}
+
+// Flux of pair (k, l) for one group, k as the left state: face states (Eq.
+// rt-riemann-problem with s = minmod(grad Q_k . d, grad Q_l . d)), M1 fluxes (Eq.
+// eddington-group), GLF (Eq. riemann-GLF).  The jump of the dissipation is R - L =
+// (Q_l - Q_k) - s, because the two weights of s add to one: it keeps the digits that the
+// rounded face states lose.  The surface enters halved, so that the central term is a plain
+// sum.
 template <bool HLL, class T>
-__device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T gk[12], const T gl[12], T dx, T dy,
-                                          T dz, T wk, T wl, T Ax, T Ay, T Az, T diss, T c, const T* wave, T An,
-                                          T phi[4]) {
-    T L[4], R[4];
+__device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T gk[12], const T gl[12],
+                                          const PairGeo<T>& p, T c, const T* wave, T phi[4]) {
+    T L[4], R[4], D[4];
+    const T wl = T(1) - p.wk;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        T dqk = gk[3 * q] * dx + gk[3 * q + 1] * dy + gk[3 * q + 2] * dz;
-        T dql = gl[3 * q] * dx + gl[3 * q + 1] * dy + gl[3 * q + 2] * dz;
+        T dqk = gk[3 * q] * p.dx + gk[3 * q + 1] * p.dy + gk[3 * q + 2] * p.dz;
+        T dql = gl[3 * q] * p.dx + gl[3 * q + 1] * p.dy + gl[3 * q + 2] * p.dz;
         T s = minmod_(dqk, dql);
-        L[q] = fma_rn(wk, s, uk[q]);
+        L[q] = fma_rn(p.wk, s, uk[q]);
         R[q] = fma_rn(-wl, s, ul[q]);
+        D[q] = (ul[q] - uk[q]) - s;
     }
-    T fL[4], fR[4];
-    m1_dot_(L[0], L[1], L[2], L[3], Ax, Ay, Az, c, fL[0], fL[1], fL[2], fL[3]);
-    m1_dot_(R[0], R[1], R[2], R[3], Ax, Ay, Az, c, fR[0], fR[1], fR[2], fR[3]);
+    T FL, PL, tL, FR, PR, tR;
     if constexpr (HLL) {
+        const T Ax = T(2) * p.hx, Ay = T(2) * p.hy, Az = T(2) * p.hz;
+        T fL[4], fR[4];
+        m1_terms(L[0], L[1], L[2], L[3], Ax, Ay, Az, c, fL[0], PL, tL);
+        m1_terms(R[0], R[1], R[2], R[3], Ax, Ay, Az, c, fR[0], PR, tR);
+        fL[1] = PL * Ax + tL * L[1];
+        fL[2] = PL * Ay + tL * L[2];
+        fL[3] = PL * Az + tL * L[3];
+        fR[1] = PR * Ax + tR * R[1];
+        fR[2] = PR * Ay + tR * R[2];
+        fR[3] = PR * Az + tR * R[3];
         // HLL (Eq. riemann-HLL): (l+ F_L.A - l- F_R.A + l+ l- |A| (U_R - U_L)) / (l+ - l-),
         // l+ = max(0, lmax_L, lmax_R), l- = min(0, lmin_L, lmin_R); central flux if l+ = l-
         T xL, nL, xR, nR;
@@ -347,18 +463,23 @@ __device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T 
         const T lp = fmax_(T(0), fmax_(xL, xR)), lm = fmin_(T(0), fmin_(nL, nR));
         const T den = lp - lm;
         if (den > T(0)) {
-            const T jm = lp * lm * An;
+            const T jm = lp * lm * (T(2) * p.diss * rcp_(c));
             const T iden = T(1) / den;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) phi[q] = (lp * fL[q] - lm * fR[q] + jm * (R[q] - L[q])) * iden;
+            for (int q = 0; q < 4; ++q) phi[q] = (lp * fL[q] - lm * fR[q] + jm * D[q]) * iden;
         } else {
 #pragma unroll
             for (int q = 0; q < 4; ++q) phi[q] = T(0.5) * (fL[q] + fR[q]);
         }
         return;
     }
-#pragma unroll
-    for (int q = 0; q < 4; ++q) phi[q] = T(0.5) * (fL[q] + fR[q]) - diss * (R[q] - L[q]);
+    m1_terms(L[0], L[1], L[2], L[3], p.hx, p.hy, p.hz, c, FL, PL, tL);
+    m1_terms(R[0], R[1], R[2], R[3], p.hx, p.hy, p.hz, c, FR, PR, tR);
+    const T P = PL + PR;
+    phi[0] = fma_rn(-p.diss, D[0], FL + FR);
+    phi[1] = fma_rn(-p.diss, D[1], P * p.hx + (tL * L[1] + tR * R[1]));
+    phi[2] = fma_rn(-p.diss, D[2], P * p.hy + (tL * L[2] + tR * R[2]));
+    phi[3] = fma_rn(-p.diss, D[3], P * p.hz + (tL * L[3] + tR * R[3]));
 }
 
 // update parameters of the flux stage
@@ -399,6 +520,10 @@ inline PairArgs<T> pair_args(rt_ctx* c) {
     a.up_off = c->up_off.as<int64_t>();
     a.low_slot = c->low_slot.as<int32_t>();
     a.ends = c->pair_ends.as<int2>();
+    const bool kept = std::is_same<T, double>::value && c->pair_geo_ready;
+    a.pg = kept ? static_cast<const PairGeo<T>*>(c->pair_geo.p) : nullptr;
+    a.wd = kept ? c->row_wd.as<T>() : nullptr;
+    a.wkl = kept ? c->pair_w.as<T>() : nullptr;
     a.n_pairs = c->n_directed / 2;
     a.G = c->cfg.n_groups;
     a.frec = nullptr;

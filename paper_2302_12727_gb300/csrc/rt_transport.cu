@@ -229,6 +229,125 @@ __global__ void __launch_bounds__(128) k_gradient(PairArgs<T> a, const T* __rest
     }
 }
 
+// The double path's kept pair geometry (load_pair_geo, k_gradient_wd): one thread per pair slot
+// writes the flux geometry and the two spline weights, one warp per row the entries' w d.
+// The double pipe bounds this path, and every sub-cycle and reverse step of a build shares
+// the geometry, which is a third of the flux kernel's double instructions and three quarters of
+// the gradient's; reading it back costs 64 bytes a pair and 24 an entry.
+__global__ void __launch_bounds__(128) k_pair_geometry(PairArgs<double> a, double c, PairGeo<double>* pg,
+                                                       double* wkl) {
+    const int64_t slot = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (slot >= a.n_pairs) return;
+    const int2 kl = a.ends[slot];
+    PairGeo<double> p;
+    double sk, sl;
+    load_pair_geo(a, slot, kl.x, kl.y, c, p, sk, sl);
+    vstore<8>(reinterpret_cast<double*>(pg + slot), reinterpret_cast<const double*>(&p));
+    *reinterpret_cast<double2*>(wkl + 2 * slot) = make_double2(sk, sl);
+}
+
+__global__ void __launch_bounds__(256) k_row_weights(PairArgs<double> a, double* __restrict__ wd) {
+    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (i >= a.n) return;
+    const double* tag = nullptr;
+    const Pos<double> pi = load_pos(tag, a.pos, i);
+    const double iH = a.geo[8 * i];
+    for (int64_t e = a.row_off[i] + lane; e < a.row_off[i + 1]; e += 32) {
+        const Pos<double> pj = load_pos(tag, a.pos, a.cols[e]);
+        double dx, dy, dz;
+        sep(a.sp, pi, pj, dx, dy, dz);
+        const double w = spline_w_(sqrt_(dx * dx + dy * dy + dz * dz) * iH);
+        wd[3 * e] = w * dx;
+        wd[3 * e + 1] = w * dy;
+        wd[3 * e + 2] = w * dz;
+    }
+}
+
+rt_status prepare_pair_geometry(rt_ctx* c) {
+    if (!c->fp64 || c->pair_geo_ready || !c->pair_geo.p) return RT_OK;
+    const PairArgs<double> a = pair_args<double>(c);   // pair_geo_ready is false: computes
+    k_pair_geometry<<<nblk(std::max<int64_t>(a.n_pairs, 1), 128), 128, 0, c->stream>>>(
+        a, c->cfg.c_red, static_cast<PairGeo<double>*>(c->pair_geo.p), c->pair_w.as<double>());
+    k_row_weights<<<nblk(c->n * 32, 256), 256, 0, c->stream>>>(a, c->row_wd.as<double>());
+    c->launches += 2;
+    RT_CUDA(c, cudaGetLastError());
+    c->pair_geo_ready = true;
+    return RT_OK;
+}
+
+// Double gradient from the kept row weights: 16 double instructions per entry and group are
+// left.  LN lanes share the row of one (particle, group), every LN-th entry each, so that small
+// sets still fill the double pipes of all SMs; at LN = 4 the sums are reduced so that each
+// lane ends with one component and applies B_i to it alone.
+template <int GC, int LN, bool BINS>
+__global__ void __launch_bounds__(128) k_gradient_wd(PairArgs<double> a, const double* __restrict__ rec,
+                                                     double* __restrict__ grad, int g0) {
+    static_assert(LN == 1 || LN == 4, "lanes per (particle, group)");
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int sub = (int)(t % LN);
+    const int64_t q = t / LN;
+    int64_t i = q / GC;
+    const int g = (int)(q - i * GC);
+    const bool act = i < (BINS ? a.count : a.n);
+    i = act ? (BINS ? (int64_t)a.order[i] : i) : 0;
+    const int RS = 4 * a.G, off = 4 * (g0 + g);
+    double ui[4], acc[4][3];
+    vload<4>(rec + i * RS + off, ui);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c][0] = acc[c][1] = acc[c][2] = 0.0;
+    const int64_t e1 = act ? a.row_off[i + 1] : 0;
+#pragma unroll 2
+    for (int64_t e = act ? a.row_off[i] + sub : 0; e < e1; e += LN) {
+        double u[4];
+        vload<4>(rec + (int64_t)a.cols[e] * RS + off, u);
+        const double wx = a.wd[3 * e], wy = a.wd[3 * e + 1], wz = a.wd[3 * e + 2];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const double dq = u[c] - ui[c];
+            acc[c][0] += dq * wx;
+            acc[c][1] += dq * wy;
+            acc[c][2] += dq * wz;
+        }
+    }
+    if constexpr (LN == 4) {
+        const bool hi = sub & 2, odd = sub & 1;
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {   // lanes 0, 1 keep components 0, 1; lanes 2, 3 the others
+                const double give = hi ? acc[c][d] : acc[c + 2][d], keep = hi ? acc[c + 2][d] : acc[c][d];
+                acc[c][d] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
+            }
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const double give = odd ? acc[0][d] : acc[1][d], keep = odd ? acc[1][d] : acc[0][d];
+            acc[0][d] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
+        }
+    }
+    if (!act) return;
+    double M[6];
+    const double om = a.omega[i];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) M[k] = om * a.geo[8 * i + 2 + k];
+    double* out = grad + i * 12 * a.G + 12 * (g0 + g) + 3 * sub;
+#pragma unroll
+    for (int c = 0; c < (LN == 4 ? 1 : 4); ++c)
+        sym_mv(M, acc[c][0], acc[c][1], acc[c][2], out[3 * c], out[3 * c + 1], out[3 * c + 2]);
+}
+
+// lanes per (particle, group) of the double gradient: four up to the size where one lane each
+// gives every SM's four double pipes eight warps
+template <int GC, bool BINS>
+static void launch_gradient_wd(rt_ctx* c, cudaStream_t s, const PairArgs<double>& a, const double* rec, double* grad,
+                               int g0) {
+    const int64_t m = (BINS ? a.count : a.n) * GC;
+    if (c->n * GC < (int64_t)c->sm_count * 1024)
+        k_gradient_wd<GC, 4, BINS><<<nblk(4 * m, 128), 128, 0, s>>>(a, rec, grad, g0);
+    else
+        k_gradient_wd<GC, 1, BINS><<<nblk(m, 128), 128, 0, s>>>(a, rec, grad, g0);
+}
+
 // Float gradient with one thread per (particle, group): the GC lanes of a particle read the
 // same neighbour position and neighbouring 16-byte pieces of the same state record, so a
 // warp request touches about 32 / GC records instead of 32.  Same neighbour pairing and
@@ -419,32 +538,14 @@ __global__ void __launch_bounds__(128) k_flux(PairArgs<T> a, FluxExtra<T> x, con
         if (slot >= a.n_pairs) return;
     }
     constexpr int NC = 4 * GC;
-    const T* tag = nullptr;
     const int G = a.G, RS = 4 * G;
     const int2 kl = a.ends[slot];
     const int64_t i = kl.x, j = kl.y;
     T wgt = T(1);
     if constexpr (BINS) wgt = T(1 << min(a.bins[i], a.bins[j]));   // min(dt_k, dt_l) / dt_min
-    const Pos<T> pi = load_pos(tag, a.pos, i);
-    const Pos<T> pj = load_pos(tag, a.pos, j);
-    T gi8[8], gj8[8];
-    vload<8>(a.geo + 8 * i, gi8);
-    vload<8>(a.geo + 8 * j, gj8);
-    T dx, dy, dz;
-    sep(a.sp, pi, pj, dx, dy, dz);              // d = x_l - x_k
-    // A_kl = (Bp_k w_k + Bp_l w_l) d  (Eq. HopkinsAij)
-    T r = sqrt_(dx * dx + dy * dy + dz * dz);
-    T si = spline_w_(r * gi8[0]);
-    T sj = spline_w_(r * gj8[0]);
-    T M[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) M[q] = gi8[2 + q] * si + gj8[2 + q] * sj;
-    T Ax, Ay, Az;
-    sym_mv(M, dx, dy, dz, Ax, Ay, Az);
-    T An = sqrt_(Ax * Ax + Ay * Ay + Az * Az);
-    T diss = T(0.5) * x.c * An;
-    T ih = rcp_(gi8[1] + gj8[1]);
-    T wi = gi8[1] * ih, wj = gj8[1] * ih;
+    PairGeo<T> pr;
+    T sk, sl;
+    load_pair_geo(a, slot, i, j, x.c, pr, sk, sl);
     const T* ri = rec + i * RS;
     const T* rj = rec + j * RS;
     const T* qi = a.grad + i * 12 * G;
@@ -458,7 +559,7 @@ __global__ void __launch_bounds__(128) k_flux(PairArgs<T> a, FluxExtra<T> x, con
         vload<4>(rj + 4 * gg, uj);
         vload<12>(qi + 12 * gg, gri);
         vload<12>(qj + 12 * gg, grj);
-        pair_flux<HLL>(ui, uj, gri, grj, dx, dy, dz, wi, wj, Ax, Ay, Az, diss, x.c, x.wave, An, &out[4 * g]);
+        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
     }
     if constexpr (BINS) {
 #pragma unroll
@@ -781,18 +882,9 @@ __global__ void __launch_bounds__(128) k_flux_staged(PairArgs<float> a, FluxExtr
     vload<8>(mine + 4, gj8);
     float dx, dy, dz;
     sep(a.sp, pi, pj, dx, dy, dz);
-    float r = sqrt_(dx * dx + dy * dy + dz * dz);
-    float si = spline_w_(r * gi8[0]);
-    float sj = spline_w_(r * gj8[0]);
-    float M[6];
-#pragma unroll
-    for (int q = 0; q < 6; ++q) M[q] = gi8[2 + q] * si + gj8[2 + q] * sj;
-    float Ax, Ay, Az;
-    sym_mv(M, dx, dy, dz, Ax, Ay, Az);
-    float An = sqrt_(Ax * Ax + Ay * Ay + Az * Az);
-    float diss = 0.5f * x.c * An;
-    float ih = rcp_(gi8[1] + gj8[1]);
-    float wi = gi8[1] * ih, wj = gj8[1] * ih;
+    PairGeo<float> pr;
+    float sk, sl;
+    pair_geo(dx, dy, dz, gi8, gj8, x.c, pr, sk, sl);
     const float* ri = rec + i * RS;
     const float* qi = a.grad + i * 12 * G;
     float out[NC];
@@ -804,7 +896,7 @@ __global__ void __launch_bounds__(128) k_flux_staged(PairArgs<float> a, FluxExtr
         vload<4>(mine + 12 + 4 * g, uj);
         vload<12>(qi + 12 * gg, gri);
         vload<12>(mine + 12 + 4 * GC + 12 * g, grj);
-        pair_flux<HLL>(ui, uj, gri, grj, dx, dy, dz, wi, wj, Ax, Ay, Az, diss, x.c, x.wave, An, &out[4 * g]);
+        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
     }
     if (act) vstore<NC>(pairbuf + slot * NC, out);
 }
@@ -900,18 +992,9 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
     vload<8>(lrow(1), gj8);
     float dx, dy, dz;
     sep(a.sp, pi, pj, dx, dy, dz);
-    float r = sqrt_(dx * dx + dy * dy + dz * dz);
-    float si = spline_w_(r * gi8[0]);
-    float sj = spline_w_(r * gj8[0]);
-    float M[6];
-#pragma unroll
-    for (int k = 0; k < 6; ++k) M[k] = gi8[2 + k] * si + gj8[2 + k] * sj;
-    float Ax, Ay, Az;
-    sym_mv(M, dx, dy, dz, Ax, Ay, Az);
-    float An = sqrt_(Ax * Ax + Ay * Ay + Az * Az);
-    float diss = 0.5f * x.c * An;
-    float ih = rcp_(gi8[1] + gj8[1]);
-    float wi = gi8[1] * ih, wj = gj8[1] * ih;
+    PairGeo<float> pr;
+    float sk, sl;
+    pair_geo(dx, dy, dz, gi8, gj8, x.c, pr, sk, sl);
     float out[NC];
 #pragma unroll
     for (int g = 0; g < G; ++g) {
@@ -922,7 +1005,7 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
         vload<4>(lrow(3 + G + 3 * g), grj);
         vload<4>(lrow(4 + G + 3 * g), grj + 4);
         vload<4>(lrow(5 + G + 3 * g), grj + 8);
-        pair_flux<HLL>(ui, uj, gri, grj, dx, dy, dz, wi, wj, Ax, Ay, Az, diss, x.c, x.wave, An, &out[4 * g]);
+        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
     }
     if constexpr (BINS) {
         const float wgt = (float)(1 << min(a.bins[kl.x], a.bins[kl.y]));   // min(dt_k, dt_l) / dt_min
@@ -1106,6 +1189,19 @@ static void launch_gradient_t(rt_ctx* c, cudaStream_t s, T* rec, bool packed = f
                     case 2: k_gradient_g<2><<<nbg, gb, 0, s>>>(a, rec, gr, g0); break;
                     case 3: k_gradient_g<3><<<nbg, gb, 0, s>>>(a, rec, gr, g0); break;
                     default: k_gradient_g<4><<<nbg, gb, 0, s>>>(a, rec, gr, g0); break;
+                }
+                prof_end(c, s, pr);
+                ++c->launches;
+                continue;
+            }
+        }
+        if constexpr (std::is_same<T, double>::value) {
+            if (a.wd) {
+                switch (gc) {
+                    case 1: launch_gradient_wd<1, false>(c, s, a, rec, c->grad_t.as<T>(), g0); break;
+                    case 2: launch_gradient_wd<2, false>(c, s, a, rec, c->grad_t.as<T>(), g0); break;
+                    case 3: launch_gradient_wd<3, false>(c, s, a, rec, c->grad_t.as<T>(), g0); break;
+                    default: launch_gradient_wd<4, false>(c, s, a, rec, c->grad_t.as<T>(), g0); break;
                 }
                 prof_end(c, s, pr);
                 ++c->launches;
@@ -1373,6 +1469,7 @@ rt_status set_fields(rt_ctx* c, int64_t first, int64_t count, const double* omeg
                                                        c->geo_t.as<float>(), c->omega_t.as<float>());
     ++c->launches;
     RT_CUDA(c, cudaGetLastError());
+    c->pair_geo_ready = false;   // B changed: the kept surfaces are computed again
     return RT_OK;
 }
 
@@ -1458,6 +1555,18 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
     for (int g0 = 0; g0 < G; g0 += kMaxGC) {
         const int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
         if (n_start == 0) break;
+        if constexpr (std::is_same<T, double>::value) {
+            if (ag.wd) {
+                switch (gc) {
+                    case 1: launch_gradient_wd<1, true>(c, s, ag, rec, gr, g0); break;
+                    case 2: launch_gradient_wd<2, true>(c, s, ag, rec, gr, g0); break;
+                    case 3: launch_gradient_wd<3, true>(c, s, ag, rec, gr, g0); break;
+                    default: launch_gradient_wd<4, true>(c, s, ag, rec, gr, g0); break;
+                }
+                ++c->launches;
+                continue;
+            }
+        }
         switch (gc) {
             case 1: k_gradient<T, 1, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
             case 2: k_gradient<T, 2, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
