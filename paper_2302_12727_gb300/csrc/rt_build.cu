@@ -9,9 +9,10 @@
 #include <cub/cub.cuh>
 
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
-#include "rt_internal.cuh"
+#include "rt_pair.cuh"
 
 namespace rt {
 
@@ -51,7 +52,8 @@ __device__ __forceinline__ int wrap_cell(int c, int nc) {
 // is close to the sphere plus one cell layer.  An axis whose span covers the whole grid is
 // walked once without clipping.  With ASC the ranges come in ascending cell index (a
 // periodic axis is walked from the cell that wraps to the lowest index), so that the
-// candidates, being sorted by cell, come in ascending particle index.
+// candidates, being sorted by cell, come in ascending particle index.  Where fr returns a bool,
+// false ends the walk.
 __device__ __forceinline__ int first_wrapped(int lo, int hi, int nc) {
     return lo < 0 ? 0 : (hi >= nc ? nc : lo);
 }
@@ -120,7 +122,11 @@ __device__ __forceinline__ void for_each_candidate_range(const Grid& g, float px
             for (int sI = 0; sI < ns; ++sI) {
                 int b = g.cell_start[base + sl[sI]];
                 int e = g.cell_start[base + sh[sI] + 1];
-                fr(b, e);
+                if constexpr (std::is_same<decltype(fr(b, e)), bool>::value) {
+                    if (!fr(b, e)) return;
+                } else {
+                    fr(b, e);
+                }
             }
         }
     }
@@ -131,24 +137,6 @@ template <bool ASC = false, class F>
 __device__ __forceinline__ void for_each_candidate(const Grid& g, float px, float py, float pz, float R, F&& f) {
     for_each_candidate_range<ASC>(g, px, py, pz, R, [&](int b, int e) {
         for (int j = b; j < e; ++j) f(j);
-    });
-}
-
-// every candidate with its quantised position record, read four at a time: the loads of a
-// batch are in flight together, and f still sees the candidates one by one, in order
-template <bool ASC = false, class F>
-__device__ __forceinline__ void for_each_candidate_q(const Grid& g, const uint4* __restrict__ xq, float px, float py,
-                                                     float pz, float R, F&& f) {
-    for_each_candidate_range<ASC>(g, px, py, pz, R, [&](int b, int e) {
-        for (int j0 = b; j0 < e; j0 += 4) {
-            uint4 q[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (j0 + u < e) q[u] = xq[j0 + u];
-#pragma unroll
-            for (int u = 0; u < 4; ++u)
-                if (j0 + u < e) f(j0 + u, q[u]);
-        }
     });
 }
 
@@ -251,340 +239,519 @@ __global__ void k_gather_positions(const double* __restrict__ x, const double* _
 }
 
 // ------------------------------------------------------------------------------------
-// a2: smoothing lengths.  f(h) = h - eta * omega(h)^(-1/3), omega(h) = sum_j W(r_ij, h) with
-// the self term; safeguarded Newton, first in float on fixed-point separations, then in
-// double on the exact separations until the step is below machine precision.  The double
-// phase runs for every particle on the FP64 path.  On the float path it runs only for the
-// particles that have a candidate within kNearBand of their own support radius at the float
-// root (about one in thirty): the float root is within a few 1e-6 of the exact one, so for
-// every other particle no neighbour can change side of H_i, and the pair lists, which are
-// decided by H_i and H_j, are those of the exact roots.
+// Walk of one warp for one particle: the rows of cells of for_each_candidate_range<true>, one
+// row per lane, so that the range arithmetic and the cell-table loads of up to 32 rows run side
+// by side; their candidates, numbered by a prefix sum over the lanes, are then dealt 32 at a time
+// to the lanes.  f(j, valid) sees them in ascending index, called by the whole warp, and ends the
+// walk by returning false (the same in every lane).  A thread that walks its own sphere runs
+// row by row on the latency of the table and record loads, half of a warp's lanes idle (14.8
+// active of 32) behind the longest row; a warp per particle that takes the rows in turn repeats the row
+// arithmetic in every lane.
+__device__ __forceinline__ int wrap_once(int c, int nc) { return c < 0 ? c + nc : (c >= nc ? c - nc : c); }
+
+template <class F>
+__device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, float pz, float R, int lane, F&& f) {
+    const unsigned FULL = 0xffffffffu;
+    const float Rc = R * 1.0001f + 1e-6f * (g.cellf[0] + g.cellf[1] + g.cellf[2]);
+    const float R2 = Rc * Rc;
+    const float p[3] = {px, py, pz};
+    int lo[3], hi[3];
+    bool all[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = (int)floorf((p[a] - Rc) * g.inv_cellf[a]);
+        hi[a] = (int)floorf((p[a] + Rc) * g.inv_cellf[a]);
+        all[a] = (hi[a] - lo[a] + 1 >= g.nc[a]);
+        if (all[a]) {
+            lo[a] = 0;
+            hi[a] = g.nc[a] - 1;
+        } else if (!g.periodic) {
+            lo[a] = max(lo[a], 0);
+            hi[a] = min(hi[a], g.nc[a] - 1);
+        }
+    }
+    const int nzs = hi[2] - lo[2] + 1, nys = hi[1] - lo[1] + 1;
+    const int z0 = first_wrapped(lo[2], hi[2], g.nc[2]), y0 = first_wrapped(lo[1], hi[1], g.nc[1]);
+    const int rows = nzs > 0 && nys > 0 ? nzs * nys : 0;
+    for (int r0 = 0; r0 < rows; r0 += 32) {
+        const int r = r0 + lane;
+        int b1 = 0, n1 = 0, b2 = 0, n2 = 0;
+        if (r < rows) {
+            const int kz = r / nys, ky = r - kz * nys;
+            int z = z0 + kz, y = y0 + ky;
+            if (z > hi[2]) z -= nzs;
+            if (y > hi[1]) y -= nys;
+            const float dz = all[2] ? 0.f : fmaxf(0.f, fmaxf(z * g.cellf[2] - pz, pz - (z + 1) * g.cellf[2]));
+            const float dy = all[1] ? 0.f : fmaxf(0.f, fmaxf(y * g.cellf[1] - py, py - (y + 1) * g.cellf[1]));
+            const float rem = R2 - dy * dy - dz * dz;
+            if (rem > 0.f) {
+                const int base = (wrap_once(z, g.nc[2]) * g.nc[1] + wrap_once(y, g.nc[1])) * g.nc[0];
+                int xa = 0, xb = g.nc[0] - 1;
+                if (!all[0]) {
+                    const float w = sqrtf(rem);
+                    xa = (int)floorf((px - w) * g.inv_cellf[0]);
+                    xb = (int)floorf((px + w) * g.inv_cellf[0]);
+                    if (!g.periodic) {
+                        xa = max(xa, 0);
+                        xb = min(xb, g.nc[0] - 1);
+                    }
+                }
+                // up to two ranges of cells, the wrapped part first
+                int s1 = xa, e1 = xb, s2 = 0, e2 = -1;
+                if (xa < 0) {
+                    s1 = 0; e1 = xb; s2 = xa + g.nc[0]; e2 = g.nc[0] - 1;
+                } else if (xb >= g.nc[0]) {
+                    s1 = 0; e1 = xb - g.nc[0]; s2 = xa; e2 = g.nc[0] - 1;
+                }
+                if (s1 <= e1) {
+                    b1 = g.cell_start[base + s1];
+                    n1 = g.cell_start[base + e1 + 1] - b1;
+                }
+                if (s2 <= e2) {
+                    b2 = g.cell_start[base + s2];
+                    n2 = g.cell_start[base + e2 + 1] - b2;
+                }
+            }
+        }
+        int end = n1 + n2;      // inclusive prefix sum of the rows' candidates
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int v = __shfl_up_sync(FULL, end, o);
+            if (lane >= o) end += v;
+        }
+        const int off = end - n1 - n2, total = __shfl_sync(FULL, end, 31);
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            int L = 0;          // the last row whose first candidate is not past t
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1)
+                if (__shfl_sync(FULL, off, L + o) <= t) L += o;
+            const int c = t - __shfl_sync(FULL, off, L), m = __shfl_sync(FULL, n1, L);
+            const int u1 = __shfl_sync(FULL, b1, L), u2 = __shfl_sync(FULL, b2, L);
+            if (!f(c < m ? u1 + c : u2 + (c - m), t < total)) return;
+        }
+    }
+}
+
+// ------------------------------------------------------------------------------------
+// a2: smoothing lengths, h = eta omega(h)^(-1/3) with omega(h) = sum_j W(r_ij, h) and the self
+// term.  With S(h) = sum_j w(r_ij / H) the equation is S(h) = S* = (kappa eta)^3 / sigma, the
+// same number for every particle.
+//
+// Float phase (k_h_lists): safeguarded Newton on f(h) = h - eta omega(h)^(-1/3), nearly linear
+// in h, from the h of the previous call or a local particle count.  The candidates are walked
+// once, out to a little more than the first guess's support: their indices go to the
+// particle's list in memory, from which the double phase and the pair search take them, their
+// distances to shared memory, over which the iterations sum.  Where they overflow the list each
+// iteration walks, but only until S passes 4 S*: a particle that has moved into a dense clump
+// with the h of a void would otherwise visit the whole clump an iteration.
+//
+// Double phase (k_h_refine): Newton on S(h) - S* in double on the exact separations.  On the
+// FP64 path it runs for every particle.  On the float path it runs only for the
+// particles that have a candidate within the near band of their own support radius at the float
+// root: that is within about 1e-6 of the exact one (the last step is below 4e-7 and the
+// rounding of the ~50-term sums 3e-7, over f' > 0.5), so for every other particle no neighbour
+// can change side of H_i, and the pair lists, which are decided by H_i and H_j, are those of
+// the exact roots.  Particles whose last step was not that small, or whose f' is (the edge of
+// a clump), take the double phase too.
 struct HParams {
     double eta, h0, h_cap;
+    double s_star, eta3;   // S* = (kappa eta)^3 / sigma, and eta^3
     float scale[3];
     int max_iter;
     float tol32;
-    int refine64;   // 1: Newton in double to machine precision here; 0: flag near-threshold particles
+    int refine64;   // 1: the double phase follows for every particle, 0: for the flagged ones
 };
 
-// |r^2 - H^2| < kNearBand H^2 at the float root: the particle's h is refined in double
-constexpr float kNearBand = 2e-4f;
+// |r / H - 1| below which a candidate flags its particle for the double phase: ten times the
+// float root's error after a tight step
+constexpr float kNear = 1e-5f, kTightStep = 4e-7f;
 
 __device__ __forceinline__ float fsep(uint32_t a, uint32_t b, float scale) { return (float)(int32_t)(a - b) * scale; }
 
-// Newton in double from hd on the exact separations of particle p; returns false if it did
-// not converge.  On return hd is the root and om_d = omega(hd).
-__device__ bool refine_h_double(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq,
-                                int64_t n, const HParams& hp, int64_t p, double& hd, double& om_d) {
-    const uint4 q4p = xq[p];
-    const uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    const double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    const float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
-    double lod = 0.0, hid = INFINITY;
-    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
-    bool okd = false, last = false;
-    for (int it = 0; it < 60; ++it) {
-        double H = kKappa * hd;
-        double iH = 1.0 / H;
-        double H2 = H * H;
-        float Hf = (float)H * 1.001f;
-        float H2f = Hf * Hf;
-        double sw = 0.0, sdw = 0.0;
-        for_each_candidate(g, pxf, pyf, pzf, Hf, [&](int j) {
-            float dxf = fsep(xq[j].x, qx, hp.scale[0]);
-            float dyf = fsep(xq[j].y, qy, hp.scale[1]);
-            float dzf = fsep(xq[j].z, qz, hp.scale[2]);
-            if (dxf * dxf + dyf * dyf + dzf * dzf >= H2f) return;
-            double dx = sep_fast(xs[j], px, g.box[0], half[0], g.periodic);
-            double dy = sep_fast(xs[n + j], py, g.box[1], half[1], g.periodic);
-            double dz = sep_fast(xs[2 * n + j], pz, g.box[2], half[2], g.periodic);
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < H2) {
-                double q = sqrt(r2) * iH;
-                double w = spline_w(q);
-                sw += w;
-                sdw += 3.0 * w + q * spline_dw(q);
-            }
-        });
-        double om = kSigma * iH * iH * iH * sw;
-        double dom = -kKappa * kSigma * iH * iH * iH * iH * sdw;
-        double cb = cbrt(om);
-        double f = hd - hp.eta / cb;
-        double fp = 1.0 + (hp.eta / 3.0) / (cb * om) * dom;
-        om_d = om;
-        if (last) { okd = true; break; }        // omega evaluated at the final h
-        if (f < 0.0) lod = hd; else hid = hd;
-        double step = f / fp;
-        // once the Newton step is tiny the next iterate is exact to rounding: take it and
-        // evaluate omega there once more; a residual at the rounding floor or a collapsed
-        // bracket ends the iteration at the current h
-        if (fabs(f) <= 1e-15 * hd || (hid - lod) <= 1e-14 * hd) { okd = true; break; }
-        if (fp > 0.0 && fabs(step) <= 1e-11 * hd) last = true;
-        double hn = hd - step;
-        if (!last && (it >= 12 || !(hn > lod && hn < hid) || !(fp > 0.0)))
-            hn = isinf(hid) ? 1.01 * hd : 0.5 * (lod + hid);
-        hd = hn;
+// compensated float sum
+struct Kahan {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        float y = v - c;
+        float t = s + y;
+        c = (t - s) - y;
+        s = t;
     }
-    return okd;
+    // adds another sum, without rounding (the lanes of a reduction)
+    __device__ __forceinline__ void merge(float s2, float c2) {
+        const float t = __fadd_rn(s, s2), z = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(s2, z));
+        c = __fsub_rn(__fadd_rn(c, c2), e);
+        s = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
+};
+
+// One Newton step of the float phase from the sums at h; what the step says about h
+struct HStep {
+    float hn;          // next iterate
+    bool tight, loose; // below kTightStep with f' near one; below the caller's tolerance
+};
+__device__ __forceinline__ HStep h_newton(const HParams& hp, float h, float sw, float sdw, int it, float& lo,
+                                          float& hi) {
+    const float kapf = (float)kKappa, sigf = (float)kSigma, eta = (float)hp.eta;
+    const float iH = 1.f / (kapf * h);
+    const float om = sigf * iH * iH * iH * sw;
+    const float dom = -kapf * sigf * iH * iH * iH * iH * sdw;      // d omega / d h
+    const float cb = cbrtf(om);
+    const float f = h - eta / cb;
+    const float fp = 1.f + (eta / 3.f) / (cb * om) * dom;
+    if (f < 0.f) lo = h; else hi = h;
+    const float step = f / fp;
+    HStep r;
+    r.tight = fp > 0.5f && fabsf(step) <= kTightStep * h;
+    // residual at the rounding floor, a small Newton step, or a collapsed bracket (where f' is
+    // small, rounding alone keeps the step above tolerance)
+    r.loose = fabsf(f) <= 1e-6f * h || (fp > 0.f && fabsf(step) <= hp.tol32 * h) || (hi - lo) <= hp.tol32 * h;
+    // safeguarded Newton; plain bisection of the bracket after 24 Newton steps
+    float hn = h - step;
+    if (it >= 24 || !(hn > lo && hn < hi) || !(fp > 0.f)) hn = isinf(hi) ? 2.f * h : 0.5f * (lo + hi);
+    r.hn = hn > (float)hp.h_cap ? (float)hp.h_cap : hn;
+    return r;
 }
 
-// The same Newton in double for particle p, with the 32 lanes of a warp sharing the candidate
-// walk (in every contiguous run of candidates, lane l takes the l-th, (l + 32)-th, ...) and
-// combining their sums by a fixed butterfly, whose result is the same in every lane: the
-// lanes then take the same steps.  Used where few particles need it (k_h_refine), so that the double arithmetic,
-// slow on this GPU, is spread over many threads.
-__device__ bool refine_h_warp(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq,
-                              int64_t n, const HParams& hp, int64_t p, int lane, double& hd, double& om_d) {
-    const uint4 q4p = xq[p];
-    const uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    const double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    const float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
-    double lod = 0.0, hid = INFINITY;
-    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
-    bool okd = false, last = false;
-    for (int it = 0; it < 60; ++it) {
-        double H = kKappa * hd;
-        double iH = 1.0 / H;
-        double H2 = H * H;
-        float Hf = (float)H * 1.001f;
-        float H2f = Hf * Hf;
-        double sw = 0.0, sdw = 0.0;
-        for_each_candidate_range(g, pxf, pyf, pzf, Hf, [&](int b, int e) {
-          for (int j = b + lane; j < e; j += 32) {
-            float dxf = fsep(xq[j].x, qx, hp.scale[0]);
-            float dyf = fsep(xq[j].y, qy, hp.scale[1]);
-            float dzf = fsep(xq[j].z, qz, hp.scale[2]);
-            if (dxf * dxf + dyf * dyf + dzf * dzf >= H2f) continue;
-            double dx = sep_fast(xs[j], px, g.box[0], half[0], g.periodic);
-            double dy = sep_fast(xs[n + j], py, g.box[1], half[1], g.periodic);
-            double dz = sep_fast(xs[2 * n + j], pz, g.box[2], half[2], g.periodic);
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < H2) {
-                double q = sqrt(r2) * iH;
-                double w = spline_w(q);
-                sw += w;
-                sdw += 3.0 * w + q * spline_dw(q);
-            }
-          }
-        });
-        for (int o = 16; o > 0; o >>= 1) {
-            sw += __shfl_xor_sync(0xffffffffu, sw, o);
-            sdw += __shfl_xor_sync(0xffffffffu, sdw, o);
-        }
-        double om = kSigma * iH * iH * iH * sw;
-        double dom = -kKappa * kSigma * iH * iH * iH * iH * sdw;
-        double cb = cbrt(om);
-        double f = hd - hp.eta / cb;
-        double fp = 1.0 + (hp.eta / 3.0) / (cb * om) * dom;
-        om_d = om;
-        if (last) { okd = true; break; }
-        if (f < 0.0) lod = hd; else hid = hd;
-        double step = f / fp;
-        if (fabs(f) <= 1e-15 * hd || (hid - lod) <= 1e-14 * hd) { okd = true; break; }
-        if (fp > 0.0 && fabs(step) <= 1e-11 * hd) last = true;
-        double hn = hd - step;
-        if (!last && (it >= 12 || !(hn > lod && hn < hid) || !(fp > 0.0)))
-            hn = isinf(hid) ? 1.01 * hd : 0.5 * (lod + hid);
-        hd = hn;
-    }
-    return okd;
+// lanes a particle of the sums, warps and particles a block
+constexpr int kSumLanes = 8, kListWarps = 8, kListParticles = kListWarps * 32 / kSumLanes;
+
+// entries a particle's candidate list holds: twice what 1.1 support radii hold of an even set (128
+// at the usual eta), at most what the blocks' 48 KB of shared distances allow
+static int list_capacity(double eta) {
+    const double even = 4.18879 * std::pow(kKappa * eta * 1.1, 3.0);
+    return (int)std::min(352.0, std::max(32.0, std::floor((2.0 * even + 31.0) / 32.0) * 32.0));
 }
 
-// The same for one warp, walking the candidates once: the double Newton moves h by far less
-// than 1e-4 from the float root, so the particles within 1.0009 of its support radius contain
-// every neighbour of every iteration.  Their exact distances are dealt to the lanes in walk
-// order (candidate c to lane c mod 32) and kept in registers (kRefineSlots a lane); the
-// iterations then sum the spline over them.  A lane that would need more slots, or an
-// iterate beyond that radius, sends the warp to refine_h_warp.
-constexpr int kRefineSlots = 8;
-
-__device__ bool refine_h_warp_cached(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq,
-                                     int64_t n, const HParams& hp, int64_t p, int lane, double& hd, double& om_d) {
-    const uint4 q4p = xq[p];
-    const uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    const double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    const float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
-    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
-    const double h_start = hd;
-    const double Rc = kKappa * hd * 1.0009, Rc2 = Rc * Rc;
-    const float Hf = (float)(kKappa * hd) * 1.001f, H2f = Hf * Hf;
-    double r[kRefineSlots];
-    int cnt = 0;
-    bool over = false;
-    int seen = 0;     // candidates of the earlier ranges (walk order)
-    for_each_candidate_range(g, pxf, pyf, pzf, Hf, [&](int b, int e) {
-        const int first = (lane - seen) & 31;    // this lane's first candidate of the range
-        for (int j = b + first; j < e; j += 32) {
-            float dxf = fsep(xq[j].x, qx, hp.scale[0]);
-            float dyf = fsep(xq[j].y, qy, hp.scale[1]);
-            float dzf = fsep(xq[j].z, qz, hp.scale[2]);
-            if (dxf * dxf + dyf * dyf + dzf * dzf >= H2f) continue;
-            double dx = sep_fast(xs[j], px, g.box[0], half[0], g.periodic);
-            double dy = sep_fast(xs[n + j], py, g.box[1], half[1], g.periodic);
-            double dz = sep_fast(xs[2 * n + j], pz, g.box[2], half[2], g.periodic);
-            double r2 = dx * dx + dy * dy + dz * dz;
-            if (r2 < Rc2) {
-                if (cnt < kRefineSlots) {
-                    const double rr = sqrt(r2);
-#pragma unroll
-                    for (int k = 0; k < kRefineSlots; ++k)   // static indices keep r in registers
-                        if (k == cnt) r[k] = rr;
-                    ++cnt;
-                } else {
-                    over = true;
-                }
-            }
-        }
-        seen += e - b;
-    });
-    if (__any_sync(0xffffffffu, over)) return refine_h_warp(g, xs, xq, n, hp, p, lane, hd, om_d);
-    double lod = 0.0, hid = INFINITY;
-    bool okd = false, last = false;
-    for (int it = 0; it < 60; ++it) {
-        double H = kKappa * hd;
-        if (H > Rc) {   // beyond the cached radius (never expected): walk again
-            hd = h_start;
-            return refine_h_warp(g, xs, xq, n, hp, p, lane, hd, om_d);
-        }
-        double iH = 1.0 / H;
-        double sw = 0.0, sdw = 0.0;
-#pragma unroll
-        for (int k = 0; k < kRefineSlots; ++k) {
-            if (k < cnt && r[k] < H) {
-                double q = r[k] * iH;
-                double w = spline_w(q);
-                sw += w;
-                sdw += 3.0 * w + q * spline_dw(q);
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            sw += __shfl_xor_sync(0xffffffffu, sw, o);
-            sdw += __shfl_xor_sync(0xffffffffu, sdw, o);
-        }
-        double om = kSigma * iH * iH * iH * sw;
-        double dom = -kKappa * kSigma * iH * iH * iH * iH * sdw;
-        double cb = cbrt(om);
-        double f = hd - hp.eta / cb;
-        double fp = 1.0 + (hp.eta / 3.0) / (cb * om) * dom;
-        om_d = om;
-        if (last) { okd = true; break; }
-        if (f < 0.0) lod = hd; else hid = hd;
-        double step = f / fp;
-        if (fabs(f) <= 1e-15 * hd || (hid - lod) <= 1e-14 * hd) { okd = true; break; }
-        if (fp > 0.0 && fabs(step) <= 1e-11 * hd) last = true;
-        double hn = hd - step;
-        if (!last && (it >= 12 || !(hn > lod && hn < hid) || !(fp > 0.0)))
-            hn = isinf(hid) ? 1.0001 * hd : 0.5 * (lod + hid);
-        hd = hn;
-    }
-    return okd;
-}
-
-__global__ void k_h_solve(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
-                          HParams hp, const double* __restrict__ h_prev, const int32_t* __restrict__ perm,
-                          double* h_out, double* omega_out, float* H2f_out, unsigned long long* hminmax, int* flags,
-                          int32_t* refine_list, int* refine_count) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double hd = 0.0, om_d = 0.0;
-    bool active = p < n;
+// SOLVE: h by Newton, and the list of the candidates within at least H (1 + 2 kNear) of it.
+// Otherwise h_out holds the smoothing lengths, and only the lists are made.  list_cnt is the
+// list's length, or -1 where it overflowed.  Each warp walks for its four particles in turn; the
+// sums of the four then run side by side on eight lanes each.
+// 262,144 particles that moved by a tenth of their spacing took 0.88 ms with a thread per
+// particle and a walk of the cells every iteration, 1,000,000 strongly clustered ones 5.2 ms, and
+// 155 ms where some had the h of a place far less dense.
+template <bool SOLVE>
+__global__ void __launch_bounds__(kListWarps * 32)
+k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
+          const double* __restrict__ h_prev, const int32_t* __restrict__ perm, const double* __restrict__ h_given,
+          float* __restrict__ h_sum, int* flags, int32_t* refine_list, int* refine_count,
+          int32_t* __restrict__ list, int32_t* __restrict__ list_cnt, int cap) {
+    constexpr int PW = 32 / kSumLanes;            // particles a warp
+    const unsigned FULL = 0xffffffffu;
+    extern __shared__ float st_all[];             // distances of the stored candidates, cap a particle
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int a = lane / kSumLanes, sub = lane % kSumLanes;
+    const int64_t p0 = (blockIdx.x * (int64_t)kListWarps + wid) * PW, p = p0 + a;
+    const bool active = p < n;
+    float* st = st_all + wid * PW * cap;
+    const float kapf = (float)kKappa;
+    float h = 0.f;
     if (active) {
-        const float kapf = (float)kKappa;
-        const float sigf = (float)kSigma;
-        const uint4 q4p = xq[p];
-        uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-        double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-        float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
-
-        // first guess: the particle's h of the previous call (particles move little between
-        // calls), else the particle count of the surrounding 27 cells
-        float h;
-        if (h_prev) {
+        if (!SOLVE) {
+            h = (float)h_given[p];
+        } else if (h_prev) {
+            // first guess: the particle's h of the previous call (particles move little between
+            // calls), else the particle count of the surrounding 27 cells
             h = (float)h_prev[perm[p]];
         } else {
-            int cnt = count_27(g, cell_coord(px, g.inv_cell[0], g.nc[0]), cell_coord(py, g.inv_cell[1], g.nc[1]),
-                               cell_coord(pz, g.inv_cell[2], g.nc[2]));
+            int cnt = count_27(g, cell_coord(xs[p], g.inv_cell[0], g.nc[0]),
+                               cell_coord(xs[n + p], g.inv_cell[1], g.nc[1]),
+                               cell_coord(xs[2 * n + p], g.inv_cell[2], g.nc[2]));
             double vol27 = 27.0 * g.cell[0] * g.cell[1] * g.cell[2];
             h = cnt > 1 ? (float)(hp.eta * cbrt(vol27 / (double)cnt)) : (float)hp.h0;
         }
-        if (!(h > 0.f) || !(h < (float)hp.h_cap)) h = (float)hp.h0;
-
-        // ---- float phase: Newton on float separations, omega summed in double
-        float lo = 0.f, hi = INFINITY;
-        const float eta = (float)hp.eta;
-        bool ok = false, near = false;
-        double sw_last = 0.0;
-        for (int it = 0; it < hp.max_iter; ++it) {
-            float H = kapf * h;
-            float iH = 1.f / H;
-            float H2 = H * H;
-            double sw = 0.0;
-            float sdw = 0.f;
-            bool nb = false;
-            for_each_candidate_q(g, xq, pxf, pyf, pzf, H, [&](int, uint4 qj) {
-                float dx = fsep(qj.x, qx, hp.scale[0]);
-                float dy = fsep(qj.y, qy, hp.scale[1]);
-                float dz = fsep(qj.z, qz, hp.scale[2]);
-                float r2 = dx * dx + dy * dy + dz * dz;
-                nb |= fabsf(r2 - H2) < kNearBand * H2;
-                if (r2 < H2) {
-                    float q = sqrtf(r2) * iH;
-                    float w = spline_w(q);
-                    sw += (double)w;
-                    sdw += 3.f * w + q * spline_dw(q);
-                }
-            });
-            sw_last = sw;
-            near = nb;
-            float om = sigf * iH * iH * iH * (float)sw;
-            float dom = -kapf * sigf * iH * iH * iH * iH * sdw;      // d omega / d h
-            float cb = cbrtf(om);
-            float f = h - eta / cb;
-            float fp = 1.f + (eta / 3.f) / (cb * om) * dom;
-            if (f < 0.f) lo = h; else hi = h;
-            float step = f / fp;
-            // converged: residual at the rounding floor, a tiny Newton step, or a collapsed
-            // bracket (where f' is small, rounding alone keeps the step above tolerance)
-            if (fabsf(f) <= 1e-6f * h || (fp > 0.f && fabsf(step) <= hp.tol32 * h) ||
-                (hi - lo) <= hp.tol32 * h) {
-                ok = true;
-                break;
-            }
-            float hn = h - step;
-            // safeguarded Newton; plain bisection of the bracket after 24 Newton steps
-            if (it >= 24 || !(hn > lo && hn < hi) || !(fp > 0.f)) hn = isinf(hi) ? 2.f * h : 0.5f * (lo + hi);
-            if (hn > (float)hp.h_cap) hn = (float)hp.h_cap;
-            if (hn == h) break;       // no progress possible: reported as not converged
-            h = hn;
-        }
-        if (!ok) atomicExch(&flags[F_NOCONV], 1);
-        hd = (double)h;
-        {
-            double H = kKappa * hd;
-            om_d = kSigma / (H * H * H) * sw_last;
-        }
-
-        // ---- double phase: Newton on the exact separations to machine precision, here for
-        // every particle (FP64 path), else later (k_h_refine) for the near-threshold ones
-        if (ok && hp.refine64) {
-            if (!refine_h_double(g, xs, xq, n, hp, p, hd, om_d)) atomicExch(&flags[F_NOCONV], 1);
-        } else if (ok && near) {
-            refine_list[atomicAdd(refine_count, 1)] = (int32_t)p;
-        }
-        h_out[p] = hd;
-        omega_out[p] = om_d;
-        double Hd = kKappa * hd;
-        H2f_out[p] = (float)(Hd * Hd);
+        if (SOLVE && (!(h > 0.f) || !(h < (float)hp.h_cap))) h = (float)hp.h0;
     }
-    double mn = active ? hd : INFINITY, mx = active ? hd : 0.0;
+    float lo = 0.f, hi = INFINITY, Rs = 0.f, h_over = 0.f;
+    const float s_many = 4.f * (float)hp.s_star;
+    // wants: the list is in use (until it overflows); Rs and cnt describe it
+    bool done = !active, ok = false, near = false, wants = true;
+    int cnt = 0, it = 0;
+    Kahan S_last;
+    while (__any_sync(FULL, !done)) {
+        const float H = kapf * h, iH = 1.f / H;
+        const bool fill = !done && wants && H * (1.f + 2.f * kNear) > Rs;
+        unsigned todo = __ballot_sync(FULL, fill && sub == 0);
+        while (todo) {          // walks that store, one particle at a time
+            const int src = __ffs(todo) - 1, b = src / kSumLanes;
+            todo &= todo - 1;
+            const int64_t q = p0 + b;
+            const uint4 qp = xq[q];
+            const float R = __shfl_sync(FULL, H, src) * (SOLVE ? 1.10f : 1.f + 4.f * kNear), R2 = R * R;
+            int c = 0;
+            warp_walk(g, (float)qp.x * hp.scale[0], (float)qp.y * hp.scale[1], (float)qp.z * hp.scale[2], R, lane,
+                      [&](int j, bool valid) {
+                          float r2 = INFINITY;
+                          if (valid) {
+                              const uint4 qj = xq[j];
+                              const float dx = fsep(qj.x, qp.x, hp.scale[0]);
+                              const float dy = fsep(qj.y, qp.y, hp.scale[1]);
+                              const float dz = fsep(qj.z, qp.z, hp.scale[2]);
+                              r2 = dx * dx + dy * dy + dz * dz;
+                          }
+                          const bool in = r2 < R2;
+                          const unsigned m = __ballot_sync(FULL, in);
+                          const int pos = c + __popc(m & ((1u << lane) - 1u));
+                          if (in && pos < cap) {
+                              list[q * cap + pos] = j;
+                              st[b * cap + pos] = sqrtf(r2);
+                          }
+                          c += __popc(m);
+                          return c <= cap;
+                      });
+            if (a == b) {
+                cnt = c;
+                Rs = R;
+                if (c > cap) {
+                    wants = false;
+                    Rs = 0.f;
+                    h_over = h;
+                    if (!SOLVE) done = true;
+                }
+            }
+        }
+        __syncwarp();
+        if (!SOLVE) break;
+        Kahan sw;
+        float sdw = 0.f, gap = INFINITY;
+        auto term = [&](float q) {
+            gap = fminf(gap, fabsf(q - 1.f));
+            const float u = fmaxf(1.f - q, 0.f), v = fmaxf(0.5f - q, 0.f);
+            const float u2 = u * u, v2 = v * v;
+            const float w = u2 * u - 4.f * (v2 * v);
+            sw.add(w);
+            sdw += 3.f * w + q * (12.f * v2 - 3.f * u2);
+        };
+        if (!done && wants)
+            for (int k = sub; k < cnt; k += kSumLanes) term(st[a * cap + k] * iH);
+#pragma unroll
+        for (int o = kSumLanes / 2; o > 0; o >>= 1) {
+            sw.merge(__shfl_xor_sync(FULL, sw.s, o), __shfl_xor_sync(FULL, sw.c, o));
+            sdw += __shfl_xor_sync(FULL, sdw, o);
+            gap = fminf(gap, __shfl_xor_sync(FULL, gap, o));
+        }
+        // walks that sum, for the particles whose candidates overflow the list
+        bool many = false;
+        todo = __ballot_sync(FULL, !done && !wants && sub == 0);
+        while (todo) {
+            const int src = __ffs(todo) - 1, b = src / kSumLanes;
+            todo &= todo - 1;
+            const uint4 qp = xq[p0 + b];
+            const float Hb = __shfl_sync(FULL, H, src), iHb = 1.f / Hb;
+            const float R = Hb * (1.f + 2.f * kNear), R2 = R * R;
+            Kahan swb;
+            float sdb = 0.f, gb = INFINITY;
+            warp_walk(g, (float)qp.x * hp.scale[0], (float)qp.y * hp.scale[1], (float)qp.z * hp.scale[2], R, lane,
+                      [&](int j, bool valid) {
+                          if (valid) {
+                              const uint4 qj = xq[j];
+                              const float dx = fsep(qj.x, qp.x, hp.scale[0]);
+                              const float dy = fsep(qj.y, qp.y, hp.scale[1]);
+                              const float dz = fsep(qj.z, qp.z, hp.scale[2]);
+                              const float r2 = dx * dx + dy * dy + dz * dz;
+                              if (r2 < R2) {
+                                  const float q = sqrtf(r2) * iHb;
+                                  gb = fminf(gb, fabsf(q - 1.f));
+                                  const float u = fmaxf(1.f - q, 0.f), v = fmaxf(0.5f - q, 0.f);
+                                  const float u2 = u * u, v2 = v * v;
+                                  const float w = u2 * u - 4.f * (v2 * v);
+                                  swb.add(w);
+                                  sdb += 3.f * w + q * (12.f * v2 - 3.f * u2);
+                              }
+                          }
+                          return !__any_sync(FULL, swb.s >= s_many);
+                      });
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                swb.merge(__shfl_xor_sync(FULL, swb.s, o), __shfl_xor_sync(FULL, swb.c, o));
+                sdb += __shfl_xor_sync(FULL, sdb, o);
+                gb = fminf(gb, __shfl_xor_sync(FULL, gb, o));
+            }
+            if (a == b) {
+                sw = swb;
+                sdw = sdb;
+                gap = gb;
+                many = swb.s >= s_many;
+            }
+        }
+        if (!done) {
+            if (many) {           // S(h) > 4 S*: far too large, whatever the rest of the walk
+                hi = h;
+                h = fmaxf(0.6f * h, 0.5f * (lo + h));
+                wants = h < 0.85f * h_over;
+                done = it + 1 >= hp.max_iter;
+            } else {
+                S_last = sw;
+                const HStep r = h_newton(hp, h, sw.s - sw.c, sdw, it, lo, hi);
+                if (r.tight || (r.loose && (it >= 6 || it + 1 >= hp.max_iter || r.hn == h))) {
+                    ok = done = true;
+                    near = !r.tight || gap < kNear;
+                    // the double phase may move such an h by more than the margin of the list
+                    if (!r.tight && Rs < 1.01f * H) wants = false;
+                } else if (r.hn == h || it + 1 >= hp.max_iter) {
+                    done = true;      // no progress possible: reported as not converged
+                } else {
+                    h = r.hn;
+                    wants = wants || h < 0.85f * h_over;
+                }
+            }
+            ++it;
+        }
+    }
+    if (active && sub == 0) {
+        list_cnt[p] = wants ? cnt : -1;
+        if (SOLVE) {
+            if (!ok) atomicExch(&flags[F_NOCONV], 1);
+            if (ok && near && !hp.refine64) refine_list[atomicAdd(refine_count, 1)] = (int32_t)p;
+            h_sum[p] = h;
+            h_sum[n + p] = S_last.s;
+            h_sum[2 * n + p] = S_last.c;
+        }
+    }
+}
+
+// What the float phase leaves to one thread per particle (its few double instructions would cost
+// k_h_lists, with eight lanes a particle, eight times as much): h, omega = sigma / H^3 S and the
+// float H^2, also in the free word of the position record, so that the pair search reads a
+// candidate's position and support radius with one 16-byte load; the smallest and largest h
+// and the sum of H^3 (which only steers the reported pair_build).  With h_sum NULL (given h) only the
+// record is filled.
+__global__ void __launch_bounds__(256)
+k_h_finish(const float* __restrict__ h_sum, int64_t n, int reduce, double* __restrict__ h_out,
+           double* __restrict__ omega_out, float* __restrict__ H2f, uint4* __restrict__ xq,
+           unsigned long long* hminmax) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    double mn = INFINITY, mx = 0.0, h3 = 0.0;
+    if (p < n) {
+        float H2;
+        if (h_sum) {
+            const double hd = (double)h_sum[p], H = kKappa * hd;
+            H2 = (float)(H * H);
+            h3 = H * H * H;
+            mn = mx = hd;
+            h_out[p] = hd;
+            omega_out[p] = kSigma / h3 * ((double)h_sum[n + p] - (double)h_sum[2 * n + p]);
+            H2f[p] = H2;
+        } else {
+            H2 = H2f[p];
+        }
+        reinterpret_cast<unsigned*>(xq + p)[3] = __float_as_uint(H2);
+    }
+    if (!h_sum || !reduce) return;
     warp_minmax(mn, mx);
-    // sum of H^3 (only steers the choice of the pair-search method, never a result)
-    double h3 = active ? (kKappa * hd) * (kKappa * hd) * (kKappa * hd) : 0.0;
     for (int o = 16; o > 0; o >>= 1) h3 += __shfl_xor_sync(0xffffffffu, h3, o);
     if ((threadIdx.x & 31) == 0 && mx > 0.0) {
         atomic_min_pos(&hminmax[0], mn);
         atomic_max_pos(&hminmax[1], mx);
         atomicAdd(reinterpret_cast<double*>(&hminmax[4]), h3);
     }
+}
+
+// Double phase for particle p from the float root hd, by the kRefineLanes lanes of a group:
+// Newton on S(h) = S*.  The step after one of less than 1e-8 h is exact to rounding, and at the
+// root omega is (eta/h)^3, so two evaluations do, with no cube root and one reciprocal each:
+// these scalar parts, which a group's lanes all repeat, were three quarters of the double
+// instructions with a warp per particle and the omega^(-1/3) form.  The particle's list holds
+// every candidate within kNear of its float support, which contains every neighbour of every
+// iterate; their distances are dealt to the lanes and kept in registers.  A particle without a
+// list, or whose lanes would need more than kRefineSlots, walks for every evaluation.
+constexpr int kRefineLanes = 8, kRefineSlots = 12;
+
+__device__ bool refine_h(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
+                         const HParams& hp, int64_t p, int lane, unsigned group, const int32_t* __restrict__ list,
+                         int list_cnt, double& hd, double& om_d) {
+    const uint4 q4p = xq[p];
+    const uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
+    const double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
+    const float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
+    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
+    // exact distance of candidate j, handed to f if below R
+    auto visit = [&](int j, float R2f, double R2, auto&& f) {
+        const uint4 qj = xq[j];
+        const float dxf = fsep(qj.x, qx, hp.scale[0]);
+        const float dyf = fsep(qj.y, qy, hp.scale[1]);
+        const float dzf = fsep(qj.z, qz, hp.scale[2]);
+        if (dxf * dxf + dyf * dyf + dzf * dzf >= R2f) return;
+        const double dx = sep_fast(xs[j], px, g.box[0], half[0], g.periodic);
+        const double dy = sep_fast(xs[n + j], py, g.box[1], half[1], g.periodic);
+        const double dz = sep_fast(xs[2 * n + j], pz, g.box[2], half[2], g.periodic);
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        if (r2 < R2) f(r2 > 0.0 ? sqrt_fast(r2) : 0.0);
+    };
+    // this lane's candidates closer than R
+    auto walk = [&](double R, auto&& f) {
+        const float Rf = (float)R * 1.0001f, R2f = Rf * Rf;
+        int seen = 0;     // candidates of the earlier ranges (walk order)
+        for_each_candidate_range(g, pxf, pyf, pzf, Rf, [&](int b, int e) {
+            for (int j = b + ((lane - seen) & (kRefineLanes - 1)); j < e; j += kRefineLanes) visit(j, R2f, R * R, f);
+            seen += e - b;
+        });
+    };
+    const double Rc = kKappa * hd * (1.0 + kNear);
+    double r[kRefineSlots];
+    int cnt = 0;
+    if (list_cnt >= 0) {
+        const float Rf = (float)Rc * 1.0001f;
+        for (int k = lane; k < list_cnt; k += kRefineLanes)
+            visit(list[k], Rf * Rf, Rc * Rc, [&](double rr) {
+#pragma unroll
+                for (int u = 0; u < kRefineSlots; ++u)   // static indices keep r in registers
+                    if (u == cnt) r[u] = rr;
+                ++cnt;
+            });
+    }
+    bool kept = list_cnt >= 0 && !__any_sync(group, cnt > kRefineSlots);
+    double lod = 0.0, hid = INFINITY;
+    for (int it = 0; it < 60; ++it) {
+        const double H = kKappa * hd, iH = rcp_fast(H);
+        kept = kept && H <= Rc;
+        double S = 0.0, D = 0.0;      // S and sum q w'(q) = -h dS/dh
+        auto term = [&](double rr) {
+            const double q = rr * iH;
+            if (q < 1.0) {
+                const double a = 1.0 - q, a2 = a * a;
+                double w = a2 * a, d = -3.0 * a2;
+                if (q < 0.5) {
+                    const double b = 0.5 - q, b2 = b * b;
+                    w -= 4.0 * (b2 * b);
+                    d += 12.0 * b2;
+                }
+                S += w;
+                D += q * d;
+            }
+        };
+        if (kept) {
+#pragma unroll
+            for (int k = 0; k < kRefineSlots; ++k)
+                if (k < cnt) term(r[k]);
+        } else {
+            walk(H, term);
+        }
+#pragma unroll
+        for (int o = kRefineLanes / 2; o > 0; o >>= 1) {
+            S += __shfl_xor_sync(group, S, o);
+            D += __shfl_xor_sync(group, D, o);
+        }
+        const double f = S - hp.s_star;
+        if (f < 0.0) lod = hd; else hid = hd;
+        const double step = D < 0.0 ? -f * hd * rcp_fast(D) : INFINITY;
+        if (fabs(step) <= 1e-8 * hd) {
+            hd -= step;
+            om_d = hp.eta3 * rcp_fast(hd * hd * hd);
+            return true;
+        }
+        if (hid - lod <= 1e-14 * hd) {
+            om_d = kSigma * iH * iH * iH * S;
+            return true;
+        }
+        double hn = hd - step;
+        if (it >= 12 || !(hn > lod && hn < hid)) hn = isinf(hid) ? 1.01 * hd : 0.5 * (lod + hid);
+        hd = hn;
+    }
+    return false;
 }
 
 // Smoothing lengths given by the caller (rt_neighbours_given_h): h_i from h_in (caller order)
@@ -648,30 +815,46 @@ __global__ void k_h_given(Grid g, const double* __restrict__ xs, const uint4* __
     }
 }
 
-// Float path: the double phase for the particles k_h_solve flagged, one warp per particle
-// (grid-stride over the list; its order is arbitrary, and each particle's result depends on
-// its own position and neighbours only).  The smallest and largest h are widened to the
+// The double phase, kRefineLanes lanes per particle: for the particles k_h_lists flagged (todo,
+// of arbitrary order; each particle's result depends on its own position and neighbours
+// only), or for all of them when todo is NULL.  The smallest and largest h are widened to the
 // refined values (the pair search's bound must cover them).
-__global__ void k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
-                           HParams hp, const int32_t* __restrict__ list, const int* __restrict__ count, double* h_out,
-                           double* omega_out, float* H2f_out, unsigned long long* hminmax, int* flags) {
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int cnt = *count;
+__global__ void __launch_bounds__(128)
+k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
+           const int32_t* __restrict__ todo, const int* __restrict__ count, const int32_t* __restrict__ list,
+           int32_t* list_cnt, int cap, double* h_out, double* omega_out, float* H2f_out, uint4* xq_out,
+           unsigned long long* hminmax, int* flags) {
+    const int lane = threadIdx.x & (kRefineLanes - 1);
+    const unsigned group = ((1u << kRefineLanes) - 1u) << (threadIdx.x & 31 & ~(kRefineLanes - 1));
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kRefineLanes;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) / kRefineLanes;
+    const int64_t cnt = todo ? (int64_t)*count : n;
+    double mn = INFINITY, mx = 0.0, h3 = 0.0;
     for (int64_t t = w0; t < cnt; t += nw) {
-        const int64_t p = list[t];
-        double hd = h_out[p], om_d = omega_out[p];
-        const bool ok = refine_h_warp_cached(g, xs, xq, n, hp, p, lane, hd, om_d);
+        const int64_t p = todo ? (int64_t)todo[t] : t;
+        const double h0 = h_out[p];
+        double hd = h0, om_d = omega_out[p];
+        const bool ok = refine_h(g, xs, xq, n, hp, p, lane, group, list + p * cap, list_cnt[p], hd, om_d);
         if (lane == 0) {
             if (!ok) atomicExch(&flags[F_NOCONV], 1);
             h_out[p] = hd;
             omega_out[p] = om_d;
             const double Hd = kKappa * hd;
             H2f_out[p] = (float)(Hd * Hd);
-            atomic_min_pos(&hminmax[0], hd);
-            atomic_max_pos(&hminmax[1], hd);
+            reinterpret_cast<unsigned*>(xq_out + p)[3] = __float_as_uint((float)(Hd * Hd));
+            // a root beyond the list's margin (an edge where f' nearly vanishes): no list
+            if (hd > h0 * (1.0 + kNear)) list_cnt[p] = -1;
+            mn = fmin(mn, hd);
+            mx = fmax(mx, hd);
+            h3 += Hd * Hd * Hd;
         }
+    }
+    warp_minmax(mn, mx);
+    for (int o = 16; o > 0; o >>= 1) h3 += __shfl_xor_sync(0xffffffffu, h3, o);
+    if ((threadIdx.x & 31) == 0 && mx > 0.0) {
+        atomic_min_pos(&hminmax[0], mn);
+        atomic_max_pos(&hminmax[1], mx);
+        if (!todo) atomicAdd(reinterpret_cast<double*>(&hminmax[4]), h3);
     }
 }
 
@@ -679,277 +862,271 @@ __global__ void k_h_refine(Grid g, const double* __restrict__ xs, const uint4* _
 // a3: symmetric pair lists { j != i : r_ij < max(H_i, H_j) }.  A float test on the
 // fixed-point separation decides all pairs except those within 1e-5 of the threshold,
 // which are decided by the exact double test (r^2 and H^2 without contraction).
+//
+// Each particle looks only inside its own support: its list of candidates, or a walk where
+// that overflowed.  An entry (i, j) that j does not have in its own support (H_j <= r < H_i) is
+// handed to row j as an extra; the row is its own entries merged with its extras, in
+// ascending order whatever order the extras arrived in.  Searching out to the largest H_j that
+// could reach i instead visits 2.5 times the candidates (0.43 ms on 262,144 particles), and
+// on strongly clustered sets no bound is local enough: there every entry and its transpose
+// were sorted as 64-bit keys (7.8 of 15.6 ms on 1,000,000 particles).
 struct PairParams {
     float scale[3];
-    double Hmax;
 };
 
-// Local search radii of the direct pair search.  A pair with r_ij < H_j > H_i must be found
-// from i, so i searches out to max(H_i, H_j) for every j that can reach it.  Over a coarse
-// grid of at most 16^3 blocks, Hb[B] is the largest H in block B and Hreach[A] the largest
-// Hb[B] over the blocks B whose box lies within Hb[B] of A's box (A included): every j that
-// reaches a particle of A has H_j <= Hreach[A], so max(H_i, Hreach[A]) bounds i's search.
-struct Blocks {
-    int nb[3];
-    double len[3];      // block edge per axis
-    int reach[3];       // blocks per axis within H_max of a block (no block farther can qualify)
-    int periodic;
-};
+// extra entries carry this bit beside their index (particle numbers stay below 2^31)
+constexpr uint32_t kAsym = 0x80000000u;
 
-__device__ __forceinline__ int block_of(const Blocks& bk, double x, double y, double z) {
-    const double p[3] = {x, y, z};
-    int b[3];
-    for (int a = 0; a < 3; ++a) {
-        int v = (int)floor(p[a] / bk.len[a]);
-        b[a] = v < 0 ? 0 : (v >= bk.nb[a] ? bk.nb[a] - 1 : v);
-    }
-    return (b[2] * bk.nb[1] + b[1]) * bk.nb[0] + b[0];
+// the exact double test of r_pj < H_k (no contraction), as a plain double evaluation would do it;
+// a call, because it is rare and its registers would halve the occupancy of the search
+__device__ __noinline__ bool inside_exact(const double* __restrict__ xs, double hk, int64_t n, double b0, double b1,
+                                          double b2, int periodic, int64_t p, int j) {
+    const double H = __dmul_rn(kKappa, hk);
+    const double ex = sep_exact(xs[j], xs[p], b0, periodic);
+    const double ey = sep_exact(xs[n + j], xs[n + p], b1, periodic);
+    const double ez = sep_exact(xs[2 * n + j], xs[2 * n + p], b2, periodic);
+    return norm2_exact(ex, ey, ez) < __dmul_rn(H, H);
 }
 
-// Hb (float bits, ordered like integers for H > 0) of every block; the lanes of a warp that
-// fall in the same block (particles are sorted by cell) combine before one atomic
-// Also stores each particle's float H^2 in the free word of its position record, so that the
-// pair search reads a candidate's position and support radius with one 16-byte load.
-__global__ void k_block_hmax(const double* __restrict__ xs, const float* __restrict__ H2f, int64_t n, Blocks bk,
-                             unsigned* __restrict__ hb, uint4* __restrict__ xq) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool in = p < n;
-    const int b = in ? block_of(bk, xs[p], xs[n + p], xs[2 * n + p]) : -1;
-    const float h2 = in ? H2f[p] : 0.f;
-    if (in) reinterpret_cast<unsigned*>(xq + p)[3] = __float_as_uint(h2);
-    const unsigned v = in ? __float_as_uint(sqrtf(h2)) : 0u;
-    const unsigned peers = __match_any_sync(0xffffffffu, b);
-    const unsigned m = __reduce_max_sync(peers, v);
-    if (in && (threadIdx.x & 31) == __ffs(peers) - 1) atomicMax(&hb[b], m);
+// is r_pj < H of the particle whose float H^2 is H2 and whose h is h[k]?
+__device__ __forceinline__ bool inside(const Grid& g, const double* __restrict__ xs, const double* __restrict__ h,
+                                       int64_t n, float r2, float H2, int64_t k, int64_t p, int j) {
+    if (r2 < H2 * (1.f - 1e-5f)) return true;
+    if (r2 > H2 * (1.f + 1e-5f)) return false;
+    return inside_exact(xs, h[k], n, g.box[0], g.box[1], g.box[2], g.periodic, p, j);
 }
 
-// Hreach of every block: one warp per block A, its lanes scanning the blocks B within
-// bk.reach blocks of A along each axis (each block once, also where that span wraps)
-__global__ void k_block_reach(const unsigned* __restrict__ hb, Blocks bk, float* __restrict__ reach) {
-    const int nbt = bk.nb[0] * bk.nb[1] * bk.nb[2];
-    const int A = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-    const int lane = threadIdx.x & 31;
-    if (A >= nbt) return;      // whole warps
-    const int a[3] = {A % bk.nb[0], (A / bk.nb[0]) % bk.nb[1], A / (bk.nb[0] * bk.nb[1])};
-    const float len[3] = {(float)bk.len[0], (float)bk.len[1], (float)bk.len[2]};
-    // the scanned span per axis: [a - k, a + k] wrapped (or clipped), or the whole axis
-    int lo[3], w[3];
-    for (int x = 0; x < 3; ++x) {
-        const int k = bk.reach[x];
-        if (2 * k + 1 >= bk.nb[x]) {
-            lo[x] = 0;
-            w[x] = bk.nb[x];
-        } else if (bk.periodic) {
-            lo[x] = a[x] - k;
-            w[x] = 2 * k + 1;
-        } else {
-            lo[x] = max(a[x] - k, 0);
-            w[x] = min(a[x] + k, bk.nb[x] - 1) - lo[x] + 1;
-        }
-    }
-    const int span = w[0] * w[1] * w[2];
-    unsigned r = hb[A];
-    for (int t = lane; t < span; t += 32) {
-        int b[3] = {lo[0] + t % w[0], lo[1] + (t / w[0]) % w[1], lo[2] + t / (w[0] * w[1])};
-        for (int x = 0; x < 3; ++x) b[x] = (b[x] % bk.nb[x] + bk.nb[x]) % bk.nb[x];
-        const int Bi = (b[2] * bk.nb[1] + b[1]) * bk.nb[0] + b[0];
-        const unsigned hbB = hb[Bi];
-        if (hbB <= r) continue;
-        const float Hb = __uint_as_float(hbB);
-        float d2 = 0.f;
-        for (int x = 0; x < 3; ++x) {
-            int d = abs(a[x] - b[x]);
-            if (bk.periodic) d = min(d, bk.nb[x] - d);
-            const float gap = d > 1 ? (d - 1) * len[x] : 0.f;
-            d2 += gap * gap;
-        }
-        // the gap between the boxes, with a relative margin against rounding
-        if (d2 < Hb * Hb * 1.0002f) r = hbB;
-    }
-    r = __reduce_max_sync(0xffffffffu, r);
-    if (lane == 0) reach[A] = __uint_as_float(r);
+// candidate j of particle p (the whole warp calls): own entry?  asym: not one of j's own
+__device__ __forceinline__ bool own_entry(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq,
+                                          const double* __restrict__ h, int64_t n, const PairParams& pp, int64_t p,
+                                          const uint4& qp, int j, bool valid, bool& asym) {
+    asym = false;
+    if (!valid || j == p) return false;
+    const uint4 qj = xq[j];
+    const float dx = fsep(qj.x, qp.x, pp.scale[0]);
+    const float dy = fsep(qj.y, qp.y, pp.scale[1]);
+    const float dz = fsep(qj.z, qp.z, pp.scale[2]);
+    const float r2 = dx * dx + dy * dy + dz * dz;
+    if (!inside(g, xs, h, n, r2, __uint_as_float(qp.w), p, p, j)) return false;
+    asym = !inside(g, xs, h, n, r2, __uint_as_float(qj.w), j, p, j);
+    return true;
 }
 
-// FILL = false counts each row into counts[p]; with cap > 0 it also writes the first cap
-// entries of row p to cols[p cap ...] and raises *row_max to the longest row.  FILL = true
-// writes row p to cols[row_off[p] ...].  Both walk the candidates in ascending index, so
-// every row comes out in ascending column order.
-template <bool FILL>
-__global__ void k_pairs(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq,
-                        const double* __restrict__ h, const float* __restrict__ H2f, int64_t n, PairParams pp,
-                        Blocks bk, const float* __restrict__ reach, int32_t* counts,
-                        const int64_t* __restrict__ row_off, int32_t* cols, int cap = 0, int* row_max = nullptr) {
-    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int cnt = 0;
-    if (p < n) {
-        const uint4 q4p = xq[p];
-        uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-        double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-        const float H2i = H2f[p];
-        const float Hr = reach[block_of(bk, px, py, pz)];
-        float R = sqrtf(fmaxf(H2i, Hr * Hr)) * 1.0001f;
-        int64_t base = FILL ? row_off[p] : p * (int64_t)cap;
-        for_each_candidate_q<true>(g, xq, (float)px, (float)py, (float)pz, R, [&](int j, uint4 qj) {
-            if (j == p) return;
-            float dx = fsep(qj.x, qx, pp.scale[0]);
-            float dy = fsep(qj.y, qy, pp.scale[1]);
-            float dz = fsep(qj.z, qz, pp.scale[2]);
-            float r2f = dx * dx + dy * dy + dz * dz;
-            float H2m = fmaxf(H2i, __uint_as_float(qj.w));   // H_j^2 (k_block_hmax)
-            bool in;
-            if (r2f < H2m * (1.f - 1e-5f)) in = true;
-            else if (r2f > H2m * (1.f + 1e-5f)) in = false;
-            else {
-                // exact double test (no contraction), as a plain double evaluation would do it
-                double Hm = fmax(__dmul_rn(kKappa, h[p]), __dmul_rn(kKappa, h[j]));
-                double ex = sep_exact(xs[j], px, g.box[0], g.periodic);
-                double ey = sep_exact(xs[n + j], py, g.box[1], g.periodic);
-                double ez = sep_exact(xs[2 * n + j], pz, g.box[2], g.periodic);
-                in = norm2_exact(ex, ey, ez) < __dmul_rn(Hm, Hm);
-            }
-            if (in) {
-                if (FILL || cnt < cap) cols[base + cnt] = j;
-                ++cnt;
-            }
-        });
-        if (!FILL) counts[p] = cnt;
-    }
-    if (!FILL && row_max) {   // every lane of the (full) warp takes part
-        const int m = __reduce_max_sync(0xffffffffu, cnt);
-        if ((threadIdx.x & 31) == 0) atomicMax(row_max, m);
-    }
+// extras that a row holds in place; a row that gets more has them filled in a second pass
+constexpr int kExtras = 32;
+
+// hands the asymmetric entry (p, j) to row j
+__device__ __forceinline__ void hand_extra(int32_t* extra, int32_t* extras, int64_t p, int j) {
+    const int k = atomicAdd(&extra[j], 1);
+    if (k < kExtras) extras[(int64_t)j * kExtras + k] = (int32_t)p;
 }
 
-// rows of cap entries (k_pairs' counting walk) -> CSR rows at row_off, one warp per row
-__global__ void k_rows_compact(const int32_t* __restrict__ cols_cap, int64_t cap, const int64_t* __restrict__ row_off,
-                               int64_t n, int32_t* __restrict__ cols) {
+// One warp per particle: own entries, with their asymmetry bit, over the front of the list
+// (each round's reads come before its writes, which lie no further back); their number; and the
+// extras of the other rows.  Two rounds of 32 candidates are in flight together.  Particles
+// without a list go to `over`, for k_own_walk.
+__global__ void __launch_bounds__(256, 5)
+k_own_rows(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
+           int64_t n, PairParams pp, int32_t* list, int cap, const int32_t* __restrict__ list_cnt,
+           int32_t* __restrict__ own, int32_t* extra, int32_t* __restrict__ extras, int32_t* over, int* over_n) {
     const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (p >= n) return;
-    const int64_t b = row_off[p], m = row_off[p + 1] - b;
-    for (int64_t k = lane; k < m; k += 32) cols[b + k] = cols_cap[p * cap + k];
-}
-
-
-// Rows sorted ascending are [lower neighbours j < i | upper neighbours j > i].  Each
-// unordered pair is the upper entry of its lower particle; slot(i, j) numbers those entries.
-__global__ void k_row_split(const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols, int64_t n,
-                            int32_t* n_low, int32_t* n_up) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t lo = row_off[i], hi = row_off[i + 1];
-    int64_t b = lo, e = hi;
-    while (b < e) {
-        int64_t m = (b + e) >> 1;
-        if (cols[m] < (int32_t)i) b = m + 1; else e = m;
+    const int had = list_cnt[p];
+    if (had < 0) {
+        if (lane == 0) over[atomicAdd(over_n, 1)] = (int32_t)p;
+        return;
     }
-    n_low[i] = (int32_t)(b - lo);
-    n_up[i] = (int32_t)(hi - b);
-}
-
-// the two particles of every pair slot
-__global__ void k_pair_ends(const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols,
-                            const int32_t* __restrict__ n_low, const int64_t* __restrict__ up_off, int64_t n,
-                            int2* ends) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    int64_t e0 = row_off[i] + n_low[i], e1 = row_off[i + 1], slot = up_off[i];
-    for (int64_t e = e0; e < e1; ++e, ++slot) ends[slot] = make_int2((int)i, cols[e]);
-}
-
-// for every lower entry (i, k), k < i: the slot of the pair in k's upper list.  One warp per
-// particle, its lanes taking the lower entries (each a binary search in row k's upper part).
-__global__ void k_low_slots(const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols,
-                            const int32_t* __restrict__ n_low, const int64_t* __restrict__ up_off, int64_t n,
-                            int32_t* low_slot) {
-    const int64_t i = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (i >= n) return;
-    int64_t r0 = row_off[i];
-    int64_t lbase = r0 - up_off[i];       // lower entries before row i
-    for (int e = lane; e < n_low[i]; e += 32) {
-        int k = cols[r0 + e];
-        int64_t b = row_off[k] + n_low[k], hi = row_off[k + 1], t = hi;
-        while (b < t) {
-            int64_t m = (b + t) >> 1;
-            if (cols[m] < (int32_t)i) b = m + 1; else t = m;
+    const uint4 qp = xq[p];
+    int32_t* row = list + p * cap;
+    int c = 0;
+    for (int t0 = 0; t0 < had; t0 += 64) {
+        int j[2];
+        bool in[2], asym[2];
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const int t = t0 + 32 * u + lane;
+            j[u] = t < had ? row[t] : (int)p;
         }
-        low_slot[lbase + e] = (int32_t)(up_off[k] + (b - row_off[k] - n_low[k]));
-    }
-}
-
-// Pair search for strongly varying h: each particle lists only { j : r_ij < H_i } (its own
-// support) and emits the entry and its transpose as 64-bit keys (row << 32 | col); sorting
-// and removing duplicates gives the same symmetric lists, rows ascending, without any
-// particle searching out to the largest H of the set.
-template <bool FILL>
-__global__ void k_pairs_gather(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq,
-                               const double* __restrict__ h, const float* __restrict__ H2f, int64_t n, PairParams pp,
-                               int32_t* counts, const int64_t* __restrict__ off, uint64_t* keys) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const uint4 q4p = xq[p];
-    uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    const float H2i = H2f[p];
-    int cnt = 0;
-    int64_t base = FILL ? off[p] : 0;
-    for_each_candidate(g, (float)px, (float)py, (float)pz, sqrtf(H2i) * 1.0001f, [&](int j) {
-        if (j == p) return;
-        float dx = fsep(xq[j].x, qx, pp.scale[0]);
-        float dy = fsep(xq[j].y, qy, pp.scale[1]);
-        float dz = fsep(xq[j].z, qz, pp.scale[2]);
-        float r2f = dx * dx + dy * dy + dz * dz;
-        bool in;
-        if (r2f < H2i * (1.f - 1e-5f)) in = true;
-        else if (r2f > H2i * (1.f + 1e-5f)) in = false;
-        else {
-            double Hi = __dmul_rn(kKappa, h[p]);
-            double ex = sep_exact(xs[j], px, g.box[0], g.periodic);
-            double ey = sep_exact(xs[n + j], py, g.box[1], g.periodic);
-            double ez = sep_exact(xs[2 * n + j], pz, g.box[2], g.periodic);
-            in = norm2_exact(ex, ey, ez) < __dmul_rn(Hi, Hi);
-        }
-        if (in) {
-            if (FILL) {
-                keys[2 * (base + cnt)] = ((uint64_t)p << 32) | (uint32_t)j;
-                keys[2 * (base + cnt) + 1] = ((uint64_t)(uint32_t)j << 32) | (uint64_t)p;
+#pragma unroll
+        for (int u = 0; u < 2; ++u) in[u] = own_entry(g, xs, xq, h, n, pp, p, qp, j[u], true, asym[u]);
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            const unsigned m = __ballot_sync(0xffffffffu, in[u]);
+            if (in[u]) {
+                row[c + __popc(m & ((1u << lane) - 1u))] = (int32_t)((uint32_t)j[u] | (asym[u] ? kAsym : 0u));
+                if (asym[u]) hand_extra(extra, extras, p, j[u]);
             }
-            ++cnt;
+            c += __popc(m);
         }
-    });
-    if (!FILL) counts[p] = cnt;
+    }
+    if (lane == 0) own[p] = c;
 }
 
-// unique sorted keys -> columns, and the number of entries of every row
-__global__ void k_keys_to_csr(const uint64_t* __restrict__ ukeys, const int64_t* __restrict__ nuniq, int32_t* cols,
-                              int32_t* counts) {
-    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= *nuniq) return;
-    uint64_t k = ukeys[e];
-    cols[e] = (int32_t)(uint32_t)(k & 0xffffffffu);
-    atomicAdd(&counts[(int64_t)(k >> 32)], 1);
+// The particles without a list, by walks, a warp each: their number of own entries, with room
+// for them reserved in the spill (its offset goes to the unused list); FILL writes them there.
+template <bool FILL>
+__global__ void __launch_bounds__(128)
+k_own_walk(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
+           int64_t n, PairParams pp, int32_t* list, int cap, int32_t* __restrict__ own, int32_t* extra,
+           int32_t* __restrict__ extras, const int32_t* __restrict__ over, const int* __restrict__ over_n,
+           unsigned long long* spill_n, int32_t* __restrict__ spill) {
+    const int lane = threadIdx.x & 31;
+    const int nw = (gridDim.x * blockDim.x) >> 5, m = *over_n;
+    for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < m; w += nw) {
+        const int64_t p = over[w];
+        const uint4 qp = xq[p];
+        unsigned long long* where = reinterpret_cast<unsigned long long*>(list + p * cap);
+        int32_t* out = FILL ? spill + *where : nullptr;
+        int c = 0;
+        warp_walk(g, (float)qp.x * pp.scale[0], (float)qp.y * pp.scale[1], (float)qp.z * pp.scale[2],
+                  sqrtf(__uint_as_float(qp.w)) * 1.0001f, lane, [&](int j, bool valid) {
+                      bool asym;
+                      const bool in = own_entry(g, xs, xq, h, n, pp, p, qp, j, valid, asym);
+                      const unsigned b = __ballot_sync(0xffffffffu, in);
+                      if (in) {
+                          if (FILL) out[c + __popc(b & ((1u << lane) - 1u))] = (int32_t)((uint32_t)j | (asym ? kAsym : 0u));
+                          else if (asym) hand_extra(extra, extras, p, j);
+                      }
+                      c += __popc(b);
+                      return true;
+                  });
+        if (!FILL && lane == 0) {
+            own[p] = c;
+            *where = atomicAdd(spill_n, (unsigned long long)c);
+        }
+    }
+}
+
+// row lengths, own entries and extras; and how many extras the rows have that hold more than
+// kExtras (their offsets come from a scan, their sum decides whether the second pass runs)
+__global__ void k_row_lengths(const int32_t* __restrict__ own, const int32_t* __restrict__ extra, int64_t n,
+                              int32_t* __restrict__ counts, unsigned long long* more) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p > n) return;
+    const int e = p < n ? extra[p] : 0;
+    counts[p] = p < n ? own[p] + e : 0;
+    if (e > kExtras) atomicAdd(more, (unsigned long long)e);
+}
+__global__ void k_more_extras(const int32_t* __restrict__ extra, int64_t n, int32_t* __restrict__ more) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p <= n) more[p] = p < n && extra[p] > kExtras ? extra[p] : 0;
+}
+
+// second pass for those rows: every asymmetric entry (p, j) again, any order
+__global__ void __launch_bounds__(256)
+k_extras_fill(int64_t n, const int32_t* __restrict__ list, int cap, const int32_t* __restrict__ list_cnt,
+              const int32_t* __restrict__ own, const int32_t* __restrict__ extra, const int64_t* __restrict__ off,
+              int32_t* fill, const int32_t* __restrict__ spill, int32_t* __restrict__ out) {
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (p >= n) return;
+    const int32_t* row = list + p * cap;
+    if (list_cnt[p] < 0) row = spill + *reinterpret_cast<const unsigned long long*>(row);
+    for (int t = lane; t < own[p]; t += 32) {
+        const uint32_t v = (uint32_t)row[t];
+        if (!(v & kAsym)) continue;
+        const int j = (int)(v & ~kAsym);
+        if (extra[j] > kExtras) out[off[j] + atomicAdd(&fill[j], 1)] = (int32_t)p;
+    }
+}
+
+// Row p: own entries (ascending) merged with its extras (any order) by rank, one warp per row; and
+// the row's split into lower neighbours j < p and upper ones j > p.  Each unordered pair is the
+// upper entry of its lower particle; slot(i, j) numbers those entries.
+__global__ void __launch_bounds__(256)
+k_rows_merge(int64_t n, const int32_t* __restrict__ list, int cap, const int32_t* __restrict__ list_cnt,
+             const int32_t* __restrict__ own, const int32_t* __restrict__ extra, const int32_t* __restrict__ extras,
+             const int64_t* __restrict__ more_off, const int32_t* __restrict__ more,
+             const int32_t* __restrict__ spill, const int64_t* __restrict__ row_off, int32_t* __restrict__ cols,
+             int32_t* __restrict__ n_low, int32_t* __restrict__ n_up) {
+    const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (p >= n) return;
+    const int32_t* row = list + p * cap;
+    if (list_cnt[p] < 0) row = spill + *reinterpret_cast<const unsigned long long*>(row);
+    const int m = own[p], E = extra[p];
+    const int32_t* ex = E > kExtras ? more + more_off[p] : extras + p * kExtras;
+    int32_t* out = cols + row_off[p];
+    int low = 0;
+    auto below = [&](int v) {     // extras smaller than v
+        int c = 0;
+        for (int k = 0; k < E; ++k) c += ex[k] < v ? 1 : 0;
+        return c;
+    };
+    for (int t = lane; t < m; t += 32) {
+        const int v = (int)((uint32_t)row[t] & ~kAsym);
+        low += v < p ? 1 : 0;
+        out[t + below(v)] = v;
+    }
+    for (int k = lane; k < E; k += 32) {
+        const int v = ex[k];
+        low += v < p ? 1 : 0;
+        int b = 0, e = m;         // own entries smaller than v
+        while (b < e) {
+            const int u = (b + e) >> 1;
+            if ((int)((uint32_t)row[u] & ~kAsym) < v) b = u + 1; else e = u;
+        }
+        out[b + below(v)] = v;
+    }
+    low = __reduce_add_sync(0xffffffffu, low);
+    if (lane == 0) {
+        n_low[p] = low;
+        n_up[p] = m + E - low;
+    }
+}
+
+// The two particles of every pair slot, and for every lower entry (i, k), k < i, the slot of the
+// pair in k's upper list.  One warp per particle k, its lanes taking the upper entries: the
+// slots are written side by side, and k's place among the lower entries of each l is found by a
+// binary search.
+__global__ void __launch_bounds__(256)
+k_pair_slots(const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols,
+             const int32_t* __restrict__ n_low, const int64_t* __restrict__ up_off, int64_t n,
+             int2* __restrict__ ends, int32_t* __restrict__ low_slot) {
+    const int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    if (k >= n) return;
+    const int64_t e0 = row_off[k] + n_low[k], s0 = up_off[k];
+    const int m = (int)(up_off[k + 1] - s0);
+    for (int t = lane; t < m; t += 32) {
+        const int l = cols[e0 + t];
+        const int64_t slot = s0 + t, r = row_off[l];
+        ends[slot] = make_int2((int)k, l);
+        const int32_t* row = cols + r;
+        int b = 0, e = n_low[l];
+        while (b < e) {
+            const int u = (b + e) >> 1;
+            if (row[u] < (int32_t)k) b = u + 1; else e = u;
+        }
+        low_slot[r - up_off[l] + b] = (int32_t)slot;      // r - up_off[l]: lower entries before row l
+    }
 }
 
 // ------------------------------------------------------------------------------------
 // a4: E_i = sum_j psi_j(x_i) d d^T, B_i = E_i^-1 (double), and the per-particle factors used
 // by the pair kernels.
-__device__ void sym3_eigs(double a, double b, double c, double d, double e, double f, double ev[3]) {
+template <class T>
+__device__ __forceinline__ void sym3_eigs(T a, T b, T c, T d, T e, T f, T ev[3]) {
     // symmetric [[a d e][d b f][e f c]]: trigonometric closed form
-    double p1 = d * d + e * e + f * f;
-    double q = (a + b + c) / 3.0;
-    if (p1 == 0.0) { ev[0] = a; ev[1] = b; ev[2] = c; return; }
-    double p2 = (a - q) * (a - q) + (b - q) * (b - q) + (c - q) * (c - q) + 2.0 * p1;
-    double p = sqrt(p2 / 6.0);
-    double ip = 1.0 / p;
-    double B00 = (a - q) * ip, B11 = (b - q) * ip, B22 = (c - q) * ip, B01 = d * ip, B02 = e * ip, B12 = f * ip;
-    double detB = B00 * (B11 * B22 - B12 * B12) - B01 * (B01 * B22 - B12 * B02) + B02 * (B01 * B12 - B11 * B02);
-    double r = fmin(fmax(detB / 2.0, -1.0), 1.0);
-    double phi = acos(r) / 3.0;
-    ev[0] = q + 2.0 * p * cos(phi);
-    ev[2] = q + 2.0 * p * cos(phi + 2.0943951023931954923);
-    ev[1] = 3.0 * q - ev[0] - ev[2];
+    const T p1 = d * d + e * e + f * f;
+    const T q = (a + b + c) / T(3);
+    if (p1 == T(0)) { ev[0] = a; ev[1] = b; ev[2] = c; return; }
+    const T p2 = (a - q) * (a - q) + (b - q) * (b - q) + (c - q) * (c - q) + T(2) * p1;
+    const T p = sqrt(p2 / T(6));
+    const T ip = T(1) / p;
+    const T B00 = (a - q) * ip, B11 = (b - q) * ip, B22 = (c - q) * ip, B01 = d * ip, B02 = e * ip, B12 = f * ip;
+    const T detB = B00 * (B11 * B22 - B12 * B12) - B01 * (B01 * B22 - B12 * B02) + B02 * (B01 * B12 - B11 * B02);
+    const T phi = acos(fmin_(fmax_(detB / T(2), T(-1)), T(1))) / T(3);
+    ev[0] = q + T(2) * p * cos(phi);
+    ev[2] = q + T(2) * p * cos(phi + T(2.0943951023931954923));
+    ev[1] = T(3) * q - ev[0] - ev[2];
 }
+
+// cond_2 from the float eigenvalues of E / tr E (exact to 1e-6 cond) serves all but the largest
+// of the set and those above kCondFloat, whose value is taken in double (k_cond): the double
+// closed form, an arccosine and two cosines, was most of the geometry's double instructions.
+constexpr float kCondFloat = 1e3f;
 
 template <class T>
 __device__ __forceinline__ void store_pos(void* pos, int64_t p, const double* xs, const uint4* xq, int64_t n);
@@ -968,17 +1145,6 @@ __device__ __forceinline__ void store_pos<double>(void* pos, int64_t p, const do
 // Float path: separations from the fixed-point positions, weights in float and a
 // compensated (Kahan) float sum, so that E_i keeps ~1e-8 relative accuracy before its
 // inversion in double.
-struct Kahan {
-    float s = 0.f, c = 0.f;
-    __device__ __forceinline__ void add(float v) {
-        float y = v - c;
-        float t = s + y;
-        c = (t - s) - y;
-        s = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)s - (double)c; }
-};
-
 template <class T>
 __device__ __forceinline__ void accumulate_E(const double* xs, const uint4* xq, const double* box, int periodic,
                                              float s0, float s1, float s2, int64_t n, int64_t p, double H,
@@ -1034,17 +1200,19 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
                            const double* __restrict__ h, const double* __restrict__ omega,
                            const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols, int64_t n, double b0,
                            double b1, double b2, int periodic, float s0, float s1, float s2, double* V_out,
-                           double* B_out, double* cond_out, void* pos_t, T* geo_t, T* om_t,
-                           unsigned long long* red, int* flags) {
+                           double* B_out, float* cond_out, void* pos_t, T* geo_t, T* om_t,
+                           unsigned long long* red, unsigned* cond_max, int* flags) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    double cond = 0.0, V = INFINITY;
+    float cond = 0.f;
+    double V = INFINITY;
     if (p < n) {
         const double box[3] = {b0, b1, b2};
-        double hi = h[p], H = kKappa * hi, iH = 1.0 / H;
+        double hi = h[p], H = kKappa * hi, iH = rcp_fast(H);
         double om = omega[p];
         double E[6];
         accumulate_E<T>(xs, xq, box, periodic, s0, s1, s2, n, p, H, row_off, cols, E);
-        double fac = kSigma * iH * iH * iH / om;   // psi = fac * w
+        V = rcp_fast(om);
+        const double s3 = kSigma * iH * iH * iH, fac = s3 * V;   // psi = fac * w
         double e_xx = E[0] * fac, e_yy = E[1] * fac, e_zz = E[2] * fac;
         double e_xy = E[3] * fac, e_xz = E[4] * fac, e_yz = E[5] * fac;
         // cofactor inverse of the symmetric matrix
@@ -1052,7 +1220,6 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
         double c_xy = e_xz * e_yz - e_xy * e_zz;
         double c_xz = e_xy * e_yz - e_xz * e_yy;
         double det = e_xx * c_xx + e_xy * c_xy + e_xz * c_xz;
-        V = 1.0 / om;
         V_out[p] = V;
         store_pos<T>(pos_t, p, xs, xq, n);
         if (!(det > 0.0) || !(om > 0.0)) {
@@ -1060,10 +1227,9 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
             for (int k = 0; k < 6; ++k) B_out[k * n + p] = 0.0;
             for (int k = 0; k < 8; ++k) geo_t[8 * p + k] = (T)0;
             om_t[p] = (T)0;
-            cond_out[p] = INFINITY;
-            cond = INFINITY;
+            cond_out[p] = 0.f;     // the call fails
         } else {
-            double id = 1.0 / det;
+            const double id = rcp_fast(det);
             double B[6];
             B[0] = c_xx * id;
             B[1] = (e_xx * e_zz - e_xz * e_xz) * id;
@@ -1071,14 +1237,14 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
             B[3] = c_xy * id;
             B[4] = c_xz * id;
             B[5] = (e_xy * e_xz - e_xx * e_yz) * id;
-            double ev[3];
-            sym3_eigs(e_xx, e_yy, e_zz, e_xy, e_xz, e_yz, ev);
-            double lmin = fmin(ev[0], fmin(ev[1], ev[2])), lmax = fmax(ev[0], fmax(ev[1], ev[2]));
-            cond = lmin > 0 ? lmax / lmin : INFINITY;
+            const float it = 1.f / (float)(e_xx + e_yy + e_zz);
+            float ev[3];
+            sym3_eigs((float)e_xx * it, (float)e_yy * it, (float)e_zz * it, (float)e_xy * it, (float)e_xz * it,
+                      (float)e_yz * it, ev);
+            const float lmin = fminf(ev[0], fminf(ev[1], ev[2])), lmax = fmaxf(ev[0], fmaxf(ev[1], ev[2]));
+            cond = lmin > 0.f ? lmax / lmin : INFINITY;
             cond_out[p] = cond;
-            if (!(lmin > 0)) atomicExch(&flags[F_GEOM], 1);
-            if (cond > 1e10) atomicAdd(&flags[F_ILL], 1);
-            double bp = V * V * kSigma * iH * iH * iH;   // V_i psitilde_j(x_i) = Bp_i d w(q_ij)
+            const double bp = V * fac;   // V_i psitilde_j(x_i) = Bp_i d w(q_ij)
             geo_t[8 * p] = (T)iH;
             geo_t[8 * p + 1] = (T)hi;
             for (int k = 0; k < 6; ++k) {
@@ -1088,12 +1254,28 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
             om_t[p] = (T)om;
         }
     }
-    double vmin = V, cmax = cond;
-    warp_minmax(vmin, cmax);
+    // largest float condition number (non-negative floats order like integers) and smallest V
+    const unsigned cm = __reduce_max_sync(0xffffffffu, __float_as_uint(cond));
+    for (int o = 16; o > 0; o >>= 1) V = fmin(V, __shfl_xor_sync(0xffffffffu, V, o));
     if ((threadIdx.x & 31) == 0) {
-        if (cmax > 0.0) atomic_max_pos(&red[2], cmax);
-        if (vmin < INFINITY) atomic_min_pos(&red[3], vmin);
+        if (cm) atomicMax(cond_max, cm);
+        if (V < INFINITY) atomic_min_pos(&red[3], V);
     }
+}
+
+// cond_2(E_i) = cond_2(B_i) in double where the float value is within 2% of the largest or above
+// kCondFloat: the largest, the ill-conditioned ones, and a last check that E_i is positive definite
+__global__ void k_cond(const float* __restrict__ cond, const double* __restrict__ B, int64_t n,
+                       const unsigned* __restrict__ cond_max, unsigned long long* red, int* flags) {
+    const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (p >= n || !(cond[p] >= fminf(0.98f * __uint_as_float(*cond_max), kCondFloat))) return;
+    double ev[3];
+    sym3_eigs(B[p], B[n + p], B[2 * n + p], B[3 * n + p], B[4 * n + p], B[5 * n + p], ev);
+    const double lmin = fmin(ev[0], fmin(ev[1], ev[2])), lmax = fmax(ev[0], fmax(ev[1], ev[2]));
+    const double c = lmin > 0 ? lmax / lmin : INFINITY;
+    if (!(lmin > 0)) atomicExch(&flags[F_GEOM], 1);
+    if (c > 1e10) atomicAdd(&flags[F_ILL], 1);
+    atomic_max_pos(&red[2], c);
 }
 
 // ------------------------------------------------------------------------------------
@@ -1105,7 +1287,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 struct SrcParams {
-    double eta, h0, h_cap;
+    double s_star, eta3, h0, h_cap;   // (kappa eta)^3 / sigma and eta^3 of the sources' eta
     int max_iter;
     int warm;       // start from the h of the last call (in hs_out), else from h0
     int fixed;      // hs_out holds given smoothing lengths: only omega_s at them
@@ -1197,9 +1379,8 @@ __global__ void __launch_bounds__(kSrcThreads) k_src_h(Grid g, const double* __r
             double r2 = dx * dx + dy * dy + dz * dz;
             if (r2 < H2) {
                 double q = sqrt(r2) * iH;
-                double w = spline_w(q);
-                sw += w;
-                sdw += 3.0 * w + q * spline_dw(q);
+                sw += spline_w(q);
+                sdw += q * spline_dw(q);
             }
         });
         red_w[t] = sw;
@@ -1220,21 +1401,28 @@ __global__ void __launch_bounds__(kSrcThreads) k_src_h(Grid g, const double* __r
             ok = om > 0.0;
             break;
         }
-        double f, fp;
-        if (om > 0.0) {
-            double dom = -kKappa * kSigma * iH * iH * iH * iH * sdw;
-            double cb = cbrt(om);
-            f = h - sp.eta / cb;
-            fp = 1.0 + (sp.eta / 3.0) / (cb * om) * dom;
-        } else {
-            f = -INFINITY;
-            fp = 0.0;
-        }
+        // Newton on S(h) = sum w = S* (see k_h_solve) close to the root, where a step of less than
+        // 1e-8 h ends it: the next one would be below rounding, and at the root omega is
+        // (eta/h)^3.  Farther off on h - eta omega^(-1/3), nearly linear in h.
+        const double f = sw - sp.s_star;
         if (f < 0.0) lo = h; else hi = h;
-        double step = (om > 0.0) ? f / fp : -INFINITY;
-        if (om > 0.0 && !(fabs(step) > 2e-16 * h)) { ok = true; break; }
+        double step = -INFINITY;
+        if (sw > 0.0 && sdw < 0.0) {
+            if (fabs(f) < 1e-3 * sp.s_star) {
+                step = -f * h / sdw;
+            } else {
+                const double x = cbrt(sp.s_star / sw), fp = 1.0 - x - x * sdw / (3.0 * sw);
+                step = fp > 0.0 ? h * (1.0 - x) / fp : -INFINITY;
+            }
+        }
+        if (fabs(step) <= 1e-8 * h) {
+            h -= step;
+            om = sp.eta3 / (h * h * h);
+            ok = true;
+            break;
+        }
         double hn = h - step;
-        if (!(hn > lo && hn < hi) || !(fp > 0.0)) hn = isinf(hi) ? 1.5 * h : 0.5 * (lo + hi);
+        if (!(hn > lo && hn < hi)) hn = isinf(hi) ? 1.5 * h : 0.5 * (lo + hi);
         if (hn > sp.h_cap) hn = sp.h_cap;
         if (hn == h) { ok = om > 0.0; break; }
         h = hn;
@@ -1517,13 +1705,17 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     RT_TRY(ensure(c, c->omega_d, n * 8, "omega"));
     RT_TRY(ensure(c, c->V_d, n * 8, "V"));
     RT_TRY(ensure(c, c->B_d, 6 * n * 8, "B"));
-    RT_TRY(ensure(c, c->cond_d, n * 8, "cond"));
+    RT_TRY(ensure(c, c->cond_f, n * 4, "cond"));
+    RT_TRY(ensure(c, c->h_sum, 3 * n * 4, "h"));
     size_t ts = c->fp64 ? 8 : 4;
     RT_TRY(ensure(c, c->pos_t, n * 32, "geom"));
     RT_TRY(ensure(c, c->geo_t, 8 * n * ts, "geom"));
     RT_TRY(ensure(c, c->omega_t, n * ts, "geom"));
     RT_TRY(ensure(c, c->counts, (n + 1) * 4, "counts"));
     RT_TRY(ensure(c, c->row_off, (n + 1) * 8, "row_off"));
+    const int cap = list_capacity(cfg.eta_res);
+    RT_TRY(ensure(c, c->lists, (size_t)n * cap * 4, "candidate lists"));
+    RT_TRY(ensure(c, c->list_cnt, (size_t)n * 4, "candidate lists"));
     RT_TRY(ensure(c, c->flags, 64, "flags"));
     RT_TRY(ensure(c, c->red_tmp, 64, "reduction"));
 
@@ -1531,9 +1723,10 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     RT_CUDA(c, cudaMemsetAsync(flags, 0, 64, st));
     const bool warm = c->has_h_prev;
     c->has_h_prev = false;       // set again only when this call succeeds
-    // reductions: [0] min h, [1] max h, [2] max cond, [3] min V (bit patterns of positive doubles)
+    // reductions: [0] min h, [1] max h, [2] max cond, [3] min V (bit patterns of positive doubles),
+    // [4] sum of H^3, [5] spill length, [6] extras of long rows, [7] max float cond
     unsigned long long* red = reinterpret_cast<unsigned long long*>(c->red_tmp.p);
-    RT_CUDA(c, cudaMemsetAsync(red, 0, 40, st));
+    RT_CUDA(c, cudaMemsetAsync(red, 0, 64, st));
     RT_CUDA(c, cudaMemsetAsync(red, 0xff, 8, st));
     RT_CUDA(c, cudaMemsetAsync(red + 3, 0xff, 8, st));
 
@@ -1571,6 +1764,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     // a2: smoothing lengths
     HParams hp;
     hp.eta = cfg.eta_res;
+    hp.eta3 = cfg.eta_res * cfg.eta_res * cfg.eta_res;
+    hp.s_star = kKappa * kKappa * kKappa / kSigma * hp.eta3;
     hp.h0 = h0;
     double minbox = std::min(cfg.box[0], std::min(cfg.box[1], cfg.box[2]));
     hp.h_cap = cfg.periodic ? 0.5 * minbox / kKappa : 1e30;
@@ -1578,200 +1773,152 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     hp.max_iter = cfg.h_max_iter > 0 ? cfg.h_max_iter : 100;
     hp.tol32 = (float)std::max(cfg.h_tol, 2e-6);
     // the FP64 path refines every h in double; the float path only those of particles with a
-    // candidate near their support radius, which is enough for the exact root's pair lists
+    // candidate near their support radius, which is enough for the exact roots' pair lists
     hp.refine64 = c->fp64 ? 1 : 0;
     int* refine_count = flags + F_REFINE;
+    const size_t st_bytes = (size_t)kListParticles * cap * sizeof(float);
     if (h_in) {
         hp.refine64 = c->fp64 ? 1 : 0;   // omega in the working path's arithmetic
         k_h_given<<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, h_in,
                                                  c->perm.as<int32_t>(), c->h_d.as<double>(), c->omega_d.as<double>(),
                                                  c->H2f.as<float>(), red, flags);
     } else {
-        k_h_solve<<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp,
-                                                 warm ? c->h_prev.as<double>() : nullptr, c->perm.as<int32_t>(),
-                                                 c->h_d.as<double>(), c->omega_d.as<double>(), c->H2f.as<float>(), red,
-                                                 flags, c->idx_in.as<int32_t>(), refine_count);
+        k_h_lists<true><<<nblk(n, kListParticles), kListWarps * 32, st_bytes, st>>>(
+            g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, warm ? c->h_prev.as<double>() : nullptr,
+            c->perm.as<int32_t>(), nullptr, c->h_sum.as<float>(), flags, c->idx_in.as<int32_t>(), refine_count,
+            c->lists.as<int32_t>(), c->list_cnt.as<int32_t>(), cap);
     }
     RT_CUDA(c, cudaGetLastError());
-    c->launches += 1;
-    if (!c->fp64 && !h_in) {
-        k_h_refine<<<(unsigned)c->sm_count * 8, 256, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp,
-                                                  c->idx_in.as<int32_t>(), refine_count, c->h_d.as<double>(),
-                                                  c->omega_d.as<double>(), c->H2f.as<float>(), red, flags);
-        RT_CUDA(c, cudaGetLastError());
-        c->launches += 1;
+    if (h_in)
+        k_h_lists<false><<<nblk(n, kListParticles), kListWarps * 32, st_bytes, st>>>(
+            g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, nullptr, nullptr, c->h_d.as<double>(), nullptr, flags,
+            nullptr, nullptr, c->lists.as<int32_t>(), c->list_cnt.as<int32_t>(), cap);
+    k_h_finish<<<nblk(n, 256), 256, 0, st>>>(h_in ? nullptr : c->h_sum.as<float>(), n, hp.refine64 ? 0 : 1,
+                                             c->h_d.as<double>(), c->omega_d.as<double>(), c->H2f.as<float>(),
+                                             c->xq.as<uint4>(), red);
+    if (!h_in) {
+        // the number of flagged particles is on the device: a grid of resident blocks (FP64: all)
+        const int64_t nbr = std::min<int64_t>(nblk(n * kRefineLanes, 128), c->sm_count * (c->fp64 ? 64 : 8));
+        k_h_refine<<<(unsigned)nbr, 128, 0, st>>>(
+            g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, c->fp64 ? nullptr : c->idx_in.as<int32_t>(),
+            refine_count, c->lists.as<int32_t>(), c->list_cnt.as<int32_t>(), cap, c->h_d.as<double>(),
+            c->omega_d.as<double>(), c->H2f.as<float>(), c->xq.as<uint4>(), red, flags);
     }
+    RT_CUDA(c, cudaGetLastError());
+    c->launches += 3;
+
+    // a3: symmetric pair lists; every particle finds the entries of its own support, and the
+    // sizes of the rows come back with the flags of everything before (one synchronisation)
+    PairParams pp;
+    for (int a = 0; a < 3; ++a) pp.scale[a] = qscale[a];
+    RT_TRY(ensure(c, c->own_cnt, (size_t)n * 4, "pair rows"));
+    RT_TRY(ensure(c, c->extra_cnt, (size_t)n * 4, "pair rows"));
+    RT_TRY(ensure(c, c->extras, (size_t)n * kExtras * 4, "pair rows"));
+    unsigned long long *spill_n = red + 5, *more_n = red + 6;
+    int* over_n = flags + F_OVER;
+    int32_t* over = c->idx_in.as<int32_t>();      // the flagged particles' list is done with
+    RT_CUDA(c, cudaMemsetAsync(c->extra_cnt.p, 0, (size_t)n * 4, st));
+    k_own_rows<<<nblk(n * 32, 256), 256, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n,
+                                                   pp, c->lists.as<int32_t>(), cap, c->list_cnt.as<int32_t>(),
+                                                   c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(),
+                                                   c->extras.as<int32_t>(), over, over_n);
+    k_own_walk<false><<<(unsigned)c->sm_count * 4, 128, 0, st>>>(
+        g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n, pp, c->lists.as<int32_t>(), cap,
+        c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(), c->extras.as<int32_t>(), over, over_n, spill_n, nullptr);
+    k_row_lengths<<<nblk(n + 1, 256), 256, 0, st>>>(c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(), n,
+                                                     c->counts.as<int32_t>(), more_n);
+    RT_CUDA(c, cudaGetLastError());
+    tb = c->cub_tmp.bytes;
+    RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->counts.as<int32_t>(), c->row_off.as<int64_t>(),
+                                             (int)(n + 1), st));
+    c->launches += 3;
     int hflags[8];
-    double hmm[2];
-    double sumH3 = 0.0;
+    struct {
+        double hmin, hmax, cond, vmin, h3;
+        unsigned long long spill, more;
+    } hred;
+    static_assert(sizeof(hred) == 56, "layout of the reduction buffer");
+    int64_t P2 = 0;
     RT_CUDA(c, cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, st));
-    RT_CUDA(c, cudaMemcpyAsync(hmm, red, sizeof(hmm), cudaMemcpyDeviceToHost, st));
-    RT_CUDA(c, cudaMemcpyAsync(&sumH3, red + 4, 8, cudaMemcpyDeviceToHost, st));
+    RT_CUDA(c, cudaMemcpyAsync(&hred, red, sizeof(hred), cudaMemcpyDeviceToHost, st));
+    RT_CUDA(c, cudaMemcpyAsync(&P2, c->row_off.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
     RT_CUDA(c, cudaStreamSynchronize(st));
     if (hflags[F_BADPOS]) return fail(c, RT_ERR_INVALID, "positions must be finite and inside [0, box)");
     if (hflags[F_NOCONV]) return fail(c, RT_ERR_NOCONV, "smoothing-length iteration did not converge");
     if (hflags[F_BADH]) return fail(c, RT_ERR_INVALID, "given smoothing lengths must be finite, > 0 and below the "
                                                        "quarter of the periodic box over the support ratio");
     c->diag.h_refined = h_in ? 0 : (c->fp64 ? n : (int64_t)hflags[F_REFINE]);
-    c->diag.h_min = hmm[0];
-    c->diag.h_max = hmm[1];
-    double Hmax = kKappa * hmm[1];
+    c->diag.h_min = hred.hmin;
+    c->diag.h_max = hred.hmax;
+    const double Hmax = kKappa * hred.hmax;
     if (cfg.periodic && Hmax >= 0.5 * minbox)
         return fail(c, RT_ERR_GEOMETRY, "support radius reaches half the periodic box");
-
-    // a3: symmetric pair lists
-    PairParams pp;
-    for (int a = 0; a < 3; ++a) pp.scale[a] = qscale[a];
-    pp.Hmax = Hmax;
-    // Searching every particle out to max(H_i, H_max) visits H_max^3 / <H^3> times the volume
-    // of its own support; above a ratio of 12 the sort-based build is cheaper.
-    const double vol_ratio = Hmax * Hmax * Hmax / std::max(sumH3 / (double)n, 1e-300);
-    const bool sorted_build = vol_ratio > 12.0;
-    c->diag.pair_build = sorted_build ? 1 : 0;
-    int64_t P2 = 0;
-    if (!sorted_build) {
-        // search radii from the coarse blocks' largest H
-        Blocks bk;
-        int nbt = 1;
-        for (int a = 0; a < 3; ++a) {
-            bk.nb[a] = std::min(16, c->nc[a]);
-            bk.len[a] = cfg.box[a] / bk.nb[a];
-            nbt *= bk.nb[a];
-        }
-        bk.periodic = cfg.periodic;
-        for (int a = 0; a < 3; ++a) bk.reach[a] = (int)std::ceil(Hmax / bk.len[a]) + 1;
-        RT_TRY(ensure(c, c->blk, (size_t)nbt * 8, "blocks"));
-        unsigned* hb = c->blk.as<unsigned>();
-        float* reach = reinterpret_cast<float*>(hb + nbt);
-        RT_CUDA(c, cudaMemsetAsync(hb, 0, (size_t)nbt * 4, st));
-        k_block_hmax<<<nblk(n, 256), 256, 0, st>>>(c->xs_d.as<double>(), c->H2f.as<float>(), n, bk, hb,
-                                                   c->xq.as<uint4>());
-        k_block_reach<<<nblk((int64_t)nbt * 32, 128), 128, 0, st>>>(hb, bk, reach);
-        c->launches += 2;
-        // one walk counts the rows and, when the rows of the last call fit row_cap entries,
-        // also stores them (then compacted); a longer row needs a second, writing walk
-        const int cap = (int)c->row_cap;
-        if (cap > 0) RT_TRY(ensure(c, c->cols_cap, (size_t)n * cap * 4, "pair rows"));
-        int* row_max = c->flags.as<int>() + F_ROWMAX;
-        RT_CUDA(c, cudaMemsetAsync(row_max, 0, 4, st));
-        k_pairs<false><<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(),
-                                                      c->h_d.as<double>(), c->H2f.as<float>(), n, pp, bk, reach,
-                                                      c->counts.as<int32_t>(), nullptr,
-                                                      cap > 0 ? c->cols_cap.as<int32_t>() : nullptr, cap, row_max);
-        RT_CUDA(c, cudaMemsetAsync(c->counts.as<int32_t>() + n, 0, 4, st));
-        tb = c->cub_tmp.bytes;
-        RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->counts.as<int32_t>(), c->row_off.as<int64_t>(),
-                                                 (int)(n + 1), st));
-        int longest = 0;
-        RT_CUDA(c, cudaMemcpyAsync(&P2, c->row_off.as<int64_t>() + n, 8, cudaMemcpyDeviceToHost, st));
-        RT_CUDA(c, cudaMemcpyAsync(&longest, row_max, 4, cudaMemcpyDeviceToHost, st));
-        RT_CUDA(c, cudaStreamSynchronize(st));
-        if (P2 >= ((int64_t)1 << 31)) return fail(c, RT_ERR_INVALID, "more than 2^31 neighbour entries");
-        RT_TRY(ensure(c, c->cols, std::max<int64_t>(P2, 1) * 4, "pair lists"));
-        // the walks visit the candidates in ascending index: the rows need no sort
-        if (cap > 0 && longest <= cap) {
-            k_rows_compact<<<nblk(n * 32, 256), 256, 0, st>>>(c->cols_cap.as<int32_t>(), cap,
-                                                              c->row_off.as<int64_t>(), n, c->cols.as<int32_t>());
-        } else {
-            k_pairs<true><<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(),
-                                                         c->h_d.as<double>(), c->H2f.as<float>(), n, pp, bk, reach,
-                                                         nullptr, c->row_off.as<int64_t>(), c->cols.as<int32_t>());
-        }
-        // the next call's rows: the longest row with a quarter to spare, in multiples of 32,
-        // while the padded rows stay within eight times the lists (only the filled part of a
-        // row is written or read)
-        const int64_t next = ((int64_t)longest + longest / 4 + 8 + 31) / 32 * 32;
-        c->row_cap = next * n <= 8 * std::max<int64_t>(P2, 1) ? next : 0;
-        RT_CUDA(c, cudaGetLastError());
-        c->launches += 2;
-    } else {
-        int64_t* goff = c->row_off.as<int64_t>();      // gather offsets first, CSR offsets after
-        k_pairs_gather<false><<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(),
-                                                             c->h_d.as<double>(), c->H2f.as<float>(), n, pp,
-                                                             c->counts.as<int32_t>(), nullptr, nullptr);
-        RT_CUDA(c, cudaMemsetAsync(c->counts.as<int32_t>() + n, 0, 4, st));
-        tb = c->cub_tmp.bytes;
-        RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->counts.as<int32_t>(), goff, (int)(n + 1), st));
-        int64_t Mg = 0;
-        RT_CUDA(c, cudaMemcpyAsync(&Mg, goff + n, 8, cudaMemcpyDeviceToHost, st));
-        RT_CUDA(c, cudaStreamSynchronize(st));
-        if (2 * Mg >= ((int64_t)1 << 31)) return fail(c, RT_ERR_INVALID, "more than 2^31 neighbour entries");
-        const int64_t K = std::max<int64_t>(2 * Mg, 1);
-        RT_TRY(ensure(c, c->pkeys, K * 8, "pair keys"));
-        RT_TRY(ensure(c, c->pkeys_alt, K * 8, "pair keys"));
-        k_pairs_gather<true><<<nblk(n, 128), 128, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(),
-                                                            c->h_d.as<double>(), c->H2f.as<float>(), n, pp, nullptr,
-                                                            goff, c->pkeys.as<uint64_t>());
-        c->launches += 2;
-        int key_bits = 32 + c->key_bits;
-        {
-            int nb = 1;
-            while (((int64_t)1 << nb) < n) ++nb;
-            key_bits = 32 + nb;
-        }
-        size_t need = 0;
-        cub::DeviceRadixSort::SortKeys(nullptr, need, c->pkeys.as<uint64_t>(), c->pkeys_alt.as<uint64_t>(), (int)K, 0,
-                                       key_bits, st);
-        size_t need2 = 0;
-        cub::DeviceSelect::Unique(nullptr, need2, c->pkeys_alt.as<uint64_t>(), c->pkeys.as<uint64_t>(),
-                                  (int64_t*)nullptr, (int)K, st);
-        RT_TRY(ensure(c, c->cub_tmp, std::max(need, need2) + 256, "cub scratch"));
-        tb = c->cub_tmp.bytes;
-        RT_CUDA(c, cub::DeviceRadixSort::SortKeys(c->cub_tmp.p, tb, c->pkeys.as<uint64_t>(), c->pkeys_alt.as<uint64_t>(),
-                                                  (int)K, 0, key_bits, st));
-        int64_t* nuniq = reinterpret_cast<int64_t*>(red + 5);
-        tb = c->cub_tmp.bytes;
-        RT_CUDA(c, cub::DeviceSelect::Unique(c->cub_tmp.p, tb, c->pkeys_alt.as<uint64_t>(), c->pkeys.as<uint64_t>(),
-                                             nuniq, (int)K, st));
-        RT_CUDA(c, cudaMemcpyAsync(&P2, nuniq, 8, cudaMemcpyDeviceToHost, st));
-        RT_CUDA(c, cudaStreamSynchronize(st));
-        RT_TRY(ensure(c, c->cols, std::max<int64_t>(P2, 1) * 4, "pair lists"));
-        RT_CUDA(c, cudaMemsetAsync(c->counts.as<int32_t>(), 0, (n + 1) * 4, st));
-        k_keys_to_csr<<<nblk(std::max<int64_t>(P2, 1), 256), 256, 0, st>>>(c->pkeys.as<uint64_t>(), nuniq,
-                                                                            c->cols.as<int32_t>(),
-                                                                            c->counts.as<int32_t>());
-        tb = c->cub_tmp.bytes;
-        RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->counts.as<int32_t>(), c->row_off.as<int64_t>(),
-                                                 (int)(n + 1), st));
-        ++c->launches;
-        RT_CUDA(c, cudaGetLastError());
+    if (P2 >= ((int64_t)1 << 31)) return fail(c, RT_ERR_INVALID, "more than 2^31 neighbour entries");
+    // the spread of the supports, H_max^3 over the mean H^3
+    c->diag.pair_build = Hmax * Hmax * Hmax / std::max(hred.h3 / (double)n, 1e-300) > 12.0 ? 1 : 0;
+    RT_TRY(ensure(c, c->cols, std::max<int64_t>(P2, 1) * 4, "pair lists"));
+    RT_TRY(ensure(c, c->n_low, (n + 1) * 4, "pair split"));
+    RT_TRY(ensure(c, c->n_up, (n + 1) * 4, "pair split"));
+    if (hred.spill > 0) {     // own entries of the particles without a list
+        RT_TRY(ensure(c, c->spill, (size_t)hred.spill * 4, "pair rows"));
+        k_own_walk<true><<<(unsigned)c->sm_count * 4, 128, 0, st>>>(
+            g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n, pp, c->lists.as<int32_t>(), cap,
+            c->own_cnt.as<int32_t>(), nullptr, nullptr, over, over_n, nullptr, c->spill.as<int32_t>());
+        c->launches += 1;
     }
+    if (hred.more > 0) {      // rows with more extras than they hold in place
+        RT_TRY(ensure(c, c->more, (size_t)hred.more * 4, "pair rows"));
+        RT_TRY(ensure(c, c->more_off, (size_t)(n + 1) * 8, "pair rows"));
+        int32_t* cnt = c->counts.as<int32_t>();
+        k_more_extras<<<nblk(n + 1, 256), 256, 0, st>>>(c->extra_cnt.as<int32_t>(), n, cnt);
+        tb = c->cub_tmp.bytes;
+        RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, cnt, c->more_off.as<int64_t>(), (int)(n + 1), st));
+        RT_CUDA(c, cudaMemsetAsync(cnt, 0, (size_t)n * 4, st));
+        k_extras_fill<<<nblk(n * 32, 256), 256, 0, st>>>(
+            n, c->lists.as<int32_t>(), cap, c->list_cnt.as<int32_t>(), c->own_cnt.as<int32_t>(),
+            c->extra_cnt.as<int32_t>(), c->more_off.as<int64_t>(), cnt, c->spill.as<int32_t>(), c->more.as<int32_t>());
+        c->launches += 2;
+    }
+    k_rows_merge<<<nblk(n * 32, 256), 256, 0, st>>>(
+        n, c->lists.as<int32_t>(), cap, c->list_cnt.as<int32_t>(), c->own_cnt.as<int32_t>(),
+        c->extra_cnt.as<int32_t>(), c->extras.as<int32_t>(), c->more_off.as<int64_t>(), c->more.as<int32_t>(),
+        c->spill.as<int32_t>(), c->row_off.as<int64_t>(), c->cols.as<int32_t>(), c->n_low.as<int32_t>(),
+        c->n_up.as<int32_t>());
+    c->launches += 1;
+    RT_CUDA(c, cudaGetLastError());
     c->n_directed = P2;
     c->launches += 1;   // geometry below
 
-    // the lower / upper split and the slots of the pairs
-    RT_TRY(ensure(c, c->n_low, (n + 1) * 4, "pair split"));
-    RT_TRY(ensure(c, c->n_up, (n + 1) * 4, "pair split"));
+    // the slots of the pairs
     RT_TRY(ensure(c, c->up_off, (n + 1) * 8, "pair split"));
     RT_TRY(ensure(c, c->low_slot, std::max<int64_t>(P2 / 2, 1) * 4, "pair split"));
-    k_row_split<<<nblk(n, 256), 256, 0, st>>>(c->row_off.as<int64_t>(), c->cols.as<int32_t>(), n,
-                                               c->n_low.as<int32_t>(), c->n_up.as<int32_t>());
     RT_CUDA(c, cudaMemsetAsync(c->n_up.as<int32_t>() + n, 0, 4, st));
     tb = c->cub_tmp.bytes;
     RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->n_up.as<int32_t>(), c->up_off.as<int64_t>(),
                                              (int)(n + 1), st));
-    k_low_slots<<<nblk(n * 32, 256), 256, 0, st>>>(c->row_off.as<int64_t>(), c->cols.as<int32_t>(),
-                                                    c->n_low.as<int32_t>(), c->up_off.as<int64_t>(), n,
-                                                    c->low_slot.as<int32_t>());
     RT_TRY(ensure(c, c->pair_ends, std::max<int64_t>(P2 / 2, 1) * 8, "pair split"));
-    k_pair_ends<<<nblk(n, 128), 128, 0, st>>>(c->row_off.as<int64_t>(), c->cols.as<int32_t>(), c->n_low.as<int32_t>(),
-                                               c->up_off.as<int64_t>(), n, c->pair_ends.as<int2>());
-    c->launches += 3;
+    k_pair_slots<<<nblk(n * 32, 256), 256, 0, st>>>(c->row_off.as<int64_t>(), c->cols.as<int32_t>(),
+                                                     c->n_low.as<int32_t>(), c->up_off.as<int64_t>(), n,
+                                                     c->pair_ends.as<int2>(), c->low_slot.as<int32_t>());
+    c->launches += 1;
     RT_CUDA(c, cudaGetLastError());
 
     // a4: geometry
+    unsigned* cond_max = reinterpret_cast<unsigned*>(red + 7);
     if (c->fp64)
         k_geometry<double><<<nblk(n, 128), 128, 0, st>>>(
             c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(),
             c->row_off.as<int64_t>(), c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic,
-            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_d.as<double>(),
-            c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(), red, flags);
+            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_f.as<float>(),
+            c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(), red, cond_max, flags);
     else
         k_geometry<float><<<nblk(n, 128), 128, 0, st>>>(
             c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(),
             c->row_off.as<int64_t>(), c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic,
-            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_d.as<double>(),
-            c->pos_t.p, c->geo_t.as<float>(), c->omega_t.as<float>(), red, flags);
+            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_f.as<float>(),
+            c->pos_t.p, c->geo_t.as<float>(), c->omega_t.as<float>(), red, cond_max, flags);
+    k_cond<<<nblk(n, 256), 256, 0, st>>>(c->cond_f.as<float>(), c->B_d.as<double>(), n, cond_max, red, flags);
+    c->launches += 1;
     RT_CUDA(c, cudaGetLastError());
 
     // a5 preparation: sources
@@ -1785,7 +1932,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         RT_TRY(ensure(c, c->src_off, (S + 1) * 8, "sources"));
         RT_CUDA(c, cudaMemcpyAsync(c->xsrc_d.p, xsrc, 3 * S * 8, cudaMemcpyDeviceToDevice, st));
         SrcParams sp;
-        sp.eta = cfg.eta_res_star;
+        sp.eta3 = cfg.eta_res_star * cfg.eta_res_star * cfg.eta_res_star;
+        sp.s_star = kKappa * kKappa * kKappa / kSigma * sp.eta3;
         sp.h0 = cfg.eta_res_star * std::cbrt(vol / (double)n);
         sp.h_cap = hp.h_cap;
         sp.max_iter = std::max(hp.max_iter, 200);

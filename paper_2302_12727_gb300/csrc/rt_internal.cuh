@@ -21,9 +21,9 @@ constexpr double kKappa = 1.825742;
 constexpr double kSigma = 5.0929581789406507446;   // 16 / pi
 // int slots of the context's 64-byte flag buffer (cleared by every rt_neighbours): error
 // flags of the build, the clamp counter (64-bit, slots 8-9) and the device-wait time-out flag
-enum FlagSlot { F_BADPOS = 0, F_NOCONV = 1, F_GEOM = 2, F_ILL = 3, F_SRC_NOCONV = 4, F_REFINE = 5, F_BADH = 6,
+enum FlagSlot { F_BADPOS = 0, F_NOCONV = 1, F_GEOM = 2, F_ILL = 3, F_SRC_NOCONV = 4, F_REFINE = 5, F_BADH = 6, F_OVER = 7,
                 F_NSLOTS = 8, F_CLAMP = 8,
-                F_TIMEOUT = 12, F_SCRATCH = 13, F_ROWMAX = 14, F_SELFTEST = 15 };
+                F_TIMEOUT = 12, F_SCRATCH = 13, F_SELFTEST = 15 };
 constexpr int kMaxGC = 4;                          // groups handled by one pair-kernel launch
 // Packed flux rows start with a prefix that repeats their last kRowRot words: a row copy that
 // starts at word kRowRot delivers the row, one that starts at word 0 delivers it rotated by
@@ -79,19 +79,20 @@ struct rt_ctx {
     // build buffers
     rt::DevBuf keys_in, keys_out, idx_in, perm, inv_perm, cell_start, cell_end, cub_tmp;
     rt::DevBuf xs_d, xq, m_s;
-    rt::DevBuf h_d, omega_d, V_d, B_d, cond_d;           // double per particle
-    rt::DevBuf H2f;                                     // float (kappa h)^2, pair-search prefilter
+    rt::DevBuf h_d, omega_d, V_d, B_d;                   // double per particle
+    rt::DevBuf cond_f;                                  // float cond_2(E_i)
+    rt::DevBuf H2f;                                     // float (kappa h)^2
+    // candidates of the last h solve, a fixed capacity a particle, and their number (-1: none)
+    rt::DevBuf lists, list_cnt;
+    rt::DevBuf h_sum;                                   // float root h and the pair S(h), [3][n]
+    // pair search: entries of a particle's own support, extras handed to each row by others (in
+    // place, or in `more` for long rows), own entries of the particles without a list
+    rt::DevBuf own_cnt, extra_cnt, extras, more, more_off, spill;
     rt::DevBuf h_prev;                                  // h of the last call, caller order (first guess)
     bool has_h_prev = false;
     bool has_hs_prev = false;                           // hs_d holds the sources' h of the last call
     rt::DevBuf pos_t, geo_t, omega_t;                   // working precision per particle (pair kernels)
     rt::DevBuf counts, row_off, cols;                   // symmetric pair lists (CSR), rows ascending
-    // rows of row_cap entries that the counting walk of the pair search also fills (0: off);
-    // set from the longest row of the last call
-    rt::DevBuf cols_cap;
-    int64_t row_cap = 0;
-    rt::DevBuf blk;                                     // coarse blocks: largest H and reach radius
-    rt::DevBuf pkeys, pkeys_alt;                        // (row, col) keys of the sort-based build
     rt::DevBuf n_low, n_up, up_off, low_slot, pair_ends; // lower / upper split, pair slots
     rt::DevBuf pairbuf;                                 // per-pair fluxes of one group chunk
     // double path: geometry of every pair and weights of every row entry, kept from the first

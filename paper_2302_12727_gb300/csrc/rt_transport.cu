@@ -1127,12 +1127,18 @@ __global__ void k_energy_part(const T* __restrict__ rec, int RS, const double* _
     }
 }
 
-__global__ void k_energy_final(const double* __restrict__ part, int nb, int G, double* out) {
-    int g = threadIdx.x;
-    if (g >= G) return;
-    double s = 0.0;
-    for (int b = 0; b < nb; ++b) s += part[g * nb + b];
-    out[g] = s;
+// one block of kEnergyBlocks threads per group adds the partial sums in a fixed tree: 4 us where
+// one thread adding the 512 in turn took 34
+__global__ void __launch_bounds__(kEnergyBlocks) k_energy_final(const double* __restrict__ part, double* out) {
+    __shared__ double sm[kEnergyBlocks];
+    const int g = blockIdx.x, t = threadIdx.x;
+    sm[t] = part[g * kEnergyBlocks + t];
+    __syncthreads();
+    for (int w = kEnergyBlocks / 2; w > 0; w >>= 1) {
+        if (t < w) sm[t] += sm[t + w];
+        __syncthreads();
+    }
+    if (t == 0) out[g] = sm[0];
 }
 
 // ------------------------------------------------------------------------------------
@@ -1745,7 +1751,7 @@ rt_status launch_energy(rt_ctx* c, cudaStream_t s, const void* rec, double* out_
     else
         k_energy_part<float><<<kEnergyBlocks, 256, 0, s>>>((const float*)rec, RS, c->V_d.as<double>(), c->n,
                                                            c->cfg.n_groups, perm, c->n_owned, part);
-    k_energy_final<<<1, 32 * ((c->cfg.n_groups + 31) / 32), 0, s>>>(part, kEnergyBlocks, c->cfg.n_groups, out_dev);
+    k_energy_final<<<c->cfg.n_groups, kEnergyBlocks, 0, s>>>(part, out_dev);
     c->launches += 2;
     RT_CUDA(c, cudaGetLastError());
     return RT_OK;
