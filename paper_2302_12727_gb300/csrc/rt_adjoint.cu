@@ -469,8 +469,8 @@ static void launch_adj_step(rt_ctx* c, cudaStream_t s, const T* lamN, const T* W
         const unsigned nbp = nblk_(std::max<int64_t>(a.n_pairs, 1), 128);
         k_adj_mu<T><<<nblk_(c->n * G, 256), 256, 0, s>>>(a, x, lamN, mu);
         ++c->launches;
-        for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-            const int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+        for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+            const int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
             const unsigned nbg = nblk_(c->n * gc, 128);
 #define RT_ADJ_PAIRS(GC_)                                                                      \
     k_adj_pair<T, GC_><<<nbp, 128, 0, s>>>(a, x.c, mu, W, slots, sel, g0);                      \
@@ -488,8 +488,8 @@ static void launch_adj_step(rt_ctx* c, cudaStream_t s, const T* lamN, const T* W
         }
         return;
     }
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
         const unsigned nbg = nblk_(c->n * gc, 128);
         switch (gc) {
             case 1: k_adj_flux<T, 1><<<nbg, 128, 0, s>>>(a, x, lamN, W, ub, gam, g0); break;
@@ -498,8 +498,8 @@ static void launch_adj_step(rt_ctx* c, cudaStream_t s, const T* lamN, const T* W
             default: k_adj_flux<T, 4><<<nbg, 128, 0, s>>>(a, x, lamN, W, ub, gam, g0); break;
         }
     }
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
         const unsigned nbg = nblk_(c->n * gc, 128);
         switch (gc) {
             case 1: k_adj_grad<T, 1><<<nbg, 128, 0, s>>>(a, ub, gam, lamO, g0); break;
@@ -508,7 +508,7 @@ static void launch_adj_step(rt_ctx* c, cudaStream_t s, const T* lamN, const T* W
             default: k_adj_grad<T, 4><<<nbg, 128, 0, s>>>(a, ub, gam, lamO, g0); break;
         }
     }
-    c->launches += 2 * ((G + kMaxGC - 1) / kMaxGC);
+    c->launches += 2 * ((G + chunk_groups(G) - 1) / chunk_groups(G));
 }
 
 rt_status run_adjoint(rt_ctx* c, int n_sub, int k, bool has_src, bool has_alpha, const void* U0s,

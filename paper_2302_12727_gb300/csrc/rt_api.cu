@@ -140,8 +140,7 @@ static rt_status ensure_state(rt_ctx* c) {
             ++g_generation;
         }
     }
-    if (!c->fp64 && G <= kMaxGC)
-        RT_TRY(ensure(c, c->frec, (size_t)(12 + 16 * G + kRowRot) * n * 4, "packed flux rows"));
+    if (!c->fp64) RT_TRY(ensure(c, c->frec, (size_t)(12 + 16 * gc + kRowRot) * n * 4, "packed flux rows"));
     return RT_OK;
 }
 
@@ -304,9 +303,9 @@ rt_status rt_gradients(rt_ctx* c, const void* U, void* gradU) {
     if (!U || !gradU) return fail(c, RT_ERR_INVALID, "NULL array");
     const int G = c->cfg.n_groups;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(launch_gradient(c, c->stream, c->U_a.p));
-    RT_TRY(state_out(c, c->grad_t.p, gradU, 12 * G, 12 * G, 0));
+    RT_TRY(state_out(c, c->grad_t.p, gradU, 12 * G));
     return RT_OK;
 }
 
@@ -317,12 +316,12 @@ rt_status rt_step_bins(rt_ctx* c, void* U, const double* Lsrc, const double* alp
     const int G = c->cfg.n_groups;
     const bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(set_step_inputs(c, c->dt_min, Lsrc, alpha));
     RT_CUDA(c, cudaMemsetAsync(c->acc_t.p, 0, (size_t)32 * G * c->n, c->stream));   // 32 B per (particle, group)
     for (int s = 0; s < (1 << c->bins_max); ++s)
         RT_TRY(launch_step_bins(c, c->stream, s, c->U_a.p, has_src, alpha != nullptr));
-    RT_TRY(state_out(c, c->U_a.p, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->U_a.p, U, 4 * G));
     return RT_OK;
 }
 
@@ -332,10 +331,10 @@ rt_status rt_drift(rt_ctx* c, void* U, const double* v, double dt_drift) {
     if (!std::isfinite(dt_drift)) return fail(c, RT_ERR_INVALID, "dt_drift must be finite");
     const int G = c->cfg.n_groups;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(launch_gradient(c, c->stream, c->U_a.p));
     RT_TRY(launch_drift(c, c->stream, c->U_a.p, v, dt_drift));
-    RT_TRY(state_out(c, c->U_a.p, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->U_a.p, U, 4 * G));
     return RT_OK;
 }
 
@@ -346,7 +345,7 @@ rt_status rt_transport_step(rt_ctx* c, double dt, void* U, const double* Lsrc, c
     const int G = c->cfg.n_groups;
     bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     if (c->profiling) {
         destroy_prof(c->plain_prof);
@@ -357,7 +356,7 @@ rt_status rt_transport_step(rt_ctx* c, double dt, void* U, const double* Lsrc, c
     c->prof_sink = nullptr;
     if (c->profiling) c->last_prof = &c->plain_prof;
     RT_TRY(s);
-    RT_TRY(state_out(c, c->U_b.p, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->U_b.p, U, 4 * G));
     return RT_OK;
 }
 
@@ -367,11 +366,11 @@ rt_status rt_transport_step_given_gradients(rt_ctx* c, double dt, void* U, const
     if (!std::isfinite(dt) || dt < 0) return fail(c, RT_ERR_INVALID, "dt must be finite and >= 0");
     const int G = c->cfg.n_groups;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
-    RT_TRY(state_in(c, gradU, c->grad_t.p, 12 * G, 12 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
+    RT_TRY(state_in(c, gradU, c->grad_t.p, 12 * G));
     RT_TRY(set_step_inputs(c, dt, nullptr, alpha));
     RT_TRY(launch_flux_given(c, c->stream, c->U_a.p, c->U_b.p, alpha != nullptr));
-    RT_TRY(state_out(c, c->U_b.p, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->U_b.p, U, 4 * G));
     return RT_OK;
 }
 
@@ -389,10 +388,10 @@ rt_status rt_inject(rt_ctx* c, double dt, void* U, const double* Lsrc) {
     if (!std::isfinite(dt) || dt < 0) return fail(c, RT_ERR_INVALID, "dt must be finite and >= 0");
     if (!Lsrc || c->n_src == 0 || c->n_inj_targets == 0) return RT_OK;
     const int G = c->cfg.n_groups;
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(set_step_inputs(c, dt, Lsrc, nullptr));
     RT_TRY(launch_inject(c, c->stream, c->U_a.p));
-    RT_TRY(state_out(c, c->U_a.p, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->U_a.p, U, 4 * G));
     return RT_OK;
 }
 
@@ -406,7 +405,7 @@ rt_status rt_subcycle(rt_ctx* c, int32_t n_sub, double dt, void* U, const double
     bool has_src = Lsrc && c->n_src > 0 && c->n_inj_targets > 0;
     bool has_alpha = alpha != nullptr;
     RT_TRY(prepare_pair_geometry(c));
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U, c->U_a.p, 4 * G));
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     // sub-cycles after the first take their injection from the previous gather
     RT_TRY(set_dense_injection(c, has_src && n_sub > 1));
@@ -448,7 +447,7 @@ rt_status rt_subcycle(rt_ctx* c, int32_t n_sub, double dt, void* U, const double
     c->launches += it->second.kernels;
     if (c->profiling) c->last_prof = &it->second.prof;
     void* fin = (n_sub % 2 == 0) ? c->U_a.p : c->U_b.p;
-    RT_TRY(state_out(c, fin, U, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, fin, U, 4 * G));
     return RT_OK;
 }
 
@@ -469,13 +468,13 @@ rt_status rt_adjoint(rt_ctx* c, int32_t n_sub, double dt, int32_t ckpt_every, co
     RT_TRY(set_step_inputs(c, dt, Lsrc, alpha));
     RT_TRY(ensure(c, c->lam_a, (size_t)4 * G * c->n * tsize(c), "adjoint"));
     RT_TRY(ensure(c, c->lam_b, (size_t)4 * G * c->n * tsize(c), "adjoint"));
-    RT_TRY(state_in(c, U0, c->U_a.p, 4 * G, 4 * G, 0));
-    RT_TRY(state_in(c, dLdU_final, c->lam_a.p, 4 * G, 4 * G, 0));
+    RT_TRY(state_in(c, U0, c->U_a.p, 4 * G));
+    RT_TRY(state_in(c, dLdU_final, c->lam_a.p, 4 * G));
     if (dLdLsrc && c->n_src > 0)
         RT_CUDA(c, cudaMemsetAsync(dLdLsrc, 0, (size_t)c->n_src * G * sizeof(double), c->stream));
     RT_TRY(run_adjoint(c, n_sub, ckpt_every, has_src, alpha != nullptr, c->U_a.p, c->lam_a.p, c->lam_b.p,
                        (dLdLsrc && c->n_src > 0) ? dLdLsrc : nullptr));
-    RT_TRY(state_out(c, c->lam_b.p, dLdU0, 4 * G, 4 * G, 0));
+    RT_TRY(state_out(c, c->lam_b.p, dLdU0, 4 * G));
     return RT_OK;
 }
 
@@ -483,9 +482,8 @@ rt_status rt_energy(rt_ctx* c, const void* U, double* E_host) {
     RT_TRY(check_ready(c));
     if (!U || !E_host) return fail(c, RT_ERR_INVALID, "NULL array");
     const int G = c->cfg.n_groups;
-    RT_TRY(state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0));
     double* out = c->energy_part.as<double>() + (size_t)G * 512;
-    RT_TRY(launch_energy(c, c->stream, c->U_a.p, out));
+    RT_TRY(launch_energy(c, c->stream, U, out));
     RT_CUDA(c, cudaMemcpyAsync(E_host, out, G * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     int timed_out = 0;
     RT_CUDA(c, cudaMemcpyAsync(&timed_out, c->flags.as<int>() + F_TIMEOUT, sizeof(int), cudaMemcpyDeviceToHost,
@@ -683,7 +681,7 @@ rt_status rt_autotune(rt_ctx* c, const void* U, double dt, int32_t n_sub, const 
         }
         double kbest = 0.0;
         for (int r = 0; r <= repeats && st == RT_OK; ++r) {   // r = 0 warms up
-            st = state_in(c, U, c->U_a.p, 4 * G, 4 * G, 0);
+            st = state_in(c, U, c->U_a.p, 4 * G);
             if (st != RT_OK) break;
             void* a = c->U_a.p;
             void* b = c->U_b.p;

@@ -1207,12 +1207,12 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
     double V = INFINITY;
     if (p < n) {
         const double box[3] = {b0, b1, b2};
-        double hi = h[p], H = kKappa * hi, iH = rcp_fast(H);
+        double hi = h[p], H = kKappa * hi, iH = 1.0 / H;
         double om = omega[p];
         double E[6];
         accumulate_E<T>(xs, xq, box, periodic, s0, s1, s2, n, p, H, row_off, cols, E);
-        V = rcp_fast(om);
-        const double s3 = kSigma * iH * iH * iH, fac = s3 * V;   // psi = fac * w
+        V = 1.0 / om;                              // V, 1/H and bp as in k_set_fields
+        const double fac = kSigma * iH * iH * iH * V;   // psi = fac * w
         double e_xx = E[0] * fac, e_yy = E[1] * fac, e_zz = E[2] * fac;
         double e_xy = E[3] * fac, e_xz = E[4] * fac, e_yz = E[5] * fac;
         // cofactor inverse of the symmetric matrix
@@ -1244,7 +1244,7 @@ __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restric
             const float lmin = fminf(ev[0], fminf(ev[1], ev[2])), lmax = fmaxf(ev[0], fmaxf(ev[1], ev[2]));
             cond = lmin > 0.f ? lmax / lmin : INFINITY;
             cond_out[p] = cond;
-            const double bp = V * fac;   // V_i psitilde_j(x_i) = Bp_i d w(q_ij)
+            const double bp = V * V * kSigma * iH * iH * iH;   // V_i psitilde_j(x_i) = Bp_i d w(q_ij)
             geo_t[8 * p] = (T)iH;
             geo_t[8 * p + 1] = (T)hi;
             for (int k = 0; k < 6; ++k) {

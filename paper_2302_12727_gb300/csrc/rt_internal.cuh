@@ -24,7 +24,13 @@ constexpr double kSigma = 5.0929581789406507446;   // 16 / pi
 enum FlagSlot { F_BADPOS = 0, F_NOCONV = 1, F_GEOM = 2, F_ILL = 3, F_SRC_NOCONV = 4, F_REFINE = 5, F_BADH = 6, F_OVER = 7,
                 F_NSLOTS = 8, F_CLAMP = 8,
                 F_TIMEOUT = 12, F_SCRATCH = 13, F_SELFTEST = 15 };
-constexpr int kMaxGC = 4;                          // groups handled by one pair-kernel launch
+constexpr int kMaxGC = 4;                          // most groups handled by one pair-kernel launch
+// groups of a chunk: G groups in as few chunks as kMaxGC allows, of even size (five groups as
+// 3 + 2: a chunk of one pays the pair geometry for itself alone)
+inline int chunk_groups(int G) {
+    const int chunks = (G + kMaxGC - 1) / kMaxGC;
+    return (G + chunks - 1) / chunks;
+}
 // Packed flux rows start with a prefix that repeats their last kRowRot words: a row copy that
 // starts at word kRowRot delivers the row, one that starts at word 0 delivers it rotated by
 // four 16-byte chunks (the pair pass uses both, see k_flux_tma).
@@ -117,7 +123,7 @@ struct rt_ctx {
     rt::DevBuf U_a, U_b, grad_t, alpha_s, L_dev, dt_dev, energy_part;
     rt::DevBuf inj_dense;                               // dt sum coef L per (particle, group), [N][G] double
     bool inj_dense_ready = false;                       // filled by set_step_inputs for this call
-    rt::DevBuf frec;                                    // packed float flux-input rows (G <= 4)
+    rt::DevBuf frec;                                    // packed float flux-input rows of a group chunk
     rt::DevBuf wave_t;                                  // HLL wave-speed table, working precision
     // photo-ionisation sink per group (rt_set_absorbers): alpha in caller order [G][N]
     // (double), its sorted working-precision copy [N][G], the cross sections
@@ -135,9 +141,10 @@ struct rt_ctx {
     // prefix (cum_*[level] = entries with a key <= level)
     rt::DevBuf bins_nmin, order_b, order_m, order_q, bin_keys, bin_keys2, bin_vals, bin_cub, bin_hist;
     std::vector<int64_t> cum_b, cum_m, cum_q;
-    CUtensorMap rows_map{};                             // tensor map of frec (tile::gather4)
-    const void* rows_map_for = nullptr;
-    int64_t rows_map_n = 0;
+    // tensor maps of frec (tile::gather4), by the number of groups of a chunk
+    CUtensorMap rows_map[rt::kMaxGC + 1]{};
+    const void* rows_map_for[rt::kMaxGC + 1]{};
+    int64_t rows_map_n[rt::kMaxGC + 1]{};
     // adjoint
     rt::DevBuf ck, seg, lam_a, lam_b, adj_w, adj_x, adj_ub, adj_gam, adj_lam;
     int64_t ck_cap = 0, seg_cap = 0;
@@ -191,9 +198,9 @@ namespace rt {
 rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const double* xsrc,
                            const double* h_in = nullptr, const double* hs_in = nullptr,
                            const double* oms_in = nullptr, const double* octw_in = nullptr);
-// caller-order component-major arrays <-> sorted records (comps values at record offset off)
-rt_status state_in(rt_ctx* c, const void* U_user, void* rec, int comps, int RS, int off);
-rt_status state_out(rt_ctx* c, const void* rec, void* U_user, int comps, int RS, int off);
+// caller-order component-major arrays <-> sorted records of comps values (a multiple of four)
+rt_status state_in(rt_ctx* c, const void* U_user, void* rec, int comps);
+rt_status state_out(rt_ctx* c, const void* rec, void* U_user, int comps);
 // sorted double per-particle fields [comps][N] -> caller order
 rt_status field_out(rt_ctx* c, const double* src_sorted, double* dst_user, int comps);
 rt_status set_step_inputs(rt_ctx* c, double dt, const double* Lsrc, const double* alpha);
@@ -218,7 +225,8 @@ rt_status launch_step_bins(rt_ctx* c, cudaStream_t s, int step, void* U, bool ha
 // rec += grad_t . (v dt) per component (needs launch_gradient on rec first)
 rt_status launch_drift(rt_ctx* c, cudaStream_t s, void* rec, const double* v, double dt);
 rt_status launch_inject(rt_ctx* c, cudaStream_t s, void* rec);
-rt_status launch_energy(rt_ctx* c, cudaStream_t s, const void* rec, double* out_dev);
+// energies per group of the caller's state U
+rt_status launch_energy(rt_ctx* c, cudaStream_t s, const void* U, double* out_dev);
 rt_status run_adjoint(rt_ctx* c, int n_sub, int ckpt_every, bool has_src, bool has_alpha, const void* U0_sorted,
                       const void* lam_final_sorted, void* lam0_sorted, double* dLdL_dev);
 }  // namespace rt

@@ -46,22 +46,32 @@ static int pair_warps(const rt_ctx* c) { return c->tune.pair_warps > 0 ? c->tune
 
 // ------------------------------------------------------------------------------------
 // caller order <-> cell-sorted records
+// One thread per particle (caller order) and four components: the caller's planes are read and
+// written side by side, the records in pieces of four values.  Records filled in sorted order
+// instead, each value a 4-byte read at a random place, took 0.385 ms for 2,097,152 particles of
+// four groups.
 template <class T>
-__global__ void k_state_in(const T* __restrict__ src, const int32_t* __restrict__ perm, int64_t n, int comps, int RS,
-                           int off, T* __restrict__ rec) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int64_t i = perm[p];
-    for (int c = 0; c < comps; ++c) rec[p * RS + off + c] = src[c * n + i];
+__global__ void __launch_bounds__(256) k_state_in(const T* __restrict__ src, const int32_t* __restrict__ inv_perm,
+                                                  int64_t n, int RS, T* __restrict__ rec) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int c = 4 * blockIdx.y;
+    T v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = src[(c + q) * n + i];
+    vstore<4>(rec + (int64_t)inv_perm[i] * RS + c, v);
 }
 
 template <class T>
-__global__ void k_state_out(const T* __restrict__ rec, const int32_t* __restrict__ inv_perm, int64_t n, int comps,
-                            int RS, int off, T* __restrict__ dst) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(256) k_state_out(const T* __restrict__ rec, const int32_t* __restrict__ inv_perm,
+                                                   int64_t n, int RS, T* __restrict__ dst) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
-    int64_t p = inv_perm[i];
-    for (int c = 0; c < comps; ++c) dst[c * n + i] = rec[p * RS + off + c];
+    const int c = 4 * blockIdx.y;
+    T v[4];
+    vload<4>(rec + (int64_t)inv_perm[i] * RS + c, v);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) dst[(c + q) * n + i] = v[q];
 }
 
 // plain SoA gathers (double per-particle fields)
@@ -207,9 +217,9 @@ __global__ void __launch_bounds__(128) k_gradient(PairArgs<T> a, const T* __rest
         for (int c = 0; c < NC; ++c) {
             T dq0 = u0[c] - ui[c];
             T dq1 = u1[c] - ui[c];
-            acc[c][0] += dq0 * wx0 + dq1 * wx1;
-            acc[c][1] += dq0 * wy0 + dq1 * wy1;
-            acc[c][2] += dq0 * wz0 + dq1 * wz1;
+            acc[c][0] = fma_rn(dq1, wx1, fma_rn(dq0, wx0, acc[c][0]));
+            acc[c][1] = fma_rn(dq1, wy1, fma_rn(dq0, wy0, acc[c][1]));
+            acc[c][2] = fma_rn(dq1, wz1, fma_rn(dq0, wz0, acc[c][2]));
         }
     }
     T M[6];
@@ -221,9 +231,9 @@ __global__ void __launch_bounds__(128) k_gradient(PairArgs<T> a, const T* __rest
     for (int c = 0; c < NC; ++c) sym_mv(M, acc[c][0], acc[c][1], acc[c][2], out[3 * c], out[3 * c + 1], out[3 * c + 2]);
     if (a.frec) {
         T* row = packed_row(a, i);
-        row_store<3 * NC>(a, row, 12 + 4 * a.G + 12 * g0, out);
-        row_store<NC>(a, row, 12 + 4 * g0, ui);
-        if (g0 == 0) packed_static(a, i, row);
+        row_store<3 * NC>(a, row, 12 + NC, out);
+        row_store<NC>(a, row, 12, ui);
+        packed_static(a, i, row);
     } else {
         vstore<3 * NC>(grad + i * 12 * a.G + 12 * g0, out);
     }
@@ -390,9 +400,9 @@ __global__ void __launch_bounds__(256) k_gradient_g(PairArgs<float> a, const flo
         for (int c = 0; c < 4; ++c) {
             float dq0 = u0[c] - ui[c];
             float dq1 = u1[c] - ui[c];
-            acc[c][0] += dq0 * wx0 + dq1 * wx1;
-            acc[c][1] += dq0 * wy0 + dq1 * wy1;
-            acc[c][2] += dq0 * wz0 + dq1 * wz1;
+            acc[c][0] = fma_rn(dq1, wx1, fma_rn(dq0, wx0, acc[c][0]));
+            acc[c][1] = fma_rn(dq1, wy1, fma_rn(dq0, wy0, acc[c][1]));
+            acc[c][2] = fma_rn(dq1, wz1, fma_rn(dq0, wz0, acc[c][2]));
         }
     }
     float M[6];
@@ -404,9 +414,9 @@ __global__ void __launch_bounds__(256) k_gradient_g(PairArgs<float> a, const flo
     for (int c = 0; c < 4; ++c) sym_mv(M, acc[c][0], acc[c][1], acc[c][2], out[3 * c], out[3 * c + 1], out[3 * c + 2]);
     if (a.frec) {
         float* row = packed_row(a, i);
-        row_store<12>(a, row, 12 + 4 * a.G + 12 * (g0 + g), out);
-        row_store<4>(a, row, 12 + off, ui);
-        if (g0 + g == 0) packed_static(a, i, row);
+        row_store<12>(a, row, 12 + 4 * GC + 12 * g, out);
+        row_store<4>(a, row, 12 + 4 * g, ui);
+        if (g == 0) packed_static(a, i, row);
     } else {
         vstore<12>(grad + i * 12 * a.G + 12 * (g0 + g), out);
     }
@@ -493,9 +503,9 @@ __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax 
             for (int c = 0; c < 4; ++c) {
                 float dq0 = u0[c] - ui[c];
                 float dq1 = u1[c] - ui[c];
-                acc[c][0] += dq0 * X0 + dq1 * X1;
-                acc[c][1] += dq0 * Y0 + dq1 * Y1;
-                acc[c][2] += dq0 * Z0 + dq1 * Z1;
+                acc[c][0] = fma_rn(dq1, X1, fma_rn(dq0, X0, acc[c][0]));
+                acc[c][1] = fma_rn(dq1, Y1, fma_rn(dq0, Y0, acc[c][1]));
+                acc[c][2] = fma_rn(dq1, Z1, fma_rn(dq0, Z0, acc[c][2]));
             }
         }
         ea = en;
@@ -514,9 +524,9 @@ __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax 
     for (int c = 0; c < 4; ++c) sym_mv(M, acc[c][0], acc[c][1], acc[c][2], out[3 * c], out[3 * c + 1], out[3 * c + 2]);
     if (a.frec) {
         float* row = packed_row(a, i);
-        row_store<12>(a, row, 12 + 4 * a.G + 12 * (g0 + g), out);
-        row_store<4>(a, row, 12 + off, ui);
-        if (g0 + g == 0) packed_static(a, i, row);
+        row_store<12>(a, row, 12 + 4 * GC + 12 * g, out);
+        row_store<4>(a, row, 12 + 4 * g, ui);
+        if (g == 0) packed_static(a, i, row);
     } else {
         vstore<12>(grad + i * 12 * a.G + 12 * (g0 + g), out);
     }
@@ -1015,6 +1025,104 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
     if (act) vstore<NC>(pairbuf + slot * NC, out);
 }
 
+// The same pair pass for the HLL solver, with the wave-speed table (81,608 bytes) in shared memory: one
+// block per SM, as many warps as rows fit beside the table, each walking batches of 32 slots.
+// A batch's 32 lanes read 32 scattered nodes of the table in each of its 8 lookups a group:
+// from L1 that is a wavefront a line and the kernel's bound (0.251 ms on 131,071 particles and
+// three groups), from shared memory a few bank conflicts.
+template <int G>
+struct HllShape {
+    static constexpr int table = RT_WAVE_NF * RT_WAVE_NTH * 8;
+    static constexpr int warps = (226 * 1024 - 512 - table) / (PackedRows<G>::WF * 4) < 20
+                                     ? (226 * 1024 - 512 - table) / (PackedRows<G>::WF * 4)
+                                     : 20;
+    static constexpr int smem = 128 + warps * PackedRows<G>::WF * 4 + table;
+};
+template <int G>
+__global__ void __launch_bounds__(HllShape<G>::warps * 32, 1)
+k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
+           const __grid_constant__ CUtensorMap rows, int* err_flag, unsigned long long budget) {
+    using R = PackedRows<G>;
+    constexpr int NC = 4 * G, RW = R::RW;
+    extern __shared__ __align__(128) float sm_dyn[];
+    __shared__ __align__(8) uint64_t bar[32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t sm0 = smem_u32(sm_dyn);
+    float* sm = sm_dyn + (((sm0 + 127u) & ~127u) - sm0) / 4u;
+    float* ws = sm + wid * R::WF;
+    const float2* tab = reinterpret_cast<const float2*>(sm + (blockDim.x >> 5) * R::WF);
+    for (int k = threadIdx.x; k < RT_WAVE_NF * RT_WAVE_NTH; k += blockDim.x)
+        const_cast<float2*>(tab)[k] = reinterpret_cast<const float2*>(x.wave)[k];
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t mb = smem_u32(&bar[wid]);
+    if (lane == 0) mbar_init(mb, 1);
+    __syncthreads();
+    const int64_t np = a.n_pairs, stride = gridDim.x * (int64_t)blockDim.x;
+    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    // lanes past the last slot gather particle 0 (always present) and store nothing
+    int2 kl = t < np ? a.ends[t] : make_int2(0, 0);
+    for (uint32_t parity = 0; t - lane < np; parity ^= 1) {
+        if (lane == 0) mbar_expect_tx(mb, R::bytes);
+        __syncwarp();
+        const int q = lane & 7;
+        const int r0 = __shfl_sync(FULL, kl.y, 4 * q), r1 = __shfl_sync(FULL, kl.y, 4 * q + 1);
+        const int r2 = __shfl_sync(FULL, kl.y, 4 * q + 2), r3 = __shfl_sync(FULL, kl.y, 4 * q + 3);
+        // even slots get the rows as they are (copy from word kRowRot), odd slots rotated by four
+        // chunks (copy from word 0 of the prefixed row)
+        if (lane < 8) tma_gather4(smem_u32(ws + q * R::SLOT), &rows, (q & 1) ? 0 : kRowRot, r0, r1, r2, r3, mb);
+        // the next batch's ends, under this batch's copies and arithmetic
+        const int64_t slot = t;
+        t += stride;
+        const int2 kl_next = t < np ? a.ends[t] : make_int2(0, 0);
+        const float* rk = packed_row(a, (int64_t)kl.x);
+        const uint4 pkv = *reinterpret_cast<const uint4*>(rk);
+        const Pos<float> pi = {pkv.x, pkv.y, pkv.z};
+        float gi8[8], gj8[8];
+        vload<8>(rk + 4, gi8);
+        if (!mbar_wait(mb, parity, budget)) {
+            atomicExch(err_flag, 1);
+            // let the copies still in flight land before the block exits, however short the
+            // caller's budget (a copy lands in microseconds; this wait too is bounded)
+            mbar_wait(mb, parity, budget > 2000000000ull ? budget : 2000000000ull);
+            return;
+        }
+        // this lane's row: slot lane / 4, row lane % 4 within it.  A quarter-warp reads the rows
+        // of one even and one odd slot; the slots start on the same bank, and the rows of a slot
+        // cover four of the eight 16-byte bank groups at any one chunk, so the odd slot's rotation
+        // by four chunks sends its lanes to the other four (all but the last four chunks).
+        // Logical chunk c is at chunk c (even slot), c + 4 or, for the last four, c + 4 - RW / 4.
+        const float* rl = ws + (lane >> 2) * R::SLOT + (lane & 3) * RW;
+        const bool odd = (lane >> 2) & 1;
+        const float* rlA = rl + (odd ? kRowRot : 0);
+        const float* rlB = rl + (odd ? kRowRot - RW : 0);
+        constexpr int NCH = RW / 4;
+        auto lrow = [&](int c) -> const float* { return (c < NCH - kRowRot / 4 ? rlA : rlB) + 4 * c; };
+        const uint4 pv = *reinterpret_cast<const uint4*>(lrow(0));
+        const Pos<float> pj = {pv.x, pv.y, pv.z};
+        vload<8>(lrow(1), gj8);
+        float dx, dy, dz;
+        sep(a.sp, pi, pj, dx, dy, dz);
+        PairGeo<float> pr;
+        float sk, sl;
+        pair_geo(dx, dy, dz, gi8, gj8, x.c, pr, sk, sl);
+        float out[NC];
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+            float ui[4], uj[4], gri[12], grj[12];
+            vload<4>(rk + 12 + 4 * g, ui);
+            vload<4>(lrow(3 + g), uj);
+            vload<12>(rk + 12 + 4 * G + 12 * g, gri);
+            vload<4>(lrow(3 + G + 3 * g), grj);
+            vload<4>(lrow(4 + G + 3 * g), grj + 4);
+            vload<4>(lrow(5 + G + 3 * g), grj + 8);
+            pair_flux<true>(ui, uj, gri, grj, pr, x.c, reinterpret_cast<const float*>(tab), &out[4 * g]);
+        }
+        if (slot < np) vstore<NC>(pairbuf + slot * NC, out);
+        kl = kl_next;
+        __syncwarp();      // every lane has read its row before the next copies overwrite it
+    }
+}
+
 // Float pass 2 with one thread per (particle, group): the lanes of one particle read the
 // 16-byte pieces of a slot that lie side by side, so a warp request touches about 32 / GC
 // slots instead of 32.  Same order of additions and subtractions as k_flux_gather.
@@ -1107,23 +1215,32 @@ rt_status launch_drift(rt_ctx* c, cudaStream_t s, void* rec, const double* v, do
 // a10: energy per group, sum_i V_i E_i,g in double; fixed grid and tree order.
 constexpr int kEnergyBlocks = 512;
 
-// Particles of caller index >= owned (the ghost copies of a domain decomposition) are left out.
+// Reads the caller's state, particles [0, owned) (the ghost copies of a domain decomposition come
+// after them); V is in sorted order.
 template <class T>
-__global__ void k_energy_part(const T* __restrict__ rec, int RS, const double* __restrict__ V, int64_t n, int G,
-                              const int32_t* __restrict__ perm, int64_t owned, double* part) {
+__global__ void __launch_bounds__(256)
+k_energy_part(const T* __restrict__ U, const double* __restrict__ V, int64_t n, int G,
+              const int32_t* __restrict__ inv_perm, int64_t owned, double* __restrict__ part) {
     __shared__ double sm[256];
-    for (int g = 0; g < G; ++g) {
-        double s = 0.0;
-        for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x)
-            if (owned >= n || perm[p] < owned) s += V[p] * (double)rec[p * RS + 4 * g];
-        sm[threadIdx.x] = s;
-        __syncthreads();
-        for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sm[threadIdx.x] += sm[threadIdx.x + w];
+    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
+        double s[kMaxGC] = {0.0, 0.0, 0.0, 0.0};
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < owned;
+             i += (int64_t)gridDim.x * blockDim.x) {
+            const double v = V[inv_perm[i]];
+#pragma unroll
+            for (int g = 0; g < kMaxGC; ++g)
+                if (g0 + g < G) s[g] += v * (double)U[(int64_t)4 * (g0 + g) * n + i];
+        }
+        for (int g = 0; g < kMaxGC && g0 + g < G; ++g) {
+            sm[threadIdx.x] = s[g];
+            __syncthreads();
+            for (int w = blockDim.x / 2; w > 0; w >>= 1) {
+                if (threadIdx.x < w) sm[threadIdx.x] += sm[threadIdx.x + w];
+                __syncthreads();
+            }
+            if (threadIdx.x == 0) part[(g0 + g) * gridDim.x + blockIdx.x] = sm[0];
             __syncthreads();
         }
-        if (threadIdx.x == 0) part[g * gridDim.x + blockIdx.x] = sm[0];
-        __syncthreads();
     }
 }
 
@@ -1161,14 +1278,18 @@ static void set_carveouts() {
 }
 
 template <class T>
-static void launch_gradient_t(rt_ctx* c, cudaStream_t s, T* rec, bool packed = false) {
+static void launch_gradient_t(rt_ctx* c, cudaStream_t s, T* rec, bool packed = false, int only = -1) {
     set_carveouts<T>();
     PairArgs<T> a = pair_args<T>(c);
-    if (packed) a.frec = c->frec.as<T>();
     const int G = c->cfg.n_groups;
     unsigned nb = nblk(c->n, 128);
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        if (only >= 0 && g0 != only) continue;
+        int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
+        if (packed) {
+            a.frec = c->frec.as<T>();
+            a.RW = 12 + 16 * gc;
+        }
         int pr = prof_begin(c, s, RT_KERNEL_GRADIENT);
         if constexpr (std::is_same<T, float>::value) {
             if (c->tune.gradient_variant == 2 && gc > 1) {
@@ -1242,11 +1363,12 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
     return fn;
 }
 
-// tensor map of the packed rows [n][kRowRot + 12 + 16G] floats, box of the 12 + 16G logical
-// words of a row (for tile::gather4); encoded again whenever the buffer or its shape changes
-static bool packed_rows_map(rt_ctx* c) {
-    const int RW = 12 + 16 * c->cfg.n_groups;
-    if (c->rows_map_for == c->frec.p && c->rows_map_n == c->n) return true;
+// tensor map of the packed rows [n][kRowRot + 12 + 16 gc] floats of a chunk of gc groups, box of
+// the 12 + 16 gc logical words of a row (for tile::gather4); encoded again whenever the buffer or
+// its shape changes
+static bool packed_rows_map(rt_ctx* c, int gc) {
+    const int RW = 12 + 16 * gc;
+    if (c->rows_map_for[gc] == c->frec.p && c->rows_map_n[gc] == c->n) return true;
     PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
     if (!enc || !c->frec.p) return false;
     // rows of kRowRot + RW words (the prefix first); the box is the RW logical words
@@ -1254,12 +1376,21 @@ static bool packed_rows_map(rt_ctx* c) {
     cuuint64_t strides[1] = {(cuuint64_t)(RW + kRowRot) * 4};
     cuuint32_t box[2] = {(cuuint32_t)RW, 1};
     cuuint32_t estr[2] = {1, 1};
-    CUresult r = enc(&c->rows_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->frec.p, dims, strides, box, estr,
+    CUresult r = enc(&c->rows_map[gc], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, c->frec.p, dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return false;
-    c->rows_map_for = c->frec.p;
-    c->rows_map_n = c->n;
+    c->rows_map_for[gc] = c->frec.p;
+    c->rows_map_n[gc] = c->n;
+    return true;
+}
+
+// whether the float pair pass fetches packed rows: its variant, and tensor maps for the chunks
+static bool packed_rows(rt_ctx* c) {
+    const int G = c->cfg.n_groups, cs = chunk_groups(G);
+    if (c->fp64 || c->tune.flux_variant != 2) return false;
+    for (int g0 = 0; g0 < G; g0 += cs)
+        if (!packed_rows_map(c, G - g0 < cs ? G - g0 : cs)) return false;
     return true;
 }
 
@@ -1275,6 +1406,9 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
         cudaFuncSetAttribute((const void*)k_flux_gather_g<GC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
         cudaFuncSetAttribute((const void*)k_flux_tma<GC, HLL>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
+        if (HLL)
+            cudaFuncSetAttribute((const void*)k_flux_hll<GC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 HllShape<GC>::smem);
         (void)cudaGetLastError();
     }
     unsigned npb = nblk(std::max<int64_t>(a.n_pairs, 1), 128);
@@ -1285,9 +1419,15 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
         unsigned long long budget = c->cfg.device_wait_budget_cycles ? c->cfg.device_wait_budget_cycles
                                                                      : 4000000000ull;
         const int pw = pair_warps(c);
-        k_flux_tma<GC, HLL><<<nblk(std::max<int64_t>(a.n_pairs, 1), pw * 32), pw * 32,
-                              (size_t)pw * PackedRows<GC>::WF * sizeof(float) + 128, s>>>(
-            a, x, pb, c->rows_map, c->flags.as<int>() + F_TIMEOUT, budget);
+        int* ef = c->flags.as<int>() + F_TIMEOUT;
+        // HLL: with two batches a warp or more, the table in shared memory is worth loading
+        if (HLL && a.n_pairs >= (int64_t)c->sm_count * HllShape<GC>::warps * 64)
+            k_flux_hll<GC><<<c->sm_count, HllShape<GC>::warps * 32, HllShape<GC>::smem, s>>>(
+                a, x, pb, c->rows_map[GC], ef, budget);
+        else
+            k_flux_tma<GC, HLL><<<nblk(std::max<int64_t>(a.n_pairs, 1), pw * 32), pw * 32,
+                                  (size_t)pw * PackedRows<GC>::WF * sizeof(float) + 128, s>>>(
+                a, x, pb, c->rows_map[GC], ef, budget);
     } else if (variant == 1) {
         k_flux_staged<GC, HLL><<<npb, 128, 0, s>>>(a, x, rec, pb, g0);
     } else {
@@ -1305,9 +1445,8 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
 
 template <class T>
 static void launch_flux_t(rt_ctx* c, cudaStream_t s, const T* rec, T* out, bool has_alpha, bool packed = false,
-                          bool inject_after = false) {
+                          bool inject_after = false, int only = -1) {
     PairArgs<T> a = pair_args<T>(c);
-    if (packed) a.frec = c->frec.as<T>();
     FluxExtra<T> x;
     const bool hll = c->cfg.riemann_solver == RT_RIEMANN_HLL;
     x.wave = hll ? c->wave_t.as<T>() : nullptr;
@@ -1323,8 +1462,13 @@ static void launch_flux_t(rt_ctx* c, cudaStream_t s, const T* rec, T* out, bool 
     unsigned nb = nblk(c->n, 128);
     T* pb = c->pairbuf.as<T>();
     unsigned npb = nblk(std::max<int64_t>(a.n_pairs, 1), 128);
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        if (only >= 0 && g0 != only) continue;
+        int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
+        if (packed) {
+            a.frec = c->frec.as<T>();
+            a.RW = 12 + 16 * gc;
+        }
         if constexpr (std::is_same<T, float>::value) {
             if (hll) {
                 switch (gc) {
@@ -1398,18 +1542,19 @@ rt_status launch_gradient(rt_ctx* c, cudaStream_t s, void* rec) {
     return RT_OK;
 }
 
-// packed flux rows from sorted states and gradients given in grad_t (one thread per
-// particle and group): what the gradient kernels write beside their gradients
-__global__ void k_pack_rows(PairArgs<float> a, const float* __restrict__ rec, const float* __restrict__ grad) {
+// packed flux rows of the groups [g0, g0 + gc) from sorted states and gradients given in grad_t
+// (one thread per particle and group): what the gradient kernels write beside their gradients
+__global__ void k_pack_rows(PairArgs<float> a, const float* __restrict__ rec, const float* __restrict__ grad, int g0,
+                            int gc) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t i = t / a.G;
+    const int64_t i = t / gc;
     if (i >= a.n) return;
-    const int g = (int)(t - i * a.G);
+    const int g = (int)(t - i * gc);
     float* row = packed_row(a, i);
     float gq[12], u[4];
-    vload<12>(grad + i * 12 * a.G + 12 * g, gq);
-    vload<4>(rec + i * 4 * a.G + 4 * g, u);
-    row_store<12>(a, row, 12 + 4 * a.G + 12 * g, gq);
+    vload<12>(grad + i * 12 * a.G + 12 * (g0 + g), gq);
+    vload<4>(rec + i * 4 * a.G + 4 * (g0 + g), u);
+    row_store<12>(a, row, 12 + 4 * gc + 12 * g, gq);
     row_store<4>(a, row, 12 + 4 * g, u);
     if (g == 0) packed_static(a, i, row);
 }
@@ -1418,15 +1563,20 @@ rt_status launch_flux_given(rt_ctx* c, cudaStream_t s, void* Uin, void* Uout, bo
     if (c->fp64) {
         launch_flux_t<double>(c, s, (const double*)Uin, (double*)Uout, has_alpha);
     } else {
-        const bool packed = c->tune.flux_variant == 2 && c->cfg.n_groups <= kMaxGC && packed_rows_map(c);
-        if (packed) {
-            PairArgs<float> a = pair_args<float>(c);
-            a.frec = c->frec.as<float>();
-            k_pack_rows<<<nblk(c->n * c->cfg.n_groups, 256), 256, 0, s>>>(a, (const float*)Uin,
-                                                                          c->grad_t.as<float>());
-            ++c->launches;
+        const int G = c->cfg.n_groups, cs = chunk_groups(G);
+        if (!packed_rows(c)) {
+            launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha);
+        } else {
+            for (int g0 = 0; g0 < G; g0 += cs) {
+                const int gc = G - g0 < cs ? G - g0 : cs;
+                PairArgs<float> a = pair_args<float>(c);
+                a.frec = c->frec.as<float>();
+                a.RW = 12 + 16 * gc;
+                k_pack_rows<<<nblk(c->n * gc, 256), 256, 0, s>>>(a, (const float*)Uin, c->grad_t.as<float>(), g0, gc);
+                ++c->launches;
+                launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha, true, false, g0);
+            }
         }
-        launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha, packed);
     }
     RT_CUDA(c, cudaGetLastError());
     return RT_OK;
@@ -1496,15 +1646,14 @@ static void bins_flux_tma(rt_ctx* c, cudaStream_t s, const PairArgs<T>& af, cons
                                  cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
             (void)cudaGetLastError();
         }
-        const unsigned nbf = nblk(std::max<int64_t>(af.count, 1), 128);
         const unsigned long long budget = c->cfg.device_wait_budget_cycles ? c->cfg.device_wait_budget_cycles
                                                                            : 4000000000ull;
         int* ef = c->flags.as<int>() + F_TIMEOUT;
         const int pw = pair_warps(c);
         const size_t smem = (size_t)pw * PackedRows<GC>::WF * sizeof(float) + 128;
         const unsigned nbt = nblk(std::max<int64_t>(af.count, 1), pw * 32);
-        if (hll) k_flux_tma<GC, true, true><<<nbt, pw * 32, smem, s>>>(af, x, pb, c->rows_map, ef, budget);
-        else k_flux_tma<GC, false, true><<<nbt, pw * 32, smem, s>>>(af, x, pb, c->rows_map, ef, budget);
+        if (hll) k_flux_tma<GC, true, true><<<nbt, pw * 32, smem, s>>>(af, x, pb, c->rows_map[GC], ef, budget);
+        else k_flux_tma<GC, false, true><<<nbt, pw * 32, smem, s>>>(af, x, pb, c->rows_map[GC], ef, budget);
     }
 }
 
@@ -1553,13 +1702,13 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
     // step start, which is what its pairs use until its step ends
     bool packed = false;
     if constexpr (std::is_same<T, float>::value)
-        packed = c->tune.flux_variant == 2 && G <= kMaxGC && packed_rows_map(c);
+        packed = G <= kMaxGC && packed_rows(c);
     if (packed) {
         ag.frec = c->frec.as<T>();
         af.frec = c->frec.as<T>();
     }
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        const int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        const int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
         if (n_start == 0) break;
         if constexpr (std::is_same<T, double>::value) {
             if (ag.wd) {
@@ -1581,8 +1730,8 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
         }
         ++c->launches;
     }
-    for (int g0 = 0; g0 < G; g0 += kMaxGC) {
-        const int gc = G - g0 < kMaxGC ? G - g0 : kMaxGC;
+    for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+        const int gc = G - g0 < chunk_groups(G) ? G - g0 : chunk_groups(G);
 #define RT_BINS_FLUX(GC_)                                                                    \
     if (n_pairs > 0) {                                                                       \
         if (packed)                                                                          \
@@ -1630,36 +1779,46 @@ rt_status launch_step(rt_ctx* c, cudaStream_t s, void* Uin, void* Uout, bool has
         launch_flux_t<double>(c, s, (const double*)Uin, (double*)Uout, has_alpha, false, inject_after);
     } else {
         if (inject_first) launch_inject_t<float>(c, s, (float*)Uin);
-        // packed rows for the tensor-memory-accelerator pair pass (one group chunk only)
-        const bool packed = c->tune.flux_variant == 2 && c->cfg.n_groups <= kMaxGC && packed_rows_map(c);
-        launch_gradient_t<float>(c, s, (float*)Uin, packed);
-        launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha, packed, inject_after);
+        // packed rows for the tensor-memory-accelerator pair pass, which hold one chunk of groups:
+        // each chunk's gradient, fluxes and update in turn (a chunk reads and writes its own
+        // groups only).  99,991 particles and five groups: 0.166 ms of pair passes a sub-cycle
+        // with direct loads
+        if (packed_rows(c)) {
+            const int G = c->cfg.n_groups;
+            for (int g0 = 0; g0 < G; g0 += chunk_groups(G)) {
+                launch_gradient_t<float>(c, s, (float*)Uin, true, g0);
+                launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha, true, inject_after, g0);
+            }
+        } else {
+            launch_gradient_t<float>(c, s, (float*)Uin);
+            launch_flux_t<float>(c, s, (const float*)Uin, (float*)Uout, has_alpha, false, inject_after);
+        }
     }
     RT_CUDA(c, cudaGetLastError());
     return RT_OK;
 }
 
-rt_status state_in(rt_ctx* c, const void* U_user, void* rec, int comps, int RS, int off) {
-    unsigned nb = nblk(c->n, 256);
+rt_status state_in(rt_ctx* c, const void* U_user, void* rec, int comps) {
+    const dim3 nb(nblk(c->n, 256), comps / 4);
     if (c->fp64)
-        k_state_in<double><<<nb, 256, 0, c->stream>>>((const double*)U_user, c->perm.as<int32_t>(), c->n, comps, RS,
-                                                       off, (double*)rec);
+        k_state_in<double><<<nb, 256, 0, c->stream>>>((const double*)U_user, c->inv_perm.as<int32_t>(), c->n, comps,
+                                                      (double*)rec);
     else
-        k_state_in<float><<<nb, 256, 0, c->stream>>>((const float*)U_user, c->perm.as<int32_t>(), c->n, comps, RS, off,
-                                                      (float*)rec);
+        k_state_in<float><<<nb, 256, 0, c->stream>>>((const float*)U_user, c->inv_perm.as<int32_t>(), c->n, comps,
+                                                     (float*)rec);
     ++c->launches;
     RT_CUDA(c, cudaGetLastError());
     return RT_OK;
 }
 
-rt_status state_out(rt_ctx* c, const void* rec, void* U_user, int comps, int RS, int off) {
-    unsigned nb = nblk(c->n, 256);
+rt_status state_out(rt_ctx* c, const void* rec, void* U_user, int comps) {
+    const dim3 nb(nblk(c->n, 256), comps / 4);
     if (c->fp64)
-        k_state_out<double><<<nb, 256, 0, c->stream>>>((const double*)rec, c->inv_perm.as<int32_t>(), c->n, comps, RS,
-                                                        off, (double*)U_user);
+        k_state_out<double><<<nb, 256, 0, c->stream>>>((const double*)rec, c->inv_perm.as<int32_t>(), c->n, comps,
+                                                       (double*)U_user);
     else
-        k_state_out<float><<<nb, 256, 0, c->stream>>>((const float*)rec, c->inv_perm.as<int32_t>(), c->n, comps, RS,
-                                                       off, (float*)U_user);
+        k_state_out<float><<<nb, 256, 0, c->stream>>>((const float*)rec, c->inv_perm.as<int32_t>(), c->n, comps,
+                                                      (float*)U_user);
     ++c->launches;
     RT_CUDA(c, cudaGetLastError());
     return RT_OK;
@@ -1741,16 +1900,15 @@ rt_status set_dense_injection(rt_ctx* c, bool on) {
     return RT_OK;
 }
 
-rt_status launch_energy(rt_ctx* c, cudaStream_t s, const void* rec, double* out_dev) {
+rt_status launch_energy(rt_ctx* c, cudaStream_t s, const void* U, double* out_dev) {
     double* part = c->energy_part.as<double>();
-    int RS = 4 * c->cfg.n_groups;
-    const int32_t* perm = c->perm.as<int32_t>();
+    const int32_t* inv = c->inv_perm.as<int32_t>();
     if (c->fp64)
-        k_energy_part<double><<<kEnergyBlocks, 256, 0, s>>>((const double*)rec, RS, c->V_d.as<double>(), c->n,
-                                                            c->cfg.n_groups, perm, c->n_owned, part);
+        k_energy_part<double><<<kEnergyBlocks, 256, 0, s>>>((const double*)U, c->V_d.as<double>(), c->n,
+                                                            c->cfg.n_groups, inv, c->n_owned, part);
     else
-        k_energy_part<float><<<kEnergyBlocks, 256, 0, s>>>((const float*)rec, RS, c->V_d.as<double>(), c->n,
-                                                           c->cfg.n_groups, perm, c->n_owned, part);
+        k_energy_part<float><<<kEnergyBlocks, 256, 0, s>>>((const float*)U, c->V_d.as<double>(), c->n,
+                                                           c->cfg.n_groups, inv, c->n_owned, part);
     k_energy_final<<<c->cfg.n_groups, kEnergyBlocks, 0, s>>>(part, out_dev);
     c->launches += 2;
     RT_CUDA(c, cudaGetLastError());
