@@ -402,8 +402,8 @@ __global__ void __launch_bounds__(128) k_adj_grad(PairArgs<T> a, const T* __rest
         T dx, dy, dz;
         sep(a.sp, pi, pj, dx, dy, dz);              // d_ij = x_j - x_i
         const T r = sqrt_(dx * dx + dy * dy + dz * dz);
-        const T wi = spline_w_(r * iHi);
-        const T wj = spline_w_(r * a.geo[8 * j]);
+        const T wi = spline_w_(r, iHi);
+        const T wj = spline_w_(r, a.geo[8 * j]);
         T gj[12];
         vload<12>(gam + j * 12 * G + 12 * gg, gj);
 #pragma unroll

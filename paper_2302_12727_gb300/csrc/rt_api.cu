@@ -20,23 +20,28 @@ rt_status cuda_fail(rt_ctx* c, cudaError_t e, const char* what) {
     return e == cudaErrorMemoryAllocation ? RT_ERR_OOM : RT_ERR_CUDA;
 }
 
-static int64_t g_generation = 0;
-
-rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what) {
+rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what, bool slack) {
     if (bytes == 0) bytes = 16;
     if (b.bytes >= bytes) return RT_OK;
+    const size_t least = bytes;
+    if (slack) bytes += (bytes / 16 + 255) / 256 * 256;
     if (b.p) {
         cudaFree(b.p);
         b.p = nullptr;
         b.bytes = 0;
     }
     cudaError_t e = cudaMalloc(&b.p, bytes);
+    if (e != cudaSuccess && bytes > least) {     // no room for the slack
+        (void)cudaGetLastError();
+        bytes = least;
+        e = cudaMalloc(&b.p, bytes);
+    }
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         return fail(c, RT_ERR_OOM, std::string("device allocation failed: ") + what);
     }
     b.bytes = bytes;
-    ++g_generation;   // buffers captured in graphs moved
+    ++c->generation;   // buffers captured in graphs moved
     return RT_OK;
 }
 
@@ -119,7 +124,7 @@ static rt_status ensure_state(rt_ctx* c) {
     if (c->n_src > 0) RT_TRY(ensure(c, c->inj_dense, (size_t)G * n * 8, "injection"));
     // per-pair flux slots of one group chunk (at most 4 groups)
     const int gc = G < kMaxGC ? G : kMaxGC;
-    RT_TRY(ensure(c, c->pairbuf, (size_t)std::max<int64_t>(c->n_directed / 2, 1) * 4 * gc * tsize(c), "pair fluxes"));
+    RT_TRY(ensure(c, c->pairbuf, (size_t)std::max<int64_t>(c->n_directed / 2, 1) * 4 * gc * tsize(c), "pair fluxes", true));
     // double path: the kept pair geometry (80 bytes a pair and 24 an entry), where it takes no
     // more than a quarter of the memory that is free; without it the kernels compute it
     if (c->fp64) {
@@ -130,14 +135,14 @@ static rt_status ensure_state(rt_ctx* c) {
         const bool fits = P * 64 <= c->pair_geo.bytes && P * 16 <= c->pair_w.bytes && P * 48 <= c->row_wd.bytes;
         if (!fits) RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
         if (fits || need <= (free_b + have) / 4) {
-            RT_TRY(ensure(c, c->pair_geo, P * 64, "pair geometry"));
-            RT_TRY(ensure(c, c->pair_w, P * 16, "pair geometry"));
-            RT_TRY(ensure(c, c->row_wd, P * 48, "pair geometry"));
+            RT_TRY(ensure(c, c->pair_geo, P * 64, "pair geometry", true));
+            RT_TRY(ensure(c, c->pair_w, P * 16, "pair geometry", true));
+            RT_TRY(ensure(c, c->row_wd, P * 48, "pair geometry", true));
         } else {
             free_buf(c->pair_geo);
             free_buf(c->pair_w);
             free_buf(c->row_wd);
-            ++g_generation;
+            ++c->generation;
         }
     }
     if (!c->fp64) RT_TRY(ensure(c, c->frec, (size_t)(12 + 16 * gc + kRowRot) * n * 4, "packed flux rows"));
@@ -229,19 +234,21 @@ static rt_status neighbours(rt_ctx* c, const double* x, const double* m, const d
     RT_CUDA(c, cudaSetDevice(c->device));
     c->built = false;
     c->has_bins = false;   // bins live in the sorted order and depend on the pair lists
-    int64_t gen0 = g_generation;
-    int64_t targets0 = c->n_inj_targets;
+    const int64_t gen0 = c->generation;
     rt_status s = build_neighbours(c, x, m, xsrc, h_in, hs_in, oms_in, octw_in);
     if (s != RT_OK) {
         drop_graphs(c);
         return s;
     }
     RT_TRY(ensure_state(c));
-    // captured graphs hold buffer addresses, the injection grid size and the pair count (the
-    // pair pass's grid and slot bound), which a rebuild can change without moving a buffer
-    std::vector<int64_t> shape{c->n_directed, c->n_inj_targets, c->n_inj_entries};
-    if (g_generation != gen0 || c->n_inj_targets != targets0 || shape != c->graph_shape) drop_graphs(c);
-    c->graph_shape = shape;
+    const int64_t pairs = c->n_directed / 2;
+    if (c->generation != gen0 || pairs > c->pair_cap || c->n_inj_targets > c->target_cap) drop_graphs(c);
+    if (c->graphs.empty()) {
+        // the grids of the next captures cover a little more: moving particles change the number
+        // of pairs by fractions of a percent, and every empty block costs its launch
+        c->pair_cap = pairs + pairs / 64 + 1024;
+        c->target_cap = c->n_inj_targets + c->n_inj_targets / 4 + 128;
+    }
     if (h_out) {
         // h in caller order
         RT_TRY(field_out(c, c->h_d.as<double>(), h_out, 1));
@@ -421,10 +428,12 @@ rt_status rt_subcycle(rt_ctx* c, int32_t n_sub, double dt, void* U, const double
         int64_t l0 = c->launches;
         c->prof_sink = c->profiling ? &entry.prof : nullptr;
         c->prof_pairs = 0;
+        c->capturing = true;
         for (int k = 0; k < n_sub && s == RT_OK; ++k) {
             s = launch_step(c, c->cap_stream, a, b, has_src, has_alpha, k == 0, k + 1 < n_sub);
             std::swap(a, b);
         }
+        c->capturing = false;
         c->prof_sink = nullptr;
         entry.kernels = c->launches - l0;
         c->launches = l0;
@@ -752,7 +761,7 @@ void rt_destroy(rt_ctx* c) {
                       &c->sigma_d, &c->bins_s, &c->bins_tmp, &c->acc_t, &c->bins_nmin, &c->order_b, &c->order_m,
                       &c->order_q, &c->bin_keys, &c->bin_keys2, &c->bin_vals, &c->bin_cub, &c->bin_hist, &c->alpha_s,
                       &c->L_dev, &c->dt_dev, &c->energy_part, &c->ck, &c->seg, &c->lam_a, &c->lam_b, &c->adj_w,
-                      &c->adj_x, &c->adj_ub, &c->adj_gam, &c->adj_lam, &c->pair_geo, &c->pair_w, &c->row_wd, &c->adj_slots,
+                      &c->adj_x, &c->adj_ub, &c->adj_gam, &c->adj_lam, &c->inj_dense, &c->pair_geo, &c->pair_w, &c->row_wd, &c->adj_slots,
                       &c->adj_sel};
     for (DevBuf* b : bufs) free_buf(*b);
     if (c->cap_stream) cudaStreamDestroy(c->cap_stream);

@@ -1856,18 +1856,18 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     if (P2 >= ((int64_t)1 << 31)) return fail(c, RT_ERR_INVALID, "more than 2^31 neighbour entries");
     // the spread of the supports, H_max^3 over the mean H^3
     c->diag.pair_build = Hmax * Hmax * Hmax / std::max(hred.h3 / (double)n, 1e-300) > 12.0 ? 1 : 0;
-    RT_TRY(ensure(c, c->cols, std::max<int64_t>(P2, 1) * 4, "pair lists"));
+    RT_TRY(ensure(c, c->cols, std::max<int64_t>(P2, 1) * 4, "pair lists", true));
     RT_TRY(ensure(c, c->n_low, (n + 1) * 4, "pair split"));
     RT_TRY(ensure(c, c->n_up, (n + 1) * 4, "pair split"));
     if (hred.spill > 0) {     // own entries of the particles without a list
-        RT_TRY(ensure(c, c->spill, (size_t)hred.spill * 4, "pair rows"));
+        RT_TRY(ensure(c, c->spill, (size_t)hred.spill * 4, "pair rows", true));
         k_own_walk<true><<<(unsigned)c->sm_count * 4, 128, 0, st>>>(
             g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n, pp, c->lists.as<int32_t>(), cap,
             c->own_cnt.as<int32_t>(), nullptr, nullptr, over, over_n, nullptr, c->spill.as<int32_t>());
         c->launches += 1;
     }
     if (hred.more > 0) {      // rows with more extras than they hold in place
-        RT_TRY(ensure(c, c->more, (size_t)hred.more * 4, "pair rows"));
+        RT_TRY(ensure(c, c->more, (size_t)hred.more * 4, "pair rows", true));
         RT_TRY(ensure(c, c->more_off, (size_t)(n + 1) * 8, "pair rows"));
         int32_t* cnt = c->counts.as<int32_t>();
         k_more_extras<<<nblk(n + 1, 256), 256, 0, st>>>(c->extra_cnt.as<int32_t>(), n, cnt);
@@ -1891,12 +1891,12 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
 
     // the slots of the pairs
     RT_TRY(ensure(c, c->up_off, (n + 1) * 8, "pair split"));
-    RT_TRY(ensure(c, c->low_slot, std::max<int64_t>(P2 / 2, 1) * 4, "pair split"));
+    RT_TRY(ensure(c, c->low_slot, std::max<int64_t>(P2 / 2, 1) * 4, "pair split", true));
     RT_CUDA(c, cudaMemsetAsync(c->n_up.as<int32_t>() + n, 0, 4, st));
     tb = c->cub_tmp.bytes;
     RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->n_up.as<int32_t>(), c->up_off.as<int64_t>(),
                                              (int)(n + 1), st));
-    RT_TRY(ensure(c, c->pair_ends, std::max<int64_t>(P2 / 2, 1) * 8, "pair split"));
+    RT_TRY(ensure(c, c->pair_ends, std::max<int64_t>(P2 / 2, 1) * 8, "pair split", true));
     k_pair_slots<<<nblk(n * 32, 256), 256, 0, st>>>(c->row_off.as<int64_t>(), c->cols.as<int32_t>(),
                                                      c->n_low.as<int32_t>(), c->up_off.as<int64_t>(), n,
                                                      c->pair_ends.as<int2>(), c->low_slot.as<int32_t>());
@@ -1962,17 +1962,17 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         if (hflags[F_SRC_NOCONV]) return fail(c, RT_ERR_NOCONV, "source smoothing-length iteration did not converge");
         if (NE > Smax) return fail(c, RT_ERR_INVALID, "too many injection entries");
         c->n_inj_entries = NE;
-        int64_t NEa = std::max<int64_t>(NE, 1);
-        RT_TRY(ensure(c, c->src_entry_gas, NEa * 4, "injection"));
-        RT_TRY(ensure(c, c->src_entry_xi, NEa * 8, "injection"));
-        RT_TRY(ensure(c, c->inj_key, NEa * 8, "injection"));
-        RT_TRY(ensure(c, c->inj_key_out, NEa * 8, "injection"));
-        RT_TRY(ensure(c, c->inj_val, NEa * 4, "injection"));
-        RT_TRY(ensure(c, c->inj_val_out, NEa * 4, "injection"));
-        RT_TRY(ensure(c, c->inj_src, NEa * 4, "injection"));
-        RT_TRY(ensure(c, c->inj_coef, NEa * 8, "injection"));
-        RT_TRY(ensure(c, c->inj_targets, NEa * 4, "injection"));
-        RT_TRY(ensure(c, c->inj_off, (NEa + 1) * 4, "injection"));
+        const int64_t NEa = std::max<int64_t>(NE, 1);
+        RT_TRY(ensure(c, c->src_entry_gas, NEa * 4, "injection", true));
+        RT_TRY(ensure(c, c->src_entry_xi, NEa * 8, "injection", true));
+        RT_TRY(ensure(c, c->inj_key, NEa * 8, "injection", true));
+        RT_TRY(ensure(c, c->inj_key_out, NEa * 8, "injection", true));
+        RT_TRY(ensure(c, c->inj_val, NEa * 4, "injection", true));
+        RT_TRY(ensure(c, c->inj_val_out, NEa * 4, "injection", true));
+        RT_TRY(ensure(c, c->inj_src, NEa * 4, "injection", true));
+        RT_TRY(ensure(c, c->inj_coef, NEa * 8, "injection", true));
+        RT_TRY(ensure(c, c->inj_targets, NEa * 4, "injection", true));
+        RT_TRY(ensure(c, c->inj_off, (NEa + 1) * 4, "injection", true));
         double* octw = c->omegas_d.as<double>() + S;   // 8 per source after omega_s
         k_src_entries<true><<<sb, kSrcWarps * 32, 0, st>>>(g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S,
                                                 c->hs_d.as<double>(), c->omegas_d.as<double>(), nullptr,

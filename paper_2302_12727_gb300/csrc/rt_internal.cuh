@@ -106,9 +106,10 @@ struct rt_ctx {
     rt::DevBuf pair_geo, pair_w, row_wd;
     bool pair_geo_ready = false;
     rt::DevBuf adj_slots, adj_sel;                      // adjoint: per-pair values of one group chunk
-    // sizes that captured graphs bake in besides buffer addresses (pair count, injection
-    // targets and entries): a rebuild that changes them drops the graphs
-    std::vector<int64_t> graph_shape;
+    // captured graphs hold buffer addresses and launch grids: they are dropped when a buffer moves
+    // (generation) or a rebuild has more pairs or targets than their grids cover
+    int64_t generation = 0, pair_cap = 0, target_cap = 0;
+    bool capturing = false;                             // launch grids from the capacities
     rt::DevBuf flags;                                   // int32 error flags + counters
     rt::DevBuf red_tmp;                                 // small reduction scratch (double)
     int64_t n_directed = 0;
@@ -170,7 +171,8 @@ struct rt_ctx {
 namespace rt {
 rt_status fail(rt_ctx* c, rt_status s, const std::string& msg);
 rt_status cuda_fail(rt_ctx* c, cudaError_t e, const char* what);
-rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what);
+// with slack, a buffer that grows gets a sixteenth more than asked
+rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what, bool slack = false);
 void free_buf(DevBuf& b);
 // HLL wave speeds over (f, theta), [RT_WAVE_NF][RT_WAVE_NTH] each (rt_hll.cu)
 void build_wave_table(double* lmax, double* lmin);

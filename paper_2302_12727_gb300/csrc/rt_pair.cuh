@@ -27,17 +27,26 @@ __device__ __forceinline__ float sqrt_(float x) {
 // explicitly rounded fused multiply-add
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+// explicitly rounded product (never contracted into a sum)
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
 __device__ __forceinline__ double fmax_(double a, double b) { return fmax(a, b); }
 __device__ __forceinline__ float fmax_(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double fmin_(double a, double b) { return fmin(a, b); }
 __device__ __forceinline__ float fmin_(float a, float b) { return fminf(a, b); }
 
-// cubic-spline shape without branches: (1-q)_+^3 - 4 (1/2-q)_+^3 (Eq. cubic-spline-kernel)
+// cubic-spline shape at q = r / H without branches: (1-q)_+^3 - 4 (1/2-q)_+^3 (Eq. cubic-spline-kernel)
+// (the fused multiply-adds of these helpers are explicit: the kernel variants' results are
+// compared bit by bit, whatever the compiler would contract around them)
 template <class T>
-__device__ __forceinline__ T spline_w_(T q) {
-    T a = fmax_(T(1) - q, T(0));
-    T b = fmax_(T(0.5) - q, T(0));
-    return a * a * a - T(4) * (b * b * b);
+__device__ __forceinline__ T spline_w_(T r, T iH) {
+    T a = fmax_(fma_rn(-r, iH, T(1)), T(0));
+    T b = fmax_(fma_rn(-r, iH, T(0.5)), T(0));
+    return fma_rn(T(-4), mul_rn(mul_rn(b, b), b), mul_rn(mul_rn(a, a), a));
+}
+template <class T>
+__device__ __forceinline__ T norm2_(T x, T y, T z) {
+    return fma_rn(z, z, fma_rn(y, y, mul_rn(x, x)));
 }
 
 // minmod of Eq. rt-minmod (both positive -> min, both negative -> max, else 0) as the median
@@ -288,11 +297,13 @@ struct PairArgs {
     const int64_t* up_off;    // first pair slot of each row
     const int32_t* low_slot;  // slot of each lower entry's pair
     const int2* ends;         // (k, l) of each pair slot
+    // number of pairs, from the device: a captured graph outlives a rebuild that changes it
+    __device__ __forceinline__ int64_t pairs() const { return row_off[n] >> 1; }
     // double path: the pairs' geometry, computed once per build (prepare_pair_geometry), or null
     const PairGeo<T>* pg;     // [P]
     const T* wd;              // [2P][3] per row entry: w(r_ij / H_i) d_ij
     const T* wkl;             // [P][2] w(r / H_k), w(r / H_l)
-    int64_t n_pairs;
+    int64_t n_pairs;          // what the launch grids cover: at least pairs()
     int G;
     // packed flux-input rows [N][kRowRot + RW], RW = 12 + 16G logical words {pos (4), geo
     // (8), U (4G), grad U (12G)} after a prefix that repeats the last kRowRot of them; when
@@ -312,9 +323,9 @@ struct PairArgs {
 // symmetric 3x3 (xx, yy, zz, xy, xz, yz) times vector
 template <class T>
 __device__ __forceinline__ void sym_mv(const T M[6], T x, T y, T z, T& ox, T& oy, T& oz) {
-    ox = M[0] * x + M[3] * y + M[4] * z;
-    oy = M[3] * x + M[1] * y + M[5] * z;
-    oz = M[4] * x + M[5] * y + M[2] * z;
+    ox = fma_rn(M[4], z, fma_rn(M[3], y, M[0] * x));
+    oy = fma_rn(M[5], z, fma_rn(M[1], y, M[3] * x));
+    oz = fma_rn(M[2], z, fma_rn(M[5], y, M[4] * x));
 }
 
 // Angle in [0, pi] of the vector (x, y), y >= 0.  Double: atan2.  Float: the arctangent of
@@ -386,9 +397,9 @@ __device__ __forceinline__ void wave_speeds_(const T* __restrict__ tab, T E, T F
 template <class T>
 __device__ __forceinline__ void pair_geo(T dx, T dy, T dz, const T gk[8], const T gl[8], T c, PairGeo<T>& p, T& sk,
                                          T& sl) {
-    const T r = sqrt_(dx * dx + dy * dy + dz * dz);
-    sk = spline_w_(r * gk[0]);
-    sl = spline_w_(r * gl[0]);
+    const T r = sqrt_(norm2_(dx, dy, dz));
+    sk = spline_w_(r, gk[0]);
+    sl = spline_w_(r, gl[0]);
     const T hk = T(0.5) * sk, hl = T(0.5) * sl;
     T M[6];
 #pragma unroll
@@ -524,7 +535,7 @@ inline PairArgs<T> pair_args(rt_ctx* c) {
     a.pg = kept ? static_cast<const PairGeo<T>*>(c->pair_geo.p) : nullptr;
     a.wd = kept ? c->row_wd.as<T>() : nullptr;
     a.wkl = kept ? c->pair_w.as<T>() : nullptr;
-    a.n_pairs = c->n_directed / 2;
+    a.n_pairs = c->capturing ? c->pair_cap : c->n_directed / 2;
     a.G = c->cfg.n_groups;
     a.frec = nullptr;
     a.RW = 12 + 16 * a.G;

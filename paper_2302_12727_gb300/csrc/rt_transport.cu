@@ -42,6 +42,11 @@ static int grad_block(const rt_ctx* c) {
     return c->tune.gradient_variant == 2 ? kGradBlock : 256;
 }
 static int gather_block(const rt_ctx* c) { return c->tune.gather_block > 0 ? c->tune.gather_block : kGatherBlock; }
+// fewer (particle, group)s than eight warps per SM: the gradient and the gather then take the
+// kernels with more loads in flight per thread
+static bool few_threads(const rt_ctx* c, int gc) {
+    return c->tune.gradient_variant == 2 && c->n * gc < (int64_t)c->sm_count * 256;
+}
 static int pair_warps(const rt_ctx* c) { return c->tune.pair_warps > 0 ? c->tune.pair_warps : 1; }
 
 // ------------------------------------------------------------------------------------
@@ -101,18 +106,25 @@ __global__ void k_alpha_g_sorted(const double* __restrict__ ag, const int32_t* _
     for (int g = 0; g < G; ++g) out[p * G + g] = (T)ag[(int64_t)g * n + i];
 }
 
-__global__ void k_set_scalar(double* dst, double v) { *dst = v; }
+__global__ void k_set_scalar(double* dst, double dt, int64_t n_targets) {
+    dst[0] = dt;
+    reinterpret_cast<int64_t*>(dst)[1] = n_targets;
+}
 
 // ------------------------------------------------------------------------------------
 // a5: injection, one thread per target particle: E_g += dt * sum_e coef_e L[src_e][g]
 // (coef = xi / V_target), accumulated in double.
+// the number of targets stands behind dt (set_step_inputs): a captured graph outlives a rebuild
+// that changes it
+__device__ __forceinline__ int64_t n_targets_of(const double* dt_dev) { return reinterpret_cast<const int64_t*>(dt_dev)[1]; }
+
 template <class T>
 __global__ void k_inject(const int32_t* __restrict__ targets, const int32_t* __restrict__ off,
                          const int32_t* __restrict__ src, const double* __restrict__ coef,
-                         const double* __restrict__ L, int G, const double* __restrict__ dt_dev, int64_t n_targets,
-                         int RS, T* rec, const int8_t* __restrict__ bins, int s) {
+                         const double* __restrict__ L, int G, const double* __restrict__ dt_dev, int RS, T* rec,
+                         const int8_t* __restrict__ bins, int s) {
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (t >= n_targets) return;
+    if (t >= n_targets_of(dt_dev)) return;
     double dt = *dt_dev;
     int64_t p = targets[t];
     if (bins) {   // time bins: only particles starting a step, for their own step
@@ -209,8 +221,8 @@ __global__ void __launch_bounds__(128) k_gradient(PairArgs<T> a, const T* __rest
         T dx0, dy0, dz0, dx1, dy1, dz1;
         sep(a.sp, pi, p0, dx0, dy0, dz0);
         sep(a.sp, pi, p1, dx1, dy1, dz1);
-        T w0 = spline_w_(sqrt_(dx0 * dx0 + dy0 * dy0 + dz0 * dz0) * iH);
-        T w1 = two ? spline_w_(sqrt_(dx1 * dx1 + dy1 * dy1 + dz1 * dz1) * iH) : T(0);
+        T w0 = spline_w_(sqrt_(norm2_(dx0, dy0, dz0)), iH);
+        T w1 = two ? spline_w_(sqrt_(norm2_(dx1, dy1, dz1)), iH) : T(0);
         T wx0 = w0 * dx0, wy0 = w0 * dy0, wz0 = w0 * dz0;
         T wx1 = w1 * dx1, wy1 = w1 * dy1, wz1 = w1 * dz1;
 #pragma unroll
@@ -247,7 +259,7 @@ __global__ void __launch_bounds__(128) k_gradient(PairArgs<T> a, const T* __rest
 __global__ void __launch_bounds__(128) k_pair_geometry(PairArgs<double> a, double c, PairGeo<double>* pg,
                                                        double* wkl) {
     const int64_t slot = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (slot >= a.n_pairs) return;
+    if (slot >= a.pairs()) return;
     const int2 kl = a.ends[slot];
     PairGeo<double> p;
     double sk, sl;
@@ -267,7 +279,7 @@ __global__ void __launch_bounds__(256) k_row_weights(PairArgs<double> a, double*
         const Pos<double> pj = load_pos(tag, a.pos, a.cols[e]);
         double dx, dy, dz;
         sep(a.sp, pi, pj, dx, dy, dz);
-        const double w = spline_w_(sqrt_(dx * dx + dy * dy + dz * dz) * iH);
+        const double w = spline_w_(sqrt_(norm2_(dx, dy, dz)), iH);
         wd[3 * e] = w * dx;
         wd[3 * e + 1] = w * dy;
         wd[3 * e + 2] = w * dz;
@@ -392,9 +404,9 @@ __global__ void __launch_bounds__(256) k_gradient_g(PairArgs<float> a, const flo
         float dx0, dy0, dz0, dx1, dy1, dz1;
         sep(a.sp, pi, p0, dx0, dy0, dz0);
         sep(a.sp, pi, p1, dx1, dy1, dz1);
-        float w0 = spline_w_(sqrt_(dx0 * dx0 + dy0 * dy0 + dz0 * dz0) * iH);
-        float w1 = two ? spline_w_(sqrt_(dx1 * dx1 + dy1 * dy1 + dz1 * dz1) * iH) : 0.f;
-        float wx0 = w0 * dx0, wy0 = w0 * dy0, wz0 = w0 * dz0;
+        float w0 = spline_w_(sqrt_(norm2_(dx0, dy0, dz0)), iH);
+        float w1 = two ? spline_w_(sqrt_(norm2_(dx1, dy1, dz1)), iH) : 0.f;
+        float wx0 = mul_rn(w0, dx0), wy0 = mul_rn(w0, dy0), wz0 = mul_rn(w0, dz0);
         float wx1 = w1 * dx1, wy1 = w1 * dy1, wz1 = w1 * dz1;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
@@ -417,6 +429,76 @@ __global__ void __launch_bounds__(256) k_gradient_g(PairArgs<float> a, const flo
         row_store<12>(a, row, 12 + 4 * GC + 12 * g, out);
         row_store<4>(a, row, 12 + 4 * g, ui);
         if (g == 0) packed_static(a, i, row);
+    } else {
+        vstore<12>(grad + i * 12 * a.G + 12 * (g0 + g), out);
+    }
+}
+
+// k_gradient_g for sets too small to fill the GPU, where the gradient is the latency of one
+// thread's chain of loads: eight neighbours' indices, then their positions and states in
+// flight together instead of two.  Same order and sums.  4,096 particles, one group: 24.1 us a
+// launch with two in flight.
+constexpr int kWide = 8;
+template <int GC>
+__global__ void __launch_bounds__(64) k_gradient_w(PairArgs<float> a, const float* __restrict__ rec,
+                                                   float* __restrict__ grad, int g0) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t i = t / GC;
+    if (i >= a.n) return;
+    const int g = (int)(t - i * GC);
+    const float* tag = nullptr;
+    const Pos<float> pi = load_pos(tag, a.pos, i);
+    const int RS = 4 * a.G;
+    const int off = 4 * (g0 + g);
+    const int64_t e0 = a.row_off[i];
+    const int m = (int)(a.row_off[i + 1] - e0);
+    const int32_t* row = a.cols + e0;
+    float ui[4], geo[8];
+    vload<4>(rec + i * RS + off, ui);
+    vload<8>(a.geo + 8 * i, geo);
+    const float om = a.omega[i], iH = geo[0];
+    float acc[4][3];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c][0] = acc[c][1] = acc[c][2] = 0.f;
+    int j[kWide];
+#pragma unroll
+    for (int k = 0; k < kWide; ++k) j[k] = m > 0 ? row[min(k, m - 1)] : (int)i;   // past the end: weight zero
+    for (int b = 0; b < m; b += kWide) {
+        Pos<float> p[kWide];
+        float u[kWide][4];
+#pragma unroll
+        for (int k = 0; k < kWide; ++k) {
+            p[k] = load_pos(tag, a.pos, j[k]);
+            vload<4>(rec + (int64_t)j[k] * RS + off, u[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < kWide; ++k) j[k] = row[min(b + kWide + k, m - 1)];
+#pragma unroll
+        for (int k = 0; k < kWide; ++k) {
+            float dx, dy, dz;
+            sep(a.sp, pi, p[k], dx, dy, dz);
+            const float w = b + k < m ? spline_w_(sqrt_(norm2_(dx, dy, dz)), iH) : 0.f;
+            const float wx = w * dx, wy = w * dy, wz = w * dz;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float dq = u[k][c] - ui[c];
+                acc[c][0] = fma_rn(dq, wx, acc[c][0]);
+                acc[c][1] = fma_rn(dq, wy, acc[c][1]);
+                acc[c][2] = fma_rn(dq, wz, acc[c][2]);
+            }
+        }
+    }
+    float M[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) M[k] = om * geo[2 + k];
+    float out[12];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) sym_mv(M, acc[c][0], acc[c][1], acc[c][2], out[3 * c], out[3 * c + 1], out[3 * c + 2]);
+    if (a.frec) {
+        float* to = packed_row(a, i);
+        row_store<12>(a, to, 12 + 4 * GC + 12 * g, out);
+        row_store<4>(a, to, 12 + 4 * g, ui);
+        if (g == 0) packed_static(a, i, to);
     } else {
         vstore<12>(grad + i * 12 * a.G + 12 * (g0 + g), out);
     }
@@ -482,9 +564,9 @@ __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax 
         float dx0, dy0, dz0, dx1, dy1, dz1;
         sep(a.sp, pi, p0, dx0, dy0, dz0);
         sep(a.sp, pi, p1, dx1, dy1, dz1);
-        float w0 = spline_w_(sqrt_(dx0 * dx0 + dy0 * dy0 + dz0 * dz0) * iH);
-        float w1 = two ? spline_w_(sqrt_(dx1 * dx1 + dy1 * dy1 + dz1 * dz1) * iH) : 0.f;
-        float wx0 = w0 * dx0, wy0 = w0 * dy0, wz0 = w0 * dz0;
+        float w0 = spline_w_(sqrt_(norm2_(dx0, dy0, dz0)), iH);
+        float w1 = two ? spline_w_(sqrt_(norm2_(dx1, dy1, dz1)), iH) : 0.f;
+        float wx0 = mul_rn(w0, dx0), wy0 = mul_rn(w0, dy0), wz0 = mul_rn(w0, dz0);
         float wx1 = w1 * dx1, wy1 = w1 * dy1, wz1 = w1 * dz1;
         const int hj0 = has ? j0 : -1;
 #pragma unroll
@@ -545,7 +627,7 @@ __global__ void __launch_bounds__(128) k_flux(PairArgs<T> a, FluxExtra<T> x, con
         if (slot >= a.count) return;
         slot = a.order[slot];
     } else {
-        if (slot >= a.n_pairs) return;
+        if (slot >= a.pairs()) return;
     }
     constexpr int NC = 4 * GC;
     const int G = a.G, RS = 4 * G;
@@ -855,7 +937,7 @@ __global__ void __launch_bounds__(128) k_flux_staged(PairArgs<float> a, FluxExtr
     const int lane = threadIdx.x & 31;
     float* ws = st + (threadIdx.x >> 5) * 32 * RW;
     const int64_t slot = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool act = slot < a.n_pairs;
+    const bool act = slot < a.pairs();
     // lanes past the last slot stage particle 0 (always present) and store nothing
     const int2 kl = act ? a.ends[slot] : make_int2(0, 0);
     const int G = a.G, RS = 4 * G;
@@ -956,7 +1038,9 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
     float* sm = sm_dyn + (((sm0 + 127u) & ~127u) - sm0) / 4u;
     float* ws = sm + wid * R::WF;
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const bool act = t < (BINS ? a.count : a.n_pairs);
+    const int64_t np = BINS ? a.count : a.pairs();
+    const bool act = t < np;
+    if (t - lane >= np) return;       // a captured grid covers more slots than a build may have
     const int64_t slot = BINS ? (act ? (int64_t)a.order[t] : 0) : t;
     // lanes past the last slot gather particle 0 (always present) and store nothing
     const int2 kl = act ? a.ends[slot] : make_int2(0, 0);
@@ -1057,7 +1141,7 @@ k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
     const uint32_t mb = smem_u32(&bar[wid]);
     if (lane == 0) mbar_init(mb, 1);
     __syncthreads();
-    const int64_t np = a.n_pairs, stride = gridDim.x * (int64_t)blockDim.x;
+    const int64_t np = a.pairs(), stride = gridDim.x * (int64_t)blockDim.x;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     // lanes past the last slot gather particle 0 (always present) and store nothing
     int2 kl = t < np ? a.ends[t] : make_int2(0, 0);
@@ -1126,11 +1210,15 @@ k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
 // Float pass 2 with one thread per (particle, group): the lanes of one particle read the
 // 16-byte pieces of a slot that lie side by side, so a warp request touches about 32 / GC
 // slots instead of 32.  Same order of additions and subtractions as k_flux_gather.
-template <int GC>
-__global__ void __launch_bounds__(kGatherBlockMax) k_flux_gather_g(PairArgs<float> a, FluxExtra<float> x,
+// B loads in flight a thread: eight, or (WIDE) 24, a whole half row, with the lower slots' indices
+// loaded beside the upper slots: for sets too small to fill the GPU, where the launch is the
+// latency of one thread's chain of loads (4,096 particles, one group: 14.4 us with eight).
+template <int GC, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(PairArgs<float> a, FluxExtra<float> x,
                                                        const float* __restrict__ rec,
                                                        const float* __restrict__ pairbuf, float* __restrict__ out,
                                                        int g0) {
+    constexpr int B = WIDE ? 24 : 8;
     // blocks run from the last particles to the first: the pair pass wrote the slots in
     // ascending order, so the most recent (still L2-resident) slots are read first
     const int64_t t = (gridDim.x - 1 - blockIdx.x) * (int64_t)blockDim.x + threadIdx.x;
@@ -1143,31 +1231,38 @@ __global__ void __launch_bounds__(kGatherBlockMax) k_flux_gather_g(PairArgs<floa
     FluxAcc<float> acc;
     acc.zero();
     const int64_t r0 = a.row_off[i], s0 = a.up_off[i], s1 = a.up_off[i + 1];
-    // batches of up to eight loads in flight (the last one predicated), added in order
-    for (int64_t sl = s0; sl < s1; sl += 8) {
-        const int m = s1 - sl < 8 ? (int)(s1 - sl) : 8;
-        float p[8][4];
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (u < m) vload<4>(pb + (sl + u) * NC, p[u]);
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (u < m) acc.add(p[u]);
-    }
     const int nl = a.n_low[i];
     const int32_t* ls = a.low_slot + (r0 - s0);
-    for (int e = 0; e < nl; e += 8) {   // up to eight slot indices, then their loads in flight
-        const int m = nl - e < 8 ? nl - e : 8;
-        int32_t q[8];
+    int32_t q[B];
+    if constexpr (WIDE) {
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-            if (u < m) q[u] = ls[e + u];
-        float p[8][4];
+        for (int u = 0; u < B; ++u)
+            if (u < nl) q[u] = ls[u];
+    }
+    // batches of up to B loads in flight (the last one predicated), added in order
+    for (int64_t sl = s0; sl < s1; sl += B) {
+        const int m = s1 - sl < B ? (int)(s1 - sl) : B;
+        float p[B][4];
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < B; ++u)
+            if (u < m) vload<4>(pb + (sl + u) * NC, p[u]);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (u < m) acc.add(p[u]);
+    }
+    for (int e = 0; e < nl; e += B) {   // up to B slot indices, then their loads in flight
+        const int m = nl - e < B ? nl - e : B;
+        if (!WIDE || e > 0) {
+#pragma unroll
+            for (int u = 0; u < B; ++u)
+                if (u < m) q[u] = ls[e + u];
+        }
+        float p[B][4];
+#pragma unroll
+        for (int u = 0; u < B; ++u)
             if (u < m) vload<4>(pb + (int64_t)q[u] * NC, p[u]);
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
+        for (int u = 0; u < B; ++u)
             if (u < m) acc.sub(p[u]);
     }
     const float dt = (float)(*x.dt_dev);
@@ -1292,6 +1387,19 @@ static void launch_gradient_t(rt_ctx* c, cudaStream_t s, T* rec, bool packed = f
         }
         int pr = prof_begin(c, s, RT_KERNEL_GRADIENT);
         if constexpr (std::is_same<T, float>::value) {
+            if (few_threads(c, gc)) {
+                float* gr = c->grad_t.as<float>();
+                const unsigned nbw = nblk(c->n * gc, 64);
+                switch (gc) {
+                    case 1: k_gradient_w<1><<<nbw, 64, 0, s>>>(a, rec, gr, g0); break;
+                    case 2: k_gradient_w<2><<<nbw, 64, 0, s>>>(a, rec, gr, g0); break;
+                    case 3: k_gradient_w<3><<<nbw, 64, 0, s>>>(a, rec, gr, g0); break;
+                    default: k_gradient_w<4><<<nbw, 64, 0, s>>>(a, rec, gr, g0); break;
+                }
+                prof_end(c, s, pr);
+                ++c->launches;
+                continue;
+            }
             if (c->tune.gradient_variant == 2 && gc > 1) {
                 // warps of 32 / gc particles: ceil(n / (32 / gc)) warps of 32 lanes
                 const int64_t warps = (c->n + 32 / gc - 1) / (32 / gc);
@@ -1435,7 +1543,9 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
     }
     prof_end(c, s, pr);
     pr = prof_begin(c, s, RT_KERNEL_FLUX_GATHER);
-    if (c->tune.gather_variant == 1)
+    if (c->tune.gather_variant == 1 && few_threads(c, GC))
+        k_flux_gather_g<GC, true><<<nblk(c->n * GC, 64), 64, 0, s>>>(a, x, rec, pb, out, g0);
+    else if (c->tune.gather_variant == 1)
         k_flux_gather_g<GC><<<nblk(c->n * GC, gather_block(c)), gather_block(c), 0, s>>>(a, x, rec, pb, out, g0);
     else
         k_flux_gather<float, GC><<<nblk(c->n, 128), 128, 0, s>>>(a, x, rec, pb, out, g0);
@@ -1520,10 +1630,9 @@ template <class T>
 static void launch_inject_t(rt_ctx* c, cudaStream_t s, T* rec, const int8_t* bins = nullptr, int step = 0) {
     if (c->n_inj_targets <= 0) return;
     int pr = prof_begin(c, s, RT_KERNEL_INJECT);
-    k_inject<T><<<nblk(c->n_inj_targets, 128), 128, 0, s>>>(
+    k_inject<T><<<nblk(c->capturing ? c->target_cap : c->n_inj_targets, 128), 128, 0, s>>>(
         c->inj_targets.as<int32_t>(), c->inj_off.as<int32_t>(), c->inj_src.as<int32_t>(), c->inj_coef.as<double>(),
-        c->L_dev.as<double>(), c->cfg.n_groups, c->dt_dev.as<double>(), c->n_inj_targets, 4 * c->cfg.n_groups, rec,
-        bins, step);
+        c->L_dev.as<double>(), c->cfg.n_groups, c->dt_dev.as<double>(), 4 * c->cfg.n_groups, rec, bins, step);
     prof_end(c, s, pr);
     ++c->launches;
 }
@@ -1834,7 +1943,7 @@ rt_status field_out(rt_ctx* c, const double* src_sorted, double* dst_user, int c
 
 rt_status set_step_inputs(rt_ctx* c, double dt, const double* Lsrc, const double* alpha) {
     cudaStream_t s = c->stream;
-    k_set_scalar<<<1, 1, 0, s>>>(c->dt_dev.as<double>(), dt);
+    k_set_scalar<<<1, 1, 0, s>>>(c->dt_dev.as<double>(), dt, c->n_inj_targets);
     ++c->launches;
     if (Lsrc && c->n_src > 0)
         RT_CUDA(c, cudaMemcpyAsync(c->L_dev.p, Lsrc, (size_t)c->n_src * c->cfg.n_groups * sizeof(double),
