@@ -755,7 +755,7 @@ void rt_destroy(rt_ctx* c) {
                       &c->geo_t, &c->omega_t, &c->counts, &c->row_off, &c->cols, &c->lists, &c->list_cnt, &c->own_cnt,
                       &c->extra_cnt, &c->extras, &c->more, &c->more_off, &c->spill, &c->n_low,
                       &c->n_up, &c->up_off, &c->low_slot, &c->pair_ends, &c->pairbuf, &c->flags, &c->red_tmp,
-                      &c->xsrc_d, &c->hs_d, &c->omegas_d, &c->src_counts, &c->src_off, &c->inj_key,
+                      &c->src_list, &c->src_list_cnt, &c->xsrc_d, &c->hs_d, &c->omegas_d, &c->src_counts, &c->src_off, &c->inj_key,
                       &c->inj_key_out, &c->inj_val, &c->inj_val_out, &c->inj_targets, &c->inj_off, &c->inj_src,
                       &c->inj_coef, &c->src_entry_gas, &c->src_entry_xi, &c->U_a, &c->U_b, &c->grad_t, &c->frec, &c->wave_t, &c->alpha_g_c, &c->alpha_g_s,
                       &c->sigma_d, &c->bins_s, &c->bins_tmp, &c->acc_t, &c->bins_nmin, &c->order_b, &c->order_m,

@@ -1145,51 +1145,72 @@ __device__ __forceinline__ void store_pos<double>(void* pos, int64_t p, const do
 // Float path: separations from the fixed-point positions, weights in float and a
 // compensated (Kahan) float sum, so that E_i keeps ~1e-8 relative accuracy before its
 // inversion in double.
+//
+// E_i, eight lanes a row (the columns are then read side by side and a row of 46 takes six rounds
+// of loads): sums of the float path compensated and merged, those of the double path in double
+constexpr int kELanes = 8;
+struct Sum {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void fold(int o) { v += __shfl_xor_sync(0xffffffffu, v, o); }
+    __device__ __forceinline__ double value() const { return v; }
+};
+struct KahanSum : Kahan {
+    __device__ __forceinline__ void fold(int o) {
+        merge(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
+    }
+};
 template <class T>
-__device__ __forceinline__ void accumulate_E(const double* xs, const uint4* xq, const double* box, int periodic,
-                                             float s0, float s1, float s2, int64_t n, int64_t p, double H,
-                                             const int64_t* row_off, const int32_t* cols, double E[6]);
-
-template <>
-__device__ __forceinline__ void accumulate_E<double>(const double* xs, const uint4*, const double* box,
-                                                     int periodic, float, float, float, int64_t n, int64_t p,
-                                                     double H, const int64_t* row_off, const int32_t* cols,
-                                                     double E[6]) {
-    const double half[3] = {0.5 * box[0], 0.5 * box[1], 0.5 * box[2]};
-    double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    double iH = 1.0 / H, H2 = H * H;
-    for (int k = 0; k < 6; ++k) E[k] = 0.0;
-    for (int64_t e = row_off[p]; e < row_off[p + 1]; ++e) {
-        int j = cols[e];
-        double dx = sep_fast(xs[j], px, box[0], half[0], periodic);
-        double dy = sep_fast(xs[n + j], py, box[1], half[1], periodic);
-        double dz = sep_fast(xs[2 * n + j], pz, box[2], half[2], periodic);
-        double r2 = dx * dx + dy * dy + dz * dz;
-        if (!(r2 < H2)) continue;
-        double w = spline_w(sqrt(r2) * iH);
-        E[0] += w * dx * dx; E[1] += w * dy * dy; E[2] += w * dz * dz;
-        E[3] += w * dx * dy; E[4] += w * dx * dz; E[5] += w * dy * dz;
+__global__ void __launch_bounds__(256)
+k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
+    const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols, int64_t n, double b0, double b1, double b2,
+    int periodic, float s0, float s1, float s2, double* __restrict__ E_out) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t p = t / kELanes;
+    const int lane = (int)(t % kELanes);
+    const bool act = p < n;
+    const int64_t pp = act ? p : 0, e1 = act ? row_off[pp + 1] : 0;
+    const double H = kKappa * h[pp];
+    typename std::conditional<std::is_same<T, float>::value, KahanSum, Sum>::type acc[6];
+    if constexpr (std::is_same<T, float>::value) {
+        const uint4 q = xq[pp];
+        const float iH = (float)(1.0 / H), H2 = (float)(H * H);
+#pragma unroll 2
+        for (int64_t e = row_off[pp] + lane; e < e1; e += kELanes) {
+            const uint4 qj = xq[cols[e]];
+            const float dx = fsep(qj.x, q.x, s0), dy = fsep(qj.y, q.y, s1), dz = fsep(qj.z, q.z, s2);
+            const float r2 = dx * dx + dy * dy + dz * dz;
+            if (!(r2 < H2)) continue;
+            const float w = spline_w(sqrtf(r2) * iH);
+            acc[0].add(w * dx * dx); acc[1].add(w * dy * dy); acc[2].add(w * dz * dz);
+            acc[3].add(w * dx * dy); acc[4].add(w * dx * dz); acc[5].add(w * dy * dz);
+        }
+    } else {
+        const double x = xs[pp], y = xs[n + pp], z = xs[2 * n + pp];
+        const double iH = 1.0 / H, H2 = H * H;
+        for (int64_t e = row_off[pp] + lane; e < e1; e += kELanes) {
+            const int j = cols[e];
+            const double dx = sep_fast(xs[j], x, b0, 0.5 * b0, periodic);
+            const double dy = sep_fast(xs[n + j], y, b1, 0.5 * b1, periodic);
+            const double dz = sep_fast(xs[2 * n + j], z, b2, 0.5 * b2, periodic);
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            if (!(r2 < H2)) continue;
+            const double w = r2 > 0.0 ? spline_w(sqrt_fast(r2) * iH) : 0.0;
+            const double wx = w * dx, wy = w * dy, wz = w * dz;
+            acc[0].add(wx * dx); acc[1].add(wy * dy); acc[2].add(wz * dz);
+            acc[3].add(wx * dy); acc[4].add(wx * dz); acc[5].add(wy * dz);
+        }
     }
-}
-
-template <>
-__device__ __forceinline__ void accumulate_E<float>(const double*, const uint4* xq, const double*, int, float s0,
-                                                    float s1, float s2, int64_t n, int64_t p, double H,
-                                                    const int64_t* row_off, const int32_t* cols, double E[6]) {
-    const uint4 q4p = xq[p];
-    uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    float iH = (float)(1.0 / H), H2 = (float)(H * H);
-    Kahan acc[6];
-    for (int64_t e = row_off[p]; e < row_off[p + 1]; ++e) {
-        int j = cols[e];
-        float dx = fsep(xq[j].x, qx, s0), dy = fsep(xq[j].y, qy, s1), dz = fsep(xq[j].z, qz, s2);
-        float r2 = dx * dx + dy * dy + dz * dz;
-        if (!(r2 < H2)) continue;
-        float w = spline_w(sqrtf(r2) * iH);
-        acc[0].add(w * dx * dx); acc[1].add(w * dy * dy); acc[2].add(w * dz * dz);
-        acc[3].add(w * dx * dy); acc[4].add(w * dx * dz); acc[5].add(w * dy * dz);
+#pragma unroll
+    for (int o = kELanes / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 6; ++k) acc[k].fold(o);
+    if (act && lane < 6) {
+        double v = 0.0;
+#pragma unroll
+        for (int k = 0; k < 6; ++k) v = k == lane ? acc[k].value() : v;
+        E_out[lane * n + p] = v;
     }
-    for (int k = 0; k < 6; ++k) E[k] = acc[k].value();
 }
 
 // Also writes the pair kernels' records: position, {1/H, h, Bp (6)} with
@@ -1198,19 +1219,16 @@ __device__ __forceinline__ void accumulate_E<float>(const double*, const uint4* 
 template <class T>
 __global__ void k_geometry(const double* __restrict__ xs, const uint4* __restrict__ xq,
                            const double* __restrict__ h, const double* __restrict__ omega,
-                           const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols, int64_t n, double b0,
-                           double b1, double b2, int periodic, float s0, float s1, float s2, double* V_out,
-                           double* B_out, float* cond_out, void* pos_t, T* geo_t, T* om_t,
+                           int64_t n, double* V_out, double* B_out, float* cond_out, void* pos_t, T* geo_t, T* om_t,
                            unsigned long long* red, unsigned* cond_max, int* flags) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     float cond = 0.f;
     double V = INFINITY;
     if (p < n) {
-        const double box[3] = {b0, b1, b2};
         double hi = h[p], H = kKappa * hi, iH = 1.0 / H;
         double om = omega[p];
         double E[6];
-        accumulate_E<T>(xs, xq, box, periodic, s0, s1, s2, n, p, H, row_off, cols, E);
+        for (int k = 0; k < 6; ++k) E[k] = B_out[k * n + p];     // E_i (k_E), replaced by B_i
         V = 1.0 / om;                              // V, 1/H and bp as in k_set_fields
         const double fac = kSigma * iH * iH * iH * V;   // psi = fac * w
         double e_xx = E[0] * fac, e_yy = E[1] * fac, e_zz = E[2] * fac;
@@ -1293,6 +1311,204 @@ struct SrcParams {
     int fixed;      // hs_out holds given smoothing lengths: only omega_s at them
 };
 
+// One step of the source solve from the sums at h: S(h) = sum w, D = sum q w'(q).  Newton on
+// S(h) = S* (see k_h_lists) close to the root, where a step of less than 1e-8 h ends it: the
+// next one would be below rounding, and at the root omega is (eta/h)^3.  Farther off on h - eta
+// omega^(-1/3), nearly linear in h.  Returns 1 when done, 0 for another evaluation at the new h,
+// -1 when h cannot move.
+__device__ __forceinline__ int src_newton(const SrcParams& sp, double S, double D, double& h, double& lo, double& hi,
+                                          double& om) {
+    const double f = S - sp.s_star;
+    if (f < 0.0) lo = h; else hi = h;
+    double step = -INFINITY;
+    if (S > 0.0 && D < 0.0) {
+        if (fabs(f) < 1e-3 * sp.s_star) {
+            step = -f * h / D;
+        } else {
+            const double x = cbrt(sp.s_star / S), fp = 1.0 - x - x * D / (3.0 * S);
+            step = fp > 0.0 ? h * (1.0 - x) / fp : -INFINITY;
+        }
+    }
+    if (fabs(step) <= 1e-8 * h) {
+        h -= step;
+        om = sp.eta3 / (h * h * h);
+        return 1;
+    }
+    double hn = h - step;
+    if (!(hn > lo && hn < hi)) hn = isinf(hi) ? 1.5 * h : 0.5 * (lo + hi);
+    if (hn > sp.h_cap) hn = sp.h_cap;
+    if (hn == h) return om > 0.0 ? 1 : -1;
+    h = hn;
+    return 0;
+}
+
+// Sources with a list of candidates (kSrcList of them within 1.1 supports, about 64 of an even
+// set): one warp each walks once (warp_walk) and iterates over the stored distances; the count
+// and the entries then come from the list.  A source whose candidates overflow it keeps
+// src_list_cnt = -1 and goes to k_src_h and k_src_entries, which walk.  One source in 4,096
+// particles: 46 + 18 + 43 us with a block of walks per iteration and two more for the entries.
+constexpr int kSrcList = 384, kSrcListWarps = 4;
+
+struct QuantParams {
+    double mul[3];      // fixed-point units per length, as in k_gather_positions
+    float scale[3];
+};
+
+__global__ void __launch_bounds__(kSrcListWarps * 32)
+k_src_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, QuantParams qp,
+            const double* __restrict__ xsrc, int64_t S, SrcParams sp, double* hs_out, double* oms_out, int* flags,
+            int32_t* __restrict__ list, int32_t* __restrict__ list_cnt) {
+    __shared__ double dist[kSrcListWarps][kSrcList];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t s_id = blockIdx.x * (int64_t)kSrcListWarps + wid;
+    if (s_id >= S) return;      // whole warps
+    const unsigned FULL = 0xffffffffu;
+    const double p[3] = {xsrc[s_id], xsrc[S + s_id], xsrc[2 * S + s_id]};
+    uint32_t q[3];
+    for (int a = 0; a < 3; ++a) q[a] = (uint32_t)fmin(fmax(floor(p[a] * qp.mul[a]), 0.0), 4294967295.0);
+    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
+    double h = (sp.warm || sp.fixed) ? hs_out[s_id] : sp.h0, lo = 0.0, hi = INFINITY, om = 0.0, Rs = 0.0;
+    if (!(h > 0.0) || !(h < sp.h_cap)) {
+        if (sp.fixed && lane == 0) atomicExch(&flags[F_BADH], 1);
+        h = sp.h0;
+    }
+    int c = 0, state = 0;
+    for (int it = 0; it < sp.max_iter && state == 0; ++it) {
+        const double H = kKappa * h, iH = 1.0 / H;
+        if (H > Rs) {
+            Rs = H * (sp.fixed ? 1.0 : 1.1);
+            const double R2 = Rs * Rs;
+            const float R2f = (float)R2 * 1.001f;
+            c = 0;
+            warp_walk(g, (float)p[0], (float)p[1], (float)p[2], (float)Rs * 1.0001f, lane, [&](int j, bool valid) {
+                double r2 = INFINITY;
+                if (valid) {
+                    const uint4 qj = xq[j];
+                    const float ax = fsep(qj.x, q[0], qp.scale[0]), ay = fsep(qj.y, q[1], qp.scale[1]),
+                                az = fsep(qj.z, q[2], qp.scale[2]);
+                    if (ax * ax + ay * ay + az * az < R2f) {
+                        const double dx = sep_fast(xs[j], p[0], g.box[0], half[0], g.periodic);
+                        const double dy = sep_fast(xs[n + j], p[1], g.box[1], half[1], g.periodic);
+                        const double dz = sep_fast(xs[2 * n + j], p[2], g.box[2], half[2], g.periodic);
+                        r2 = dx * dx + dy * dy + dz * dz;
+                    }
+                }
+                const bool in = r2 < R2;
+                const unsigned m = __ballot_sync(FULL, in);
+                const int pos = c + __popc(m & ((1u << lane) - 1u));
+                if (in && pos < kSrcList) {
+                    list[s_id * kSrcList + pos] = j;
+                    dist[wid][pos] = sqrt(r2);
+                }
+                c += __popc(m);
+                return c <= kSrcList;
+            });
+            if (c > kSrcList) {
+                if (lane == 0) list_cnt[s_id] = -1;
+                return;      // hs_out keeps the first guess for k_src_h
+            }
+            __syncwarp();
+        }
+        double sw = 0.0, sdw = 0.0;
+        for (int k = lane; k < c; k += 32) {
+            const double u = dist[wid][k] * iH;
+            sw += spline_w(u);
+            sdw += u * spline_dw(u);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            sw += __shfl_xor_sync(FULL, sw, o);
+            sdw += __shfl_xor_sync(FULL, sdw, o);
+        }
+        om = kSigma * iH * iH * iH * sw;
+        if (sp.fixed) {   // given h: omega there, no iteration
+            state = om > 0.0 ? 1 : -1;
+            break;
+        }
+        state = src_newton(sp, sw, sdw, h, lo, hi, om);
+    }
+    if (lane == 0) {
+        if (state != 1) atomicExch(&flags[F_SRC_NOCONV], 1);
+        hs_out[s_id] = h;
+        oms_out[s_id] = om;
+        // the last step moves h by less than 1e-8: the list, a tenth longer or exact, covers it
+        // unless it ends right at the support
+        list_cnt[s_id] = kKappa * h <= Rs ? c : -1;
+    }
+}
+
+// Count (FILL = false) or write (FILL = true) the gas entries of the sources with a list, one warp
+// each; the counterpart of k_src_entries
+template <bool FILL>
+__global__ void __launch_bounds__(kSrcListWarps * 32)
+k_src_list_entries(Grid g, const double* __restrict__ xs, int64_t n, const double* __restrict__ xsrc, int64_t S,
+                   const double* __restrict__ hs, const double* __restrict__ oms, const int32_t* __restrict__ list,
+                   const int32_t* __restrict__ list_cnt, int32_t* counts, const int64_t* __restrict__ off,
+                   int32_t* e_gas, double* e_xi, double* octw_out, const double* __restrict__ octw_given) {
+    __shared__ unsigned char oct_of[kSrcListWarps][kSrcList];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t src = blockIdx.x * (int64_t)kSrcListWarps + wid;
+    if (src >= S || list_cnt[src] < 0) return;
+    const unsigned FULL = 0xffffffffu;
+    const double p[3] = {xsrc[src], xsrc[S + src], xsrc[2 * S + src]};
+    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
+    const double H = kKappa * hs[src], iH = 1.0 / H, H2 = H * H, fac = kSigma * iH * iH * iH / oms[src];
+    const int m = list_cnt[src];
+    const int64_t base = FILL ? off[src] : 0;
+    double w8[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    int c = 0;
+    for (int t0 = 0; t0 < m; t0 += 32) {
+        const int t = t0 + lane;
+        bool in = false;
+        int j = 0, oct = 0;
+        double ps = 0.0;
+        if (t < m) {
+            j = list[src * kSrcList + t];
+            const double dx = sep_fast(xs[j], p[0], g.box[0], half[0], g.periodic);
+            const double dy = sep_fast(xs[n + j], p[1], g.box[1], half[1], g.periodic);
+            const double dz = sep_fast(xs[2 * n + j], p[2], g.box[2], half[2], g.periodic);
+            const double r2 = dx * dx + dy * dy + dz * dz;
+            in = r2 < H2;
+            if (FILL && in) {
+                ps = fac * spline_w(sqrt(r2) * iH);
+                oct = (dx < 0 ? 1 : 0) | (dy < 0 ? 2 : 0) | (dz < 0 ? 4 : 0);
+            }
+        }
+        const unsigned b = __ballot_sync(FULL, in);
+        if (FILL && in) {
+            const int pos = c + __popc(b & ((1u << lane) - 1u));
+            e_gas[base + pos] = j;
+            e_xi[base + pos] = ps;
+            oct_of[wid][pos] = (unsigned char)oct;
+#pragma unroll
+            for (int a = 0; a < 8; ++a) w8[a] += a == oct ? ps : 0.0;
+        }
+        c += __popc(b);
+    }
+    if (!FILL) {
+        if (lane == 0) counts[src] = c;
+        return;
+    }
+    // octant sums; xi = mu_a psi, mu_a = sum_b w_b / (q_nz w_a)
+    double wsum = 0.0;
+    int qnz = 0;
+#pragma unroll
+    for (int a = 0; a < 8; ++a) {
+        w8[a] = octw_given ? octw_given[8 * src + a] : warp_sum(w8[a]);
+        wsum += w8[a];
+        qnz += (w8[a] > 0.0);
+        if (lane == 0) octw_out[8 * src + a] = w8[a];
+    }
+    __syncwarp();
+    const double share = wsum / (double)qnz;
+    for (int e = lane; e < c; e += 32) {
+        const int oct = oct_of[wid][e];
+        double w = 0.0;
+#pragma unroll
+        for (int a = 0; a < 8; ++a) w = a == oct ? w8[a] : w;
+        e_xi[base + e] = share / w * e_xi[base + e];
+    }
+}
+
 // Rows of the culled walk of for_each_candidate handed out round-robin to the threads of a
 // block (thread t takes rows t, t + nt, ...).
 template <class F>
@@ -1356,9 +1572,11 @@ constexpr int kSrcThreads = 128;
 // term), omega summed over the rows of all threads in a fixed tree order
 __global__ void __launch_bounds__(kSrcThreads) k_src_h(Grid g, const double* __restrict__ xs, int64_t n,
                                                        const double* __restrict__ xsrc, int64_t S, SrcParams sp,
-                                                       double* hs_out, double* oms_out, int* flags) {
+                                                       double* hs_out, double* oms_out, int* flags,
+                                                       const int32_t* __restrict__ list_cnt) {
     const int s_id = blockIdx.x;
     const int t = threadIdx.x;
+    if (list_cnt[s_id] >= 0) return;     // solved by k_src_lists
     __shared__ double red_w[kSrcThreads], red_dw[kSrcThreads];
     double p[3] = {xsrc[s_id], xsrc[S + s_id], xsrc[2 * S + s_id]};
     const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
@@ -1401,31 +1619,11 @@ __global__ void __launch_bounds__(kSrcThreads) k_src_h(Grid g, const double* __r
             ok = om > 0.0;
             break;
         }
-        // Newton on S(h) = sum w = S* (see k_h_solve) close to the root, where a step of less than
-        // 1e-8 h ends it: the next one would be below rounding, and at the root omega is
-        // (eta/h)^3.  Farther off on h - eta omega^(-1/3), nearly linear in h.
-        const double f = sw - sp.s_star;
-        if (f < 0.0) lo = h; else hi = h;
-        double step = -INFINITY;
-        if (sw > 0.0 && sdw < 0.0) {
-            if (fabs(f) < 1e-3 * sp.s_star) {
-                step = -f * h / sdw;
-            } else {
-                const double x = cbrt(sp.s_star / sw), fp = 1.0 - x - x * sdw / (3.0 * sw);
-                step = fp > 0.0 ? h * (1.0 - x) / fp : -INFINITY;
-            }
-        }
-        if (fabs(step) <= 1e-8 * h) {
-            h -= step;
-            om = sp.eta3 / (h * h * h);
-            ok = true;
+        const int done = src_newton(sp, sw, sdw, h, lo, hi, om);
+        if (done) {
+            ok = done == 1;
             break;
         }
-        double hn = h - step;
-        if (!(hn > lo && hn < hi)) hn = isinf(hi) ? 1.5 * h : 0.5 * (lo + hi);
-        if (hn > sp.h_cap) hn = sp.h_cap;
-        if (hn == h) { ok = om > 0.0; break; }
-        h = hn;
     }
     if (t == 0) {
         if (!ok) atomicExch(&flags[F_SRC_NOCONV], 1);
@@ -1489,11 +1687,12 @@ __global__ void __launch_bounds__(kSrcWarps * 32)
 k_src_entries(Grid g, const double* __restrict__ xs, int64_t n, const double* __restrict__ xsrc, int64_t S,
               const double* __restrict__ hs, const double* __restrict__ oms, int32_t* counts,
               const int64_t* __restrict__ off, int32_t* e_gas, double* e_xi, double* octw_out,
-              const double* __restrict__ octw_given = nullptr) {
+              const double* __restrict__ octw_given, const int32_t* __restrict__ list_cnt) {
     __shared__ int row_n[kSrcRowsMax];
     __shared__ double w8s[kSrcWarps][8];
     __shared__ int total;
     const int src = blockIdx.x;
+    if (list_cnt[src] >= 0) return;      // k_src_list_entries
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const double p[3] = {xsrc[src], xsrc[S + src], xsrc[2 * S + src]};
     int c[3];
@@ -1905,18 +2104,27 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
 
     // a4: geometry
     unsigned* cond_max = reinterpret_cast<unsigned*>(red + 7);
-    if (c->fp64)
+    double* Bd = c->B_d.as<double>();
+    if (c->fp64) {
+        k_E<double><<<nblk(n * kELanes, 256), 256, 0, st>>>(
+            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->row_off.as<int64_t>(),
+            c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic, qscale[0], qscale[1],
+            qscale[2], Bd);
         k_geometry<double><<<nblk(n, 128), 128, 0, st>>>(
-            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(),
-            c->row_off.as<int64_t>(), c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic,
-            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_f.as<float>(),
-            c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(), red, cond_max, flags);
-    else
+            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(), n,
+            c->V_d.as<double>(), Bd, c->cond_f.as<float>(), c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(),
+            red, cond_max, flags);
+    } else {
+        k_E<float><<<nblk(n * kELanes, 256), 256, 0, st>>>(
+            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->row_off.as<int64_t>(),
+            c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic, qscale[0], qscale[1],
+            qscale[2], Bd);
         k_geometry<float><<<nblk(n, 128), 128, 0, st>>>(
-            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(),
-            c->row_off.as<int64_t>(), c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic,
-            qscale[0], qscale[1], qscale[2], c->V_d.as<double>(), c->B_d.as<double>(), c->cond_f.as<float>(),
-            c->pos_t.p, c->geo_t.as<float>(), c->omega_t.as<float>(), red, cond_max, flags);
+            c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->omega_d.as<double>(), n,
+            c->V_d.as<double>(), Bd, c->cond_f.as<float>(), c->pos_t.p, c->geo_t.as<float>(), c->omega_t.as<float>(),
+            red, cond_max, flags);
+    }
+    c->launches += 1;
     k_cond<<<nblk(n, 256), 256, 0, st>>>(c->cond_f.as<float>(), c->B_d.as<double>(), n, cond_max, red, flags);
     c->launches += 1;
     RT_CUDA(c, cudaGetLastError());
@@ -1942,18 +2150,35 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         c->has_hs_prev = false;     // set again only when this call succeeds
         if (hs_in) RT_CUDA(c, cudaMemcpyAsync(c->hs_d.p, hs_in, S * 8, cudaMemcpyDeviceToDevice, st));
         const unsigned sb = (unsigned)S;   // one block of kSrcWarps warps per source
+        RT_TRY(ensure(c, c->src_list, (size_t)S * kSrcList * 4, "sources"));
+        RT_TRY(ensure(c, c->src_list_cnt, (size_t)S * 4, "sources"));
+        int32_t* slist = c->src_list.as<int32_t>();
+        int32_t* scnt = c->src_list_cnt.as<int32_t>();
+        QuantParams qp;
+        for (int a = 0; a < 3; ++a) {
+            qp.mul[a] = qmul[a];
+            qp.scale[a] = qscale[a];
+        }
+        const unsigned sw = nblk(S, kSrcListWarps);
+        k_src_lists<<<sw, kSrcListWarps * 32, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, qp,
+                                                       c->xsrc_d.as<double>(), S, sp, c->hs_d.as<double>(),
+                                                       c->omegas_d.as<double>(), flags, slist, scnt);
         k_src_h<<<(unsigned)S, kSrcThreads, 0, st>>>(g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S, sp,
-                                                     c->hs_d.as<double>(), c->omegas_d.as<double>(), flags);
+                                                     c->hs_d.as<double>(), c->omegas_d.as<double>(), flags, scnt);
         if (hs_in && oms_in)   // the sources' own omega_s, from their owners
             RT_CUDA(c, cudaMemcpyAsync(c->omegas_d.p, oms_in, S * 8, cudaMemcpyDeviceToDevice, st));
+        k_src_list_entries<false><<<sw, kSrcListWarps * 32, 0, st>>>(
+            g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S, c->hs_d.as<double>(), c->omegas_d.as<double>(),
+            slist, scnt, c->src_counts.as<int32_t>(), nullptr, nullptr, nullptr, nullptr, nullptr);
         k_src_entries<false><<<sb, kSrcWarps * 32, 0, st>>>(g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S,
                                                  c->hs_d.as<double>(), c->omegas_d.as<double>(),
-                                                 c->src_counts.as<int32_t>(), nullptr, nullptr, nullptr, nullptr);
+                                                 c->src_counts.as<int32_t>(), nullptr, nullptr, nullptr, nullptr,
+                                                 nullptr, scnt);
         RT_CUDA(c, cudaMemsetAsync(c->src_counts.as<int32_t>() + S, 0, 4, st));
         tb = c->cub_tmp.bytes;
         RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->src_counts.as<int32_t>(),
                                                  c->src_off.as<int64_t>(), (int)(S + 1), st));
-        c->launches += 2;
+        c->launches += 4;
         int64_t NE = 0;
         RT_CUDA(c, cudaMemcpyAsync(&NE, c->src_off.as<int64_t>() + S, 8, cudaMemcpyDeviceToHost, st));
         RT_CUDA(c, cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, st));
@@ -1974,11 +2199,15 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         RT_TRY(ensure(c, c->inj_targets, NEa * 4, "injection", true));
         RT_TRY(ensure(c, c->inj_off, (NEa + 1) * 4, "injection", true));
         double* octw = c->omegas_d.as<double>() + S;   // 8 per source after omega_s
+        k_src_list_entries<true><<<sw, kSrcListWarps * 32, 0, st>>>(
+            g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S, c->hs_d.as<double>(), c->omegas_d.as<double>(),
+            slist, scnt, nullptr, c->src_off.as<int64_t>(), c->src_entry_gas.as<int32_t>(),
+            c->src_entry_xi.as<double>(), octw, hs_in ? octw_in : nullptr);
         k_src_entries<true><<<sb, kSrcWarps * 32, 0, st>>>(g, c->xs_d.as<double>(), n, c->xsrc_d.as<double>(), S,
                                                 c->hs_d.as<double>(), c->omegas_d.as<double>(), nullptr,
                                                 c->src_off.as<int64_t>(), c->src_entry_gas.as<int32_t>(),
-                                                c->src_entry_xi.as<double>(), octw, hs_in ? octw_in : nullptr);
-        ++c->launches;
+                                                c->src_entry_xi.as<double>(), octw, hs_in ? octw_in : nullptr, scnt);
+        c->launches += 2;
         if (NE > 0) {
             c->launches += 3;
             k_inj_keys<<<nblk(NE, B), B, 0, st>>>(c->src_entry_gas.as<int32_t>(), c->src_off.as<int64_t>(), S, NE,

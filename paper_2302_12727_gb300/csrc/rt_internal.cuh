@@ -116,6 +116,7 @@ struct rt_ctx {
     int64_t n_owned = 0;                                // rt_energy sums caller indices [0, n_owned)
 
     // sources / injection
+    rt::DevBuf src_list, src_list_cnt;                  // candidates of the sources, as lists
     rt::DevBuf xsrc_d, hs_d, omegas_d, src_counts, src_off, inj_key, inj_key_out, inj_val, inj_val_out;
     rt::DevBuf inj_targets, inj_off, inj_src, inj_coef, src_entry_gas, src_entry_xi;
     int64_t n_inj_entries = 0, n_inj_targets = 0;

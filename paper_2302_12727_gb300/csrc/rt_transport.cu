@@ -279,7 +279,8 @@ __global__ void __launch_bounds__(256) k_row_weights(PairArgs<double> a, double*
         const Pos<double> pj = load_pos(tag, a.pos, a.cols[e]);
         double dx, dy, dz;
         sep(a.sp, pi, pj, dx, dy, dz);
-        const double w = spline_w_(sqrt_(norm2_(dx, dy, dz)), iH);
+        const double r2 = norm2_(dx, dy, dz);
+        const double w = r2 > 0.0 ? spline_w_(sqrt_fast(r2), iH) : 0.0;
         wd[3 * e] = w * dx;
         wd[3 * e + 1] = w * dy;
         wd[3 * e + 2] = w * dz;
