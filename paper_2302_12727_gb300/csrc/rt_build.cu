@@ -349,11 +349,11 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
 // Double phase (k_h_refine): Newton on S(h) - S* in double on the exact separations.  On the
 // FP64 path it runs for every particle.  On the float path it runs only for the
 // particles that have a candidate within the near band of their own support radius at the float
-// root: that is within about 1e-6 of the exact one (the last step is below 4e-7 and the
-// rounding of the ~50-term sums 3e-7, over f' > 0.5), so for every other particle no neighbour
-// can change side of H_i, and the pair lists, which are decided by H_i and H_j, are those of
-// the exact roots.  Particles whose last step was not that small, or whose f' is (the edge of
-// a clump), take the double phase too.
+// root: that is within 2e-6 of the exact one (the last step is below 4e-7 and the rounding of
+// the ~50-term sums 3e-7, over f' > 0.25; f' is one in an even set and 1/3 in a density falling
+// as r^-2), so for every other particle no neighbour can change side of H_i, and the pair
+// lists, which are decided by H_i and H_j, are those of the exact roots.  Particles whose last
+// step was not that small, or whose f' is (the edge of a clump), take the double phase too.
 struct HParams {
     double eta, h0, h_cap;
     double s_star, eta3;   // S* = (kappa eta)^3 / sigma, and eta^3
@@ -363,8 +363,8 @@ struct HParams {
     int refine64;   // 1: the double phase follows for every particle, 0: for the flagged ones
 };
 
-// |r / H - 1| below which a candidate flags its particle for the double phase: ten times the
-// float root's error after a tight step
+// |r / H - 1| below which a candidate flags its particle for the double phase: five times the
+// largest error of the float root after a tight step
 constexpr float kNear = 1e-5f, kTightStep = 4e-7f;
 
 __device__ __forceinline__ float fsep(uint32_t a, uint32_t b, float scale) { return (float)(int32_t)(a - b) * scale; }
@@ -405,7 +405,7 @@ __device__ __forceinline__ HStep h_newton(const HParams& hp, float h, float sw, 
     if (f < 0.f) lo = h; else hi = h;
     const float step = f / fp;
     HStep r;
-    r.tight = fp > 0.5f && fabsf(step) <= kTightStep * h;
+    r.tight = fp > 0.25f && fabsf(step) <= kTightStep * h;
     // residual at the rounding floor, a small Newton step, or a collapsed bracket (where f' is
     // small, rounding alone keeps the step above tolerance)
     r.loose = fabsf(f) <= 1e-6f * h || (fp > 0.f && fabsf(step) <= hp.tol32 * h) || (hi - lo) <= hp.tol32 * h;
@@ -650,88 +650,20 @@ k_h_finish(const float* __restrict__ h_sum, int64_t n, int reduce, double* __res
     }
 }
 
-// Double phase for particle p from the float root hd, by the kRefineLanes lanes of a group:
-// Newton on S(h) = S*.  The step after one of less than 1e-8 h is exact to rounding, and at the
-// root omega is (eta/h)^3, so two evaluations do, with no cube root and one reciprocal each:
-// these scalar parts, which a group's lanes all repeat, were three quarters of the double
-// instructions with a warp per particle and the omega^(-1/3) form.  The particle's list holds
-// every candidate within kNear of its float support, which contains every neighbour of every
-// iterate; their distances are dealt to the lanes and kept in registers.  A particle without a
-// list, or whose lanes would need more than kRefineSlots, walks for every evaluation.
-constexpr int kRefineLanes = 8, kRefineSlots = 12;
-
-__device__ bool refine_h(const Grid& g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
-                         const HParams& hp, int64_t p, int lane, unsigned group, const int32_t* __restrict__ list,
-                         int list_cnt, double& hd, double& om_d) {
-    const uint4 q4p = xq[p];
-    const uint32_t qx = q4p.x, qy = q4p.y, qz = q4p.z;
-    const double px = xs[p], py = xs[n + p], pz = xs[2 * n + p];
-    const float pxf = (float)px, pyf = (float)py, pzf = (float)pz;
-    const double half[3] = {0.5 * g.box[0], 0.5 * g.box[1], 0.5 * g.box[2]};
-    // exact distance of candidate j, handed to f if below R
-    auto visit = [&](int j, float R2f, double R2, auto&& f) {
-        const uint4 qj = xq[j];
-        const float dxf = fsep(qj.x, qx, hp.scale[0]);
-        const float dyf = fsep(qj.y, qy, hp.scale[1]);
-        const float dzf = fsep(qj.z, qz, hp.scale[2]);
-        if (dxf * dxf + dyf * dyf + dzf * dzf >= R2f) return;
-        const double dx = sep_fast(xs[j], px, g.box[0], half[0], g.periodic);
-        const double dy = sep_fast(xs[n + j], py, g.box[1], half[1], g.periodic);
-        const double dz = sep_fast(xs[2 * n + j], pz, g.box[2], half[2], g.periodic);
-        const double r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 < R2) f(r2 > 0.0 ? sqrt_fast(r2) : 0.0);
-    };
-    // this lane's candidates closer than R
-    auto walk = [&](double R, auto&& f) {
-        const float Rf = (float)R * 1.0001f, R2f = Rf * Rf;
-        int seen = 0;     // candidates of the earlier ranges (walk order)
-        for_each_candidate_range(g, pxf, pyf, pzf, Rf, [&](int b, int e) {
-            for (int j = b + ((lane - seen) & (kRefineLanes - 1)); j < e; j += kRefineLanes) visit(j, R2f, R * R, f);
-            seen += e - b;
-        });
-    };
-    const double Rc = kKappa * hd * (1.0 + kNear);
-    double r[kRefineSlots];
-    int cnt = 0;
-    if (list_cnt >= 0) {
-        const float Rf = (float)Rc * 1.0001f;
-        for (int k = lane; k < list_cnt; k += kRefineLanes)
-            visit(list[k], Rf * Rf, Rc * Rc, [&](double rr) {
-#pragma unroll
-                for (int u = 0; u < kRefineSlots; ++u)   // static indices keep r in registers
-                    if (u == cnt) r[u] = rr;
-                ++cnt;
-            });
-    }
-    bool kept = list_cnt >= 0 && !__any_sync(group, cnt > kRefineSlots);
+// Newton on S(h) = S* in double from the float root hd, by the lanes of a group: sums(H, iH, S, D)
+// adds this lane's share of S and D = sum q w'(q) = -h dS/dh.  The step after one of less than
+// 1e-8 h is exact to rounding, and at the root omega is (eta/h)^3, so two evaluations do, with no
+// cube root and two reciprocals: these scalar parts, which a group's lanes all repeat, were
+// three quarters of the double instructions in the omega^(-1/3) form.
+template <int LN, class F>
+__device__ __forceinline__ bool newton_double(const HParams& hp, unsigned group, double& hd, double& om_d, F&& sums) {
     double lod = 0.0, hid = INFINITY;
     for (int it = 0; it < 60; ++it) {
         const double H = kKappa * hd, iH = rcp_fast(H);
-        kept = kept && H <= Rc;
-        double S = 0.0, D = 0.0;      // S and sum q w'(q) = -h dS/dh
-        auto term = [&](double rr) {
-            const double q = rr * iH;
-            if (q < 1.0) {
-                const double a = 1.0 - q, a2 = a * a;
-                double w = a2 * a, d = -3.0 * a2;
-                if (q < 0.5) {
-                    const double b = 0.5 - q, b2 = b * b;
-                    w -= 4.0 * (b2 * b);
-                    d += 12.0 * b2;
-                }
-                S += w;
-                D += q * d;
-            }
-        };
-        if (kept) {
+        double S = 0.0, D = 0.0;
+        sums(H, iH, S, D);
 #pragma unroll
-            for (int k = 0; k < kRefineSlots; ++k)
-                if (k < cnt) term(r[k]);
-        } else {
-            walk(H, term);
-        }
-#pragma unroll
-        for (int o = kRefineLanes / 2; o > 0; o >>= 1) {
+        for (int o = LN / 2; o > 0; o >>= 1) {
             S += __shfl_xor_sync(group, S, o);
             D += __shfl_xor_sync(group, D, o);
         }
@@ -752,6 +684,188 @@ __device__ bool refine_h(const Grid& g, const double* __restrict__ xs, const uin
         hd = hn;
     }
     return false;
+}
+
+// one distance's share of S and D
+__device__ __forceinline__ void newton_term(double rr, double iH, double& S, double& D) {
+    const double q = rr * iH;
+    if (q < 1.0) {
+        const double a = 1.0 - q, a2 = a * a;
+        double w = a2 * a, d = -3.0 * a2;
+        if (q < 0.5) {
+            const double b = 0.5 - q, b2 = b * b;
+            w -= 4.0 * (b2 * b);
+            d += 12.0 * b2;
+        }
+        S += w;
+        D += q * d;
+    }
+}
+
+// exact distance of candidate j from particle p; beyond the float bound R2f: infinite
+struct ExactDist {
+    const double* xs;
+    const uint4* xq;
+    int64_t n;
+    double px, py, pz, b0, b1, b2;
+    uint4 q;
+    float s0, s1, s2;
+    int periodic;
+    __device__ __forceinline__ ExactDist(const Grid& g, const double* xs_, const uint4* xq_, int64_t n_, const float* sc,
+                                         int64_t p)
+        : xs(xs_), xq(xq_), n(n_), px(xs_[p]), py(xs_[n_ + p]), pz(xs_[2 * n_ + p]), b0(g.box[0]), b1(g.box[1]),
+          b2(g.box[2]), q(xq_[p]), s0(sc[0]), s1(sc[1]), s2(sc[2]), periodic(g.periodic) {}
+    __device__ __forceinline__ double operator()(int j, float R2f) const {
+        const uint4 qj = xq[j];
+        const float ax = fsep(qj.x, q.x, s0), ay = fsep(qj.y, q.y, s1), az = fsep(qj.z, q.z, s2);
+        if (ax * ax + ay * ay + az * az >= R2f) return INFINITY;
+        const double dx = sep_fast(xs[j], px, b0, 0.5 * b0, periodic);
+        const double dy = sep_fast(xs[n + j], py, b1, 0.5 * b1, periodic);
+        const double dz = sep_fast(xs[2 * n + j], pz, b2, 0.5 * b2, periodic);
+        const double r2 = dx * dx + dy * dy + dz * dz;
+        return r2 > 0.0 ? sqrt_fast(r2) : 0.0;
+    }
+};
+
+// what the double phase leaves behind for particle p
+__device__ __forceinline__ void store_refined(int64_t p, bool ok, double hd, double om_d, double* h_out,
+                                              double* omega_out, float* H2f_out, uint4* xq_out, int* flags) {
+    if (!ok) atomicExch(&flags[F_NOCONV], 1);
+    h_out[p] = hd;
+    omega_out[p] = om_d;
+    const double Hd = kKappa * hd;
+    H2f_out[p] = (float)(Hd * Hd);
+    reinterpret_cast<unsigned*>(xq_out + p)[3] = __float_as_uint((float)(Hd * Hd));
+}
+__device__ __forceinline__ void reduce_refined(double mn, double mx, double h3, bool sum, unsigned long long* hminmax) {
+    warp_minmax(mn, mx);
+    for (int o = 16; o > 0; o >>= 1) h3 += __shfl_xor_sync(0xffffffffu, h3, o);
+    if ((threadIdx.x & 31) == 0 && mx > 0.0) {
+        atomic_min_pos(&hminmax[0], mn);
+        atomic_max_pos(&hminmax[1], mx);
+        if (sum) atomicAdd(reinterpret_cast<double*>(&hminmax[4]), h3);
+    }
+}
+
+// The double phase, LN lanes per particle, from the particle's list: it holds every candidate
+// within kNear of the float support, which contains every neighbour of every iterate.  It runs
+// for the particles k_h_lists flagged (todo, of arbitrary order; each particle's result depends
+// on its own position and neighbours only) or for all of them (FP64, todo NULL), eight lanes
+// each, whose repeated scalar parts the double pipe bears; on small sets, where the flagged ones
+// are a handful and each a chain of latencies, 32.  The
+// distances are dealt to the lanes and kept in registers, SLOTS a lane.  A particle without a
+// list, with more neighbours than slots or with an iterate beyond the list goes to `rest`.  The
+// smallest and largest h are widened to the refined values.
+template <int LN, int SLOTS>
+__global__ void __launch_bounds__(128)
+k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
+           const int32_t* __restrict__ todo, const int* __restrict__ count, const int32_t* __restrict__ list,
+           const int32_t* __restrict__ list_cnt, int cap, double* h_out, double* omega_out, float* H2f_out,
+           uint4* xq_out, unsigned long long* hminmax, int* flags, int32_t* rest, int* rest_n) {
+    const int lane = threadIdx.x & (LN - 1);
+    const unsigned group = LN == 32 ? 0xffffffffu : ((1u << (LN & 31)) - 1u) << (threadIdx.x & 31 & ~(LN - 1));
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LN;
+    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) / LN;
+    const int64_t cnt = todo ? (int64_t)*count : n;
+    double mn = INFINITY, mx = 0.0, h3 = 0.0;
+    for (int64_t t = w0; t < cnt; t += nw) {
+        const int64_t p = todo ? (int64_t)todo[t] : t;
+        const int have = list_cnt[p];
+        double hd = h_out[p], om_d = omega_out[p];
+        const double Rc = kKappa * hd * (1.0 + kNear);
+        const float Rf = (float)Rc * 1.0001f;
+        const ExactDist dist(g, xs, xq, n, hp.scale, p);
+        double r[SLOTS];
+        int c = 0;
+        for (int k = lane; k < have; k += LN) {
+            const double rr = dist(list[p * cap + k], Rf * Rf);
+            if (rr < Rc) {
+#pragma unroll
+                for (int u = 0; u < SLOTS; ++u)   // static indices keep r in registers
+                    if (u == c) r[u] = rr;
+                ++c;
+            }
+        }
+        bool kept = have >= 0 && !__any_sync(group, c > SLOTS);
+        bool ok = false;
+        if (kept)
+            ok = newton_double<LN>(hp, group, hd, om_d, [&](double H, double iH, double& S, double& D) {
+                if (H > Rc) kept = false;
+#pragma unroll
+                for (int k = 0; k < SLOTS; ++k)
+                    if (k < c) newton_term(r[k], iH, S, D);
+            });
+        if (lane != 0) continue;
+        if (!kept || kKappa * hd > Rc) {
+            rest[atomicAdd(rest_n, 1)] = (int32_t)p;
+            continue;
+        }
+        store_refined(p, ok, hd, om_d, h_out, omega_out, H2f_out, xq_out, flags);
+        const double Hd = kKappa * hd;
+        mn = fmin(mn, hd);
+        mx = fmax(mx, hd);
+        h3 += Hd * Hd * Hd;
+    }
+    reduce_refined(mn, mx, h3, !todo, hminmax);
+}
+
+// The double phase of the rest, a warp each: one walk a little beyond the float support, its
+// distances in shared memory (kRestDist of them; each evaluation walks where they overflow).
+// Such a particle may move far enough that its list, if any, no longer covers it: none is left.
+constexpr int kRestDist = 1024, kRestWarps = 4;
+__global__ void __launch_bounds__(kRestWarps * 32)
+k_h_refine_walk(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
+                const int32_t* __restrict__ rest, const int* __restrict__ rest_n, int32_t* list_cnt, double* h_out,
+                double* omega_out, float* H2f_out, uint4* xq_out, unsigned long long* hminmax, int sum, int* flags) {
+    __shared__ double dists[kRestWarps][kRestDist];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned FULL = 0xffffffffu;
+    double* st = dists[wid];
+    double mn = INFINITY, mx = 0.0, h3 = 0.0;
+    const int cnt = *rest_n, nw = gridDim.x * kRestWarps;
+    for (int t = blockIdx.x * kRestWarps + wid; t < cnt; t += nw) {
+        const int64_t p = rest[t];
+        double hd = h_out[p], om_d = omega_out[p], Rs = 0.0;
+        const ExactDist dist(g, xs, xq, n, hp.scale, p);
+        const float pxf = (float)dist.px, pyf = (float)dist.py, pzf = (float)dist.pz;
+        int c = 0;
+        const bool ok = newton_double<32>(hp, FULL, hd, om_d, [&](double H, double iH, double& S, double& D) {
+            if (H > Rs) {
+                Rs = H * 1.001;
+                const float Rf = (float)Rs * 1.0001f;
+                c = 0;
+                __syncwarp();
+                warp_walk(g, pxf, pyf, pzf, Rf, lane, [&](int j, bool valid) {
+                    const double rr = valid ? dist(j, Rf * Rf) : INFINITY;
+                    const bool in = rr < Rs;
+                    const unsigned m = __ballot_sync(FULL, in);
+                    const int pos = c + __popc(m & ((1u << lane) - 1u));
+                    if (in && pos < kRestDist) st[pos] = rr;
+                    c += __popc(m);
+                    return c <= kRestDist;
+                });
+                __syncwarp();
+            }
+            if (c <= kRestDist) {
+                for (int k = lane; k < c; k += 32) newton_term(st[k], iH, S, D);
+            } else {
+                const float Rf = (float)H * 1.0001f;
+                warp_walk(g, pxf, pyf, pzf, Rf, lane, [&](int j, bool valid) {
+                    if (valid) newton_term(dist(j, Rf * Rf), iH, S, D);
+                    return true;
+                });
+            }
+        });
+        if (lane == 0) {
+            store_refined(p, ok, hd, om_d, h_out, omega_out, H2f_out, xq_out, flags);
+            list_cnt[p] = -1;
+            const double Hd = kKappa * hd;
+            mn = fmin(mn, hd);
+            mx = fmax(mx, hd);
+            h3 += Hd * Hd * Hd;
+        }
+    }
+    reduce_refined(mn, mx, h3, sum != 0, hminmax);
 }
 
 // Smoothing lengths given by the caller (rt_neighbours_given_h): h_i from h_in (caller order)
@@ -812,49 +926,6 @@ __global__ void k_h_given(Grid g, const double* __restrict__ xs, const uint4* __
         atomic_min_pos(&hminmax[0], mn);
         atomic_max_pos(&hminmax[1], mx);
         atomicAdd(reinterpret_cast<double*>(&hminmax[4]), h3);
-    }
-}
-
-// The double phase, kRefineLanes lanes per particle: for the particles k_h_lists flagged (todo,
-// of arbitrary order; each particle's result depends on its own position and neighbours
-// only), or for all of them when todo is NULL.  The smallest and largest h are widened to the
-// refined values (the pair search's bound must cover them).
-__global__ void __launch_bounds__(128)
-k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
-           const int32_t* __restrict__ todo, const int* __restrict__ count, const int32_t* __restrict__ list,
-           int32_t* list_cnt, int cap, double* h_out, double* omega_out, float* H2f_out, uint4* xq_out,
-           unsigned long long* hminmax, int* flags) {
-    const int lane = threadIdx.x & (kRefineLanes - 1);
-    const unsigned group = ((1u << kRefineLanes) - 1u) << (threadIdx.x & 31 & ~(kRefineLanes - 1));
-    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / kRefineLanes;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) / kRefineLanes;
-    const int64_t cnt = todo ? (int64_t)*count : n;
-    double mn = INFINITY, mx = 0.0, h3 = 0.0;
-    for (int64_t t = w0; t < cnt; t += nw) {
-        const int64_t p = todo ? (int64_t)todo[t] : t;
-        const double h0 = h_out[p];
-        double hd = h0, om_d = omega_out[p];
-        const bool ok = refine_h(g, xs, xq, n, hp, p, lane, group, list + p * cap, list_cnt[p], hd, om_d);
-        if (lane == 0) {
-            if (!ok) atomicExch(&flags[F_NOCONV], 1);
-            h_out[p] = hd;
-            omega_out[p] = om_d;
-            const double Hd = kKappa * hd;
-            H2f_out[p] = (float)(Hd * Hd);
-            reinterpret_cast<unsigned*>(xq_out + p)[3] = __float_as_uint((float)(Hd * Hd));
-            // a root beyond the list's margin (an edge where f' nearly vanishes): no list
-            if (hd > h0 * (1.0 + kNear)) list_cnt[p] = -1;
-            mn = fmin(mn, hd);
-            mx = fmax(mx, hd);
-            h3 += Hd * Hd * Hd;
-        }
-    }
-    warp_minmax(mn, mx);
-    for (int o = 16; o > 0; o >>= 1) h3 += __shfl_xor_sync(0xffffffffu, h3, o);
-    if ((threadIdx.x & 31) == 0 && mx > 0.0) {
-        atomic_min_pos(&hminmax[0], mn);
-        atomic_max_pos(&hminmax[1], mx);
-        if (!todo) atomicAdd(reinterpret_cast<double*>(&hminmax[4]), h3);
     }
 }
 
@@ -1146,9 +1217,10 @@ __device__ __forceinline__ void store_pos<double>(void* pos, int64_t p, const do
 // compensated (Kahan) float sum, so that E_i keeps ~1e-8 relative accuracy before its
 // inversion in double.
 //
-// E_i, eight lanes a row (the columns are then read side by side and a row of 46 takes six rounds
-// of loads): sums of the float path compensated and merged, those of the double path in double
-constexpr int kELanes = 8;
+// E_i, LN lanes a row: eight for sets too small to fill the GPU with one (a row of 46 then takes
+// six rounds of loads), else one, because merging the lanes' six sums costs as much as the row (float,
+// 262,144 particles: 0.124 ms with eight).  Sums of the float path compensated and merged,
+// those of the double path in double.
 struct Sum {
     double v = 0.0;
     __device__ __forceinline__ void add(double x) { v += x; }
@@ -1160,14 +1232,14 @@ struct KahanSum : Kahan {
         merge(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
     }
 };
-template <class T>
+template <class T, int LN>
 __global__ void __launch_bounds__(256)
 k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
     const int64_t* __restrict__ row_off, const int32_t* __restrict__ cols, int64_t n, double b0, double b1, double b2,
     int periodic, float s0, float s1, float s2, double* __restrict__ E_out) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t p = t / kELanes;
-    const int lane = (int)(t % kELanes);
+    const int64_t p = t / LN;
+    const int lane = (int)(t % LN);
     const bool act = p < n;
     const int64_t pp = act ? p : 0, e1 = act ? row_off[pp + 1] : 0;
     const double H = kKappa * h[pp];
@@ -1176,7 +1248,7 @@ k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* _
         const uint4 q = xq[pp];
         const float iH = (float)(1.0 / H), H2 = (float)(H * H);
 #pragma unroll 2
-        for (int64_t e = row_off[pp] + lane; e < e1; e += kELanes) {
+        for (int64_t e = row_off[pp] + lane; e < e1; e += LN) {
             const uint4 qj = xq[cols[e]];
             const float dx = fsep(qj.x, q.x, s0), dy = fsep(qj.y, q.y, s1), dz = fsep(qj.z, q.z, s2);
             const float r2 = dx * dx + dy * dy + dz * dz;
@@ -1188,7 +1260,7 @@ k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* _
     } else {
         const double x = xs[pp], y = xs[n + pp], z = xs[2 * n + pp];
         const double iH = 1.0 / H, H2 = H * H;
-        for (int64_t e = row_off[pp] + lane; e < e1; e += kELanes) {
+        for (int64_t e = row_off[pp] + lane; e < e1; e += LN) {
             const int j = cols[e];
             const double dx = sep_fast(xs[j], x, b0, 0.5 * b0, periodic);
             const double dy = sep_fast(xs[n + j], y, b1, 0.5 * b1, periodic);
@@ -1202,10 +1274,14 @@ k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* _
         }
     }
 #pragma unroll
-    for (int o = kELanes / 2; o > 0; o >>= 1)
+    for (int o = LN / 2; o > 0; o >>= 1)
 #pragma unroll
         for (int k = 0; k < 6; ++k) acc[k].fold(o);
-    if (act && lane < 6) {
+    if (!act) return;
+    if constexpr (LN == 1) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) E_out[k * n + p] = acc[k].value();
+    } else if (lane < 6) {
         double v = 0.0;
 #pragma unroll
         for (int k = 0; k < 6; ++k) v = k == lane ? acc[k].value() : v;
@@ -1996,12 +2072,21 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
                                              c->h_d.as<double>(), c->omega_d.as<double>(), c->H2f.as<float>(),
                                              c->xq.as<uint4>(), red);
     if (!h_in) {
-        // the number of flagged particles is on the device: a grid of resident blocks (FP64: all)
-        const int64_t nbr = std::min<int64_t>(nblk(n * kRefineLanes, 128), c->sm_count * (c->fp64 ? 64 : 8));
-        k_h_refine<<<(unsigned)nbr, 128, 0, st>>>(
+        // the number of flagged particles is on the device: grids of resident blocks (FP64: all)
+        int32_t* rest = c->keys_in.as<int32_t>();     // the keys are done with
+        int* rest_n = flags + F_SCRATCH;
+        RT_CUDA(c, cudaMemsetAsync(rest_n, 0, 4, st));
+        const bool few = !c->fp64 && n < (int64_t)c->sm_count * 256;
+        const int64_t nbr = std::min<int64_t>(nblk(n * (few ? 32 : 8), 128), c->sm_count * (c->fp64 ? 64 : 8));
+        (few ? k_h_refine<32, 4> : k_h_refine<8, 12>)<<<(unsigned)nbr, 128, 0, st>>>(
             g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, c->fp64 ? nullptr : c->idx_in.as<int32_t>(),
             refine_count, c->lists.as<int32_t>(), c->list_cnt.as<int32_t>(), cap, c->h_d.as<double>(),
-            c->omega_d.as<double>(), c->H2f.as<float>(), c->xq.as<uint4>(), red, flags);
+            c->omega_d.as<double>(), c->H2f.as<float>(), c->xq.as<uint4>(), red, flags, rest, rest_n);
+        k_h_refine_walk<<<(unsigned)std::min<int64_t>(nblk(n, kRestWarps), c->sm_count * 6), kRestWarps * 32, 0, st>>>(
+            g, c->xs_d.as<double>(), c->xq.as<uint4>(), n, hp, rest, rest_n, c->list_cnt.as<int32_t>(),
+            c->h_d.as<double>(), c->omega_d.as<double>(), c->H2f.as<float>(), c->xq.as<uint4>(), red,
+            c->fp64 ? 1 : 0, flags);
+        c->launches += 1;
     }
     RT_CUDA(c, cudaGetLastError());
     c->launches += 3;
@@ -2106,7 +2191,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     unsigned* cond_max = reinterpret_cast<unsigned*>(red + 7);
     double* Bd = c->B_d.as<double>();
     if (c->fp64) {
-        k_E<double><<<nblk(n * kELanes, 256), 256, 0, st>>>(
+        const bool few = n < (int64_t)c->sm_count * 1024;
+        (few ? k_E<double, 8> : k_E<double, 1>)<<<nblk(few ? n * 8 : n, 256), 256, 0, st>>>(
             c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->row_off.as<int64_t>(),
             c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic, qscale[0], qscale[1],
             qscale[2], Bd);
@@ -2115,7 +2201,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
             c->V_d.as<double>(), Bd, c->cond_f.as<float>(), c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(),
             red, cond_max, flags);
     } else {
-        k_E<float><<<nblk(n * kELanes, 256), 256, 0, st>>>(
+        const bool few = n < (int64_t)c->sm_count * 256;
+        (few ? k_E<float, 8> : k_E<float, 1>)<<<nblk(few ? n * 8 : n, 256), 256, 0, st>>>(
             c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->row_off.as<int64_t>(),
             c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic, qscale[0], qscale[1],
             qscale[2], Bd);

@@ -17,7 +17,7 @@
 // subtract those of its lower pairs in a fixed order.  Both particles thus apply the very
 // same Phi_kl with opposite signs: the exchange is exactly antisymmetric, and so exactly
 // conservative, deterministic, and free of atomics.  With individual time bins the same
-// kernels run on the active sets of each min-step (BINS instantiations) and the fluxes are
+// kernels run on the active sets of each min-step (BINS instantiations, k_gather_bins) and the fluxes are
 // weighted by min(dt_k, dt_l) and accumulated until each particle's step ends.
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -375,13 +375,14 @@ static void launch_gradient_wd(rt_ctx* c, cudaStream_t s, const PairArgs<double>
 // same neighbour position and neighbouring 16-byte pieces of the same state record, so a
 // warp request touches about 32 / GC records instead of 32.  Same neighbour pairing and
 // order of accumulation as k_gradient.
-template <int GC>
+template <int GC, bool BINS = false>
 __global__ void __launch_bounds__(256) k_gradient_g(PairArgs<float> a, const float* __restrict__ rec,
                                                     float* __restrict__ grad, int g0) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t i = t / GC;
-    if (i >= a.n) return;
+    int64_t i = t / GC;
     const int g = (int)(t - i * GC);
+    if (i >= (BINS ? a.count : a.n)) return;
+    if constexpr (BINS) i = a.order[i];      // the particles starting a step (an ordered prefix)
     const float* tag = nullptr;
     const Pos<float> pi = load_pos(tag, a.pos, i);
     const float iH = a.geo[8 * i];
@@ -513,7 +514,7 @@ __global__ void __launch_bounds__(64) k_gradient_w(PairArgs<float> a, const floa
 // expression in the same order as k_gradient_g, so the result bits are the same.  With four
 // groups (eight particles per warp, every lane busy) five blocks per SM (48 registers, a few
 // spilled) beat four at 64 registers by 7%; with three groups they lose 2%.
-template <int GC>
+template <int GC, bool BINS = false>
 __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax : 0) k_gradient_s(PairArgs<float> a, const float* __restrict__ rec,
                                                     float* __restrict__ grad, int g0) {
     constexpr int P = 32 / GC;                     // particles per warp
@@ -521,9 +522,11 @@ __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax 
     const int lane = threadIdx.x & 31;
     const int q = lane / GC, g = lane - (lane / GC) * GC;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t i = warp * P + q;
-    const bool act = q < P && i < a.n;             // lanes past P GC and past the last particle idle
-    const int64_t ii = act ? i : 0;
+    // BINS: the particles starting a step (an ordered prefix)
+    const int64_t at = warp * P + q;
+    const bool act = q < P && at < (BINS ? a.count : a.n);   // lanes past P GC and past the last particle idle
+    const int64_t i = act ? (BINS ? (int64_t)a.order[at] : at) : 0;
+    const int64_t ii = i;
     const float* tag = nullptr;
     const Pos<float> pi = load_pos(tag, a.pos, ii);
     const float iH = a.geo[8 * ii];
@@ -766,59 +769,63 @@ __device__ __forceinline__ int update_group(T u[4], const FluxAcc<T>& acc, T f, 
 // partner starts one), in the same order as the uniform gather; at the end of its own step
 // ((s + 1) mod 2^b_i = 0) it applies U_i - dt_min / V_i acc_i, the sink over its step
 // dt_min 2^b_i and the fix-up, and clears the accumulators.  The states are updated in place
-// (this pass runs after the pair pass, and each particle writes only its own record).
+// (this pass runs after the pair pass, and each particle writes only its own record).  One
+// thread per (particle, group), the partners' bins and the slots of up to eight pairs in flight:
+// one thread per particle and a pair at a time took 0.161 ms a min-step on 262,144 particles of
+// four groups.
 template <class T, int GC>
-__device__ __forceinline__ void gather_bins(const PairArgs<T>& a, const FluxExtra<T>& x, const T* __restrict__ rec,
-                                            const T* __restrict__ pairbuf, T* __restrict__ out, int g0, int64_t i) {
-    constexpr int NC = 4 * GC, AW = AccRec<T>::words;
-    const int RS = 4 * a.G;
+__global__ void __launch_bounds__(256) k_gather_bins(PairArgs<T> a, FluxExtra<T> x, const T* __restrict__ pairbuf,
+                                                     T* __restrict__ rec, int g0) {
+    constexpr int NC = 4 * GC, AW = AccRec<T>::words, B = std::is_same<T, float>::value ? 8 : 4;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int64_t q = t / GC;
+    if (q >= a.count) return;
+    const int g = (int)(t - q * GC), gg = g0 + g;
+    const int64_t i = a.order[q];
     const int bi = a.bins[i];
     const int mask = (1 << bi) - 1;
     const bool start_i = !(a.s & mask);
-    T* accp = x.acc + (i * a.G + g0) * AW;
-    FluxAcc<T> acc[GC];
+    T* accp = x.acc + (i * a.G + gg) * AW;
+    FluxAcc<T> acc;
+    acc.load(accp);
+    const int64_t r0 = a.row_off[i], s0 = a.up_off[i];
+    const int nu = (int)(a.up_off[i + 1] - s0), nl = a.n_low[i];
+    const T* pb = pairbuf + 4 * g;
+    // the pairs [e, e + B) of one half of the row: their partners start a step, or i does
+    auto batch = [&](const int32_t* cols, int e, int m, auto&& slot, auto&& put) {
+        bool on[B];
 #pragma unroll
-    for (int g = 0; g < GC; ++g) acc[g].load(accp + g * AW);
-    const int64_t r0 = a.row_off[i], s0 = a.up_off[i], s1 = a.up_off[i + 1];
-    const int nl = a.n_low[i];
-    for (int64_t sl = s0; sl < s1; ++sl) {
-        const int l = a.cols[r0 + nl + (sl - s0)];
-        if (!start_i && (a.s & ((1 << a.bins[l]) - 1))) continue;
-        T phi[NC];
-        vload<NC>(pairbuf + sl * NC, phi);
+        for (int u = 0; u < B; ++u)
+            on[u] = e + u < m && (start_i || !(a.s & ((1 << a.bins[cols[e + u]]) - 1)));
+        T p[B][4];
 #pragma unroll
-        for (int g = 0; g < GC; ++g) acc[g].add(phi + 4 * g);
-    }
+        for (int u = 0; u < B; ++u)
+            if (on[u]) vload<4>(pb + slot(e + u) * NC, p[u]);
+#pragma unroll
+        for (int u = 0; u < B; ++u)
+            if (on[u]) put(p[u]);
+    };
+    const int32_t* up = a.cols + r0 + nl;
+    for (int e = 0; e < nu; e += B)
+        batch(up, e, nu, [&](int u) { return s0 + u; }, [&](const T* p) { acc.add(p); });
     const int32_t* ls = a.low_slot + (r0 - s0);
-    for (int e = 0; e < nl; ++e) {
-        const int k = a.cols[r0 + e];
-        if (!start_i && (a.s & ((1 << a.bins[k]) - 1))) continue;
-        T phi[NC];
-        vload<NC>(pairbuf + (int64_t)ls[e] * NC, phi);
-#pragma unroll
-        for (int g = 0; g < GC; ++g) acc[g].sub(phi + 4 * g);
-    }
+    for (int e = 0; e < nl; e += B)
+        batch(a.cols + r0, e, nl, [&](int u) { return (int64_t)ls[u]; }, [&](const T* p) { acc.sub(p); });
     if ((a.s + 1) & mask) {   // the step of i goes on (the state is updated in place)
-#pragma unroll
-        for (int g = 0; g < GC; ++g) acc[g].store(accp + g * AW);
+        acc.store(accp);
         return;
     }
-    T ui[NC];
-    vload<NC>(rec + i * RS + 4 * g0, ui);
-    const T dt = (T)(*x.dt_dev);
-    const T dti = (T)ldexp(*x.dt_dev, bi);
-    const T f = dt * a.omega[i];
+    T* u = rec + i * 4 * a.G + 4 * gg;
+    T ui[4];
+    vload<4>(u, ui);
+    const T dt = (T)(*x.dt_dev), dti = (T)ldexp(*x.dt_dev, bi);
     T sink = T(1);
     if (x.alpha) sink = fmax_(T(1) - x.c * x.alpha[i] * dti, T(0));
-    int nclamp = 0;
-#pragma unroll
-    for (int g = 0; g < GC; ++g) {
-        const T sk = x.alpha_g ? fmax_(T(1) - x.c * x.alpha_g[i * a.G + g0 + g] * dti, T(0)) : sink;
-        nclamp += update_group<T>(ui + 4 * g, acc[g], f, sk, x.clamp, nullptr);
-        acc[g].zero();
-        acc[g].store(accp + g * AW);
-    }
-    vstore<NC>(out + i * RS + 4 * g0, ui);
+    if (x.alpha_g) sink = fmax_(T(1) - x.c * x.alpha_g[i * a.G + gg] * dti, T(0));
+    const int nclamp = update_group<T>(ui, acc, dt * a.omega[i], sink, x.clamp, nullptr);
+    acc.zero();
+    acc.store(accp);
+    vstore<4>(u, ui);
     if (nclamp) atomicAdd(x.clamp_count, (unsigned long long)nclamp);
 }
 
@@ -858,14 +865,10 @@ __global__ void k_finalize_bins(PairArgs<T> a, FluxExtra<T> x, T* __restrict__ r
 // Pass 2: particle i adds the fluxes of its own upper pairs (contiguous slots) and subtracts
 // those of its lower pairs (k < i, read from k's slots), in a fixed order; then
 // U_i(t + dt) = U_i - dt / V_i sum_l F_il . A_il, the sink and the fix-up.
-template <class T, int GC, bool BINS = false>
+template <class T, int GC>
 __global__ void __launch_bounds__(128) k_flux_gather(PairArgs<T> a, FluxExtra<T> x, const T* __restrict__ rec,
                                                      const T* __restrict__ pairbuf, T* __restrict__ out, int g0) {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if constexpr (BINS) {   // the particles with a starting partner or themselves starting
-        if (i < a.count) gather_bins<T, GC>(a, x, rec, pairbuf, out, g0, a.order[i]);
-        return;
-    }
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     constexpr int NC = 4 * GC;
     const int RS = 4 * a.G;
@@ -1805,7 +1808,7 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
     ae.order = c->order_b.as<int32_t>();
     ae.count = n_end;
     const unsigned nbg = nblk(std::max<int64_t>(n_start, 1), 128), nbf = nblk(std::max<int64_t>(n_pairs, 1), 128);
-    const unsigned nbh = nblk(std::max<int64_t>(n_touch, 1), 128), nbe = nblk(std::max<int64_t>(n_end, 1), 128);
+    const unsigned nbe = nblk(std::max<int64_t>(n_end, 1), 128);
     // the float pair pass by row gathers of the packed rows: the gradient kernel writes the
     // rows of the particles starting a step (their state after injection and their new
     // gradient); every other particle's row still holds the state and gradient of its own
@@ -1832,6 +1835,18 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
                 continue;
             }
         }
+        if constexpr (std::is_same<T, float>::value) {
+            const int64_t w = (n_start + 32 / gc - 1) / (32 / gc);       // warps of the shuffle gradient
+            const unsigned nbs = nblk(w * 32, kGradBlock);
+            switch (gc) {
+                case 1: k_gradient_g<1, true><<<nblk(n_start, 256), 256, 0, s>>>(ag, rec, gr, g0); break;
+                case 2: k_gradient_s<2, true><<<nbs, kGradBlock, 0, s>>>(ag, rec, gr, g0); break;
+                case 3: k_gradient_s<3, true><<<nbs, kGradBlock, 0, s>>>(ag, rec, gr, g0); break;
+                default: k_gradient_s<4, true><<<nbs, kGradBlock, 0, s>>>(ag, rec, gr, g0); break;
+            }
+            ++c->launches;
+            continue;
+        }
         switch (gc) {
             case 1: k_gradient<T, 1, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
             case 2: k_gradient<T, 2, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
@@ -1853,7 +1868,7 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
         ++c->launches;                                                                       \
     }                                                                                        \
     if (n_touch > 0) {                                                                       \
-        k_flux_gather<T, GC_, true><<<nbh, 128, 0, s>>>(ah, x, rec, pb, rec, g0);            \
+        k_gather_bins<T, GC_><<<nblk(n_touch * GC_, 256), 256, 0, s>>>(ah, x, pb, rec, g0);   \
         ++c->launches;                                                                       \
     }                                                                                        \
     if (n_end > 0) {                                                                         \
