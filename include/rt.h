@@ -114,14 +114,14 @@ typedef struct {
     int64_t kernel_launches;  /* cumulative launches of the library's own kernels (graph
                                  replays count every kernel node; library sorts and scans
                                  that the build calls are not counted) */
-    int32_t pair_build;       /* pair-list build of the last rt_neighbours: 0 = every particle
-                                 searched to max(H_i, H_max); 1 = own supports, then sorted and
-                                 de-duplicated with their transposes (chosen when the h range is
-                                 wide); both give the same lists */
+    int32_t pair_build;       /* spread of the supports of the last rt_neighbours: 1 when H_max^3
+                                 exceeds twelve times the mean H^3 (strongly clustered sets), else
+                                 0; the lists are built in one way for both */
     int32_t wait_timeouts;    /* 1 if a device-side wait ran out since the last rt_neighbours */
     int64_t h_refined;        /* particles whose h the last rt_neighbours refined in double: all of
                                  them on the FP64 path; on the float path those with a neighbour
-                                 candidate within 1e-4 of their support radius at the float root */
+                                 candidate within 1e-5 of their support radius at the float root, or
+                                 whose float iteration did not settle as closely as that needs */
 } rt_diag;
 
 /* Launch variants of the float (RT_FP32_MIXED) pair kernels.  The paper has no counterpart:
@@ -142,7 +142,7 @@ typedef struct {
  *                     2: one thread per (particle, group), the lanes of a particle
  *                        computing the neighbour separations and kernel weights once between
  *                        them and exchanging them by warp shuffles (default; as 1 for one
- *                        group).
+ *                        group; with more neighbours in flight on sets too small to fill the GPU).
  * Changing the variants drops the context's captured sub-cycle graphs. */
 typedef struct {
     int32_t flux_variant;
@@ -271,7 +271,8 @@ rt_status rt_set_fields(rt_ctx* ctx, int64_t first, int64_t count, const double*
 /* n_sub steps of size dt without any neighbour search in between (Sec. "Dynamic
  * Sub-Cycling"), replayed from one CUDA graph that the library captures once per
  * (n_sub, source/sink presence) and reuses; dt, Lsrc and alpha live in device buffers,
- * so they may change between calls without a new capture. */
+ * so they may change between calls without a new capture, and so may the pair lists (a
+ * rebuild drops the graphs only when a buffer moves or the pairs outgrow the launch grids). */
 rt_status rt_subcycle(rt_ctx* ctx, int32_t n_sub, double dt, void* U_dev, const double* Lsrc_dev,
                       const double* alpha_dev);
 

@@ -984,7 +984,7 @@ __device__ __forceinline__ bool own_entry(const Grid& g, const double* __restric
 }
 
 // extras that a row holds in place; a row that gets more has them filled in a second pass
-constexpr int kExtras = 32;
+constexpr int kExtras = 64;
 
 // hands the asymmetric entry (p, j) to row j
 __device__ __forceinline__ void hand_extra(int32_t* extra, int32_t* extras, int64_t p, int j) {

@@ -10,7 +10,7 @@
 // V_i psitilde_j(x_i) = Bp_i d w(q).  A neighbour's data is then a few 16-byte loads.
 //
 // The gradient kernels run one thread per particle (or per particle and group) over its
-// symmetric neighbour list.  The flux of each unordered pair (k < l) is evaluated once, by
+// symmetric neighbour list; the double path keeps the geometry of pairs and rows.  The flux of each unordered pair (k < l) is evaluated once, by
 // one thread with k as the left state, and stored in the pair's slot (three launch variants:
 // direct loads, cp.async staging, or TMA row gathers of packed flux rows that the gradient
 // pass writes); a gather kernel lets every particle add the fluxes of its upper pairs and
@@ -1217,12 +1217,12 @@ k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
 // B loads in flight a thread: eight, or (WIDE) 24, a whole half row, with the lower slots' indices
 // loaded beside the upper slots: for sets too small to fill the GPU, where the launch is the
 // latency of one thread's chain of loads (4,096 particles, one group: 14.4 us with eight).
-template <int GC, bool WIDE = false>
-__global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(PairArgs<float> a, FluxExtra<float> x,
-                                                       const float* __restrict__ rec,
-                                                       const float* __restrict__ pairbuf, float* __restrict__ out,
+template <class T, int GC, bool WIDE = false>
+__global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(PairArgs<T> a, FluxExtra<T> x,
+                                                       const T* __restrict__ rec,
+                                                       const T* __restrict__ pairbuf, T* __restrict__ out,
                                                        int g0) {
-    constexpr int B = WIDE ? 24 : 8;
+    constexpr int B = (WIDE ? 24 : 8) * 4 / (int)sizeof(T);
     // blocks run from the last particles to the first: the pair pass wrote the slots in
     // ascending order, so the most recent (still L2-resident) slots are read first
     const int64_t t = (gridDim.x - 1 - blockIdx.x) * (int64_t)blockDim.x + threadIdx.x;
@@ -1231,8 +1231,8 @@ __global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(P
     const int g = (int)(t - i * GC);
     constexpr int NC = 4 * GC;
     const int RS = 4 * a.G;
-    const float* pb = pairbuf + 4 * g;
-    FluxAcc<float> acc;
+    const T* pb = pairbuf + 4 * g;
+    FluxAcc<T> acc;
     acc.zero();
     const int64_t r0 = a.row_off[i], s0 = a.up_off[i], s1 = a.up_off[i + 1];
     const int nl = a.n_low[i];
@@ -1246,7 +1246,7 @@ __global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(P
     // batches of up to B loads in flight (the last one predicated), added in order
     for (int64_t sl = s0; sl < s1; sl += B) {
         const int m = s1 - sl < B ? (int)(s1 - sl) : B;
-        float p[B][4];
+        T p[B][4];
 #pragma unroll
         for (int u = 0; u < B; ++u)
             if (u < m) vload<4>(pb + (sl + u) * NC, p[u]);
@@ -1261,7 +1261,7 @@ __global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(P
             for (int u = 0; u < B; ++u)
                 if (u < m) q[u] = ls[e + u];
         }
-        float p[B][4];
+        T p[B][4];
 #pragma unroll
         for (int u = 0; u < B; ++u)
             if (u < m) vload<4>(pb + (int64_t)q[u] * NC, p[u]);
@@ -1269,15 +1269,15 @@ __global__ void __launch_bounds__(WIDE ? 64 : kGatherBlockMax) k_flux_gather_g(P
         for (int u = 0; u < B; ++u)
             if (u < m) acc.sub(p[u]);
     }
-    const float dt = (float)(*x.dt_dev);
-    const float f = dt * a.omega[i];
-    float sink = 1.f;
-    if (x.alpha) sink = fmax_(1.f - x.c * x.alpha[i] * dt, 0.f);
-    if (x.alpha_g) sink = fmax_(1.f - x.c * x.alpha_g[i * a.G + g0 + g] * dt, 0.f);
-    float ui[4];
+    const T dt = (T)(*x.dt_dev);
+    const T f = dt * a.omega[i];
+    T sink = T(1);
+    if (x.alpha) sink = fmax_(T(1) - x.c * x.alpha[i] * dt, T(0));
+    if (x.alpha_g) sink = fmax_(T(1) - x.c * x.alpha_g[i * a.G + g0 + g] * dt, T(0));
+    T ui[4];
     const int64_t o = i * RS + 4 * (g0 + g);
     vload<4>(rec + o, ui);
-    const int nclamp = update_group<float>(ui, acc, f, sink, x.clamp, x.inj ? x.inj + i * a.G + g0 + g : nullptr);
+    const int nclamp = update_group<T>(ui, acc, f, sink, x.clamp, x.inj ? x.inj + i * a.G + g0 + g : nullptr);
     vstore<4>(out + o, ui);
     if (nclamp) atomicAdd(x.clamp_count, (unsigned long long)nclamp);
 }
@@ -1369,10 +1369,13 @@ static void set_carveouts() {
                         (const void*)k_flux<T, 2, false>, (const void*)k_flux<T, 3, false>,
                         (const void*)k_flux<T, 4, false>, (const void*)k_flux<T, 1, true>,
                         (const void*)k_flux<T, 2, true>, (const void*)k_flux<T, 3, true>,
-                        (const void*)k_flux<T, 4, true>,
-                        (const void*)k_flux_gather<T, 1>, (const void*)k_flux_gather<T, 2>,
-                        (const void*)k_flux_gather<T, 3>, (const void*)k_flux_gather<T, 4>};
+                        (const void*)k_flux<T, 4, true>};
     for (const void* f : fs) cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    if constexpr (std::is_same<T, float>::value) {
+        const void* gs[] = {(const void*)k_flux_gather<T, 1>, (const void*)k_flux_gather<T, 2>,
+                            (const void*)k_flux_gather<T, 3>, (const void*)k_flux_gather<T, 4>};
+        for (const void* f : gs) cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+    }
     (void)cudaGetLastError();
 }
 
@@ -1515,7 +1518,7 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
         attr = true;
         cudaFuncSetAttribute((const void*)k_flux_staged<GC, HLL>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
-        cudaFuncSetAttribute((const void*)k_flux_gather_g<GC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
+        cudaFuncSetAttribute((const void*)k_flux_gather_g<float, GC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
         cudaFuncSetAttribute((const void*)k_flux_tma<GC, HLL>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
         if (HLL)
@@ -1548,9 +1551,9 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
     prof_end(c, s, pr);
     pr = prof_begin(c, s, RT_KERNEL_FLUX_GATHER);
     if (c->tune.gather_variant == 1 && few_threads(c, GC))
-        k_flux_gather_g<GC, true><<<nblk(c->n * GC, 64), 64, 0, s>>>(a, x, rec, pb, out, g0);
+        k_flux_gather_g<float, GC, true><<<nblk(c->n * GC, 64), 64, 0, s>>>(a, x, rec, pb, out, g0);
     else if (c->tune.gather_variant == 1)
-        k_flux_gather_g<GC><<<nblk(c->n * GC, gather_block(c)), gather_block(c), 0, s>>>(a, x, rec, pb, out, g0);
+        k_flux_gather_g<float, GC><<<nblk(c->n * GC, gather_block(c)), gather_block(c), 0, s>>>(a, x, rec, pb, out, g0);
     else
         k_flux_gather<float, GC><<<nblk(c->n, 128), 128, 0, s>>>(a, x, rec, pb, out, g0);
     prof_end(c, s, pr);
@@ -1619,11 +1622,12 @@ static void launch_flux_t(rt_ctx* c, cudaStream_t s, const T* rec, T* out, bool 
         }
         prof_end(c, s, pr);
         pr = prof_begin(c, s, RT_KERNEL_FLUX_GATHER);
+        const unsigned nbg = nblk(c->n * gc, 128);
         switch (gc) {
-            case 1: k_flux_gather<T, 1><<<nb, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
-            case 2: k_flux_gather<T, 2><<<nb, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
-            case 3: k_flux_gather<T, 3><<<nb, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
-            default: k_flux_gather<T, 4><<<nb, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
+            case 1: k_flux_gather_g<T, 1><<<nbg, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
+            case 2: k_flux_gather_g<T, 2><<<nbg, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
+            case 3: k_flux_gather_g<T, 3><<<nbg, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
+            default: k_flux_gather_g<T, 4><<<nbg, 128, 0, s>>>(a, x, rec, pb, out, g0); break;
         }
         prof_end(c, s, pr);
         c->launches += 2;
@@ -1844,14 +1848,13 @@ static void launch_step_bins_t(rt_ctx* c, cudaStream_t s, int step, T* rec, bool
                 case 3: k_gradient_s<3, true><<<nbs, kGradBlock, 0, s>>>(ag, rec, gr, g0); break;
                 default: k_gradient_s<4, true><<<nbs, kGradBlock, 0, s>>>(ag, rec, gr, g0); break;
             }
-            ++c->launches;
-            continue;
-        }
-        switch (gc) {
-            case 1: k_gradient<T, 1, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
-            case 2: k_gradient<T, 2, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
-            case 3: k_gradient<T, 3, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
-            default: k_gradient<T, 4, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
+        } else {
+            switch (gc) {
+                case 1: k_gradient<T, 1, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
+                case 2: k_gradient<T, 2, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
+                case 3: k_gradient<T, 3, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
+                default: k_gradient<T, 4, true><<<nbg, 128, 0, s>>>(ag, rec, gr, g0); break;
+            }
         }
         ++c->launches;
     }
