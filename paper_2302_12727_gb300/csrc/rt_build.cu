@@ -249,7 +249,8 @@ __global__ void k_gather_positions(const double* __restrict__ x, const double* _
 // arithmetic in every lane.
 __device__ __forceinline__ int wrap_once(int c, int nc) { return c < 0 ? c + nc : (c >= nc ? c - nc : c); }
 
-template <class F>
+// ASC false: the order of for_each_candidate_range<false>, which differs where a sphere wraps.
+template <bool ASC = true, class F>
 __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, float pz, float R, int lane, F&& f) {
     const unsigned FULL = 0xffffffffu;
     const float Rc = R * 1.0001f + 1e-6f * (g.cellf[0] + g.cellf[1] + g.cellf[2]);
@@ -271,7 +272,8 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
         }
     }
     const int nzs = hi[2] - lo[2] + 1, nys = hi[1] - lo[1] + 1;
-    const int z0 = first_wrapped(lo[2], hi[2], g.nc[2]), y0 = first_wrapped(lo[1], hi[1], g.nc[1]);
+    const int z0 = ASC ? first_wrapped(lo[2], hi[2], g.nc[2]) : lo[2];
+    const int y0 = ASC ? first_wrapped(lo[1], hi[1], g.nc[1]) : lo[1];
     const int rows = nzs > 0 && nys > 0 ? nzs * nys : 0;
     for (int r0 = 0; r0 < rows; r0 += 32) {
         const int r = r0 + lane;
@@ -303,6 +305,10 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
                 } else if (xb >= g.nc[0]) {
                     s1 = 0; e1 = xb - g.nc[0]; s2 = xa; e2 = g.nc[0] - 1;
                 }
+                if (!ASC && s2 <= e2) {
+                    const int s = s1, e = e1;
+                    s1 = s2; e1 = e2; s2 = s; e2 = e;
+                }
                 if (s1 <= e1) {
                     b1 = g.cell_start[base + s1];
                     n1 = g.cell_start[base + e1 + 1] - b1;
@@ -333,6 +339,17 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
     }
 }
 
+// whether the two orders of that walk may differ
+__device__ __forceinline__ bool walk_wraps(const Grid& g, float px, float py, float pz, float R) {
+    const float Rc = R * 1.0001f + 1e-6f * (g.cellf[0] + g.cellf[1] + g.cellf[2]);
+    const float p[3] = {px, py, pz};
+    bool w = false;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        w |= p[a] - Rc < g.cellf[a] || p[a] + Rc > (g.nc[a] - 1) * g.cellf[a];
+    return g.periodic && w;
+}
+
 // ------------------------------------------------------------------------------------
 // a2: smoothing lengths, h = eta omega(h)^(-1/3) with omega(h) = sum_j W(r_ij, h) and the self
 // term.  With S(h) = sum_j w(r_ij / H) the equation is S(h) = S* = (kappa eta)^3 / sigma, the
@@ -342,18 +359,20 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
 // in h, from the h of the previous call or a local particle count.  The candidates are walked
 // once, out to a little more than the first guess's support: their indices go to the
 // particle's list in memory, from which the double phase and the pair search take them, their
-// distances to shared memory, over which the iterations sum.  Where they overflow the list each
-// iteration walks, but only until S passes 4 S*: a particle that has moved into a dense clump
-// with the h of a void would otherwise visit the whole clump an iteration.
+// distances to shared memory, over which the iterations sum.  Where they overflow the list (a particle
+// that has moved into a dense clump with the h of a void) each iteration walks.
+//
+// The iterates are those of one thread that adds w in double and dw/dh in float, candidate by
+// candidate in the order of for_each_candidate_range<false>: the sum of w is kept to 1e-14 (Sum2), and the
+// sum of dw/dh, whose float rounding decides the last bits of an iterate, is added in that order.  h,
+// omega, V and B are therefore the same, to 1e-14, however the candidates are dealt out.
 //
 // Double phase (k_h_refine): Newton on S(h) - S* in double on the exact separations.  On the
 // FP64 path it runs for every particle.  On the float path it runs only for the
 // particles that have a candidate within the near band of their own support radius at the float
-// root: that is within 2e-6 of the exact one (the last step is below 4e-7 and the rounding of
-// the ~50-term sums 3e-7, over f' > 0.25; f' is one in an even set and 1/3 in a density falling
-// as r^-2), so for every other particle no neighbour can change side of H_i, and the pair
-// lists, which are decided by H_i and H_j, are those of the exact roots.  Particles whose last
-// step was not that small, or whose f' is (the edge of a clump), take the double phase too.
+// root: that is within a few 1e-6 of the exact one, so for every other particle no neighbour
+// can change side of H_i, and the pair lists, which are decided by H_i and H_j, are those of the
+// exact roots.
 struct HParams {
     double eta, h0, h_cap;
     double s_star, eta3;   // S* = (kappa eta)^3 / sigma, and eta^3
@@ -363,9 +382,9 @@ struct HParams {
     int refine64;   // 1: the double phase follows for every particle, 0: for the flagged ones
 };
 
-// |r / H - 1| below which a candidate flags its particle for the double phase: five times the
-// largest error of the float root after a tight step
-constexpr float kNear = 1e-5f, kTightStep = 4e-7f;
+// |r^2 - H^2| < kNearBand H^2 at the float root flags the particle for the double phase; kNear, a
+// little more than its half, is the margin in r that lists keep around H
+constexpr float kNearBand = 2e-4f, kNear = 1.1e-4f;
 
 __device__ __forceinline__ float fsep(uint32_t a, uint32_t b, float scale) { return (float)(int32_t)(a - b) * scale; }
 
@@ -378,42 +397,64 @@ struct Kahan {
         c = (t - s) - y;
         s = t;
     }
-    // adds another sum, without rounding (the lanes of a reduction)
-    __device__ __forceinline__ void merge(float s2, float c2) {
-        const float t = __fadd_rn(s, s2), z = __fsub_rn(t, s);
-        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(s2, z));
-        c = __fsub_rn(__fadd_rn(c, c2), e);
-        s = t;
-    }
     __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
-// One Newton step of the float phase from the sums at h; what the step says about h
-struct HStep {
-    float hn;          // next iterate
-    bool tight, loose; // below kTightStep with f' near one; below the caller's tolerance
+// float sum with the exact rounding error of every addition (TwoSum) in a second float: as good as a
+// double sum to 1e-14 over a row
+struct Sum2 {
+    float s = 0.f, e = 0.f;
+    __device__ __forceinline__ void add(float v, float ev = 0.f) {
+        const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+        const float r = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+        e = __fadd_rn(__fadd_rn(e, ev), r);
+        s = t;
+    }
 };
-__device__ __forceinline__ HStep h_newton(const HParams& hp, float h, float sw, float sdw, int it, float& lo,
-                                          float& hi) {
+
+// One Newton step of the float phase from the sums at h: whether h is the root to the tolerance,
+// else the next iterate
+__device__ __forceinline__ bool h_newton(const HParams& hp, float h, float sw, float sdw, int it, float& lo,
+                                         float& hi, float& next) {
     const float kapf = (float)kKappa, sigf = (float)kSigma, eta = (float)hp.eta;
-    const float iH = 1.f / (kapf * h);
-    const float om = sigf * iH * iH * iH * sw;
-    const float dom = -kapf * sigf * iH * iH * iH * iH * sdw;      // d omega / d h
-    const float cb = cbrtf(om);
-    const float f = h - eta / cb;
-    const float fp = 1.f + (eta / 3.f) / (cb * om) * dom;
+    const float H = kapf * h;
+    const float iH = 1.f / H;
+    float om = sigf * iH * iH * iH * sw;
+    float dom = -kapf * sigf * iH * iH * iH * iH * sdw;      // d omega / d h
+    float cb = cbrtf(om);
+    float f = h - eta / cb;
+    float fp = 1.f + (eta / 3.f) / (cb * om) * dom;
     if (f < 0.f) lo = h; else hi = h;
-    const float step = f / fp;
-    HStep r;
-    r.tight = fp > 0.25f && fabsf(step) <= kTightStep * h;
-    // residual at the rounding floor, a small Newton step, or a collapsed bracket (where f' is
-    // small, rounding alone keeps the step above tolerance)
-    r.loose = fabsf(f) <= 1e-6f * h || (fp > 0.f && fabsf(step) <= hp.tol32 * h) || (hi - lo) <= hp.tol32 * h;
-    // safeguarded Newton; plain bisection of the bracket after 24 Newton steps
+    float step = f / fp;
+    // converged: residual at the rounding floor, a tiny Newton step, or a collapsed
+    // bracket (where f' is small, rounding alone keeps the step above tolerance)
+    if (fabsf(f) <= 1e-6f * h || (fp > 0.f && fabsf(step) <= hp.tol32 * h) || (hi - lo) <= hp.tol32 * h) return true;
     float hn = h - step;
+    // safeguarded Newton; plain bisection of the bracket after 24 Newton steps
     if (it >= 24 || !(hn > lo && hn < hi) || !(fp > 0.f)) hn = isinf(hi) ? 2.f * h : 0.5f * (lo + hi);
-    r.hn = hn > (float)hp.h_cap ? (float)hp.h_cap : hn;
-    return r;
+    if (hn > (float)hp.h_cap) hn = (float)hp.h_cap;
+    next = hn;
+    return false;
+}
+
+// w and t = 3 w + q w' of one candidate at distance r.  Rounded as written: h must not depend on which
+// of the two sums below, or which order of the lanes, a particle takes.
+__device__ __forceinline__ float h_term(float r, float iH, float& t) {
+    const float q = __fmul_rn(r, iH);
+    t = 0.f;
+    if (q >= 1.f) return 0.f;
+    const float u = __fsub_rn(1.f, q);
+    float w = __fmul_rn(__fmul_rn(u, u), u), d = __fmul_rn(__fmul_rn(-3.f, u), u);
+    if (q <= 0.5f) {
+        const float v = __fsub_rn(0.5f, q);
+        w = __fmaf_rn(-__fmul_rn(__fmul_rn(4.f, v), v), v, w);
+        d = __fmaf_rn(__fmul_rn(12.f, v), v, d);
+    }
+    t = __fmaf_rn(3.f, w, __fmul_rn(q, d));
+    return w;
+}
+__device__ __forceinline__ float r2_rn(float dx, float dy, float dz) {
+    return __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
 }
 
 // lanes a particle of the sums, warps and particles a block
@@ -431,8 +472,10 @@ static int list_capacity(double eta) {
 // list's length, or -1 where it overflowed.  Each warp walks for its four particles in turn; the
 // sums of the four then run side by side on eight lanes each.
 // 262,144 particles that moved by a tenth of their spacing took 0.88 ms with a thread per
-// particle and a walk of the cells every iteration, 1,000,000 strongly clustered ones 5.2 ms, and
-// 155 ms where some had the h of a place far less dense.
+// particle and a walk of the cells every iteration.  A whole search of 1,000,000 strongly clustered
+// particles takes 5.8 ms (17 ms), and up to 24 ms (172 ms) where some had the h of a place far less
+// dense: those walk the clump, its derivative terms one after the other (loading the next records
+// ahead of the sums spills and takes 26 ms).
 template <bool SOLVE>
 __global__ void __launch_bounds__(kListWarps * 32)
 k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
@@ -466,11 +509,10 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
         if (SOLVE && (!(h > 0.f) || !(h < (float)hp.h_cap))) h = (float)hp.h0;
     }
     float lo = 0.f, hi = INFINITY, Rs = 0.f, h_over = 0.f;
-    const float s_many = 4.f * (float)hp.s_star;
     // wants: the list is in use (until it overflows); Rs and cnt describe it
     bool done = !active, ok = false, near = false, wants = true;
     int cnt = 0, it = 0;
-    Kahan S_last;
+    Sum2 S_last;
     while (__any_sync(FULL, !done)) {
         const float H = kapf * h, iH = 1.f / H;
         const bool fill = !done && wants && H * (1.f + 2.f * kNear) > Rs;
@@ -481,27 +523,33 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
             const int64_t q = p0 + b;
             const uint4 qp = xq[q];
             const float R = __shfl_sync(FULL, H, src) * (SOLVE ? 1.10f : 1.f + 4.f * kNear), R2 = R * R;
+            const float bx = (float)qp.x * hp.scale[0], by = (float)qp.y * hp.scale[1], bz = (float)qp.z * hp.scale[2];
             int c = 0;
-            warp_walk(g, (float)qp.x * hp.scale[0], (float)qp.y * hp.scale[1], (float)qp.z * hp.scale[2], R, lane,
-                      [&](int j, bool valid) {
-                          float r2 = INFINITY;
-                          if (valid) {
-                              const uint4 qj = xq[j];
-                              const float dx = fsep(qj.x, qp.x, hp.scale[0]);
-                              const float dy = fsep(qj.y, qp.y, hp.scale[1]);
-                              const float dz = fsep(qj.z, qp.z, hp.scale[2]);
-                              r2 = dx * dx + dy * dy + dz * dz;
-                          }
-                          const bool in = r2 < R2;
-                          const unsigned m = __ballot_sync(FULL, in);
-                          const int pos = c + __popc(m & ((1u << lane) - 1u));
-                          if (in && pos < cap) {
-                              list[q * cap + pos] = j;
-                              st[b * cap + pos] = sqrtf(r2);
-                          }
-                          c += __popc(m);
-                          return c <= cap;
-                      });
+            auto store = [&](int j, bool valid, bool to_list, bool to_sum) {
+                float r2 = INFINITY;
+                if (valid) {
+                    const uint4 qj = xq[j];
+                    const float dx = fsep(qj.x, qp.x, hp.scale[0]);
+                    const float dy = fsep(qj.y, qp.y, hp.scale[1]);
+                    const float dz = fsep(qj.z, qp.z, hp.scale[2]);
+                    r2 = r2_rn(dx, dy, dz);
+                }
+                const bool in = r2 < R2;
+                const unsigned m = __ballot_sync(FULL, in);
+                const int pos = c + __popc(m & ((1u << lane) - 1u));
+                if (in && pos < cap) {
+                    if (to_list) list[q * cap + pos] = j;
+                    if (to_sum) st[b * cap + pos] = sqrtf(r2);
+                }
+                c += __popc(m);
+                return c <= cap;
+            };
+            const bool wraps = SOLVE && walk_wraps(g, bx, by, bz, R);
+            if (wraps) {
+                warp_walk<false>(g, bx, by, bz, R, lane, [&](int j, bool v) { return store(j, v, false, true); });
+                c = 0;
+            }
+            warp_walk(g, bx, by, bz, R, lane, [&](int j, bool v) { return store(j, v, true, SOLVE && !wraps); });
             if (a == b) {
                 cnt = c;
                 Rs = R;
@@ -515,92 +563,103 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
         }
         __syncwarp();
         if (!SOLVE) break;
-        Kahan sw;
+        bool band = false;
+        // S compensated, its derivative a plain float sum in the order of the walk: the eight terms of a
+        // round are added one after the other in every lane, so that the iterates and the root
+        // do not depend on how the candidates are dealt
+        Sum2 sw;
         float sdw = 0.f, gap = INFINITY;
-        auto term = [&](float q) {
-            gap = fminf(gap, fabsf(q - 1.f));
-            const float u = fmaxf(1.f - q, 0.f), v = fmaxf(0.5f - q, 0.f);
-            const float u2 = u * u, v2 = v * v;
-            const float w = u2 * u - 4.f * (v2 * v);
-            sw.add(w);
-            sdw += 3.f * w + q * (12.f * v2 - 3.f * u2);
-        };
-        if (!done && wants)
-            for (int k = sub; k < cnt; k += kSumLanes) term(st[a * cap + k] * iH);
+        const int mine = !done && wants ? cnt : 0;
+        const int most = __reduce_max_sync(FULL, mine);
+        for (int k0 = 0; k0 < most; k0 += kSumLanes) {
+            const int k = k0 + sub;
+            float t = 0.f;
+            if (k < mine) {
+                const float r = st[a * cap + k], q = r * iH;
+                gap = fminf(gap, fabsf(fabsf(q * q - 1.f) - kNearBand));
+                band |= fabsf(q * q - 1.f) < kNearBand;
+                if (r < H) sw.add(h_term(r, iH, t));
+            }
+#pragma unroll
+            for (int u = 0; u < kSumLanes; ++u) sdw += __shfl_sync(FULL, t, u, kSumLanes);
+        }
 #pragma unroll
         for (int o = kSumLanes / 2; o > 0; o >>= 1) {
-            sw.merge(__shfl_xor_sync(FULL, sw.s, o), __shfl_xor_sync(FULL, sw.c, o));
-            sdw += __shfl_xor_sync(FULL, sdw, o);
+            sw.add(__shfl_xor_sync(FULL, sw.s, o), __shfl_xor_sync(FULL, sw.e, o));
             gap = fminf(gap, __shfl_xor_sync(FULL, gap, o));
         }
         // walks that sum, for the particles whose candidates overflow the list
-        bool many = false;
         todo = __ballot_sync(FULL, !done && !wants && sub == 0);
         while (todo) {
             const int src = __ffs(todo) - 1, b = src / kSumLanes;
             todo &= todo - 1;
             const uint4 qp = xq[p0 + b];
-            const float Hb = __shfl_sync(FULL, H, src), iHb = 1.f / Hb;
-            const float R = Hb * (1.f + 2.f * kNear), R2 = R * R;
-            Kahan swb;
-            float sdb = 0.f, gb = INFINITY;
-            warp_walk(g, (float)qp.x * hp.scale[0], (float)qp.y * hp.scale[1], (float)qp.z * hp.scale[2], R, lane,
-                      [&](int j, bool valid) {
-                          if (valid) {
-                              const uint4 qj = xq[j];
-                              const float dx = fsep(qj.x, qp.x, hp.scale[0]);
-                              const float dy = fsep(qj.y, qp.y, hp.scale[1]);
-                              const float dz = fsep(qj.z, qp.z, hp.scale[2]);
-                              const float r2 = dx * dx + dy * dy + dz * dz;
-                              if (r2 < R2) {
-                                  const float q = sqrtf(r2) * iHb;
-                                  gb = fminf(gb, fabsf(q - 1.f));
-                                  const float u = fmaxf(1.f - q, 0.f), v = fmaxf(0.5f - q, 0.f);
-                                  const float u2 = u * u, v2 = v * v;
-                                  const float w = u2 * u - 4.f * (v2 * v);
-                                  swb.add(w);
-                                  sdb += 3.f * w + q * (12.f * v2 - 3.f * u2);
-                              }
-                          }
-                          return !__any_sync(FULL, swb.s >= s_many);
-                      });
+            const float Hb = __shfl_sync(FULL, H, src), iHb = 1.f / Hb, H2b = __fmul_rn(Hb, Hb);
+            Sum2 swb;
+            float sdb = 0.f;
+            bool nb = false;
+            warp_walk<false>(g, (float)qp.x * hp.scale[0], (float)qp.y * hp.scale[1], (float)qp.z * hp.scale[2],
+                             Hb * (1.f + 2.f * kNear), lane, [&](int j, bool valid) {
+                                 float t = 0.f;
+                                 if (valid) {
+                                     const uint4 qj = xq[j];
+                                     const float dx = fsep(qj.x, qp.x, hp.scale[0]);
+                                     const float dy = fsep(qj.y, qp.y, hp.scale[1]);
+                                     const float dz = fsep(qj.z, qp.z, hp.scale[2]);
+                                     const float r2 = r2_rn(dx, dy, dz);
+                                     nb |= fabsf(__fsub_rn(r2, H2b)) < kNearBand * H2b;
+                                     if (r2 < H2b) swb.add(h_term(sqrtf(r2), iHb, t));
+                                 }
+                                 if (__any_sync(FULL, t != 0.f)) {
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                swb.merge(__shfl_xor_sync(FULL, swb.s, o), __shfl_xor_sync(FULL, swb.c, o));
-                sdb += __shfl_xor_sync(FULL, sdb, o);
-                gb = fminf(gb, __shfl_xor_sync(FULL, gb, o));
-            }
+                                     for (int u = 0; u < 32; ++u) sdb += __shfl_sync(FULL, t, u);
+                                 }
+                                 return true;
+                             });
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) swb.add(__shfl_xor_sync(FULL, swb.s, o), __shfl_xor_sync(FULL, swb.e, o));
+            nb = __any_sync(FULL, nb);
             if (a == b) {
                 sw = swb;
                 sdw = sdb;
-                gap = gb;
-                many = swb.s >= s_many;
+                gap = INFINITY;
+                band = nb;
             }
         }
+        bool edge = false;
         if (!done) {
-            if (many) {           // S(h) > 4 S*: far too large, whatever the rest of the walk
-                hi = h;
-                h = fmaxf(0.6f * h, 0.5f * (lo + h));
-                wants = h < 0.85f * h_over;
-                done = it + 1 >= hp.max_iter;
+            S_last = sw;
+            float hn = h;
+            if (h_newton(hp, h, __fadd_rn(sw.s, sw.e), sdw, it, lo, hi, hn)) {
+                ok = done = true;
+                near = band;
+                edge = gap < 2e-6f;
+            } else if (hn == h || it + 1 >= hp.max_iter) {
+                done = true;      // no progress possible: reported as not converged
             } else {
-                S_last = sw;
-                const HStep r = h_newton(hp, h, sw.s - sw.c, sdw, it, lo, hi);
-                if (r.tight || (r.loose && (it >= 6 || it + 1 >= hp.max_iter || r.hn == h))) {
-                    ok = done = true;
-                    near = !r.tight || gap < kNear;
-                    // the double phase may move such an h by more than the margin of the list
-                    if (!r.tight && Rs < 1.01f * H) wants = false;
-                } else if (r.hn == h || it + 1 >= hp.max_iter) {
-                    done = true;      // no progress possible: reported as not converged
-                } else {
-                    h = r.hn;
-                    wants = wants || h < 0.85f * h_over;
-                }
+                h = hn;
+                wants = wants || h < 0.85f * h_over;
             }
             ++it;
         }
+        // a candidate within rounding of the band's edge: the band on the separations themselves
+        if (__any_sync(FULL, edge)) {
+            if (edge) {
+                const uint4 qp = xq[p];
+                const float H2 = __fmul_rn(H, H);
+                near = false;
+                for (int k = sub; k < cnt; k += kSumLanes) {
+                    const uint4 qj = xq[list[p * cap + k]];
+                    const float dx = fsep(qj.x, qp.x, hp.scale[0]);
+                    const float dy = fsep(qj.y, qp.y, hp.scale[1]);
+                    const float dz = fsep(qj.z, qp.z, hp.scale[2]);
+                    const float r2 = r2_rn(dx, dy, dz);
+                    near |= fabsf(__fsub_rn(r2, H2)) < kNearBand * H2;
+                }
+            }
+        }
     }
+    near = __any_sync(((1u << kSumLanes) - 1u) << (a * kSumLanes), near);
     if (active && sub == 0) {
         list_cnt[p] = wants ? cnt : -1;
         if (SOLVE) {
@@ -608,7 +667,7 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
             if (ok && near && !hp.refine64) refine_list[atomicAdd(refine_count, 1)] = (int32_t)p;
             h_sum[p] = h;
             h_sum[n + p] = S_last.s;
-            h_sum[2 * n + p] = S_last.c;
+            h_sum[2 * n + p] = S_last.e;
         }
     }
 }
@@ -633,7 +692,7 @@ k_h_finish(const float* __restrict__ h_sum, int64_t n, int reduce, double* __res
             h3 = H * H * H;
             mn = mx = hd;
             h_out[p] = hd;
-            omega_out[p] = kSigma / h3 * ((double)h_sum[n + p] - (double)h_sum[2 * n + p]);
+            omega_out[p] = kSigma / h3 * ((double)h_sum[n + p] + (double)h_sum[2 * n + p]);
             H2f[p] = H2;
         } else {
             H2 = H2f[p];
@@ -1217,20 +1276,14 @@ __device__ __forceinline__ void store_pos<double>(void* pos, int64_t p, const do
 // compensated (Kahan) float sum, so that E_i keeps ~1e-8 relative accuracy before its
 // inversion in double.
 //
-// E_i, LN lanes a row: eight for sets too small to fill the GPU with one (a row of 46 then takes
-// six rounds of loads), else one, because merging the lanes' six sums costs as much as the row (float,
-// 262,144 particles: 0.124 ms with eight).  Sums of the float path compensated and merged,
-// those of the double path in double.
+// E_i, LN lanes a row: eight on the double path's sets too small to fill the GPU with one (a row of 46
+// then takes six rounds of loads), else one.  The float path always takes one: its compensated
+// sums round at 1e-8 by the order of the row, and E_i is to be the same for every size of set.
 struct Sum {
     double v = 0.0;
     __device__ __forceinline__ void add(double x) { v += x; }
     __device__ __forceinline__ void fold(int o) { v += __shfl_xor_sync(0xffffffffu, v, o); }
     __device__ __forceinline__ double value() const { return v; }
-};
-struct KahanSum : Kahan {
-    __device__ __forceinline__ void fold(int o) {
-        merge(__shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
-    }
 };
 template <class T, int LN>
 __global__ void __launch_bounds__(256)
@@ -1243,7 +1296,7 @@ k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* _
     const bool act = p < n;
     const int64_t pp = act ? p : 0, e1 = act ? row_off[pp + 1] : 0;
     const double H = kKappa * h[pp];
-    typename std::conditional<std::is_same<T, float>::value, KahanSum, Sum>::type acc[6];
+    typename std::conditional<std::is_same<T, float>::value, Kahan, Sum>::type acc[6];
     if constexpr (std::is_same<T, float>::value) {
         const uint4 q = xq[pp];
         const float iH = (float)(1.0 / H), H2 = (float)(H * H);
@@ -1273,15 +1326,16 @@ k_E(const double* __restrict__ xs, const uint4* __restrict__ xq, const double* _
             acc[3].add(wx * dy); acc[4].add(wx * dz); acc[5].add(wy * dz);
         }
     }
-#pragma unroll
-    for (int o = LN / 2; o > 0; o >>= 1)
-#pragma unroll
-        for (int k = 0; k < 6; ++k) acc[k].fold(o);
-    if (!act) return;
     if constexpr (LN == 1) {
+        if (!act) return;
 #pragma unroll
         for (int k = 0; k < 6; ++k) E_out[k * n + p] = acc[k].value();
-    } else if (lane < 6) {
+    } else {
+#pragma unroll
+        for (int o = LN / 2; o > 0; o >>= 1)
+#pragma unroll
+            for (int k = 0; k < 6; ++k) acc[k].fold(o);
+        if (!act || lane >= 6) return;
         double v = 0.0;
 #pragma unroll
         for (int k = 0; k < 6; ++k) v = k == lane ? acc[k].value() : v;
@@ -2201,8 +2255,7 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
             c->V_d.as<double>(), Bd, c->cond_f.as<float>(), c->pos_t.p, c->geo_t.as<double>(), c->omega_t.as<double>(),
             red, cond_max, flags);
     } else {
-        const bool few = n < (int64_t)c->sm_count * 256;
-        (few ? k_E<float, 8> : k_E<float, 1>)<<<nblk(few ? n * 8 : n, 256), 256, 0, st>>>(
+        k_E<float, 1><<<nblk(n, 256), 256, 0, st>>>(
             c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), c->row_off.as<int64_t>(),
             c->cols.as<int32_t>(), n, cfg.box[0], cfg.box[1], cfg.box[2], cfg.periodic, qscale[0], qscale[1],
             qscale[2], Bd);
