@@ -246,7 +246,8 @@ __global__ void k_gather_positions(const double* __restrict__ x, const double* _
 // walk by returning false (the same in every lane).  A thread that walks its own sphere runs
 // row by row on the latency of the table and record loads, half of a warp's lanes idle (14.8
 // active of 32) behind the longest row; a warp per particle that takes the rows in turn repeats the row
-// arithmetic in every lane.
+// arithmetic in every lane.  Periodic cells wrap once, so (px, py, pz) has to lie in the box (its
+// upper edge included): no kernel walks once F_BADPOS is set (bad_positions).
 __device__ __forceinline__ int wrap_once(int c, int nc) { return c < 0 ? c + nc : (c >= nc ? c - nc : c); }
 
 // ASC false: the order of for_each_candidate_range<false>, which differs where a sphere wraps.
@@ -338,6 +339,11 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
         }
     }
 }
+
+// A position that is not finite or not in the box (k_keys): the call fails at its first
+// synchronisation, and the kernels queued before it that walk the cells, or follow lists that only
+// those make, do nothing
+__device__ __forceinline__ bool bad_positions(const int* flags) { return flags[F_BADPOS] != 0; }
 
 // whether the two orders of that walk may differ
 __device__ __forceinline__ bool walk_wraps(const Grid& g, float px, float py, float pz, float R) {
@@ -485,6 +491,7 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
     constexpr int PW = 32 / kSumLanes;            // particles a warp
     const unsigned FULL = 0xffffffffu;
     extern __shared__ float st_all[];             // distances of the stored candidates, cap a particle
+    if (bad_positions(flags)) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int a = lane / kSumLanes, sub = lane % kSumLanes;
     const int64_t p0 = (blockIdx.x * (int64_t)kListWarps + wid) * PW, p = p0 + a;
@@ -821,6 +828,7 @@ k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, 
            const int32_t* __restrict__ todo, const int* __restrict__ count, const int32_t* __restrict__ list,
            const int32_t* __restrict__ list_cnt, int cap, double* h_out, double* omega_out, float* H2f_out,
            uint4* xq_out, unsigned long long* hminmax, int* flags, int32_t* rest, int* rest_n) {
+    if (bad_positions(flags)) return;
     const int lane = threadIdx.x & (LN - 1);
     const unsigned group = LN == 32 ? 0xffffffffu : ((1u << (LN & 31)) - 1u) << (threadIdx.x & 31 & ~(LN - 1));
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LN;
@@ -934,6 +942,7 @@ k_h_refine_walk(Grid g, const double* __restrict__ xs, const uint4* __restrict__
 __global__ void k_h_given(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
                           HParams hp, const double* __restrict__ h_in, const int32_t* __restrict__ perm,
                           double* h_out, double* omega_out, float* H2f_out, unsigned long long* hminmax, int* flags) {
+    if (bad_positions(flags)) return;
     const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool active = p < n;
     double hd = 0.0;
@@ -1058,13 +1067,13 @@ __device__ __forceinline__ void hand_extra(int32_t* extra, int32_t* extras, int6
 __global__ void __launch_bounds__(256, 5)
 k_own_rows(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
            int64_t n, PairParams pp, int32_t* list, int cap, const int32_t* __restrict__ list_cnt,
-           int32_t* __restrict__ own, int32_t* extra, int32_t* __restrict__ extras, int32_t* over, int* over_n) {
+           int32_t* __restrict__ own, int32_t* extra, int32_t* __restrict__ extras, int32_t* over, int* flags) {
     const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (p >= n) return;
+    if (p >= n || bad_positions(flags)) return;
     const int had = list_cnt[p];
     if (had < 0) {
-        if (lane == 0) over[atomicAdd(over_n, 1)] = (int32_t)p;
+        if (lane == 0) over[atomicAdd(flags + F_OVER, 1)] = (int32_t)p;
         return;
     }
     const uint4 qp = xq[p];
@@ -2159,7 +2168,7 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     k_own_rows<<<nblk(n * 32, 256), 256, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n,
                                                    pp, c->lists.as<int32_t>(), cap, c->list_cnt.as<int32_t>(),
                                                    c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(),
-                                                   c->extras.as<int32_t>(), over, over_n);
+                                                   c->extras.as<int32_t>(), over, flags);
     k_own_walk<false><<<(unsigned)c->sm_count * 4, 128, 0, st>>>(
         g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n, pp, c->lists.as<int32_t>(), cap,
         c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(), c->extras.as<int32_t>(), over, over_n, spill_n, nullptr);
