@@ -185,10 +185,11 @@ rt_status rt_set_stream(rt_ctx* ctx, void* cuda_stream);
  * radii and injection weights.
  *   x_dev    [3][N] positions in [0, box)
  *   m_dev    [N] masses (kept for the caller's density; may be NULL)
- *   xsrc_dev [3][S] source positions (may be NULL when S = 0)
+ *   xsrc_dev [3][S] source positions (may be NULL when S = 0): any finite ones; they wrap into a
+ *            periodic box, and may lie outside one without walls
  *   h_out    [N] device, receives h_i in caller order (may be NULL)
  * Synchronises the stream (it sizes the pair lists).  Errors: RT_ERR_INVALID (NaN/Inf or
- * out-of-box positions), RT_ERR_NOCONV, RT_ERR_GEOMETRY, RT_ERR_OOM. */
+ * out-of-box positions, NaN/Inf source positions), RT_ERR_NOCONV, RT_ERR_GEOMETRY, RT_ERR_OOM. */
 rt_status rt_neighbours(rt_ctx* ctx, const double* x_dev, const double* m_dev, const double* xsrc_dev,
                         double* h_out_dev);
 

@@ -1443,6 +1443,28 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
+// The sources' positions as the searches take them.  A periodic one is wrapped into the box, from
+// a cell of which the walks start, and whose fixed point the float test measures from (the
+// separations themselves wrap once more).  Without walls a source may lie outside.  One that is not
+// finite ends the call (F_BADPOS) and is searched from 0 until then.
+struct SrcBox {
+    double box[3];
+    int periodic;
+};
+__global__ void k_src_positions(const double* __restrict__ x, int64_t S, SrcBox b, double* __restrict__ out, int* flags) {
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (t >= 3 * S) return;
+    const double L = b.box[t / S];
+    double v = x[t];
+    if (!isfinite(v)) {
+        atomicExch(&flags[F_BADPOS], 1);
+        v = 0.0;
+    } else if (b.periodic && !(v >= 0.0 && v <= L)) {
+        v = fmin(fmax(v - L * floor(v / L), 0.0), L);
+    }
+    out[t] = v;
+}
+
 struct SrcParams {
     double s_star, eta3, h0, h_cap;   // (kappa eta)^3 / sigma and eta^3 of the sources' eta
     int max_iter;
@@ -1670,8 +1692,9 @@ __device__ __forceinline__ void strided_rows(const Grid& g, float px, float py, 
             hi[a] = min(hi[a], g.nc[a] - 1);
         }
     }
-    const int ny = hi[1] - lo[1] + 1;
-    const int nrows = (hi[2] - lo[2] + 1) * ny;
+    // no rows beside a box without walls
+    const int ny = max(hi[1] - lo[1] + 1, 0);
+    const int nrows = lo[2] <= hi[2] ? (hi[2] - lo[2] + 1) * ny : 0;
     for (int r = t; r < nrows; r += nt) {
         int z = lo[2] + r / ny, y = lo[1] + r % ny;
         float dz = all[2] ? 0.f : fmaxf(0.f, fmaxf(z * g.cellf[2] - pz, pz - (z + 1) * g.cellf[2]));
@@ -1840,7 +1863,7 @@ k_src_entries(Grid g, const double* __restrict__ xs, int64_t n, const double* __
     const double h = hs[src], H = kKappa * h, iH = 1.0 / H, H2 = H * H;
     const double fac = kSigma * iH * iH * iH / oms[src];
     int k[3];
-    for (int a = 0; a < 3; ++a) k[a] = (int)ceil(H * g.inv_cell[a]);
+    for (int a = 0; a < 3; ++a) k[a] = (int)fmin(ceil(H * g.inv_cell[a]), (double)g.nc[a]);
     const CubeRows cr = cube_rows(g, c, k);
     const bool split = cr.rows <= kSrcRowsMax;
     const int nw = split ? kSrcWarps : 1;
@@ -2287,7 +2310,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         RT_TRY(ensure(c, c->omegas_d, S * 8 + 64 * S, "sources"));
         RT_TRY(ensure(c, c->src_counts, (S + 1) * 4, "sources"));
         RT_TRY(ensure(c, c->src_off, (S + 1) * 8, "sources"));
-        RT_CUDA(c, cudaMemcpyAsync(c->xsrc_d.p, xsrc, 3 * S * 8, cudaMemcpyDeviceToDevice, st));
+        const SrcBox sbox = {{cfg.box[0], cfg.box[1], cfg.box[2]}, cfg.periodic};
+        k_src_positions<<<nblk(3 * S, 128), 128, 0, st>>>(xsrc, S, sbox, c->xsrc_d.as<double>(), flags);
         SrcParams sp;
         sp.eta3 = cfg.eta_res_star * cfg.eta_res_star * cfg.eta_res_star;
         sp.s_star = kKappa * kKappa * kKappa / kSigma * sp.eta3;
@@ -2327,11 +2351,12 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         tb = c->cub_tmp.bytes;
         RT_CUDA(c, cub::DeviceScan::ExclusiveSum(c->cub_tmp.p, tb, c->src_counts.as<int32_t>(),
                                                  c->src_off.as<int64_t>(), (int)(S + 1), st));
-        c->launches += 4;
+        c->launches += 5;
         int64_t NE = 0;
         RT_CUDA(c, cudaMemcpyAsync(&NE, c->src_off.as<int64_t>() + S, 8, cudaMemcpyDeviceToHost, st));
         RT_CUDA(c, cudaMemcpyAsync(hflags, flags, sizeof(hflags), cudaMemcpyDeviceToHost, st));
         RT_CUDA(c, cudaStreamSynchronize(st));
+        if (hflags[F_BADPOS]) return fail(c, RT_ERR_INVALID, "source positions must be finite");
         if (hflags[F_BADH]) return fail(c, RT_ERR_INVALID, "given source smoothing lengths must be finite and > 0");
         if (hflags[F_SRC_NOCONV]) return fail(c, RT_ERR_NOCONV, "source smoothing-length iteration did not converge");
         if (NE > Smax) return fail(c, RT_ERR_INVALID, "too many injection entries");

@@ -38,3 +38,68 @@ def test_positions_out_of_the_box_are_refused(precision, periodic):
     t.rebuild(x)
     assert torch.equal(t.h, h)
     t.close()
+
+
+def _sources_set(rng, n=20000):
+    """A background with clumps, and sources in both: those in clumps overflow their candidate list."""
+    c = rng.uniform(0.2, 0.8, (3, 3))
+    x = np.mod(np.concatenate([rng.uniform(0, 1, (3, n // 2)),
+                               c[:, rng.integers(0, 3, n - n // 2)] + 0.01 * rng.normal(size=(3, n - n // 2))], axis=1), 1)
+    xsrc = np.concatenate([c, rng.uniform(0, 1, (3, 5)), [[0.0, 0.999], [0.002, 0.5], [0.998, 0.001]]], axis=1)
+    return x, np.round(xsrc * 2 ** 20) / 2 ** 20      # box lengths are added to it exactly
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_sources_outside_a_periodic_box_are_their_images(precision):
+    """The same sources whole boxes away: the same smoothing lengths, norms and injection, bit by bit."""
+    _need_gpu()
+    rng = np.random.default_rng(8)
+    x, xsrc = _sources_set(rng)
+    S = xsrc.shape[1]
+    L = rng.uniform(0.5, 2.0, (S, 1))
+    shifts = [np.zeros((3, S))] + [rng.integers(-4, 5, (3, S)).astype(float) for _ in range(2)]
+    shifts.append(np.where(np.arange(3)[:, None] == np.arange(S) % 3, -1.0, 0.0))
+    out = []
+    for d in shifts:
+        t = Transport(x, None, xsrc + d, n_groups=1, precision=precision)
+        U = t.state(np.zeros((1, 4, x.shape[1])))
+        t.inject(U, 1.0, t.luminosities(L))
+        out.append([t.source_h(), *t.source_norms(), U])
+        t.close()
+    for o in out[1:]:
+        for a, b in zip(out[0], o):
+            assert torch.equal(a, b)
+
+
+def test_sources_outside_an_open_box():
+    """Sources beside a box without periodic images, near and far: the oracle's h_s, omega_s and injection."""
+    _need_gpu()
+    rng = np.random.default_rng(9)
+    x, _ = _sources_set(rng, 6000)
+    n = x.shape[1]
+    xsrc = np.array([[1.02, 0.5, -0.1, 1.3, -2.0], [0.5, -0.03, 1.2, 1.1, 4.0], [0.5, 1.01, 0.5, -0.2, 3.0]])
+    o = oracle.Oracle(x, np.full(n, 1.0 / n), xsrc, n_groups=1, periodic=False)
+    s = o.sources()
+    t = Transport(x, None, xsrc, n_groups=1, precision="fp64", periodic=False)
+    # the tolerances of sources inside (exact roots, sums of up to thousands of weights)
+    assert np.abs(t.source_h().cpu().numpy() / s.hs - 1).max() <= 1e-12
+    assert np.abs(t.source_norms()[0].cpu().numpy() / s.omegas - 1).max() <= 1e-11
+    U = t.state(np.zeros((1, 4, n)))
+    t.inject(U, 1.0, t.luminosities(np.ones((xsrc.shape[1], 1))))
+    ref = o.inject(np.zeros((1, 4, n)), 1.0, np.ones((xsrc.shape[1], 1)))
+    ref = np.asarray(ref[0] if isinstance(ref, tuple) else ref)
+    assert np.abs(U.cpu().numpy() - ref).max() <= 1e-11 * np.abs(ref).max()
+    t.close()
+
+
+@pytest.mark.parametrize("periodic", [True, False])
+def test_source_positions_that_are_not_finite_are_refused(periodic):
+    _need_gpu()
+    rng = np.random.default_rng(10)
+    x = W.jittered_lattice(12, 0.2, rng)
+    for v in (np.nan, np.inf, -np.inf):
+        for axis in range(3):
+            xsrc = np.full((3, 2), 0.4)
+            xsrc[axis, 1] = v
+            with pytest.raises(RTError, match="RT_ERR_INVALID"):
+                Transport(x, None, xsrc, n_groups=1, precision="fp64", periodic=periodic)
