@@ -127,6 +127,7 @@ struct rt_ctx {
     bool inj_dense_ready = false;                       // filled by set_step_inputs for this call
     rt::DevBuf frec;                                    // packed float flux-input rows of a group chunk
     rt::DevBuf wave_t;                                  // HLL wave-speed table, working precision
+    signed char hll_smem[rt::kMaxGC + 1] = {};          // k_flux_hll's shared memory: 1 granted, -1 refused, 0 not asked
     // photo-ionisation sink per group (rt_set_absorbers): alpha in caller order [G][N]
     // (double), its sorted working-precision copy [N][G], the cross sections
     rt::DevBuf alpha_g_c, alpha_g_s, sigma_d;

@@ -1509,6 +1509,20 @@ static bool packed_rows(rt_ctx* c) {
     return true;
 }
 
+// whether k_flux_hll<GC>, which needs more shared memory than a launch gets unasked, may run on the
+// context's device.  The permission belongs to the function on one device: each context asks
+// for its own, once, and a refusal leaves k_flux_tma
+template <int GC>
+static bool hll_table_in_smem(rt_ctx* c) {
+    if (c->hll_smem[GC] == 0) {
+        const cudaError_t e = cudaFuncSetAttribute((const void*)k_flux_hll<GC>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, HllShape<GC>::smem);
+        if (e != cudaSuccess) (void)cudaGetLastError();
+        c->hll_smem[GC] = e == cudaSuccess ? 1 : -1;
+    }
+    return c->hll_smem[GC] > 0;
+}
+
 // float pass 1 and 2 in the variants chosen by the context's tuning
 template <int GC, bool HLL>
 static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, const FluxExtra<float>& x,
@@ -1521,9 +1535,6 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
         cudaFuncSetAttribute((const void*)k_flux_gather_g<float, GC>, cudaFuncAttributePreferredSharedMemoryCarveout, 0);
         cudaFuncSetAttribute((const void*)k_flux_tma<GC, HLL>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              cudaSharedmemCarveoutMaxShared);
-        if (HLL)
-            cudaFuncSetAttribute((const void*)k_flux_hll<GC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 HllShape<GC>::smem);
         (void)cudaGetLastError();
     }
     unsigned npb = nblk(std::max<int64_t>(a.n_pairs, 1), 128);
@@ -1536,7 +1547,7 @@ static void flux_float(rt_ctx* c, cudaStream_t s, const PairArgs<float>& a, cons
         const int pw = pair_warps(c);
         int* ef = c->flags.as<int>() + F_TIMEOUT;
         // HLL: with two batches a warp or more, the table in shared memory is worth loading
-        if (HLL && a.n_pairs >= (int64_t)c->sm_count * HllShape<GC>::warps * 64)
+        if (HLL && a.n_pairs >= (int64_t)c->sm_count * HllShape<GC>::warps * 64 && hll_table_in_smem<GC>(c))
             k_flux_hll<GC><<<c->sm_count, HllShape<GC>::warps * 32, HllShape<GC>::smem, s>>>(
                 a, x, pb, c->rows_map[GC], ef, budget);
         else
