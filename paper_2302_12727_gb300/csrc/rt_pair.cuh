@@ -109,15 +109,39 @@ __device__ __forceinline__ float sqrt_fast(float x, float& inv) {
     return x * inv;
 }
 
-// max(E, 0) and u = F2 / max(F2, cE^2), iq = 1 / max(F2, cE^2); both zero when that maximum
-// is not a normal number (|F| and cE below the square root of the smallest one: isotropic)
+// max(E, 0)
 __device__ __forceinline__ float pos_part(float v) { return fmaxf(v, 0.f); }
 __device__ __forceinline__ double pos_part(double v) { return __double2hiint(v) < 0 ? 0.0 : v; }
-__device__ __forceinline__ void m1_ratio(float F2, float cE, float& u, float& iq) {
-    iq = rcp_(fmaxf(fmaxf(F2, cE * cE), tiny_<float>()));
+
+// Whether some q = max(|F|^2, (cE)^2) that a pair's closures took was too large for 1/q to be a
+// normal number: |F| or cE of 2^63 (float), 2^511 (double) and more.  The flux kernels look
+// once a pair, after its fluxes are stored, and store_wide then takes it again with scaled
+// ratios: a compare a state is what ordinary units pay (2,097,152 particles of four groups: 0.9% of a
+// step, 2.2% with the look before the store; nothing measurable for one to three groups).
+template <class T>
+struct M1Top;
+template <>
+struct M1Top<float> {
+    bool any = false;
+    __device__ __forceinline__ void note(float q) { any |= q > 8.507059e37f; }                   // 2^126
+    static __device__ __forceinline__ float down() { return 8.2718061255302767e-25f; }           // 2^-80
+};
+template <>
+struct M1Top<double> {
+    bool any = false;
+    __device__ __forceinline__ void note(double q) { any |= __double2hiint(q) >= 0x7fd00000; }   // 2^1022
+    static __device__ __forceinline__ double down() { return 2.4099198651028841177e-181; }      // 2^-600
+};
+
+// q = max(F2, cE^2), iq = 1/q and u = F2/q; iq and u zero when q is not a normal number (|F| and cE
+// below the square root of the smallest one: isotropic)
+__device__ __forceinline__ float m1_ratio(float F2, float cE, float& u, float& iq) {
+    const float q = fmaxf(F2, cE * cE);
+    iq = rcp_(fmaxf(q, tiny_<float>()));
     u = fminf(F2 * iq, 1.f);
+    return q;
 }
-__device__ __forceinline__ void m1_ratio(double F2, double cE, double& u, double& iq) {
+__device__ __forceinline__ double m1_ratio(double F2, double cE, double& u, double& iq) {
     // non-negative doubles compare like integers: no instruction of the double pipe
     const double c2 = cE * cE;
     const double q = __double_as_longlong(F2) > __double_as_longlong(c2) ? F2 : c2;
@@ -125,6 +149,7 @@ __device__ __forceinline__ void m1_ratio(double F2, double cE, double& u, double
     const double r = rcp_fast(q);
     iq = ok ? r : 0.0;
     u = ok ? F2 * r : 0.0;
+    return q;
 }
 
 // M1 flux of one group contracted with A (Eq. eddington-group): F . A for the energy and
@@ -135,19 +160,31 @@ __device__ __forceinline__ void m1_ratio(double F2, double cE, double& u, double
 // (3 chi - 1)/2 = 2 - s = 3u/(2 + s) and (1 - chi)/2 = (1 - 3u/(2 + s))/3.  The clip is the
 // maximum in q = max(|F|^2, (cE)^2), u = |F|^2/q, and (3 chi - 1)/2 / |F|^2 = 3/((2 + s) q):
 // the direction F/|F| needs no root of its own, and three special functions a state remain
-// of five.  E <= 0 gives zero pressure.
-template <class T>
-__device__ __forceinline__ void m1_terms(T E, T Fx, T Fy, T Fz, T Ax, T Ay, T Az, T c, T& FA, T& P, T& t) {
+// of five.  E <= 0 gives zero pressure.  top notes q; WIDE takes the ratios of states beyond its
+// range from |F| and cE scaled down by a power of two, up to where F . A or c^2 E overflow.
+template <bool WIDE, class T>
+__device__ __forceinline__ void m1_terms(T E, T Fx, T Fy, T Fz, T Ax, T Ay, T Az, T c, T& FA, T& P, T& t,
+                                         M1Top<T>& top) {
     FA = Fx * Ax + Fy * Ay + Fz * Az;
     const T cE = pos_part(c * E);
     const T F2 = Fx * Fx + Fy * Fy + Fz * Fz;
-    T u, iq;
-    m1_ratio(F2, cE, u, iq);
+    T u, iq, d = T(1);
+    const T q = m1_ratio(F2, cE, u, iq);
+    top.note(q);
+    if constexpr (WIDE) {
+        M1Top<T> here;
+        here.note(q);
+        if (here.any) {
+            d = M1Top<T>::down();
+            const T x = Fx * d, y = Fy * d, z = Fz * d;
+            m1_ratio(x * x + y * y + z * z, cE * d, u, iq);
+        }
+    }
     const T s = sqrt_fast(fma_rn(T(-3), u, T(4)));
     const T r = T(3) * rcp_fast(T(2) + s);
     const T cc = c * cE;
     P = cc * fma_rn(-u * r, T(1.0 / 3.0), T(1.0 / 3.0));
-    t = (cc * (iq * r)) * FA;
+    t = WIDE ? ((cc * d) * (iq * r)) * (FA * d) : (cc * (iq * r)) * FA;
 }
 
 // ------------------------------------------------------------------------------------
@@ -440,9 +477,9 @@ __device__ __forceinline__ void load_pair_geo(const PairArgs<T>& a, int64_t slot
 // (Q_l - Q_k) - s, because the two weights of s add to one: it keeps the digits that the
 // rounded face states lose.  The surface enters halved, so that the central term is a plain
 // sum.
-template <bool HLL, class T>
+template <bool HLL, bool WIDE, class T>
 __device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T gk[12], const T gl[12],
-                                          const PairGeo<T>& p, T c, const T* wave, T phi[4]) {
+                                          const PairGeo<T>& p, T c, const T* wave, T phi[4], M1Top<T>& top) {
     T L[4], R[4], D[4];
     const T wl = T(1) - p.wk;
 #pragma unroll
@@ -458,8 +495,8 @@ __device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T 
     if constexpr (HLL) {
         const T Ax = T(2) * p.hx, Ay = T(2) * p.hy, Az = T(2) * p.hz;
         T fL[4], fR[4];
-        m1_terms(L[0], L[1], L[2], L[3], Ax, Ay, Az, c, fL[0], PL, tL);
-        m1_terms(R[0], R[1], R[2], R[3], Ax, Ay, Az, c, fR[0], PR, tR);
+        m1_terms<WIDE>(L[0], L[1], L[2], L[3], Ax, Ay, Az, c, fL[0], PL, tL, top);
+        m1_terms<WIDE>(R[0], R[1], R[2], R[3], Ax, Ay, Az, c, fR[0], PR, tR, top);
         fL[1] = PL * Ax + tL * L[1];
         fL[2] = PL * Ay + tL * L[2];
         fL[3] = PL * Az + tL * L[3];
@@ -484,8 +521,8 @@ __device__ __forceinline__ void pair_flux(const T uk[4], const T ul[4], const T 
         }
         return;
     }
-    m1_terms(L[0], L[1], L[2], L[3], p.hx, p.hy, p.hz, c, FL, PL, tL);
-    m1_terms(R[0], R[1], R[2], R[3], p.hx, p.hy, p.hz, c, FR, PR, tR);
+    m1_terms<WIDE>(L[0], L[1], L[2], L[3], p.hx, p.hy, p.hz, c, FL, PL, tL, top);
+    m1_terms<WIDE>(R[0], R[1], R[2], R[3], p.hx, p.hy, p.hz, c, FR, PR, tR, top);
     const T P = PL + PR;
     phi[0] = fma_rn(-p.diss, D[0], FL + FR);
     phi[1] = fma_rn(-p.diss, D[1], P * p.hx + (tL * L[1] + tR * R[1]));

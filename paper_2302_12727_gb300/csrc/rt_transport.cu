@@ -621,6 +621,26 @@ __global__ void __launch_bounds__(kGradBlockMax, GC == 4 ? 1280 / kGradBlockMax 
 // ------------------------------------------------------------------------------------
 // a7 + a8: pair fluxes, explicit update, grey sink, optional fix-up, groups [g0, g0 + GC).
 
+// The fluxes of a pair with a state beyond the closure's range (M1Top) again, over its slot: the groups'
+// states lie at uk, ul, their gradients at gk, gl, side by side
+template <bool HLL, int GC, class T>
+__device__ __forceinline__ void store_wide(const T* uk, const T* ul, const T* gk, const T* gl, const PairGeo<T>& pr, T c,
+                                           const T* wave, T wgt, T* to) {
+    M1Top<T> top;
+#pragma unroll 1
+    for (int g = 0; g < GC; ++g) {
+        T ui[4], uj[4], gri[12], grj[12], phi[4];
+        vload<4>(uk + 4 * g, ui);
+        vload<4>(ul + 4 * g, uj);
+        vload<12>(gk + 12 * g, gri);
+        vload<12>(gl + 12 * g, grj);
+        pair_flux<HLL, true>(ui, uj, gri, grj, pr, c, wave, phi, top);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) phi[q] *= wgt;
+        vstore<4>(to + 4 * g, phi);
+    }
+}
+
 // Pass 1 of the flux: one thread per unordered pair (k, l), k < l, evaluates Phi_kl once with
 // k as the left state and stores it in the pair's slot.
 template <class T, int GC, bool HLL, bool BINS = false>
@@ -647,6 +667,7 @@ __global__ void __launch_bounds__(128) k_flux(PairArgs<T> a, FluxExtra<T> x, con
     const T* qi = a.grad + i * 12 * G;
     const T* qj = a.grad + j * 12 * G;
     T out[NC];
+    M1Top<T> top;
 #pragma unroll
     for (int g = 0; g < GC; ++g) {
         const int gg = g0 + g;
@@ -655,13 +676,16 @@ __global__ void __launch_bounds__(128) k_flux(PairArgs<T> a, FluxExtra<T> x, con
         vload<4>(rj + 4 * gg, uj);
         vload<12>(qi + 12 * gg, gri);
         vload<12>(qj + 12 * gg, grj);
-        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
+        pair_flux<HLL, false>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g], top);
     }
     if constexpr (BINS) {
 #pragma unroll
         for (int c = 0; c < NC; ++c) out[c] *= wgt;
     }
     vstore<NC>(pairbuf + slot * NC, out);
+    if (top.any)
+        store_wide<HLL, GC>(ri + 4 * g0, rj + 4 * g0, qi + 12 * g0, qj + 12 * g0, pr, x.c, x.wave, wgt,
+                            pairbuf + slot * NC);
 }
 
 // ------------------------------------------------------------------------------------
@@ -984,6 +1008,7 @@ __global__ void __launch_bounds__(128) k_flux_staged(PairArgs<float> a, FluxExtr
     const float* ri = rec + i * RS;
     const float* qi = a.grad + i * 12 * G;
     float out[NC];
+    M1Top<float> top;
 #pragma unroll
     for (int g = 0; g < GC; ++g) {
         const int gg = g0 + g;
@@ -992,9 +1017,12 @@ __global__ void __launch_bounds__(128) k_flux_staged(PairArgs<float> a, FluxExtr
         vload<4>(mine + 12 + 4 * g, uj);
         vload<12>(qi + 12 * gg, gri);
         vload<12>(mine + 12 + 4 * GC + 12 * g, grj);
-        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
+        pair_flux<HLL, false>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g], top);
     }
     if (act) vstore<NC>(pairbuf + slot * NC, out);
+    if (act && top.any)
+        store_wide<HLL, GC>(ri + 4 * g0, rec + kl.y * (int64_t)RS + 4 * g0, qi + 12 * g0,
+                            a.grad + kl.y * (int64_t)(12 * G) + 12 * g0, pr, x.c, x.wave, 1.f, pairbuf + slot * NC);
 }
 
 // Float pass 1 with the neighbour rows fetched by the tensor memory accelerator.  The
@@ -1094,6 +1122,7 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
     float sk, sl;
     pair_geo(dx, dy, dz, gi8, gj8, x.c, pr, sk, sl);
     float out[NC];
+    M1Top<float> top;
 #pragma unroll
     for (int g = 0; g < G; ++g) {
         float ui[4], uj[4], gri[12], grj[12];
@@ -1103,14 +1132,19 @@ __global__ void __launch_bounds__(kTmaWarpsMax * 32, TmaMinBlocks<G>::value) k_f
         vload<4>(lrow(3 + G + 3 * g), grj);
         vload<4>(lrow(4 + G + 3 * g), grj + 4);
         vload<4>(lrow(5 + G + 3 * g), grj + 8);
-        pair_flux<HLL>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g]);
+        pair_flux<HLL, false>(ui, uj, gri, grj, pr, x.c, x.wave, &out[4 * g], top);
     }
+    float wgt = 1.f;
     if constexpr (BINS) {
-        const float wgt = (float)(1 << min(a.bins[kl.x], a.bins[kl.y]));   // min(dt_k, dt_l) / dt_min
+        wgt = (float)(1 << min(a.bins[kl.x], a.bins[kl.y]));   // min(dt_k, dt_l) / dt_min
 #pragma unroll
         for (int c = 0; c < NC; ++c) out[c] *= wgt;
     }
     if (act) vstore<NC>(pairbuf + slot * NC, out);
+    if (act && top.any) {
+        const float* rg = packed_row(a, (int64_t)kl.y);
+        store_wide<HLL, G>(rk + 12, rg + 12, rk + 12 + 4 * G, rg + 12 + 4 * G, pr, x.c, x.wave, wgt, pairbuf + slot * NC);
+    }
 }
 
 // The same pair pass for the HLL solver, with the wave-speed table (81,608 bytes) in shared memory: one
@@ -1194,6 +1228,7 @@ k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
         float sk, sl;
         pair_geo(dx, dy, dz, gi8, gj8, x.c, pr, sk, sl);
         float out[NC];
+        M1Top<float> top;
 #pragma unroll
         for (int g = 0; g < G; ++g) {
             float ui[4], uj[4], gri[12], grj[12];
@@ -1203,9 +1238,14 @@ k_flux_hll(PairArgs<float> a, FluxExtra<float> x, float* __restrict__ pairbuf,
             vload<4>(lrow(3 + G + 3 * g), grj);
             vload<4>(lrow(4 + G + 3 * g), grj + 4);
             vload<4>(lrow(5 + G + 3 * g), grj + 8);
-            pair_flux<true>(ui, uj, gri, grj, pr, x.c, reinterpret_cast<const float*>(tab), &out[4 * g]);
+            pair_flux<true, false>(ui, uj, gri, grj, pr, x.c, reinterpret_cast<const float*>(tab), &out[4 * g], top);
         }
         if (slot < np) vstore<NC>(pairbuf + slot * NC, out);
+        if (slot < np && top.any) {
+            const float* rg = packed_row(a, (int64_t)kl.y);
+            store_wide<true, G>(rk + 12, rg + 12, rk + 12 + 4 * G, rg + 12 + 4 * G, pr, x.c, x.wave, 1.f,
+                                pairbuf + slot * NC);
+        }
         kl = kl_next;
         __syncwarp();      // every lane has read its row before the next copies overwrite it
     }

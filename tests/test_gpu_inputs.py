@@ -103,3 +103,56 @@ def test_source_positions_that_are_not_finite_are_refused(periodic):
             xsrc[axis, 1] = v
             with pytest.raises(RTError, match="RT_ERR_INVALID"):
                 Transport(x, None, xsrc, n_groups=1, precision="fp64", periodic=periodic)
+
+
+def _beamed(G, n, rng):
+    """States from isotropic to beyond the closure's clip, |F| up to 1.2 c E (c = 1), E in [1/2, 1]."""
+    U = np.zeros((G, 4, n))
+    U[:, 0] = rng.uniform(0.5, 1.0, (G, n))
+    d = W.random_unit_vectors(G * n, rng).reshape(3, G, n).transpose(1, 0, 2)
+    U[:, 1:] = rng.uniform(0, 1.2, (G, 1, n)) * U[:, :1] * d
+    return U.astype(np.float32).astype(np.float64)
+
+
+# the squares of 2^63 reach the top of the float range; the HLL wave speeds square F x A, and so reach
+# neither as far down (F A of 2^-63) nor beyond |F| = 2^64
+@pytest.mark.parametrize("riemann,powers", [("glf", (-50, 62, 63, 64, 100)), ("hll", (62, 63))])
+@pytest.mark.parametrize("variant", [(0, 0, 0), (1, 1, 1), (2, 1, 2)])
+@pytest.mark.parametrize("side,G", [(8, 2), (24, 3)])
+def test_float_step_scales_over_the_exponent_range(side, G, variant, riemann, powers):
+    """The step is homogeneous of degree one, and a power of two is exact: a scaled state gives the scaled
+    result to a few roundings, in the plain step and with time bins."""
+    _need_gpu()
+    rng = np.random.default_rng(side)
+    x = W.jittered_lattice(side, 0.2, rng)
+    n = x.shape[1]
+    U0 = _beamed(G, n, rng)
+    t = Transport(x, None, None, n_groups=G, precision="fp32", riemann=riemann)
+    t.set_tuning(*variant)
+    dt = 0.2 * t.diagnostics()["dx_min"]
+    t.set_time_bins(rng.integers(0, 3, n).astype(np.int32), dt_min=dt)
+    base = None
+    for k in (0,) + powers:
+        a, b = t.state(np.ldexp(U0, k)), t.state(np.ldexp(U0, k))
+        t.step(a, dt)
+        t.step_bins(b)
+        out = [np.ldexp(v.cpu().numpy().astype(np.float64), -k) for v in (a, b)]
+        base = base or out
+        for v, w in zip(out, base):
+            assert np.abs(v - w).max() <= 1e-6 * np.abs(w).max(), k
+    t.close()
+
+
+@pytest.mark.parametrize("power", [505, 512, 700])
+def test_double_step_scales_beyond_the_squares_of_the_states(power):
+    _need_gpu()
+    rng = np.random.default_rng(7)
+    x = W.jittered_lattice(8, 0.2, rng)
+    U0 = _beamed(2, x.shape[1], rng)
+    t = Transport(x, None, None, n_groups=2, precision="fp64")
+    a, b = t.state(U0), t.state(np.ldexp(U0, power))
+    t.step(a, 0.01)
+    t.step(b, 0.01)
+    a, b = a.cpu().numpy(), np.ldexp(b.cpu().numpy(), -power)
+    assert np.abs(a - b).max() <= 1e-14 * np.abs(a).max()
+    t.close()
