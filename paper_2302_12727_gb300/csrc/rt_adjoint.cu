@@ -28,7 +28,9 @@ static inline unsigned nblk_(int64_t n, int b) { return (unsigned)((n + b - 1) /
 // Pi = c e (a A + g (f.A) f), a = (s - 1)/3, and a' = -1/(2s), g' = g^2/(2s), so
 //   d(p.Pi)/de = c [(a + u/s) p.A - (g + u g^2/s) (f.A)(p.f)]
 //   d(p.Pi)/dF = c [(g^2 (f.A)(p.f) - p.A)/s f + g ((p.f) A + (f.A) p)];
-// where |f| > 1 is clipped, Pi = c e (f.A) f / u.  f keeps every term scale-free.
+// where |f| > 1 is clipped, Pi = c e (f.A) f / u.  f keeps every term scale-free; a clipped state
+// with u beyond the range (E far below |F|, as at a front) takes F itself for f: Pi does not
+// change, and d(p.Pi)/dF is e times what f gives.
 template <class T>
 __device__ __forceinline__ void m1_vjp(const T u4[4], T Ax, T Ay, T Az, T c, const T pb[4], T ub[4]) {
     ub[0] = T(0);
@@ -38,15 +40,25 @@ __device__ __forceinline__ void m1_vjp(const T u4[4], T Ax, T Ay, T Az, T c, con
     const T e = c * u4[0];
     if (!(e > tiny_<T>())) return;
     const T ie = rcp_fast(e);
-    const T fx = u4[1] * ie, fy = u4[2] * ie, fz = u4[3] * ie;
-    const T fA = fx * Ax + fy * Ay + fz * Az;
+    T fx = u4[1] * ie, fy = u4[2] * ie, fz = u4[3] * ie;
+    T fA = fx * Ax + fy * Ay + fz * Az;
     const T pA = pb[1] * Ax + pb[2] * Ay + pb[3] * Az;
-    const T pf = pb[1] * fx + pb[2] * fy + pb[3] * fz;
-    const T u = fx * fx + fy * fy + fz * fz;
+    T pf = pb[1] * fx + pb[2] * fy + pb[3] * fz;
+    T u = fx * fx + fy * fy + fz * fz;
     T ce, cf, cg;   // d/de, and the coefficients of f and of (p.f) A + (f.A) p
     if (u > T(1)) {
+        const bool far = !(u <= T(1) / tiny_<T>());     // 1/u below the normal numbers, or u infinite
+        if (far) {
+            fx = u4[1];
+            fy = u4[2];
+            fz = u4[3];
+            fA = fx * Ax + fy * Ay + fz * Az;
+            pf = pb[1] * fx + pb[2] * fy + pb[3] * fz;
+            u = fx * fx + fy * fy + fz * fz;
+        }
         cg = rcp_fast(u);
         ce = cg * fA * pf;
+        if (far) cg *= e;
         cf = T(-2) * cg * ce;
     } else {
         T is;

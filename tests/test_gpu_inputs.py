@@ -156,3 +156,26 @@ def test_double_step_scales_beyond_the_squares_of_the_states(power):
     a, b = a.cpu().numpy(), np.ldexp(b.cpu().numpy(), -power)
     assert np.abs(a - b).max() <= 1e-14 * np.abs(a).max()
     t.close()
+
+
+@pytest.mark.parametrize("precision,near,far,tol", [("fp64", -300, -560, 1e-12), ("fp32", -40, -70, 1e-5)])
+def test_adjoint_of_states_with_little_energy(precision, near, far, tol):
+    """|F| >> c E: the clipped closure is linear in E along F, so the gradient is the same for E of 2^near
+    and of 2^far, up to terms of E / |F| (below the tolerance, a few roundings of sums of ~50 terms)."""
+    _need_gpu()
+    rng = np.random.default_rng(4)
+    x = W.jittered_lattice(8, 0.2, rng)
+    n = x.shape[1]
+    U0 = _beamed(2, n, rng)
+    U0[:, 1:] = W.random_unit_vectors(2 * n, rng).reshape(3, 2, n).transpose(1, 0, 2)
+    lam = rng.normal(size=U0.shape)
+    t = Transport(x, None, None, n_groups=2, precision=precision)
+    out = []
+    for k in (near, far):
+        U = U0.copy()
+        U[:, 0] = np.ldexp(U[:, 0], k)
+        dU0, _ = t.adjoint(t.state(U), 1, 0.01, t.state(lam), None, None, 1)
+        out.append(dU0.double().cpu().numpy())
+    t.close()
+    assert np.isfinite(out[1]).all()
+    assert np.abs(out[0] - out[1]).max() <= tol * np.abs(out[0]).max()
