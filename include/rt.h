@@ -28,7 +28,13 @@
  *      alpha [N]           grey absorption coefficient (double), or NULL for none
  *  - The library owns its workspaces, its cell-sorted copies and the permutation.  Memory is
  *    allocated only in rt_create, rt_neighbours and on the first call of rt_adjoint with a
- *    larger checkpoint count; rt_transport_step and rt_subcycle allocate nothing.
+ *    larger checkpoint count; rt_transport_step and rt_subcycle allocate nothing.  The FP64 path
+ *    keeps the geometry of the pairs (128 bytes each) where that takes at most a quarter of the
+ *    free device memory at rt_neighbours, and rt_adjoint per-pair values where they take at most
+ *    half of it; both stay until rt_destroy unless another allocation of the context needs
+ *    the room.  Without them the same quantities are computed in each kernel: the results then
+ *    differ by rounding, and so FP64 results may in their last bits between an empty and a
+ *    nearly full device.
  *  - All work is asynchronous on the stream given to rt_create, except where a function
  *    says it synchronises.  Nothing aborts or prints: every call returns an rt_status and
  *    rt_last_error() gives a message for the last failure.

@@ -548,8 +548,12 @@ rt_status run_adjoint(rt_ctx* c, int n_sub, int k, bool has_src, bool has_alpha,
         free_buf(c->adj_sel);
         RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
         if (pg * (12 * ts + 1) <= free_b / 2) {
-            RT_TRY(ensure(c, c->adj_slots, pg * 12 * ts, "adjoint slots"));
-            RT_TRY(ensure(c, c->adj_sel, pg, "adjoint slots"));
+            if (ensure(c, c->adj_slots, pg * 12 * ts, "adjoint slots") != RT_OK ||
+                ensure(c, c->adj_sel, pg, "adjoint slots") != RT_OK) {
+                c->err.clear();          // the stages without slots run
+                free_buf(c->adj_slots);
+                free_buf(c->adj_sel);
+            }
         }
     }
     char* ck = c->ck.as<char>();

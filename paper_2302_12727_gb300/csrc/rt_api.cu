@@ -20,6 +20,32 @@ rt_status cuda_fail(rt_ctx* c, cudaError_t e, const char* what) {
     return e == cudaErrorMemoryAllocation ? RT_ERR_OOM : RT_ERR_CUDA;
 }
 
+static void drop_graphs(rt_ctx* c);
+
+// Gives back what the context runs without, when an allocation has failed: the adjoint's slots, the
+// double path's kept pair geometry (with the graphs that hold its address) and, outside the search,
+// the search's lists.  False when there is none.
+static bool give_back(rt_ctx* c) {
+    size_t had = 0;
+    auto drop = [&](DevBuf& b) {
+        had += b.bytes;
+        free_buf(b);
+    };
+    drop(c->adj_slots);
+    drop(c->adj_sel);
+    if (c->pair_geo.bytes + c->pair_w.bytes + c->row_wd.bytes > 0) {
+        cudaStreamSynchronize(c->stream);
+        drop_graphs(c);
+        drop(c->pair_geo);
+        drop(c->pair_w);
+        drop(c->row_wd);
+        c->pair_geo_ready = false;
+    }
+    if (!c->searching)
+        for (DevBuf* b : {&c->lists, &c->extras, &c->more, &c->spill, &c->src_list}) drop(*b);
+    return had > 0;
+}
+
 rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what, bool slack) {
     if (bytes == 0) bytes = 16;
     if (b.bytes >= bytes) return RT_OK;
@@ -34,6 +60,10 @@ rt_status ensure(rt_ctx* c, DevBuf& b, size_t bytes, const char* what, bool slac
     if (e != cudaSuccess && bytes > least) {     // no room for the slack
         (void)cudaGetLastError();
         bytes = least;
+        e = cudaMalloc(&b.p, bytes);
+    }
+    if (e != cudaSuccess && give_back(c)) {
+        (void)cudaGetLastError();
         e = cudaMalloc(&b.p, bytes);
     }
     if (e != cudaSuccess) {
@@ -134,15 +164,16 @@ static rt_status ensure_state(rt_ctx* c) {
         size_t free_b = 0, total_b = 0;
         const bool fits = P * 64 <= c->pair_geo.bytes && P * 16 <= c->pair_w.bytes && P * 48 <= c->row_wd.bytes;
         if (!fits) RT_CUDA(c, cudaMemGetInfo(&free_b, &total_b));
-        if (fits || need <= (free_b + have) / 4) {
-            RT_TRY(ensure(c, c->pair_geo, P * 64, "pair geometry", true));
-            RT_TRY(ensure(c, c->pair_w, P * 16, "pair geometry", true));
-            RT_TRY(ensure(c, c->row_wd, P * 48, "pair geometry", true));
-        } else {
+        const bool keep = (fits || need <= (free_b + have) / 4) &&
+                          ensure(c, c->pair_geo, P * 64, "pair geometry", true) == RT_OK &&
+                          ensure(c, c->pair_w, P * 16, "pair geometry", true) == RT_OK &&
+                          ensure(c, c->row_wd, P * 48, "pair geometry", true) == RT_OK;
+        if (!keep || !c->pair_geo.p || !c->pair_w.p) {     // a failed one may have given the others back
+            c->err.clear();
+            if (c->pair_geo.p || c->pair_w.p || c->row_wd.p) ++c->generation;
             free_buf(c->pair_geo);
             free_buf(c->pair_w);
             free_buf(c->row_wd);
-            ++c->generation;
         }
     }
     if (!c->fp64) RT_TRY(ensure(c, c->frec, (size_t)(12 + 16 * gc + kRowRot) * n * 4, "packed flux rows"));
@@ -235,7 +266,9 @@ static rt_status neighbours(rt_ctx* c, const double* x, const double* m, const d
     c->built = false;
     c->has_bins = false;   // bins live in the sorted order and depend on the pair lists
     const int64_t gen0 = c->generation;
+    c->searching = true;
     rt_status s = build_neighbours(c, x, m, xsrc, h_in, hs_in, oms_in, octw_in);
+    c->searching = false;
     if (s != RT_OK) {
         drop_graphs(c);
         return s;

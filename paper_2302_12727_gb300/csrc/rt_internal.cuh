@@ -105,6 +105,7 @@ struct rt_ctx {
     // transport call after a build (empty when device memory is short)
     rt::DevBuf pair_geo, pair_w, row_wd;
     bool pair_geo_ready = false;
+    bool searching = false;                             // in build_neighbours, which needs its lists
     rt::DevBuf adj_slots, adj_sel;                      // adjoint: per-pair values of one group chunk
     // captured graphs hold buffer addresses and launch grids: they are dropped when a buffer moves
     // (generation) or a rebuild has more pairs or targets than their grids cover

@@ -179,3 +179,35 @@ def test_adjoint_of_states_with_little_energy(precision, near, far, tol):
     t.close()
     assert np.isfinite(out[1]).all()
     assert np.abs(out[0] - out[1]).max() <= tol * np.abs(out[0]).max()
+
+
+def test_adjoint_slots_make_room_for_more_checkpoints():
+    """A second adjoint with more checkpoints, on a device with little memory left: the context's optional
+    buffers (the slots and pair geometry, about 500 MB here) go, and the result stays, to rounding."""
+    _need_gpu()
+    rng = np.random.default_rng(6)
+    x = W.jittered_lattice(40, 0.2, rng)
+    n = x.shape[1]
+    U0, lam = _beamed(2, n, rng), rng.normal(size=(2, 4, n))
+    n_sub = 160                                   # checkpoints of 4.1 MB each: 656 MB
+    t = Transport(x, None, None, n_groups=2, precision="fp64")
+    U, w = t.state(U0), t.state(lam)
+    t.adjoint(U, 2, 1e-4, w, None, None, 1)
+    sub = t.state(U0)
+    t.subcycle(sub, 4, 1e-3)
+    free = torch.cuda.mem_get_info()[0]
+    hold = torch.empty(max(free - (250 << 20), 1), dtype=torch.uint8, device="cuda")
+    try:
+        lean = t.adjoint(U, n_sub, 1e-4, w, None, None, 1)[0].cpu().numpy()
+        again = t.state(U0)
+        t.subcycle(again, 4, 1e-3)                # the captured graph held the geometry's address
+        again = again.cpu().numpy()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    t.rebuild(x)
+    full = t.adjoint(U, n_sub, 1e-4, w, None, None, 1)[0].cpu().numpy()
+    t.close()
+    # the two evaluation orders differ by a few roundings a step
+    assert np.abs(lean - full).max() <= n_sub * 1e-14 * np.abs(full).max()
+    assert np.abs(again - sub.cpu().numpy()).max() <= 1e-13 * np.abs(again).max()
