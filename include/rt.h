@@ -115,8 +115,9 @@ typedef struct {
     double dx_min;            /* min_i (V_i / (4 pi / 3))^(1/3), the cell size of Eq. rt-cfl */
     int64_t clamp_events;     /* cumulative count of E < 0 fix-ups */
     int32_t grid[3];          /* cell-list dimensions used by rt_neighbours */
-    int32_t threads_per_particle;  /* threads per particle of the float gradient kernel (G,
-                                      at most 4, in gradient_variants 1 and 2; else 1) */
+    int32_t threads_per_particle;  /* threads per particle of the float gradient kernel (in
+                                      gradient_variants 1 and 2 the groups of one of its
+                                      launches, G / ceil(G / 4) rounded up; else 1) */
     int64_t kernel_launches;  /* cumulative launches of the library's own kernels (graph
                                  replays count every kernel node; library sorts and scans
                                  that the build calls are not counted) */
@@ -126,8 +127,7 @@ typedef struct {
     int32_t wait_timeouts;    /* 1 if a device-side wait ran out since the last rt_neighbours */
     int64_t h_refined;        /* particles whose h the last rt_neighbours refined in double: all of
                                  them on the FP64 path; on the float path those with a neighbour
-                                 candidate within 1e-5 of their support radius at the float root, or
-                                 whose float iteration did not settle as closely as that needs */
+                                 candidate within 1e-4 of their support radius at the float root */
 } rt_diag;
 
 /* Launch variants of the float (RT_FP32_MIXED) pair kernels.  The paper has no counterpart:

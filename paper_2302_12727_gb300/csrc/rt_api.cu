@@ -620,8 +620,8 @@ rt_status rt_diagnostics(rt_ctx* c, rt_diag* out) {
     }
     c->diag.clamp_events = (int64_t)cl;
     c->diag.wait_timeouts = timed_out;
-    // the float gradient runs one thread per (particle, group) in variants 1 and 2
-    const int gc = c->cfg.n_groups < kMaxGC ? c->cfg.n_groups : kMaxGC;
+    // the float gradient runs one thread per (particle, group of a chunk) in variants 1 and 2
+    const int gc = chunk_groups(c->cfg.n_groups);
     c->diag.threads_per_particle = (!c->fp64 && c->tune.gradient_variant >= 1) ? gc : 1;
     c->diag.kernel_launches = c->launches;
     *out = c->diag;

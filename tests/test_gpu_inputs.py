@@ -211,3 +211,13 @@ def test_adjoint_slots_make_room_for_more_checkpoints():
     # the two evaluation orders differ by a few roundings a step
     assert np.abs(lean - full).max() <= n_sub * 1e-14 * np.abs(full).max()
     assert np.abs(again - sub.cpu().numpy()).max() <= 1e-13 * np.abs(again).max()
+
+
+@pytest.mark.parametrize("G,threads", [(1, 1), (3, 3), (4, 4), (5, 3), (7, 4), (9, 3)])
+def test_threads_per_particle_are_those_of_the_launch(G, threads):
+    """Groups run in even chunks of at most four: 5 as 3 + 2, 7 as 4 + 3, 9 as 3 + 3 + 3."""
+    _need_gpu()
+    x = W.jittered_lattice(8, 0.2, np.random.default_rng(1))
+    t = Transport(x, None, None, n_groups=G, precision="fp32")
+    assert t.diagnostics()["threads_per_particle"] == threads
+    t.close()
