@@ -17,6 +17,11 @@
 namespace rt {
 
 
+struct Box {
+    double box[3];
+    int periodic;
+};
+
 struct Grid {
     int nc[3];
     double cell[3];
@@ -192,15 +197,26 @@ __device__ __forceinline__ double sep_fast(double xj, double xi, double box, dou
 
 // ------------------------------------------------------------------------------------
 // a1: cell keys, validation
+// A coordinate that is not finite or not in the box is refused, but the host learns of it only after
+// the search has been queued.  Until then a value spread over the box by the particle's index
+// stands in for it, in the keys and in the sorted copies, so that every walk stays in the cell
+// table and meets no more candidates than an even set has.
+__device__ __forceinline__ double position_in_box(double v, double box, int64_t i, int axis, bool& bad) {
+    if (v >= 0.0 && v < box) return v;
+    bad = true;
+    uint32_t u = (uint32_t)i * 0x9e3779b9u + (uint32_t)axis * 0x85ebca6bu;   // a multiplicative hash
+    u = (u ^ (u >> 16)) * 0x7feb352du;
+    u = (u ^ (u >> 15)) * 0x846ca68bu;
+    return box * ((double)(u ^ (u >> 16)) * 0x1p-32);
+}
+
 __global__ void k_keys(const double* __restrict__ x, int64_t n, Grid g, uint32_t* keys, int32_t* idx, int* flags) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= n) return;
     int c[3];
     bool bad = false;
     for (int a = 0; a < 3; ++a) {
-        double v = x[a * n + i];
-        if (!(v >= 0.0 && v < g.box[a])) bad = true;
-        c[a] = bad ? 0 : cell_coord(v, g.inv_cell[a], g.nc[a]);
+        c[a] = cell_coord(position_in_box(x[a * n + i], g.box[a], i, a, bad), g.inv_cell[a], g.nc[a]);
     }
     if (bad) atomicExch(&flags[F_BADPOS], 1);
     keys[i] = (uint32_t)(((int64_t)c[2] * g.nc[1] + c[1]) * g.nc[0] + c[0]);
@@ -219,7 +235,7 @@ __global__ void k_cell_start(const uint32_t* __restrict__ keys, int64_t n, int64
 }
 
 __global__ void k_gather_positions(const double* __restrict__ x, const double* __restrict__ m,
-                                   const int32_t* __restrict__ perm, int64_t n, double q0, double q1, double q2,
+                                   const int32_t* __restrict__ perm, int64_t n, Box b, double q0, double q1, double q2,
                                    double* xs, uint4* xq, double* ms, int32_t* inv_perm) {
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (p >= n) return;
@@ -227,7 +243,8 @@ __global__ void k_gather_positions(const double* __restrict__ x, const double* _
     double qs[3] = {q0, q1, q2};
     uint32_t qv[3];
     for (int a = 0; a < 3; ++a) {
-        double v = x[a * n + i];
+        bool bad = false;
+        const double v = position_in_box(x[a * n + i], b.box[a], i, a, bad);
         xs[a * n + p] = v;
         double f = floor(v * qs[a]);
         f = fmin(fmax(f, 0.0), 4294967295.0);
@@ -246,8 +263,8 @@ __global__ void k_gather_positions(const double* __restrict__ x, const double* _
 // walk by returning false (the same in every lane).  A thread that walks its own sphere runs
 // row by row on the latency of the table and record loads, half of a warp's lanes idle (14.8
 // active of 32) behind the longest row; a warp per particle that takes the rows in turn repeats the row
-// arithmetic in every lane.  Periodic cells wrap once, so (px, py, pz) has to lie in the box (its
-// upper edge included): no kernel walks once F_BADPOS is set (bad_positions).
+// arithmetic in every lane.  Periodic cells wrap once, so (px, py, pz) has to lie in the box, its
+// upper edge included (position_in_box, k_src_positions).
 __device__ __forceinline__ int wrap_once(int c, int nc) { return c < 0 ? c + nc : (c >= nc ? c - nc : c); }
 
 // ASC false: the order of for_each_candidate_range<false>, which differs where a sphere wraps.
@@ -339,11 +356,6 @@ __device__ __forceinline__ void warp_walk(const Grid& g, float px, float py, flo
         }
     }
 }
-
-// A position that is not finite or not in the box (k_keys): the call fails at its first
-// synchronisation, and the kernels queued before it that walk the cells, or follow lists that only
-// those make, do nothing
-__device__ __forceinline__ bool bad_positions(const int* flags) { return flags[F_BADPOS] != 0; }
 
 // whether the two orders of that walk may differ
 __device__ __forceinline__ bool walk_wraps(const Grid& g, float px, float py, float pz, float R) {
@@ -491,7 +503,6 @@ k_h_lists(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, i
     constexpr int PW = 32 / kSumLanes;            // particles a warp
     const unsigned FULL = 0xffffffffu;
     extern __shared__ float st_all[];             // distances of the stored candidates, cap a particle
-    if (bad_positions(flags)) return;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int a = lane / kSumLanes, sub = lane % kSumLanes;
     const int64_t p0 = (blockIdx.x * (int64_t)kListWarps + wid) * PW, p = p0 + a;
@@ -828,7 +839,6 @@ k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, 
            const int32_t* __restrict__ todo, const int* __restrict__ count, const int32_t* __restrict__ list,
            const int32_t* __restrict__ list_cnt, int cap, double* h_out, double* omega_out, float* H2f_out,
            uint4* xq_out, unsigned long long* hminmax, int* flags, int32_t* rest, int* rest_n) {
-    if (bad_positions(flags)) return;
     const int lane = threadIdx.x & (LN - 1);
     const unsigned group = LN == 32 ? 0xffffffffu : ((1u << (LN & 31)) - 1u) << (threadIdx.x & 31 & ~(LN - 1));
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / LN;
@@ -942,7 +952,6 @@ k_h_refine_walk(Grid g, const double* __restrict__ xs, const uint4* __restrict__
 __global__ void k_h_given(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n,
                           HParams hp, const double* __restrict__ h_in, const int32_t* __restrict__ perm,
                           double* h_out, double* omega_out, float* H2f_out, unsigned long long* hminmax, int* flags) {
-    if (bad_positions(flags)) return;
     const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const bool active = p < n;
     double hd = 0.0;
@@ -1067,13 +1076,13 @@ __device__ __forceinline__ void hand_extra(int32_t* extra, int32_t* extras, int6
 __global__ void __launch_bounds__(256, 5)
 k_own_rows(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, const double* __restrict__ h,
            int64_t n, PairParams pp, int32_t* list, int cap, const int32_t* __restrict__ list_cnt,
-           int32_t* __restrict__ own, int32_t* extra, int32_t* __restrict__ extras, int32_t* over, int* flags) {
+           int32_t* __restrict__ own, int32_t* extra, int32_t* __restrict__ extras, int32_t* over, int* over_n) {
     const int64_t p = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
-    if (p >= n || bad_positions(flags)) return;
+    if (p >= n) return;
     const int had = list_cnt[p];
     if (had < 0) {
-        if (lane == 0) over[atomicAdd(flags + F_OVER, 1)] = (int32_t)p;
+        if (lane == 0) over[atomicAdd(over_n, 1)] = (int32_t)p;
         return;
     }
     const uint4 qp = xq[p];
@@ -1447,11 +1456,7 @@ __device__ __forceinline__ double warp_sum(double v) {
 // a cell of which the walks start, and whose fixed point the float test measures from (the
 // separations themselves wrap once more).  Without walls a source may lie outside.  One that is not
 // finite ends the call (F_BADPOS) and is searched from 0 until then.
-struct SrcBox {
-    double box[3];
-    int periodic;
-};
-__global__ void k_src_positions(const double* __restrict__ x, int64_t S, SrcBox b, double* __restrict__ out, int* flags) {
+__global__ void k_src_positions(const double* __restrict__ x, int64_t S, Box b, double* __restrict__ out, int* flags) {
     const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t >= 3 * S) return;
     const double L = b.box[t / S];
@@ -2116,7 +2121,8 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         qmul[a] = units / cfg.box[a];
         qscale[a] = (float)(cfg.box[a] / units);
     }
-    k_gather_positions<<<nblk(n, B), B, 0, st>>>(x, m, c->perm.as<int32_t>(), n, qmul[0], qmul[1], qmul[2],
+    const Box box = {{cfg.box[0], cfg.box[1], cfg.box[2]}, cfg.periodic};
+    k_gather_positions<<<nblk(n, B), B, 0, st>>>(x, m, c->perm.as<int32_t>(), n, box, qmul[0], qmul[1], qmul[2],
                                                   c->xs_d.as<double>(), c->xq.as<uint4>(), c->m_s.as<double>(),
                                                   c->inv_perm.as<int32_t>());
     RT_CUDA(c, cudaGetLastError());
@@ -2191,7 +2197,7 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
     k_own_rows<<<nblk(n * 32, 256), 256, 0, st>>>(g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n,
                                                    pp, c->lists.as<int32_t>(), cap, c->list_cnt.as<int32_t>(),
                                                    c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(),
-                                                   c->extras.as<int32_t>(), over, flags);
+                                                   c->extras.as<int32_t>(), over, over_n);
     k_own_walk<false><<<(unsigned)c->sm_count * 4, 128, 0, st>>>(
         g, c->xs_d.as<double>(), c->xq.as<uint4>(), c->h_d.as<double>(), n, pp, c->lists.as<int32_t>(), cap,
         c->own_cnt.as<int32_t>(), c->extra_cnt.as<int32_t>(), c->extras.as<int32_t>(), over, over_n, spill_n, nullptr);
@@ -2310,8 +2316,7 @@ rt_status build_neighbours(rt_ctx* c, const double* x, const double* m, const do
         RT_TRY(ensure(c, c->omegas_d, S * 8 + 64 * S, "sources"));
         RT_TRY(ensure(c, c->src_counts, (S + 1) * 4, "sources"));
         RT_TRY(ensure(c, c->src_off, (S + 1) * 8, "sources"));
-        const SrcBox sbox = {{cfg.box[0], cfg.box[1], cfg.box[2]}, cfg.periodic};
-        k_src_positions<<<nblk(3 * S, 128), 128, 0, st>>>(xsrc, S, sbox, c->xsrc_d.as<double>(), flags);
+        k_src_positions<<<nblk(3 * S, 128), 128, 0, st>>>(xsrc, S, box, c->xsrc_d.as<double>(), flags);
         SrcParams sp;
         sp.eta3 = cfg.eta_res_star * cfg.eta_res_star * cfg.eta_res_star;
         sp.s_star = kKappa * kKappa * kKappa / kSigma * sp.eta3;
