@@ -164,7 +164,11 @@ typedef struct {
      *                   0 = the variant's default (64 for variant 2, 256 for variant 1).
      *   gather_block    threads per block of gather_variant 1: a multiple of 32 from 64 to 512;
      *                   0 = 256.
-     *   pair_warps      warps per block of flux_variant 2: 1, 2 or 4; 0 = 1. */
+     *   pair_warps      warps per block of flux_variant 2: 1, 2 or 4; 0 = 1.
+     * With gradient_variant 2, sets of fewer than 256 (particle, group)s per SM (groups of one
+     * launch) run a gradient and a gather of their own block size, and with flux_variant 2 the HLL
+     * pair pass of sets that fill the GPU runs one block per SM: the block sizes above do not
+     * apply there. */
     int32_t cell_eighths;
     int32_t gradient_block;
     int32_t gather_block;

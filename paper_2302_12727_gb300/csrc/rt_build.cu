@@ -831,8 +831,9 @@ __device__ __forceinline__ void reduce_refined(double mn, double mx, double h3, 
 // each, whose repeated scalar parts the double pipe bears; on small sets, where the flagged ones
 // are a handful and each a chain of latencies, 32.  The
 // distances are dealt to the lanes and kept in registers, SLOTS a lane.  A particle without a
-// list, with more neighbours than slots or with an iterate beyond the list goes to `rest`.  The
-// smallest and largest h are widened to the refined values.
+// list, with more neighbours than slots (eta above about 1.55: nearly all; a search of 110,592
+// particles at 1.6 in double takes 6.4 ms, 15.6 with a thread each) or with an iterate beyond the
+// list goes to `rest`.  The smallest and largest h are widened to the refined values.
 template <int LN, int SLOTS>
 __global__ void __launch_bounds__(128)
 k_h_refine(Grid g, const double* __restrict__ xs, const uint4* __restrict__ xq, int64_t n, HParams hp,
