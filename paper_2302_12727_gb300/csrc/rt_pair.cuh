@@ -83,8 +83,8 @@ __device__ __forceinline__ float rsqrt_(float x) {
 // instructions of the double pipe instead of the eight to twenty of the IEEE routines.  The
 // double path's time is that pipe's, which runs at 1/64 of the float rate.  From approximations
 // good to 2^-20 their errors are at most 0.51 ulp (1/x), 0.75 (sqrt) and 0.95 (1/sqrt), in exact
-// arithmetic; against the equations in 64 bits 16 sub-cycles of 32,768 particles are off by 4.4e-16, 4.3e-16
-// with IEEE routines (mean of four sets).
+// arithmetic; 16 sub-cycles of 32,768 particles are 4.4e-16 off the equations in 64 bits with them and
+// with the IEEE routines alike (mean of four sets).
 __device__ __forceinline__ double rcp_fast(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));

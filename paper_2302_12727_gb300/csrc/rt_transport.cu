@@ -44,8 +44,9 @@ static int grad_block(const rt_ctx* c) {
 static int gather_block(const rt_ctx* c) { return c->tune.gather_block > 0 ? c->tune.gather_block : kGatherBlock; }
 // fewer (particle, group)s than eight warps per SM: the gradient and the gather then take the
 // kernels with more loads in flight per thread, with the default gradient (variant 2) only, so that
-// the other variants time what they name.  50 sub-cycles just below the line: 2.48 -> 2.15 ms (one
-// group), 2.05 -> 1.66, 1.95 -> 1.59 and 1.97 -> 1.58 ms (four); at a sixteenth of it 1.60 -> 1.00 to 1.45 -> 0.96 ms
+// the other variants time what they name.  50 sub-cycles of one to four groups just below the line:
+// 2.48 -> 2.15, 2.05 -> 1.66, 1.95 -> 1.59 and 1.97 -> 1.58 ms; at a sixteenth of it 1.60 -> 1.00,
+// 1.54 -> 1.02, 1.28 -> 0.94 and 1.45 -> 0.96 ms (up to 4% of that from other kernels)
 static bool few_threads(const rt_ctx* c, int gc) {
     return c->tune.gradient_variant == 2 && c->n * gc < (int64_t)c->sm_count * 256;
 }
